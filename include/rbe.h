@@ -54,7 +54,9 @@ typedef enum {
 } rbe_status;
 
 typedef enum {
-    RBE_FP64 = 0,        /* phases, sincos and accumulation in FP64 */
+    RBE_FP64 = 0,        /* FP64 accuracy: the phase m.s mod 1 exact in 64-bit fixed point, its sine and
+                            cosine to about 2^-53, sums over particles and frequencies in 64- and
+                            128-bit integers, per-frequency and per-particle results in FP64 */
     RBE_FP32_PHASE = 1   /* exact 32-bit fixed-point phase m.s mod 1, FP32 sine and cosine (rho pass)
                             and one FP32 sine of the phase shifted by arg rho (force pass),
                             float-float sums across tiles */

@@ -132,8 +132,8 @@ static void free_npt(NptBuffers& b)
 static void free_buffers(DeviceBuffers& d)
 {
     cudaFree(d.cum); cudaFree(d.ks); cudaFree(d.m); cudaFree(d.w); cudaFree(d.rho); cudaFree(d.terms);
-    cudaFree(d.coef_m); cudaFree(d.coef_f); cudaFree(d.coef_d); cudaFree(d.partials); cudaFree(d.counter);
-    cudaFree(d.status); cudaFree(d.pos); cudaFree(d.q); cudaFree(d.F); cudaFree(d.WE);
+    cudaFree(d.coef_m); cudaFree(d.coef_f); cudaFree(d.coef_d); cudaFree(d.partials);
+    cudaFree(d.status); cudaFree(d.pos); cudaFree(d.q); cudaFree(d.F); cudaFree(d.WE); cudaFree(d.trig);
     d = DeviceBuffers{};
 }
 
@@ -165,9 +165,9 @@ rbe_status rbe_create(const double box[3], double alpha, int32_t P, uint64_t see
     ctx->seed = seed;
     DeviceBuffers& d = ctx->d;
     if ((err = cudaMalloc(&d.ks, sizeof(KState))) != cudaSuccess ||
-        (err = cudaMalloc(&d.counter, sizeof(unsigned))) != cudaSuccess ||
         (err = cudaMalloc(&d.status, sizeof(unsigned))) != cudaSuccess ||
-        (err = cudaMemset(d.counter, 0, sizeof(unsigned))) != cudaSuccess ||
+        (err = cudaMalloc(&d.trig, trig_table_bytes())) != cudaSuccess ||
+        (err = launch_trig_table(d.trig, nullptr)) != cudaSuccess ||
         (err = cudaMemset(d.status, 0, sizeof(unsigned))) != cudaSuccess) {
         std::string msg = std::string("device allocation failed: ") + cudaGetErrorString(err);
         free_buffers(d);

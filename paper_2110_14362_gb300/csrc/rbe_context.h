@@ -30,7 +30,8 @@ struct KState {
     double H[3];        // per-axis sums (Eq. (psf))
     double S;           // H_x H_y H_z - 1 (Eq. (S))
     double wP;          // S / P
-    FixScaleH sc[3];    // 1/l as a 64-bit mantissa and a power of two (FP32-phase path)
+    FixScaleH sc[3];    // the double 1/l as a 64-bit mantissa and a power of two (FP32-phase path)
+    FixScaleH sc64[3];  // 1/l itself, rounded to 64 bits (FP64 path)
     float cx, cy, cz;   // 2 pi / l
     int P;
     double ce;          // 2 pi / V
@@ -103,11 +104,11 @@ struct DeviceBuffers {
     double* terms = nullptr;          // [kcap + 1][8] per-frequency energy/virial terms
     int4* coef_m = nullptr;           // [kcap] FP32 force data (mx, my, mz, bits of A)
     float4* coef_f = nullptr;         // [kcap] FP32 force data (B, mx, my, mz)
-    double2* coef_d = nullptr;        // [kcap] FP64 force data (A, B)
+    double2* coef_d = nullptr;        // [kcap] FP64 path: (bits of the phase offset of arg rho, amplitude R)
+    void* trig = nullptr;             // [kTrigLen] TrigEntry (rbe_fix64.cuh), written by rbe_create
     int kcap = 0;
-    void* partials = nullptr;         // [(K + 1) * nchunks] double2 (FP64) or float4 (FP32-phase)
+    void* partials = nullptr;         // [(K + 1) * nchunks] double2 (FP64 path) or float4 (FP32-phase)
     size_t part_cap = 0;              // in 16-byte entries
-    unsigned* counter = nullptr;      // last-block counter of the reduction
     unsigned* status = nullptr;       // latched device status bits
     double* pos = nullptr;            // host-API staging
     double* q = nullptr;
@@ -195,6 +196,8 @@ rbe_status ensure_tables(rbe_ctx ctx);
 rbe_status ensure_table_capacity(rbe_ctx ctx, int need);
 rbe_status launch_tables(rbe_ctx ctx, const double* box_dev);
 rbe_status ensure_k_capacity(rbe_ctx ctx, int K);
+cudaError_t launch_trig_table(void* trig, cudaStream_t s);
+size_t trig_table_bytes();
 rbe_status launch_sample(rbe_ctx ctx, uint64_t step, int P);
 rbe_status launch_sample_device_box(rbe_ctx ctx, uint64_t step, int P, const unsigned long long* step_dev);
 rbe_status launch_tables_sample_device(rbe_ctx ctx, int P, const double* box_dev, const unsigned long long* step_dev);

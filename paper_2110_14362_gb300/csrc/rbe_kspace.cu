@@ -1,5 +1,6 @@
 // RBE k-space kernels for sm_103a and their launchers (the FP32-phase bodies live in
-// rbe_kspace_tiles.cuh, shared with the batched kernels of rbe_batch.cu).
+// rbe_kspace_tiles.cuh, shared with the batched kernels of rbe_batch.cu; the FP64 path's pair
+// passes in rbe_kspace64.cuh).
 //
 // One evaluation (Sec. 4.2 of the paper) is up to five launches on the context's stream:
 //   k_tables   per-axis weights exp(-c m^2) as exact integers, their cumulative sums, H,
@@ -8,9 +9,9 @@
 //   k_sample   one thread per frequency: Philox -> 3 uniforms -> inverse CDF  Eq. (probexpression)
 //   k_rho_*    particle-chunk x frequency-tile blocks: partial rho(k_l) per chunk
 //   k_reduce*  fixed-order sum of the partials -> rho(k_l), the per-frequency terms and
-//              force coefficients (and, on the FP64 path, the energy and virial)
+//              force coefficients
 //                                              Eq. (apppress); App. C Eq. (pressuretensorflexible)
-//   k_force_*  particle tiles x all frequencies: F_i                             Eq. (appforce)
+//   k_force_*  particle tiles x all frequencies: F_i; one more block: energy, virial  Eq. (appforce)
 // No floating-point atomics: every sum runs in an order fixed by (N, K, plan), so
 // results are bitwise reproducible run to run.  The host-buffer call can run the passes in
 // two particle groups with its copies pipelined (launch_evaluate_staged).
@@ -23,6 +24,7 @@
 
 #include "rbe_context.h"
 #include "rbe_device.cuh"
+#include "rbe_kspace64.cuh"
 #include "rbe_kspace_tiles.cuh"
 #include "rbe_sampler_variants.cuh"
 
@@ -55,9 +57,6 @@ constexpr int kRhoWideMaxSub = 8;  // particle sub-streams of a wide two-frequen
 #endif
 constexpr int kRhoMinChunk = RBE_RHO_MINCHUNK;
 constexpr double kRhoLatencyPairs = RBE_RHO_LATENCY_PAIRS;
-
-constexpr int kT = 128;               // threads per block of the FP64 force pass
-constexpr int kForceKT = 256;         // frequencies staged per tile in the FP64 force pass
 
 __global__ void __launch_bounds__(kTableThreads)
 k_tables(double bx, double by, double bz, const double* __restrict__ box_dev, double alpha, int P,
@@ -135,24 +134,6 @@ __global__ void k_weights_from_list(int K, const int32_t* __restrict__ m3, const
     w_out[l] = w[l];
 }
 
-// Fixed-order block sum of one double per thread (warp shuffles, then warp 0); the
-// result is valid in thread 0.  blockDim.x is a multiple of 32, at most 1024.
-__device__ __forceinline__ double block_sum(double v, double* scratch32)
-{
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    __syncthreads();
-    if (lane == 0) scratch32[warp] = v;
-    __syncthreads();
-    if (warp == 0) {
-        v = lane < (int)(blockDim.x >> 5) ? scratch32[lane] : 0.0;
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-    }
-    return v;
-}
-
 // Block (kt, c) handles frequency tile kt and particle chunk c_off + c (c_off: the first chunk
 // of a piece when the staged host call feeds the pass piece by piece).
 // F frequencies per thread: blocks of at most kMaxRhoThreads threads for F = 1, kRhoThreadsF
@@ -226,153 +207,6 @@ static RhoWideKernel rho_wide_kernel(int accum, bool xyzq = false)
 }
 
 
-// rho pass, FP64 path: s = r / l wrapped to [0, 1); t = m.s - rint(m.s); sincospi(2t).
-__global__ void __launch_bounds__(kMaxRhoThreads)
-k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t N, const KState* __restrict__ ks,
-          const int4* __restrict__ m, int K, int64_t chunk_len, int nchunks, double2* __restrict__ partials,
-          unsigned* __restrict__ status)
-{
-    __shared__ double4_32a sp[kMaxRhoThreads];
-    __shared__ double red[32];
-    const int tid = threadIdx.x, nt = blockDim.x;
-    const int l = blockIdx.x * nt + tid;
-    const int c = blockIdx.y;
-    const double ilx = ks->inv[0], ily = ks->inv[1], ilz = ks->inv[2];
-    const int4 mv = l < K ? m[l] : make_int4(0, 0, 0, 0);
-    const double mx = mv.x, my = mv.y, mz = mv.z;
-    double re = 0.0, im = 0.0, q2 = 0.0;
-    const int64_t start = (int64_t)c * chunk_len;
-    const int64_t end = min(N, start + chunk_len);
-    for (int64_t base = start; base < end; base += nt) {
-        const int64_t i = base + tid;
-        double4_32a rec = make_double4_32a(0.0, 0.0, 0.0, 0.0);
-        if (i < end) {
-            double sx = pos[3 * i] * ilx, sy = pos[3 * i + 1] * ily, sz = pos[3 * i + 2] * ilz;
-            sx -= floor(sx); sy -= floor(sy); sz -= floor(sz);
-            const double qi = q[i];
-            if (!isfinite(sx + sy + sz + qi)) atomicOr(status, kStatusNonFinite);
-            q2 += qi * qi;
-            rec = make_double4_32a(sx, sy, sz, qi);
-        }
-        sp[tid] = rec;
-        __syncthreads();
-        const int n_here = (int)min((int64_t)nt, end - base);
-#pragma unroll 2
-        for (int p = 0; p < n_here; ++p) {
-            const double4_32a r = sp[p];
-            double t = fma(mx, r.x, fma(my, r.y, mz * r.z));
-            t -= rint(t);
-            double sn, cs;
-            sincospi(2.0 * t, &sn, &cs);
-            re = fma(r.w, cs, re);
-            im = fma(r.w, sn, im);
-        }
-        __syncthreads();
-    }
-    if (l < K) partials[(size_t)l * nchunks + c] = make_double2(re, im);
-    if (blockIdx.x == 0) {
-        const double s = block_sum(q2, red);
-        if (tid == 0) partials[(size_t)K * nchunks + c] = make_double2(s, 0.0);
-    }
-}
-
-// =================================================================================
-// FP64 reduction: block l (of K + 1) sums its row over the chunks in a fixed order and
-// forms the per-frequency terms; the last block to finish sums those over l.
-//   e_l = (2 pi / V) w_l |rho_l|^2 / |k_l|^2
-//   W  += e_l [I - 2 (1/|k_l|^2 + 1/4a) k_l k_l]
-//   beta_l = w_l 4 pi / (V |k_l|^2), A_l = beta_l Im rho_l, B_l = beta_l Re rho_l, so that
-//   F_i = q_i sum_l k_l (sin(k_l.r_i) B_l - cos(k_l.r_i) A_l).
-__global__ void __launch_bounds__(kReduceThreads)
-k_reduce(const double2* __restrict__ partials, int nchunks, int K, const int4* __restrict__ m,
-         const double* __restrict__ w, const KState* __restrict__ ks, double2* __restrict__ rho,
-         double* __restrict__ terms, double2* __restrict__ coef_d, unsigned* __restrict__ counter,
-         unsigned* __restrict__ status, double* __restrict__ W_out, double* __restrict__ E_out)
-{
-    __shared__ double red[32];
-    __shared__ double fin[kReduceThreads / 32][7];
-    __shared__ bool is_last;
-    const int l = blockIdx.x;
-    double re = 0.0, im = 0.0;
-    const double2* row = partials + (size_t)l * nchunks;
-    for (int j = threadIdx.x; j < nchunks; j += kReduceThreads) {
-        const double2 v = row[j];
-        re += v.x;
-        im += v.y;
-    }
-    re = block_sum(re, red);
-    im = block_sum(im, red);
-    const double alpha = ks->alpha;
-    if (threadIdx.x == 0) {
-        double* t = terms + (size_t)l * 8;
-        if (l < K) {
-            const int4 mi = m[l];
-            const double bx = ks->L[0], by = ks->L[1], bz = ks->L[2];
-            const double V = bx * by * bz;
-            const double kx = 2.0 * kPi * mi.x / bx, ky = 2.0 * kPi * mi.y / by, kz = 2.0 * kPi * mi.z / bz;
-            const double kk = kx * kx + ky * ky + kz * kz;
-            const double rho2 = re * re + im * im;
-            const double e = (2.0 * kPi / V) * w[l] * rho2 / kk;
-            const double b = 2.0 * (1.0 / kk + 1.0 / (4.0 * alpha));
-            t[0] = e;
-            t[1] = e * (1.0 - b * kx * kx);
-            t[2] = e * (1.0 - b * ky * ky);
-            t[3] = e * (1.0 - b * kz * kz);
-            t[4] = -e * b * kx * ky;
-            t[5] = -e * b * kx * kz;
-            t[6] = -e * b * ky * kz;
-            t[7] = 0.0;
-            const double beta = w[l] * (4.0 * kPi / (V * kk));
-            rho[l] = make_double2(re, im);
-            coef_d[l] = make_double2(beta * im, beta * re);
-            if (!isfinite(re) || !isfinite(im)) atomicOr(status, kStatusNonFinite);
-        } else {
-            t[0] = re;  // sum of q^2
-        }
-        __threadfence();
-        is_last = (atomicAdd(counter, 1u) == gridDim.x - 1);
-    }
-    __syncthreads();
-    if (!is_last) return;
-    __threadfence();
-    double acc[7] = {0, 0, 0, 0, 0, 0, 0};
-    for (int j = threadIdx.x; j < K; j += kReduceThreads) {
-        const double* t = terms + (size_t)j * 8;
-#pragma unroll
-        for (int a = 0; a < 7; ++a) acc[a] += __ldcg(t + a);
-    }
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int a = 0; a < 7; ++a) {
-        double v = acc[a];
-#pragma unroll
-        for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-        if (lane == 0) fin[warp][a] = v;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double tot[7];
-        for (int a = 0; a < 7; ++a) {
-            tot[a] = 0.0;
-            for (int wv = 0; wv < kReduceThreads / 32; ++wv) tot[a] += fin[wv][a];
-        }
-        const double q2 = __ldcg(terms + (size_t)K * 8);
-        const double Ek = tot[0];
-        const double Es = -sqrt(alpha / kPi) * q2;
-        if (W_out) {
-            W_out[0] = tot[1]; W_out[4] = tot[2]; W_out[8] = tot[3];
-            W_out[1] = W_out[3] = tot[4];
-            W_out[2] = W_out[6] = tot[5];
-            W_out[5] = W_out[7] = tot[6];
-        }
-        if (E_out) { E_out[0] = Ek; E_out[1] = Es; }
-        bool ok = isfinite(Ek) && isfinite(Es);
-        for (int a = 1; a < 7; ++a) ok = ok && isfinite(tot[a]);
-        if (!ok) atomicOr(status, kStatusNonFinite);
-        *counter = 0u;  // ready for the next launch
-    }
-}
-
 __global__ void __launch_bounds__(kReduceThreads)
 k_reduce_f32(const float4* __restrict__ partials, int nchunks, int K, const int4* __restrict__ m,
              const double* __restrict__ w, const KState* __restrict__ ks, double2* __restrict__ rho,
@@ -399,84 +233,6 @@ k_force_f32(const void* __restrict__ pos, const double* __restrict__ q, int64_t 
         return;
     }
     force_f32_block<XYZQ>(b_off + (int64_t)blockIdx.x, pos, q, N, per_block, ks, coef_m, coef_f, K, F, status);
-}
-
-// Force pass, FP64 path: particle tiles of kT * PPT, frequencies staged kForceKT at a time.
-template <int PPT>
-__global__ void __launch_bounds__(kT) k_force_f64(const double* __restrict__ pos, const double* __restrict__ q,
-                                                  int64_t N, int64_t per_block, const KState* __restrict__ ks,
-                                                  const int4* __restrict__ mk, const double2* __restrict__ coef_d,
-                                                  int K, double* __restrict__ F)
-{
-    __shared__ double4_32a sk[kForceKT];  // (mx, my, mz, A)
-    __shared__ double sb[kForceKT];       // B
-    const int tid = threadIdx.x;
-    const double ilx = ks->inv[0], ily = ks->inv[1], ilz = ks->inv[2];
-    const bool one_tile = K <= kForceKT;
-    if (one_tile) {
-        for (int j = tid; j < K; j += kT) {
-            const int4 mm = mk[j];
-            const double2 ab = coef_d[j];
-            sk[j] = make_double4_32a((double)mm.x, (double)mm.y, (double)mm.z, ab.x);
-            sb[j] = ab.y;
-        }
-        __syncthreads();
-    }
-    const int64_t b0 = (int64_t)blockIdx.x * per_block;
-    const int64_t b1 = min(N, b0 + per_block);
-    const double cx = 2.0 * kPi * ilx, cy = 2.0 * kPi * ily, cz = 2.0 * kPi * ilz;
-    for (int64_t base = b0; base < b1; base += (int64_t)kT * PPT) {
-        double sx[PPT], sy[PPT], sz[PPT], fx[PPT], fy[PPT], fz[PPT];
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            const int64_t i = base + (int64_t)p * kT + tid;
-            if (i < b1) {
-                sx[p] = pos[3 * i] * ilx; sy[p] = pos[3 * i + 1] * ily; sz[p] = pos[3 * i + 2] * ilz;
-                sx[p] -= floor(sx[p]); sy[p] -= floor(sy[p]); sz[p] -= floor(sz[p]);
-            } else {
-                sx[p] = sy[p] = sz[p] = 0.0;
-            }
-            fx[p] = fy[p] = fz[p] = 0.0;
-        }
-        for (int k0 = 0; k0 < K; k0 += kForceKT) {
-            const int nk = min(kForceKT, K - k0);
-            if (!one_tile) {
-                __syncthreads();
-                for (int j = tid; j < nk; j += kT) {
-                    const int4 mm = mk[k0 + j];
-                    const double2 ab = coef_d[k0 + j];
-                    sk[j] = make_double4_32a((double)mm.x, (double)mm.y, (double)mm.z, ab.x);
-                    sb[j] = ab.y;
-                }
-                __syncthreads();
-            }
-            for (int l = 0; l < nk; ++l) {
-                const double4_32a a = sk[l];
-                const double B = sb[l];
-#pragma unroll
-                for (int p = 0; p < PPT; ++p) {
-                    double t = fma(a.x, sx[p], fma(a.y, sy[p], a.z * sz[p]));
-                    t -= rint(t);
-                    double sn, cs;
-                    sincospi(2.0 * t, &sn, &cs);
-                    const double g = sn * B - cs * a.w;
-                    fx[p] = fma(g, a.x, fx[p]);
-                    fy[p] = fma(g, a.y, fy[p]);
-                    fz[p] = fma(g, a.z, fz[p]);
-                }
-            }
-        }
-#pragma unroll
-        for (int p = 0; p < PPT; ++p) {
-            const int64_t i = base + (int64_t)p * kT + tid;
-            if (i < b1) {
-                const double qi = q[i];
-                F[3 * i] = qi * cx * fx[p];
-                F[3 * i + 1] = qi * cy * fy[p];
-                F[3 * i + 2] = qi * cz * fz[p];
-            }
-        }
-    }
 }
 
 // =================================================================================
@@ -763,7 +519,6 @@ static cudaError_t launch_reduce_f32(cudaStream_t s, const float4* part32, int n
 struct EvalShape {
     Plan p;
     size_t force_smem;
-    bool fp64;
 };
 
 // Frequency tiling of the FP32-phase rho pass: kf frequencies per thread (1, 2 or 4) and
@@ -826,60 +581,134 @@ static RhoShape rho_shape(int64_t N, int K, int accum)
     return best;
 }
 
-static rbe_status evaluate_shape(rbe_ctx ctx, int64_t N, int K, EvalShape* out)
+// FP64 path: frequency tiles of at most kRho64Threads lanes, split evenly, with as many particle
+// sub-streams as fit the block; particle chunks for one wave of resident blocks, of at least two
+// particles per sub-stream.  Force pass: rounds of kForce64Threads / slices particles, the slices
+// (1, 2, 4 or 8 of the frequencies) chosen for the shortest wave.
+static Plan make_plan64(rbe_ctx ctx, int64_t N, int K)
+{
+    Plan p{};
+    p.kf = 1;
+    p.ktiles = (K + kRho64Threads - 1) / kRho64Threads;
+    p.klanes = (K + p.ktiles - 1) / p.ktiles;
+    p.ksub = std::min(32, kRho64Threads / p.klanes);
+    p.kthreads = 32 * ((p.ksub * p.klanes + 31) / 32);
+    const int smem_bps = (int)((227 * 1024) / (kRho64Smem + 2048));
+    const int bps = std::max(1, std::min(smem_bps, 2 * kRho64Threads / p.kthreads));
+    const int64_t want = std::max<int64_t>(1, (int64_t)ctx->num_sms * bps / p.ktiles);
+    const int64_t least = 2 * p.ksub;
+    p.nchunks = (int)std::min<int64_t>(want, std::max<int64_t>(1, (N + least - 1) / least));
+    p.chunk_len = std::max<int64_t>(1, (N + p.nchunks - 1) / p.nchunks);
+    p.nchunks = (int)std::max<int64_t>(1, (N + p.chunk_len - 1) / p.chunk_len);
+    const int64_t resident = (int64_t)ctx->num_sms * 4;
+    double best = 1e300;
+    for (int sl : {1, 2, 4, 8}) {
+        const int64_t unit = kForce64Threads / sl, rounds = (N + unit - 1) / unit;
+        const int64_t per = (rounds + resident - 1) / resident;
+        const double cost = (double)per * ((K + sl - 1) / sl + 8.0);
+        if (cost < best - 1e-9) {
+            best = cost;
+            p.ppt = sl;  // frequency slices
+            p.per_block = per * unit;
+            p.fblocks = per > 0 ? (int)((rounds + per - 1) / per) : 0;
+        }
+    }
+    return p;
+}
+
+static rbe_status ensure_partials(rbe_ctx ctx, size_t need)
 {
     DeviceBuffers& d = ctx->d;
-    const bool fp64 = ctx->precision == RBE_FP64;
-    static int rho64_threads = 0, bps_f64 = 0;
+    if (need <= d.part_cap) return RBE_OK;
+    ctx_free(ctx, d.partials);
+    d.partials = nullptr;
+    d.part_cap = 0;
+    const cudaError_t err = ctx_alloc(ctx, &d.partials, 16 * need);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "cudaMalloc(partials)");
+    d.part_cap = need;
+    return RBE_OK;
+}
+
+cudaError_t launch_trig_table(void* trig, cudaStream_t s)
+{
+    k_trig_table<<<(kTrigLen + 127) / 128, 128, 0, s>>>(static_cast<TrigEntry*>(trig));
+    return cudaGetLastError();
+}
+
+size_t trig_table_bytes() { return kTrigBytes; }
+
+// launch_evaluate_range on the FP64 path.
+static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* pos, const double* q, int koff, int K,
+                                          bool forces, double* F, double* W, double* E)
+{
+    DeviceBuffers& d = ctx->d;
+    static const cudaError_t attr = [] {
+        cudaError_t e = cudaFuncSetAttribute(k_rho_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRho64Smem);
+        for (auto k : {k_force_f64<1>, k_force_f64<2>, k_force_f64<4>, k_force_f64<8>})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kForce64Smem);
+        return e;
+    }();
+    if (attr != cudaSuccess) return cuda_fail(ctx, attr, "shared memory of the FP64 passes");
+    const Plan p = make_plan64(ctx, N, K);
+    rbe_status st = ensure_partials(ctx, (size_t)(K + 1) * p.nchunks);
+    if (st != RBE_OK) return st;
+    cudaStream_t s = ctx->stream;
+    const int4* m = d.m + koff;
+    const double* w = d.w + koff;
+    const KState* ks = d.ks;
+    double2* part = static_cast<double2*>(d.partials);
+    const TrigEntry* trig = static_cast<const TrigEntry*>(d.trig);
+    cudaError_t err = launch_pdl(k_rho_f64, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem, s, pos, q, N, ks, m,
+                                 K, p.chunk_len, p.nchunks, part, trig, d.status, p.ksub, p.klanes);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f64");
+    record_event(ctx, 2);
+    int threads = 32;
+    while (threads < kReduceThreads && threads * 4 < p.nchunks) threads *= 2;
+    err = launch_pdl(k_reduce_f64, dim3(K + 1), dim3(threads), 0, s, (const double2*)part, p.nchunks, K, m, w, ks, trig,
+                     d.rho, d.terms, d.coef_d, d.status);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_reduce_f64");
+    record_event(ctx, 3);
+    auto force = p.ppt == 8 ? k_force_f64<8> : (p.ppt == 4 ? k_force_f64<4> : (p.ppt == 2 ? k_force_f64<2> : k_force_f64<1>));
+    err = launch_pdl(force, dim3((forces ? p.fblocks : 0) + 1), dim3(kForce64Threads), kForce64Smem, s, pos, q, N,
+                     p.per_block, ks, m, (const double2*)d.coef_d, K, F, trig, d.status, (const double*)d.terms, W, E);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_force_f64");
+    record_event(ctx, 4);
+    ctx->last_K = K;
+    return check_launch(ctx, "FP64 passes");
+}
+
+static rbe_status evaluate_shape(rbe_ctx ctx, int64_t N, int K, EvalShape* out)
+{
+    static bool force_attr = false;
     static int rho32_bps[3][4] = {{0}};  // [accum][F index, 3: wide] resident threads per SM
-    if (!rho64_threads) {
-        rho64_threads = blocks_per_sm(k_rho_f64, kMaxRhoThreads) * kMaxRhoThreads;
-        bps_f64 = blocks_per_sm(k_force_f64<2>, kT);
+    if (!force_attr) {
         cudaFuncSetAttribute(k_force_f32<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kForceSmemPerK * kForceStageK));
         cudaFuncSetAttribute(k_force_f32<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)(kForceSmemPerK * kForceStageK));
+        force_attr = true;
     }
     const int kstage = std::min(K, kForceStageK);
-    const size_t force_smem = fp64 ? 0 : (size_t)kForceSmemPerK * kstage;
+    const size_t force_smem = (size_t)kForceSmemPerK * kstage;
     static int cached_kstage = -1, cached_bps_force = 1;
-    if (!fp64 && kstage != cached_kstage) {
+    if (kstage != cached_kstage) {
         cached_bps_force = blocks_per_sm(k_force_f32<false>, kForceThreads, force_smem);
         cached_kstage = kstage;
     }
-    const int bps_force = fp64 ? bps_f64 : cached_bps_force;
-    RhoShape rs;
-    int rho_bps;
-    if (fp64) {
-        rs.kf = 1;
-        rs.ktiles = (K + kMaxRhoThreads - 1) / kMaxRhoThreads;
-        rs.kthreads = std::min(kMaxRhoThreads, 32 * (((K + rs.ktiles - 1) / rs.ktiles + 31) / 32));
-        rs.ksub = 1;
-        rs.klanes = 0;
-        rho_bps = std::max(1, std::min(32, rho64_threads / rs.kthreads));
-    } else {
-        rs = rho_shape(N, K, ctx->rho_accum);
-        const int a = ctx->rho_accum < 0 || ctx->rho_accum > 2 ? 1 : ctx->rho_accum;
-        const bool wide = rs.klanes > 0;
-        const int fi = wide ? 3 : (rs.kf == 4 ? 2 : (rs.kf == 2 ? 1 : 0));
-        int& bps = rho32_bps[a][fi];
-        if (!bps) {
-            const int tmax = rs.kf == 1 || wide ? kMaxRhoThreads : kRhoThreadsF;
-            bps = std::max(1, (wide ? blocks_per_sm(rho_wide_kernel(a), tmax) : blocks_per_sm(rho_kernel(a, rs.kf), tmax)) *
-                                  tmax);  // resident threads per SM
-        }
-        rho_bps = std::max(1, std::min(32, bps / rs.kthreads));
+    const RhoShape rs = rho_shape(N, K, ctx->rho_accum);
+    const int a = ctx->rho_accum < 0 || ctx->rho_accum > 2 ? 1 : ctx->rho_accum;
+    const bool wide = rs.klanes > 0;
+    const int fi = wide ? 3 : (rs.kf == 4 ? 2 : (rs.kf == 2 ? 1 : 0));
+    int& bps = rho32_bps[a][fi];
+    if (!bps) {
+        const int tmax = rs.kf == 1 || wide ? kMaxRhoThreads : kRhoThreadsF;
+        bps = std::max(1, (wide ? blocks_per_sm(rho_wide_kernel(a), tmax) : blocks_per_sm(rho_kernel(a, rs.kf), tmax)) *
+                              tmax);  // resident threads per SM
     }
-    const Plan p = make_plan(ctx, N, K, rs, rho_bps, bps_force,
-                             fp64 ? kT * 2 : kForceRound, fp64 ? 1 : RBE_FORCE_MIN_ROUNDS);
-    const size_t need = (size_t)(K + 1) * p.nchunks;
-    if (need > d.part_cap) {
-        ctx_free(ctx, d.partials);
-        d.partials = nullptr;
-        d.part_cap = 0;
-        cudaError_t err = ctx_alloc(ctx, &d.partials, 16 * need);
-        if (err != cudaSuccess) return cuda_fail(ctx, err, "cudaMalloc(partials)");
-        d.part_cap = need;
-    }
-    *out = EvalShape{p, force_smem, fp64};
+    const int rho_bps = std::max(1, std::min(32, bps / rs.kthreads));
+    const Plan p = make_plan(ctx, N, K, rs, rho_bps, cached_bps_force, kForceRound, RBE_FORCE_MIN_ROUNDS);
+    rbe_status st = ensure_partials(ctx, (size_t)(K + 1) * p.nchunks);
+    if (st != RBE_OK) return st;
+    *out = EvalShape{p, force_smem};
     return RBE_OK;
 }
 
@@ -889,56 +718,32 @@ static rbe_status evaluate_shape(rbe_ctx ctx, int64_t N, int K, EvalShape* out)
 static rbe_status launch_evaluate_range(rbe_ctx ctx, int64_t N, const void* pos, const double* q, int koff, int K,
                                         bool forces, double* F, double* W, double* E, bool xyzq)
 {
+    if (ctx->precision == RBE_FP64)
+        return launch_evaluate_range64(ctx, N, static_cast<const double*>(pos), q, koff, K, forces, F, W, E);
     DeviceBuffers& d = ctx->d;
     const int4* m_in = d.m + koff;
     const double* w_in = d.w + koff;
     EvalShape sh;
-    rbe_status st0 = evaluate_shape(ctx, N, K, &sh);
-    if (st0 != RBE_OK) return st0;
+    rbe_status st = evaluate_shape(ctx, N, K, &sh);
+    if (st != RBE_OK) return st;
     const Plan& p = sh.p;
-    const bool fp64 = sh.fp64;
-    const size_t force_smem = sh.force_smem;
-    const dim3 grid(p.ktiles, p.nchunks);
     cudaStream_t s = ctx->stream;
-    double2* part64 = static_cast<double2*>(d.partials);
     float4* part32 = static_cast<float4*>(d.partials);
     const KState* ks = d.ks;
-    if (fp64) {
-        k_rho_f64<<<grid, p.kthreads, 0, s>>>(static_cast<const double*>(pos), q, N, ks, m_in, K, p.chunk_len,
-                                              p.nchunks, part64, d.status);
-    } else {
-        cudaError_t err = launch_rho_f32(ctx->rho_accum, xyzq, p, grid, s, pos, q, N, ks, m_in, K, p.nchunks, part32,
-                                         d.status);
-        if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f32");
-    }
-    rbe_status st = check_launch(ctx, "k_rho");
-    if (st != RBE_OK) return st;
+    cudaError_t err = launch_rho_f32(ctx->rho_accum, xyzq, p, dim3(p.ktiles, p.nchunks), s, pos, q, N, ks, m_in, K,
+                                     p.nchunks, part32, d.status);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f32");
+    if ((st = check_launch(ctx, "k_rho")) != RBE_OK) return st;
     record_event(ctx, 2);
-    if (fp64) {
-        k_reduce<<<K + 1, kReduceThreads, 0, s>>>(part64, p.nchunks, K, m_in, w_in, ks, d.rho, d.terms, d.coef_d,
-                                                   d.counter, d.status, W, E);
-    } else {
-        cudaError_t err = launch_reduce_f32(s, (const float4*)part32, p.nchunks, K, m_in, w_in, ks, d);
-        if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_reduce_f32");
-    }
-    st = check_launch(ctx, "k_reduce");
-    if (st != RBE_OK) return st;
+    err = launch_reduce_f32(s, (const float4*)part32, p.nchunks, K, m_in, w_in, ks, d);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_reduce_f32");
+    if ((st = check_launch(ctx, "k_reduce")) != RBE_OK) return st;
     record_event(ctx, 3);
-    if (fp64) {
-        if (forces && p.fblocks > 0) {
-            k_force_f64<2><<<p.fblocks, kT, 0, s>>>(static_cast<const double*>(pos), q, N, p.per_block, ks, d.m,
-                                                    d.coef_d, K, F);
-            st = check_launch(ctx, "k_force");
-        }
-    } else {
-        // one extra block computes the energy and virial sums
-        cudaError_t err = launch_pdl(xyzq ? k_force_f32<true> : k_force_f32<false>, dim3((forces ? p.fblocks : 0) + 1),
-                                     dim3(kForceThreads), force_smem, s, pos, q,
-                                     N, p.per_block, ks, (const int4*)d.coef_m, (const float4*)d.coef_f, K, F,
-                                     d.status, (const double*)d.terms, W, E, (int64_t)0, 1);
-        st = err == cudaSuccess ? RBE_OK : cuda_fail(ctx, err, "launch k_force_f32");
-    }
-    if (st != RBE_OK) return st;
+    // one extra block computes the energy and virial sums
+    err = launch_pdl(xyzq ? k_force_f32<true> : k_force_f32<false>, dim3((forces ? p.fblocks : 0) + 1),
+                     dim3(kForceThreads), sh.force_smem, s, pos, q, N, p.per_block, ks, (const int4*)d.coef_m,
+                     (const float4*)d.coef_f, K, F, d.status, (const double*)d.terms, W, E, (int64_t)0, 1);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_force_f32");
     record_event(ctx, 4);
     ctx->last_K = K;
     return RBE_OK;

@@ -1,0 +1,420 @@
+// Pair passes of the FP64 path: rho, its reduction and the forces, on the 64-bit fixed-point sine and
+// cosine of rbe_fix64.cuh.  No FP64 instruction runs per pair; sums over particles and frequencies are
+// integers (exact, in any order), converted to double once per chunk or particle.
+//
+// What bounds them: a pair is about 120 instructions on the FMA and ALU pipes in either pass (a quarter of
+// them integer multiplications at half or quarter rate) and two random table loads from shared
+// memory; DRAM moves 32 to 56 B per particle.  Against FP64 sincospi per pair (about 35 FP64
+// instructions per pass, 76 clocks of a scheduler each): N = 3e5, P = 200 8330 -> 539 us per
+// evaluation, 1e6 x 500 67.8 -> 4.03 ms, 1e3 x 100 386 -> 21 us.
+#pragma once
+
+#include "rbe_fix64.cuh"
+#include "rbe_kspace_tiles.cuh"
+
+namespace rbe {
+
+constexpr int kRho64Threads = 512;   // threads of a rho block at most
+constexpr int kRho64Stage = 512;     // particles staged per tile at most (32 B each)
+constexpr int kRho64Group = 32;      // pairs whose products (below 2^57 each) are summed in 64 bits
+constexpr int kForce64Threads = 256;
+constexpr int kForce64Stage = 256;   // frequencies staged per tile (32 B each)
+constexpr size_t kTrigBytes = sizeof(TrigEntry) * kTrigLen;
+constexpr size_t kRho64Smem = kTrigBytes + 32 * (size_t)kRho64Stage;
+constexpr size_t kForce64Smem = kTrigBytes + 32 * (size_t)kForce64Stage;
+
+__global__ void k_trig_table(TrigEntry* __restrict__ t)
+{
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i < kTrigLen) t[i] = trig_entry(i);
+}
+
+__device__ __forceinline__ void load_trig(const TrigEntry* __restrict__ trig, TrigEntry* s_trig)
+{
+    const uint4* src = reinterpret_cast<const uint4*>(trig);
+    uint4* dst = reinterpret_cast<uint4*>(s_trig);
+    for (int i = threadIdx.x; i < kTrigLen; i += blockDim.x) dst[i] = src[i];
+}
+
+// A 128-bit integer as the nearest double or next to it (two roundings), times 2^e.
+__device__ __forceinline__ double int128_to_double(__int128 s, int e)
+{
+    const bool neg = s < 0;
+    const unsigned __int128 a = neg ? (unsigned __int128)0 - (unsigned __int128)s : (unsigned __int128)s;
+    const double d = ldexp((double)(unsigned long long)(a >> 64), 64) + (double)(unsigned long long)a;
+    return ldexp(neg ? -d : d, e);
+}
+
+// Fixed-order block sums of two doubles per thread; valid in thread 0.
+__device__ __forceinline__ void block_sum2(double& a, double& b, double (*scratch)[32])
+{
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        a += __shfl_xor_sync(0xffffffffu, a, off);
+        b += __shfl_xor_sync(0xffffffffu, b, off);
+    }
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+    if (nw == 1) return;
+    if (lane == 0) {
+        scratch[0][warp] = a;
+        scratch[1][warp] = b;
+    }
+    __syncthreads();
+    if (warp == 0) {
+        a = lane < nw ? scratch[0][lane] : 0.0;
+        b = lane < nw ? scratch[1][lane] : 0.0;
+        for (int off = 16; off > 0; off >>= 1) {
+            if (off >= nw) continue;  // the same for every lane; the lanes beyond hold zeros
+            a += __shfl_xor_sync(0xffffffffu, a, off);
+            b += __shfl_xor_sync(0xffffffffu, b, off);
+        }
+    }
+}
+
+// =================================================================================
+// rho pass.  Block (kt, c): T frequency lanes (thread j of sub-stream s owns frequency kt T + j) in S
+// particle sub-streams over the particles of chunk c, staged kRho64Stage at a time as 64-bit
+// fixed-point positions and charges and read as broadcasts.
+//
+// Charges: |q| is taken as a 59-bit fraction of twice the power of two of the chunk's largest |q| (exact
+// for charges within 2^6 of it, an error of 2^-60 of the largest one below); the sign is half a
+// revolution of the phase.  A product then has units of 2^-57 of that power of two; 32 of them are
+// summed in 64 bits, the sums of 32 in 128.
+// Partials: (Re, Im) at [l * nchunks + c]; row K holds the chunk's sum of q^2 in FP64.
+__global__ void __launch_bounds__(kRho64Threads, 2)
+k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t N, const KState* __restrict__ ks,
+          const int4* __restrict__ m, int K, int64_t chunk_len, int nchunks, double2* __restrict__ partials,
+          const TrigEntry* __restrict__ trig, unsigned* __restrict__ status, int S, int T)
+{
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    TrigEntry* st = reinterpret_cast<TrigEntry*>(s_raw);
+    int4* sp = reinterpret_cast<int4*>(s_raw + kTrigBytes);
+    __shared__ int s_eb;
+    __shared__ double s_red[2][32];
+    const int tid = threadIdx.x, nt = blockDim.x, kt = blockIdx.x, c = blockIdx.y;
+    const int64_t start = (int64_t)c * chunk_len, end = min(N, start + chunk_len);
+    if (tid == 0) s_eb = 1;
+    __syncthreads();
+    load_trig(trig, st);
+    // the largest exponent field of the chunk's charges, and the sum of their squares (inputs only)
+    int eb = 1;
+    double q2 = 0.0, zero = 0.0;
+    for (int64_t i = start + tid; i < end; i += nt) {
+        const double qi = q[i];
+        const int e = (int)(((unsigned long long)__double_as_longlong(qi) >> 52) & 0x7ffull);
+        eb = max(eb, e);
+        if (kt == 0) q2 += qi * qi;
+    }
+    eb = __reduce_max_sync(0xffffffffu, eb);
+    if ((tid & 31) == 0) atomicMax(&s_eb, eb);
+    if (kt == 0) block_sum2(q2, zero, s_red);
+    __syncthreads();
+    eb = min(s_eb, 0x7fe);
+    const bool bad_q = s_eb == 0x7ff;
+    pdl_wait();
+    pdl_trigger();
+    if (bad_q && tid == 0) atomicOr(status, kStatusNonFinite);
+    const int j = tid % T, ss = tid / T, l = kt * T + j;
+    const bool act = ss < S && l < K;
+    const int share = kRho64Stage / S, stage = share * S;
+    const int4 mv = act ? m[l] : make_int4(0, 0, 0, 0);
+    const FixScale scx = fs(ks->sc64[0]), scy = fs(ks->sc64[1]), scz = fs(ks->sc64[2]);
+    __int128 re = 0, im = 0;
+    for (int64_t base = start; base < end; base += stage) {
+        __syncthreads();  // every thread is done with the previous tile
+        const int here = (int)min((int64_t)stage, end - base);
+        for (int u = tid; u < here; u += nt) {
+            const int64_t i = base + u;
+            const unsigned long long bx = (unsigned long long)__double_as_longlong(pos[3 * i]);
+            const unsigned long long by = (unsigned long long)__double_as_longlong(pos[3 * i + 1]);
+            const unsigned long long bz = (unsigned long long)__double_as_longlong(pos[3 * i + 2]);
+            const unsigned long long bq = (unsigned long long)__double_as_longlong(q[i]);
+            if (nonfinite_bits(bx) || nonfinite_bits(by) || nonfinite_bits(bz)) atomicOr(status, kStatusNonFinite);
+            // signed halves: 2^31 added, the low word's top bit flipped
+            const unsigned long long x = fixed_frac64(bx, scx) + kMulBias, y = fixed_frac64(by, scy) + kMulBias,
+                                     z = fixed_frac64(bz, scz) + kMulBias, a = fix_magnitude(bq, eb) + kMulBias;
+            sp[2 * u] = make_int4(fx_hi(x), fx_lo(x), fx_hi(y), fx_lo(y));
+            sp[2 * u + 1] = make_int4(fx_hi(z), fx_lo(z), (int)((uint32_t)fx_hi(a) | ((uint32_t)(bq >> 63) << 31)), fx_lo(a));
+        }
+        __syncthreads();
+        if (!act) continue;
+        const int p1 = min(here, (ss + 1) * share);
+        for (int p = ss * share; p < p1; p += kRho64Group) {
+            const int n = min(kRho64Group, p1 - p);
+            unsigned long long ar = 0, ai = 0;
+#pragma unroll 2
+            for (int u = p; u < p + n; ++u) {
+                const int4 a = sp[2 * u], b = sp[2 * u + 1];
+                unsigned long long t = mad_wide(mv.x, a.y, kPhaseStart);
+                t = mad_wide(mv.y, a.w, t);
+                t = mad_wide(mv.z, b.y, t);
+                uint32_t hi = (uint32_t)(t >> 32) + (uint32_t)mv.x * (uint32_t)a.x;
+                hi += (uint32_t)mv.y * (uint32_t)a.z;
+                hi += (uint32_t)mv.z * (uint32_t)b.x;
+                hi ^= (uint32_t)b.z & 0x80000000u;
+                const PhaseX x = phase_x(hi, (uint32_t)t);
+                const TrigEntry* e = st + (hi >> 21);
+                const TrigEntry es = e[0], ec = e[kTrigN / 4];
+                const unsigned long long vs = trig_value<1>(es.v, es.h, es.l, ec.h, ec.l, x);
+                const unsigned long long vc = trig_value<-1>(ec.v, ec.h, ec.l, es.h, es.l, x);
+                const int qh = b.z & 0x7fffffff, ql = b.w;
+                ar += mul_fix(fx_hi(vc), fx_lo(vc), qh, ql);
+                ai += mul_fix(fx_hi(vs), fx_lo(vs), qh, ql);
+            }
+            const unsigned long long bias = (unsigned long long)n * kMulBias;
+            re += (long long)(ar - bias);
+            im += (long long)(ai - bias);
+        }
+    }
+    __syncthreads();
+    // the sub-streams' sums (integers: any order gives the same)
+    __int128* sum = reinterpret_cast<__int128*>(sp);
+    if (S > 1) {
+        if (act) {
+            sum[2 * (ss * T + j)] = re;
+            sum[2 * (ss * T + j) + 1] = im;
+        }
+        __syncthreads();
+        if (act && ss == 0)
+            for (int s = 1; s < S; ++s) {
+                re += sum[2 * (s * T + j)];
+                im += sum[2 * (s * T + j) + 1];
+            }
+    }
+    if (act && ss == 0) {
+        const int e = eb - 1023 - 56;  // units of 2^-57 of 2^(eb - 1023 + 1)
+        partials[(size_t)l * nchunks + c] = make_double2(int128_to_double(re, e), int128_to_double(im, e));
+    }
+    if (kt == 0 && tid == 0) partials[(size_t)K * nchunks + c] = make_double2(q2, 0.0);
+}
+
+// =================================================================================
+// Reduction: block l (of K + 1) sums its row over the chunks in a fixed order; thread 0 forms the
+// frequency's energy and virial terms (as on the FP32-phase path, freq_pre before the wait), the force
+// amplitude R = c[7] |rho| and arg rho as a 64-bit fixed-point phase.
+//
+// arg rho without an FP64 arctangent (a chain of about 60 FP64 instructions of one warp, 4 us here): the
+// FP32 arctangent, rounded to 2^-30 revolutions, as a first angle; its exact sine and cosine from the
+// table; and the remaining angle (below 2^-22) from Im(rho e^{-i phi}) / |rho|.
+__global__ void __launch_bounds__(kReduceThreads)
+k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int4* __restrict__ m,
+             const double* __restrict__ w, const KState* __restrict__ ks, const TrigEntry* __restrict__ trig,
+             double2* __restrict__ rho, double* __restrict__ terms, double2* __restrict__ coef,
+             unsigned* __restrict__ status)
+{
+    __shared__ double red[2][32];
+    const int l = blockIdx.x;
+    // the sampler completed before the rho pass passed its wait, and the rho pass lets this
+    // launch start only after that wait: m, w and ks are final here
+    double c[8];
+    if (threadIdx.x == 0 && l < K) freq_pre(m[l], w[l], ks, c);
+    pdl_wait();
+    pdl_trigger();
+    double re = 0.0, im = 0.0;
+    const double2* row = partials + (size_t)l * nchunks;
+    for (int j = threadIdx.x; j < nchunks; j += blockDim.x) {
+        const double2 v = row[j];
+        re += v.x;
+        im += v.y;
+    }
+    block_sum2(re, im, red);
+    if (threadIdx.x != 0) return;
+    double* t = terms + (size_t)l * 8;
+    if (l == K) {
+        t[0] = re;  // sum of q^2
+        return;
+    }
+    const double rho2 = re * re + im * im;
+    const double e = c[0] * rho2;
+    t[0] = e;
+#pragma unroll
+    for (int a = 1; a < 7; ++a) t[a] = e * c[a];
+    t[7] = 0.0;
+    rho[l] = make_double2(re, im);
+    if (!isfinite(re) || !isfinite(im)) atomicOr(status, kStatusNonFinite);
+    unsigned long long phi = 0ull;
+    double R = 0.0;
+    if (rho2 > 0.0) {
+        const double inv = rsqrt(rho2);
+        R = c[7] * (rho2 * inv);
+        const double cr = re * inv, ci = im * inv;  // (cos, sin) of arg rho
+        const float rev = atan2f((float)ci, (float)cr) * 0.159154943f;
+        phi = (unsigned long long)(long long)__float2int_rn(rev * 1073741824.0f) << 34;
+        const unsigned long long ph = phi + kPhaseStart;
+        const PhaseX x = phase_x((uint32_t)(ph >> 32), (uint32_t)ph);
+        const TrigEntry es = trig[ph >> 53], ec = trig[(ph >> 53) + kTrigN / 4];
+        const double s = (double)(long long)(trig_value<1>(es.v, es.h, es.l, ec.h, ec.l, x) - kMulBias);
+        const double co = (double)(long long)(trig_value<-1>(ec.v, ec.h, ec.l, es.h, es.l, x) - kMulBias);
+        // ci co - cr s = sin(arg rho - phi) in units of 2^62; revolutions in units of 2^-64: 4 / 2 pi
+        const double d = fma(ci, co, -(cr * s)) * 0.63661977236758134308;
+        phi += (unsigned long long)__double2ll_rn(d);
+    }
+    coef[l] = make_double2(__longlong_as_double((long long)(kPhaseStart - phi)), R);
+}
+
+// =================================================================================
+// Force pass: F_i,theta = q_i (2 pi / l_theta) sum_l R_l m_l,theta sin(theta_il - arg rho_l).
+// A block takes rounds of kForce64Threads / SL particles (lanes) with the frequencies of a staged tile split
+// over SL slices, whose integer sums are added at the end of the round: SL > 1 spreads small systems
+// over the GPU.  Per staged tile the amplitudes R_l become integers: scaled so that sum_l |m_l| R_l
+// (an FP32 bound, rounded up) is below 2^62, each product R sin is rounded to 2^-60 of that sum.
+// The launch carries one extra block that computes the energy and virial sums (final_sums) meanwhile.
+template <int SL>
+__global__ void __launch_bounds__(kForce64Threads, 4)
+k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t N, int64_t per_block,
+            const KState* __restrict__ ks, const int4* __restrict__ mk, const double2* __restrict__ coef, int K,
+            double* __restrict__ F, const TrigEntry* __restrict__ trig, unsigned* __restrict__ status,
+            const double* __restrict__ terms, double* __restrict__ W_out, double* __restrict__ E_out)
+{
+    if (blockIdx.x == gridDim.x - 1) {
+        pdl_wait();
+        final_sums(terms, K, ks, W_out, E_out, status);
+        return;
+    }
+    constexpr int PB = kForce64Threads / SL;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    TrigEntry* st = reinterpret_cast<TrigEntry*>(s_raw);
+    int4* sk = reinterpret_cast<int4*>(s_raw + kTrigBytes);  // (mx, my, mz, R low), (phase low, high, R high, 0)
+    __shared__ unsigned long long s_sum[SL > 1 ? 3 : 1][SL > 1 ? kForce64Threads : 1];
+    __shared__ int s_e;
+    __shared__ float s_b[3][kForce64Threads / 32];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int pl = tid % PB, sl = tid / PB;
+    load_trig(trig, st);
+    pdl_wait();  // (ks: see k_rho_f64)
+    const FixScale scx = fs(ks->sc64[0]), scy = fs(ks->sc64[1]), scz = fs(ks->sc64[2]);
+    const double cx = 2.0 * kPi * ks->inv[0], cy = 2.0 * kPi * ks->inv[1], cz = 2.0 * kPi * ks->inv[2];
+    const int64_t b0 = (int64_t)blockIdx.x * per_block, b1 = min(N, b0 + per_block);
+    const bool one_tile = K <= kForce64Stage;
+    int sh = 0;  // R as an integer is R 2^sh
+    for (int64_t base = b0; base < b1; base += PB) {
+        const int64_t i = base + pl;
+        unsigned long long x = 0, y = 0, z = 0;
+        if (i < b1) {
+            x = fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i]), scx) + kMulBias;
+            y = fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i + 1]), scy) + kMulBias;
+            z = fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i + 2]), scz) + kMulBias;
+        }
+        const int xh = fx_hi(x), xl = fx_lo(x), yh = fx_hi(y), yl = fx_lo(y), zh = fx_hi(z), zl = fx_lo(z);
+        double fx = 0.0, fy = 0.0, fz = 0.0;
+        for (int k0 = 0; k0 < K; k0 += kForce64Stage) {
+            const int nk = min(kForce64Stage, K - k0);
+            if (!one_tile || base == b0) {
+                // one frequency per thread: exponent of the largest R, then sum |m| R in its units
+                __syncthreads();
+                int4 mm = make_int4(0, 0, 0, 0);
+                double2 co = make_double2(0.0, 0.0);
+                if (tid < nk) {
+                    mm = mk[k0 + tid];
+                    co = coef[k0 + tid];
+                }
+                if (tid == 0) s_e = 1;
+                __syncthreads();
+                const unsigned long long rb = (unsigned long long)__double_as_longlong(co.y);
+                const int e = (int)((rb >> 52) & 0x7ffull);
+                const int emax = __reduce_max_sync(0xffffffffu, e);
+                if (lane == 0) atomicMax(&s_e, emax);
+                __syncthreads();
+                const int er = min(s_e, 0x7fe);
+                // R 2^(1023 - er) below 2, as FP32 (23 mantissa bits, truncated)
+                const float rf = e > 0 && e <= er && er - e < 64
+                                     ? __uint_as_float(((uint32_t)(127 + e - er) << 23) | (uint32_t)((rb >> 29) & 0x7fffffu))
+                                     : 0.0f;
+                float bx = rf * fabsf((float)mm.x), by = rf * fabsf((float)mm.y), bz = rf * fabsf((float)mm.z);
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1) {
+                    bx += __shfl_xor_sync(0xffffffffu, bx, off);
+                    by += __shfl_xor_sync(0xffffffffu, by, off);
+                    bz += __shfl_xor_sync(0xffffffffu, bz, off);
+                }
+                if (lane == 0) {
+                    s_b[0][warp] = bx;
+                    s_b[1][warp] = by;
+                    s_b[2][warp] = bz;
+                }
+                __syncthreads();
+                bx = by = bz = 0.0f;
+#pragma unroll
+                for (int v = 0; v < kForce64Threads / 32; ++v) {
+                    bx += s_b[0][v];
+                    by += s_b[1][v];
+                    bz += s_b[2][v];
+                }
+                // the bound, at least 2 (the largest R itself), rounded up well above the FP32 sums' error
+                const float bound = fmaxf(2.0f, fmaxf(bx, fmaxf(by, bz)) * 1.0001f);
+                const int lg = (int)((__float_as_uint(bound) >> 23) & 0xffu) - 127 + 1;  // bound < 2^lg
+                sh = 62 - lg + 1023 - er;  // sum |m| R 2^sh < 2^62
+                if (tid < nk) {
+                    // R 2^sh = mantissa 2^(e - 1075 + sh)
+                    const unsigned long long mant = e > 0 ? (rb & 0xFFFFFFFFFFFFFull) | (1ull << 52) : 0ull;
+                    const int k = e - 1075 + sh;
+                    const unsigned long long A =
+                        (k >= 0 ? mant << min(k, 63) : (k > -64 ? mant >> -k : 0ull)) + kMulBias;
+                    const unsigned long long off = (unsigned long long)__double_as_longlong(co.x);
+                    sk[2 * tid] = make_int4(mm.x, mm.y, mm.z, fx_lo(A));
+                    sk[2 * tid + 1] = make_int4((int)(uint32_t)off, (int)(uint32_t)(off >> 32), fx_hi(A), 0);
+                }
+                __syncthreads();
+            }
+            unsigned long long ax = 0, ay = 0, az = 0;
+            uint32_t hx = 0, hy = 0, hz = 0;
+            const int per = SL > 1 ? (nk + SL - 1) / SL : nk;
+            const int l1 = SL > 1 ? min(nk, (sl + 1) * per) : nk;
+#pragma unroll 2
+            for (int l = SL > 1 ? sl * per : 0; l < l1; ++l) {
+                const int4 a = sk[2 * l], b = sk[2 * l + 1];
+                unsigned long long t = mad_wide(a.x, xl, ((unsigned long long)(uint32_t)b.y << 32) | (uint32_t)b.x);
+                t = mad_wide(a.y, yl, t);
+                t = mad_wide(a.z, zl, t);
+                uint32_t hi = (uint32_t)(t >> 32) + (uint32_t)a.x * (uint32_t)xh;
+                hi += (uint32_t)a.y * (uint32_t)yh;
+                hi += (uint32_t)a.z * (uint32_t)zh;
+                const PhaseX p = phase_x(hi, (uint32_t)t);
+                const TrigEntry* e = st + (hi >> 21);
+                const TrigEntry es = e[0];
+                const float2 ec = *reinterpret_cast<const float2*>(&e[kTrigN / 4].h);
+                const unsigned long long v = trig_value<1>(es.v, es.h, es.l, ec.x, ec.y, p);
+                const unsigned long long h = mul_fix(fx_hi(v), fx_lo(v), b.z, a.w);
+                const int hh = fx_hi(h), hl = fx_lo(h);
+                ax = mad_wide(a.x, hl, ax);
+                ay = mad_wide(a.y, hl, ay);
+                az = mad_wide(a.z, hl, az);
+                hx += (uint32_t)a.x * (uint32_t)hh;
+                hy += (uint32_t)a.y * (uint32_t)hh;
+                hz += (uint32_t)a.z * (uint32_t)hh;
+            }
+            ax += (unsigned long long)hx << 32;
+            ay += (unsigned long long)hy << 32;
+            az += (unsigned long long)hz << 32;
+            if (SL > 1) {
+                __syncthreads();  // the previous round's sums have been read
+                s_sum[0][tid] = ax;
+                s_sum[1][tid] = ay;
+                s_sum[2][tid] = az;
+                __syncthreads();
+                if (sl == 0)
+#pragma unroll
+                    for (int s = 1; s < SL; ++s) {
+                        ax += s_sum[0][s * PB + pl];
+                        ay += s_sum[1][s * PB + pl];
+                        az += s_sum[2][s * PB + pl];
+                    }
+            }
+            // units of 2^-62 (sine) times 2^64 (product's high half) over 2^sh
+            if (sl == 0 && i < b1) {
+                const double u = ldexp(1.0, 2 - sh);
+                fx += u * (double)(long long)ax;
+                fy += u * (double)(long long)ay;
+                fz += u * (double)(long long)az;
+            }
+        }
+        if (sl == 0 && i < b1) {
+            const double qi = q[i];
+            F[3 * i] = qi * cx * fx;
+            F[3 * i + 1] = qi * cy * fy;
+            F[3 * i + 2] = qi * cz * fz;
+        }
+    }
+}
+
+}  // namespace rbe

@@ -8,6 +8,7 @@
 
 #include "rbe_context.h"
 #include "rbe_device.cuh"
+#include "rbe_fix64.cuh"
 
 namespace rbe {
 
@@ -139,6 +140,9 @@ __device__ __forceinline__ void tables_body(double bx, double by, double bz, con
         const int e = (int)((b >> 52) & 0x7ff) - 1075;
         ks->sc[t].q = ((b & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 11;
         ks->sc[t].e = e - 11;
+        const FixScale s64 = fix_scale64(sL[t], inv);
+        ks->sc64[t].q = s64.q;
+        ks->sc64[t].e = s64.e;
     } else if (tid >= 64 && tid < 67) {
         const int t = tid - 64;
         const float c = (float)(2.0 * kPi / sL[t]);
