@@ -133,7 +133,7 @@ static void free_buffers(DeviceBuffers& d)
 {
     cudaFree(d.cum); cudaFree(d.ks); cudaFree(d.m); cudaFree(d.w); cudaFree(d.rho); cudaFree(d.terms);
     cudaFree(d.coef_m); cudaFree(d.coef_f); cudaFree(d.coef_d); cudaFree(d.partials);
-    cudaFree(d.status); cudaFree(d.pos); cudaFree(d.q); cudaFree(d.F); cudaFree(d.WE); cudaFree(d.trig);
+    cudaFree(d.status); cudaFree(d.pos); cudaFree(d.q); cudaFree(d.F); cudaFree(d.WE);
     d = DeviceBuffers{};
 }
 
@@ -166,8 +166,6 @@ rbe_status rbe_create(const double box[3], double alpha, int32_t P, uint64_t see
     DeviceBuffers& d = ctx->d;
     if ((err = cudaMalloc(&d.ks, sizeof(KState))) != cudaSuccess ||
         (err = cudaMalloc(&d.status, sizeof(unsigned))) != cudaSuccess ||
-        (err = cudaMalloc(&d.trig, trig_table_bytes())) != cudaSuccess ||
-        (err = launch_trig_table(d.trig, nullptr)) != cudaSuccess ||
         (err = cudaMemset(d.status, 0, sizeof(unsigned))) != cudaSuccess) {
         std::string msg = std::string("device allocation failed: ") + cudaGetErrorString(err);
         free_buffers(d);

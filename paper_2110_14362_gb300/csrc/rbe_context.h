@@ -105,7 +105,6 @@ struct DeviceBuffers {
     int4* coef_m = nullptr;           // [kcap] FP32 force data (mx, my, mz, bits of A)
     float4* coef_f = nullptr;         // [kcap] FP32 force data (B, mx, my, mz)
     double2* coef_d = nullptr;        // [kcap] FP64 path: (bits of the phase offset of arg rho, amplitude R)
-    void* trig = nullptr;             // [kTrigLen] TrigEntry (rbe_fix64.cuh), written by rbe_create
     int kcap = 0;
     void* partials = nullptr;         // [(K + 1) * nchunks] double2 (FP64 path) or float4 (FP32-phase)
     size_t part_cap = 0;              // in 16-byte entries
@@ -196,8 +195,6 @@ rbe_status ensure_tables(rbe_ctx ctx);
 rbe_status ensure_table_capacity(rbe_ctx ctx, int need);
 rbe_status launch_tables(rbe_ctx ctx, const double* box_dev);
 rbe_status ensure_k_capacity(rbe_ctx ctx, int K);
-cudaError_t launch_trig_table(void* trig, cudaStream_t s);
-size_t trig_table_bytes();
 rbe_status launch_sample(rbe_ctx ctx, uint64_t step, int P);
 rbe_status launch_sample_device_box(rbe_ctx ctx, uint64_t step, int P, const unsigned long long* step_dev);
 rbe_status launch_tables_sample_device(rbe_ctx ctx, int P, const double* box_dev, const unsigned long long* step_dev);

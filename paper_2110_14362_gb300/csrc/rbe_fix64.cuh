@@ -6,20 +6,26 @@
 // from shared memory 9.8 clocks per warp and SM), and a pair of the FP64 formulation takes about
 // 35 of them per pass.  Here a pair takes none.
 //
-// Phase.  s = r / l is a 64-bit fraction of a revolution (error about 2^-64, against 2^-53 of a
-// double), so m.s mod 1 is exact in wrapping integer arithmetic.  The top 11 bits, rounded, pick
-// an entry a of a table of 2048 angles; the rest is x, |x| <= 2 pi 2^-12, a float-float.
+// Phase.  s = r / l is a fraction of a revolution with 64 bits, kept as an integer in units of 2^-32 and
+// an FP32 remainder (error at most 2^-58).  m.s is the wrapping integer sum of the m s_hi and the FP32
+// sum of the m s_lo: an error of about |m| 2^-59 revolutions (FP64: |m| 2^-54 from s alone).
+// The top 11 bits, rounded, pick an entry a of a table of 2048 angles; the rest is x, |x| <= 2 pi 2^-12
+// (and a little more: the FP32 sum is at most |m| units), a float-float.
 //   sin(a + x) = S + sin x (C - S t),  cos(a + x) = C - sin x (S + C t),  t = tan(x / 2)
 // (S, C the table's sine and cosine).  The bracket and the product are float-float: their result
-// is at most 2^-9.3, so 2^-46 of it is enough.  It is turned into fixed point by two FP32
-// additions of a constant (the mantissa bits of c + v hold round(v)) and added to the table's
-// 64-bit value.  Result: a 64-bit integer in units of 2^-62.  Errors: the fixed-point rounding of
-// the low part (at most 2^-53), the table (2^-61), the float-float product (about 2^-55).
+// is at most 2^-9.3, so 2^-46 of it is enough.  Its integer part is taken by an FP32 addition of a
+// constant (the mantissa bits of c + v hold round(v)) and added to the table's.  Result: an integer in
+// units of 2^-30 and an FP32 remainder.  Errors: the remainder's rounding (2^-54), the table (2^-55),
+// the float-float product (about 2^-55).
 //
 // The bracket's float-float sum is Fast2Sum-exact because |C t| < |S| for every table entry with
 // S != 0 (the smallest is sin(2 pi / 2048) = 3.1e-3, |t| <= 7.7e-4).
+//
+// A 64-bit multiply-add of 32-bit factors is a multiplication and two additions here (23 per clock and SM
+// against 61 fused 32-bit ones), so only the products that need 64 bits take it.
 #pragma once
 
+#include <cmath>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -28,14 +34,30 @@
 namespace rbe {
 
 constexpr int kTrigN = 2048;                   // table angles per revolution
-constexpr int kTrigLen = kTrigN + kTrigN / 4;  // entries: cos(a) = sin(a + 1/4 revolution)
 
-// v: sin(2 pi i / kTrigN) in units of 2^-62, made odd (so that no product of it with a power of
-// two is a rounding tie, and sin(a + pi) is the exact negative), plus kMulBias - kTrigBias; h + l: the
-// same sine times 2^30 as a float-float.
+// sin and cos of 2 pi i / kTrigN as a + r 2^-24 in units of 2^-30, a the nearest integer and r an integer
+// (TrigEntry); a is the float (float)a plus at most 32, and (that rest) + r 2^-24 as a float is the low part of
+// the value as a float-float (kept in a second plane).  Half a revolution on, every part is the exact
+// negative.  Random loads cost bank conflicts (17.7 clocks of the SM for 16 bytes per lane, 9.6 for 8):
+// with the floats stored whole beside the integers the shared-memory pipe was 80 % busy and bound the
+// passes; with everything rebuilt from the integers the conversions did.
 struct alignas(16) TrigEntry {
-    unsigned long long v;
-    float h, l;
+    int sa, sr, ca, cr;
+};
+struct alignas(8) TrigLow {
+    float s, c;
+};
+// For a sine alone: the sine's integers and the cosine's float-float; the sine's low part in its own plane.
+struct alignas(16) TrigSine {
+    int sa, sr;
+    float ch, cl;
+};
+// The table (88 KB, a constant of the library's device image: formed by the compiler).
+struct TrigTable {
+    TrigEntry entry[kTrigN];
+    TrigLow low[kTrigN];
+    TrigSine sine[kTrigN];
+    float sine_low[kTrigN];
 };
 
 #ifdef __CUDA_ARCH__
@@ -76,25 +98,19 @@ __host__ __device__ __forceinline__ unsigned long long mad_wide(int a, int b, un
     return c + (unsigned long long)((long long)a * (long long)b);
 }
 
-// kHiMagic + v holds round(v) in its mantissa (|v| < 2^22); kLoMagic + v holds v (|v| < 1; here at most
-// 0.7: half a unit and the products' rounding errors) on a grid of 2^-22.  kTrigBias removes the
-// constants' own bits from the sum.
+// kHiMagic + v holds round(v) in its mantissa (|v| < 2^22).
 constexpr float kHiMagic = 12582912.0f;  // 1.5 2^23, bits 0x4B400000
-constexpr float kLoMagic = 3.0f;         // bits 0x40000000 + (v + 1) 2^22
-constexpr unsigned long long kTrigBias = (0x4B400000ull << 32) + (1ull << 40) + (1ull << 32);
 // 2^31 on a 64-bit value makes its low word, read with the top bit flipped, the signed remainder of its
 // high word: the form in which 64-bit values enter a product.
 constexpr unsigned long long kMulBias = 1ull << 31;
 
-// Entry i: the sine by its Taylor series in 64-bit fixed point (units of 2^-63, errors of a few of
-// them) on [0, pi/4] and by symmetry elsewhere.
-__host__ __device__ inline TrigEntry trig_entry(int i)
+// sin(pi k / 1024) for k in [0, 512], in units of 2^-63: Taylor series in 64-bit fixed point (errors of a
+// few units) on [0, pi/4] and by symmetry beyond.
+constexpr unsigned long long quarter_sine(int k)
 {
-    const int j = i % kTrigN, half = j % (kTrigN / 2), quarter = kTrigN / 4;
-    const int k = half <= quarter ? half : kTrigN / 2 - half;     // angle pi k / 1024 in [0, pi/2]
-    const bool use_cos = k > quarter / 2;
-    const unsigned kk = (unsigned)(use_cos ? quarter - k : k);    // argument pi kk / 1024 in [0, pi/4]
-    const unsigned __int128 pi61 = 0x6487ED5110B4611Aull;         // floor(pi 2^61)
+    const bool use_cos = k > kTrigN / 8;
+    const unsigned kk = (unsigned)(use_cos ? kTrigN / 4 - k : k);         // argument pi kk / 1024 in [0, pi/4]
+    const unsigned __int128 pi61 = 0x6487ED5110B4611Aull;                 // floor(pi 2^61)
     const unsigned long long x = (unsigned long long)((pi61 * kk) >> 8);  // the argument in units of 2^-63
     const unsigned long long x2 = (unsigned long long)(((unsigned __int128)x * x) >> 63);
     unsigned long long term = use_cos ? 1ull << 63 : x, sum = term;
@@ -103,64 +119,105 @@ __host__ __device__ inline TrigEntry trig_entry(int i)
         term = (unsigned long long)(((unsigned __int128)term * x2) >> 63) / (unsigned)(n * (n + 1));
         sum = minus ? sum - term : sum + term;
     }
-    long long v = (long long)((sum >> 1) + (sum & 1));  // units of 2^-62
-    if ((v & 1) == 0) v += v == 0 ? 1 : -1;
-    const double s = (double)sum * 0x1.0p-33;  // the sine times 2^30
-    TrigEntry e;
-    e.h = (float)s;
-    e.l = (float)(s - (double)e.h);
-    if (j >= kTrigN / 2) {
-        v = -v;
-        e.h = -e.h;
-        e.l = -e.l;
+    return sum;
+}
+
+// A sine (u 2^-63, negated if neg) as a table entry's two parts.
+constexpr void trig_split(unsigned long long u, bool neg, int& a, int& r)
+{
+    a = (int)((u + (1ull << 32)) >> 33);
+    const long long rest = (long long)(u - ((unsigned long long)a << 33));  // units of 2^-63, up to 2^32
+    r = (int)((rest + 256) >> 9);
+    if (neg) {
+        a = -a;
+        r = -r;
     }
-    e.v = (unsigned long long)v - kTrigBias + kMulBias;
+}
+
+constexpr TrigEntry trig_entry(int i)
+{
+    const int q = kTrigN / 4, half = i % (2 * q);
+    TrigEntry e{};
+    trig_split(quarter_sine(half <= q ? half : 2 * q - half), i >= 2 * q, e.sa, e.sr);
+    trig_split(quarter_sine(half <= q ? q - half : half - q), (i >= 2 * q) != (half > q), e.ca, e.cr);
     return e;
 }
 
-// Start value of a phase sum: half a table spacing in the high word (the index is the rounded
-// phase) and half of 2^32 in the low word (which is then read as a signed remainder).
-constexpr unsigned long long kPhaseStart = (1ull << 52) + (1ull << 31);
+constexpr TrigLow trig_low(const TrigEntry& e)
+{
+    TrigLow l{};
+    l.s = (float)((double)(e.sa - (int)(float)e.sa) + (double)e.sr * 0x1.0p-24);
+    l.c = (float)((double)(e.ca - (int)(float)e.ca) + (double)e.cr * 0x1.0p-24);
+    return l;
+}
 
-// The remainder of a phase: sin x = sh + sl (|sl| at most half a unit of sh), tan(x / 2) = th + tl.
+constexpr TrigTable make_trig_table()
+{
+    TrigTable t{};
+    for (int i = 0; i < kTrigN; ++i) {
+        const TrigEntry e = trig_entry(i);
+        t.entry[i] = e;
+        t.low[i] = trig_low(e);
+        t.sine[i].sa = e.sa;
+        t.sine[i].sr = e.sr;
+        t.sine[i].ch = (float)e.ca;
+        t.sine[i].cl = t.low[i].c;
+        t.sine_low[i] = t.low[i].s;
+    }
+    return t;
+}
+
+// Start value of the integer phase sum: half a table spacing, so that the index is the rounded phase.
+constexpr uint32_t kPhaseStart = 1u << 20;
+
+// A 64-bit fraction as its nearest multiple of 2^-32 and the rest in those units.
+struct Frac {
+    int hi;
+    float lo;
+};
+
+// The remainder of a phase: sin x = sh + sl, tan(x / 2) = th + tl.
 struct PhaseX {
     float sh, sl, th, tl;
 };
 
-// hi: high word of the phase sum (with kPhaseStart), lo: low word.
-__host__ __device__ __forceinline__ PhaseX phase_x(uint32_t hi, uint32_t lo)
+// hi: integer phase sum (with kPhaseStart), lo: the FP32 sum, in units of 2^-32 revolutions.
+__host__ __device__ __forceinline__ PhaseX phase_x(uint32_t hi, float lo)
 {
-    // 2 pi 2^-32 = k1 + k2, and k1 2^-32 for the low word
-    const float k1 = 1.46291807926715968e-9f;              // RN(2 pi 2^-32)
+    // 2 pi 2^-32 = k1 + k2
+    const float k1 = 1.46291807926715968e-9f;
     const float k2 = (float)(1.46291807926715968105e-9 - (double)1.46291807926715968e-9f);
-    const float k3 = k1 * 2.3283064365386963e-10f;
-    const float dh = RBE_ADD(fx_float((hi & 0x1FFFFFu) | 0x4B000000u), -(8388608.0f + 1048576.0f));
-#ifdef __CUDA_ARCH__
-    const float dl = __int2float_rn((int)(lo ^ 0x80000000u));
-#else
-    const float dl = (float)(int)(lo ^ 0x80000000u);
-#endif
-    const float xh = RBE_MUL(dh, k1);
-    float xl = RBE_FMA(dh, k1, -xh);
-    xl = RBE_FMA(dh, k2, xl);
-    xl = RBE_FMA(dl, k3, xl);  // up to 7.3e-10: not below xh's last bit
-    // sin x = x - x^3 / 6 + x^5 / 120, tan(x/2) = x/2 + x^3 / 24 (the next term is below 2^-54)
-    const float y = RBE_ADD(xh, xl), x2 = RBE_MUL(y, y), x3 = RBE_MUL(x2, y);
-    const float sl = RBE_FMA(RBE_FMA(x2, 1.0f / 120.0f, -1.0f / 6.0f), x3, xl);
+    const float d = RBE_ADD(fx_float((hi & 0x1FFFFFu) | 0x4B000000u), -(8388608.0f + 1048576.0f));
+    // d + lo = dh + dl: exact, since d is an integer (also where |d| < |lo|)
+    const float dh = RBE_ADD(d, lo), dl = RBE_ADD(lo, -RBE_ADD(dh, -d));
     PhaseX r;
-    r.sh = RBE_ADD(xh, sl);  // Fast2Sum: |xh| >= |sl| or xh = 0
-    r.sl = RBE_ADD(sl, -RBE_ADD(r.sh, -xh));
-    r.th = RBE_MUL(0.5f, xh);
+    r.sh = RBE_MUL(dh, k1);
+    float xl = RBE_FMA(dh, k1, -r.sh);
+    xl = RBE_FMA(dh, k2, xl);
+    xl = RBE_FMA(dl, k1, xl);
+    // sin x = x - x^3 / 6 + x^5 / 120, tan(x/2) = x/2 + x^3 / 24 (the next term is below 2^-54)
+    const float x2 = RBE_MUL(r.sh, r.sh), x3 = RBE_MUL(x2, r.sh);
+    r.sl = RBE_FMA(RBE_FMA(x2, 1.0f / 120.0f, -1.0f / 6.0f), x3, xl);
+    r.th = RBE_MUL(0.5f, r.sh);
     r.tl = RBE_FMA(x3, 1.0f / 24.0f, RBE_MUL(0.5f, xl));
     return r;
 }
 
-// V + sg sin x (D - sg V' t): with (vh, vl) the float-float of the value whose entry v is given, and
-// (dh, dl) that of its derivative: sg = +1 gives sin(a + x) from (S; C), sg = -1 cos(a + x) from
-// (C; S).  Result in units of 2^-62, plus kMulBias.
+__host__ __device__ __forceinline__ float fx_i2f(int i)
+{
+#ifdef __CUDA_ARCH__
+    return __int2float_rn(i);
+#else
+    return (float)i;
+#endif
+}
+
+// V + sg sin x (D - sg V t) for a value V = (a + ...) with the float-float (vh, vl) and its derivative (dh,
+// dl): sg = +1 gives sin(a + x) from (sine, cosine), sg = -1 cos(a + x) from (cosine, sine).  Result hi + lo
+// plus the table's r 2^-24, in units of 2^-30: an integer and a float, |lo| < 1.3.
 template <int SG>
-__host__ __device__ __forceinline__ unsigned long long trig_value(unsigned long long v, float vh, float vl, float dh,
-                                                                  float dl, const PhaseX& x)
+__host__ __device__ __forceinline__ void trig_value(int a, float vh, float vl, float dh, float dl, const PhaseX& x,
+                                                    int& hi, float& lo)
 {
     const float nh = SG > 0 ? -vh : vh, nl = SG > 0 ? -vl : vl;
     const float ah = RBE_FMA(nh, x.th, dh);
@@ -173,24 +230,35 @@ __host__ __device__ __forceinline__ unsigned long long trig_value(unsigned long 
     float e = RBE_FMA(ah, sx, -p);
     e = RBE_FMA(ah, sxl, e);
     e = RBE_FMA(al, sx, e);
-    const float t1 = RBE_ADD(p, kHiMagic);
-    const float r = RBE_ADD(p, -RBE_ADD(t1, -kHiMagic));
-    const float t3 = RBE_ADD(RBE_ADD(r, e), kLoMagic);
-    const unsigned long long w = v + (unsigned long long)fx_bits(t3) * 1024ull;
-    return w + ((unsigned long long)fx_bits(t1) << 32);
+    const float t = RBE_ADD(p, kHiMagic);
+    lo = RBE_ADD(RBE_ADD(p, -RBE_ADD(t, -kHiMagic)), e);
+    hi = (int)((uint32_t)a + fx_bits(t) - 0x4B400000u);
+}
+
+// lo + r 2^-24 as a float and as an integer in units of 2^-24 (both below 1.8 in magnitude).
+__host__ __device__ __forceinline__ float trig_low_f(int r, float lo) { return RBE_FMA(fx_i2f(r), 0x1.0p-24f, lo); }
+__host__ __device__ __forceinline__ int trig_low_i(int r, float lo)
+{
+#ifdef __CUDA_ARCH__
+    return r + __float2int_rn(RBE_MUL(lo, 16777216.0f));
+#else
+    return r + (int)rintf(lo * 16777216.0f);
+#endif
 }
 
 // The signed halves of a value held with kMulBias: v = fx_hi 2^32 + fx_lo.
 __host__ __device__ __forceinline__ int fx_hi(unsigned long long v) { return (int)(uint32_t)(v >> 32); }
 __host__ __device__ __forceinline__ int fx_lo(unsigned long long v) { return (int)((uint32_t)v ^ 0x80000000u); }
 
-// a b 2^-64 for a (signed) and b (0 <= b < 2^62) given as signed halves, rounded, plus kMulBias: three
-// IMAD.WIDE.  The product of the low words (at most a quarter unit, of either sign) is left out.
-__host__ __device__ __forceinline__ unsigned long long mul_fix(int a_hi, int a_lo, int b_hi, int b_lo)
+// v b 2^-60 for v = v_hi + v_lo 2^-24 (units of 2^-30; |v_lo| < 2^25) and b = b_hi 2^30 + b_lo
+// (0 <= b < 2^60, b_lo signed), rounded, plus kMulBias: three 64-bit products; that of the low words (below
+// two units) is left out.
+__host__ __device__ __forceinline__ unsigned long long mul_fix(int v_hi, int v_lo, int b_hi, int b_lo)
 {
-    unsigned long long c = mad_wide(a_lo, b_hi, (1ull << 63) + (1ull << 31));
-    c = mad_wide(a_hi, b_lo, c);
-    return mad_wide(a_hi, b_hi, c >> 32);
+    // the constant: 2^31 as the bias (c is below 2^31 in magnitude) and one half, both shifted by 30
+    unsigned long long c = mad_wide((int)((uint32_t)v_lo << 6), b_hi, (1ull << 61) + (1ull << 29));
+    c = mad_wide(v_hi, b_lo, c);
+    return mad_wide(v_hi, b_hi, (unsigned long long)(uint32_t)(c >> 30));
 }
 
 // 1 / l as a 64-bit mantissa (rounded to the last bit) and a power of two, l a positive normal double
@@ -252,15 +320,21 @@ __host__ __device__ inline unsigned long long fixed_frac64(unsigned long long rb
     return (rb >> 63) ? 0ull - res : res;
 }
 
-// |q| as a 59-bit fraction of 2^(E + 1), E = the unbiased exponent field of a number no smaller than
-// |q|: floor(|q| 2^(58 - E)).  eb: that exponent field (1 .. 2046).
+__host__ __device__ __forceinline__ Frac frac_of(unsigned long long f)
+{
+    const unsigned long long g = f + kMulBias;
+    return Frac{fx_hi(g), fx_i2f(fx_lo(g)) * 0x1.0p-32f};
+}
+
+// |q| as a fraction of 2^(E + 1), E = the unbiased exponent of a number no smaller than |q| (eb: its
+// exponent field, 1 .. 2046), in units of 2^-55, rounded: exact for charges within a factor of 4 of it.
 __host__ __device__ inline unsigned long long fix_magnitude(unsigned long long qb, int eb)
 {
     const int e = (int)((qb >> 52) & 0x7ff);
     if (e == 0 || e > eb) return 0ull;  // zero or subnormal (below 2^-1022)
     const unsigned long long m = (qb & 0xFFFFFFFFFFFFFull) | (1ull << 52);
-    const int sh = 6 - (eb - e);  // m 2^(e - eb) 2^(58 - 52)
-    return sh >= 0 ? m << sh : (sh > -64 ? m >> -sh : 0ull);
+    const int sh = 2 - (eb - e);  // m 2^(e - eb) 2^(54 - 52)
+    return sh >= 0 ? m << sh : (sh > -55 ? (m + (1ull << (-sh - 1))) >> -sh : 0ull);
 }
 
 }  // namespace rbe

@@ -594,13 +594,13 @@ static Plan make_plan64(rbe_ctx ctx, int64_t N, int K)
     p.ksub = std::min(32, kRho64Threads / p.klanes);
     p.kthreads = 32 * ((p.ksub * p.klanes + 31) / 32);
     const int smem_bps = (int)((227 * 1024) / (kRho64Smem + 2048));
-    const int bps = std::max(1, std::min(smem_bps, 2 * kRho64Threads / p.kthreads));
+    const int bps = std::max(1, std::min(smem_bps, RBE_RHO64_MINB * kRho64Threads / p.kthreads));
     const int64_t want = std::max<int64_t>(1, (int64_t)ctx->num_sms * bps / p.ktiles);
     const int64_t least = 2 * p.ksub;
     p.nchunks = (int)std::min<int64_t>(want, std::max<int64_t>(1, (N + least - 1) / least));
     p.chunk_len = std::max<int64_t>(1, (N + p.nchunks - 1) / p.nchunks);
     p.nchunks = (int)std::max<int64_t>(1, (N + p.chunk_len - 1) / p.chunk_len);
-    const int64_t resident = (int64_t)ctx->num_sms * 4;
+    const int64_t resident = (int64_t)ctx->num_sms * RBE_FORCE64_MINB;
     double best = 1e300;
     for (int sl : {1, 2, 4, 8}) {
         const int64_t unit = kForce64Threads / sl, rounds = (N + unit - 1) / unit;
@@ -629,14 +629,6 @@ static rbe_status ensure_partials(rbe_ctx ctx, size_t need)
     return RBE_OK;
 }
 
-cudaError_t launch_trig_table(void* trig, cudaStream_t s)
-{
-    k_trig_table<<<(kTrigLen + 127) / 128, 128, 0, s>>>(static_cast<TrigEntry*>(trig));
-    return cudaGetLastError();
-}
-
-size_t trig_table_bytes() { return kTrigBytes; }
-
 // launch_evaluate_range on the FP64 path.
 static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* pos, const double* q, int koff, int K,
                                           bool forces, double* F, double* W, double* E)
@@ -658,20 +650,19 @@ static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* 
     const double* w = d.w + koff;
     const KState* ks = d.ks;
     double2* part = static_cast<double2*>(d.partials);
-    const TrigEntry* trig = static_cast<const TrigEntry*>(d.trig);
     cudaError_t err = launch_pdl(k_rho_f64, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem, s, pos, q, N, ks, m,
-                                 K, p.chunk_len, p.nchunks, part, trig, d.status, p.ksub, p.klanes);
+                                 K, p.chunk_len, p.nchunks, part, d.status, p.ksub, p.klanes);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f64");
     record_event(ctx, 2);
     int threads = 32;
     while (threads < kReduceThreads && threads * 4 < p.nchunks) threads *= 2;
-    err = launch_pdl(k_reduce_f64, dim3(K + 1), dim3(threads), 0, s, (const double2*)part, p.nchunks, K, m, w, ks, trig,
+    err = launch_pdl(k_reduce_f64, dim3(K + 1), dim3(threads), 0, s, (const double2*)part, p.nchunks, K, m, w, ks,
                      d.rho, d.terms, d.coef_d, d.status);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_reduce_f64");
     record_event(ctx, 3);
     auto force = p.ppt == 8 ? k_force_f64<8> : (p.ppt == 4 ? k_force_f64<4> : (p.ppt == 2 ? k_force_f64<2> : k_force_f64<1>));
     err = launch_pdl(force, dim3((forces ? p.fblocks : 0) + 1), dim3(kForce64Threads), kForce64Smem, s, pos, q, N,
-                     p.per_block, ks, m, (const double2*)d.coef_d, K, F, trig, d.status, (const double*)d.terms, W, E);
+                     p.per_block, ks, m, (const double2*)d.coef_d, K, F, d.status, (const double*)d.terms, W, E);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_force_f64");
     record_event(ctx, 4);
     ctx->last_K = K;

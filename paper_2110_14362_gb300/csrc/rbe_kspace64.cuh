@@ -2,38 +2,55 @@
 // cosine of rbe_fix64.cuh.  No FP64 instruction runs per pair; sums over particles and frequencies are
 // integers (exact, in any order), converted to double once per chunk or particle.
 //
-// What bounds them: a pair is about 120 instructions on the FMA and ALU pipes in either pass (a quarter of
-// them integer multiplications at half or quarter rate) and two random table loads from shared
-// memory; DRAM moves 32 to 56 B per particle.  Against FP64 sincospi per pair (about 35 FP64
-// instructions per pass, 76 clocks of a scheduler each): N = 3e5, P = 200 8330 -> 539 us per
-// evaluation, 1e6 x 500 67.8 -> 4.03 ms, 1e3 x 100 386 -> 21 us.
+// What bounds them: a pair is about 90 instructions on the FMA and ALU pipes in either pass, 5 or 6 of them
+// 64-bit products, and 25 bytes of random table loads from shared memory; at P = 500 a pair takes 106
+// clocks of a scheduler in the rho pass and 124 in the force pass (0.86 and 0.70 instructions per clock;
+// the force pass waits for the heavy FMA pipe, which the integer products run on); DRAM moves 32 to 56 B
+// per particle.  Against FP64 sincospi per pair (about 35 FP64 instructions per pass, 76 clocks of a
+// scheduler each): N = 3e5, P = 200 8330 -> 385 us per evaluation, 1e6 x 500 67.8 -> 2.87 ms, 1e3 x 100
+// 386 -> 20.5 us.
 #pragma once
+
+#include <type_traits>
 
 #include "rbe_fix64.cuh"
 #include "rbe_kspace_tiles.cuh"
 
 namespace rbe {
 
+// Resident blocks the registers are sized for, and the unrolling of the pair loops (slab, N = 3e5, P = 200:
+// rho 199 us unrolled by 2, 216 by 1, 205 by 4, 217 at one block of 128 registers; force 186 us by 4, 209
+// by 1, 197 by 2, 219 at three blocks of 80 registers, 242 at five of 48).
+#ifndef RBE_RHO64_MINB
+#define RBE_RHO64_MINB 2
+#endif
+#ifndef RBE_FORCE64_MINB
+#define RBE_FORCE64_MINB 4
+#endif
+#ifndef RBE_RHO64_UNROLL
+#define RBE_RHO64_UNROLL 2
+#endif
+#ifndef RBE_FORCE64_UNROLL
+#define RBE_FORCE64_UNROLL 4
+#endif
+constexpr int kRho64Unroll = RBE_RHO64_UNROLL, kForce64Unroll = RBE_FORCE64_UNROLL;
 constexpr int kRho64Threads = 512;   // threads of a rho block at most
 constexpr int kRho64Stage = 512;     // particles staged per tile at most (32 B each)
-constexpr int kRho64Group = 32;      // pairs whose products (below 2^57 each) are summed in 64 bits
+constexpr int kRho64Group = 32;      // pairs whose products (at most 2^57 each) are summed in 64 bits
 constexpr int kForce64Threads = 256;
-constexpr int kForce64Stage = 256;   // frequencies staged per tile (32 B each)
-constexpr size_t kTrigBytes = sizeof(TrigEntry) * kTrigLen;
-constexpr size_t kRho64Smem = kTrigBytes + 32 * (size_t)kRho64Stage;
-constexpr size_t kForce64Smem = kTrigBytes + 32 * (size_t)kForce64Stage;
+constexpr int kForce64Stage = 256;   // frequencies staged per tile (48 B each)
+constexpr size_t kRho64Trig = (sizeof(TrigEntry) + sizeof(TrigLow)) * kTrigN;  // planes entry and low
+constexpr size_t kForce64Trig = (sizeof(TrigSine) + sizeof(float)) * kTrigN;    // planes sine and sine_low
+constexpr size_t kRho64Smem = kRho64Trig + 32 * (size_t)kRho64Stage;
+constexpr size_t kForce64Smem = kForce64Trig + 48 * (size_t)kForce64Stage;
 
-__global__ void k_trig_table(TrigEntry* __restrict__ t)
-{
-    const int i = blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < kTrigLen) t[i] = trig_entry(i);
-}
+__device__ const TrigTable g_trig = make_trig_table();
 
-__device__ __forceinline__ void load_trig(const TrigEntry* __restrict__ trig, TrigEntry* s_trig)
+__device__ __forceinline__ void load_trig(const void* __restrict__ src_v, void* dst_v, int bytes)
 {
-    const uint4* src = reinterpret_cast<const uint4*>(trig);
-    uint4* dst = reinterpret_cast<uint4*>(s_trig);
-    for (int i = threadIdx.x; i < kTrigLen; i += blockDim.x) dst[i] = src[i];
+    const uint4* src = reinterpret_cast<const uint4*>(src_v);
+    uint4* dst = reinterpret_cast<uint4*>(dst_v);
+    for (int i = threadIdx.x; i < bytes / 16; i += blockDim.x) dst[i] = src[i];
 }
 
 // A 128-bit integer as the nearest double or next to it (two roundings), times 2^e.
@@ -76,26 +93,29 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double (*scratc
 // particle sub-streams over the particles of chunk c, staged kRho64Stage at a time as 64-bit
 // fixed-point positions and charges and read as broadcasts.
 //
-// Charges: |q| is taken as a 59-bit fraction of twice the power of two of the chunk's largest |q| (exact
-// for charges within 2^6 of it, an error of 2^-60 of the largest one below); the sign is half a
-// revolution of the phase.  A product then has units of 2^-57 of that power of two; 32 of them are
-// summed in 64 bits, the sums of 32 in 128.
+// Charges: |q| is taken as a 55-bit fraction qh 2^-27 + ql 2^-55 of twice the power of two of the chunk's
+// largest |q| (exact for charges within a factor of 4 of it, an error of 2^-56 of that power below); the
+// sign is half a revolution of the phase.  With the sine (or cosine) as v + w, v an integer in units of
+// 2^-30, a product takes two integer multiplications, v qh and v ql, summed in 64 bits over 32 pairs,
+// and one FP32 FMA for w qh (2^-57 of the charge at most, so the FP32 sum of 32 of them is good to
+// 2^-78); the groups' sums are added in 128 bits.  Where every charge of the staged tile has ql = 0 (27
+// significant bits do: integers, equal magnitudes that are a power of two) v ql is left out.
 // Partials: (Re, Im) at [l * nchunks + c]; row K holds the chunk's sum of q^2 in FP64.
-__global__ void __launch_bounds__(kRho64Threads, 2)
+__global__ void __launch_bounds__(kRho64Threads, RBE_RHO64_MINB)
 k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t N, const KState* __restrict__ ks,
           const int4* __restrict__ m, int K, int64_t chunk_len, int nchunks, double2* __restrict__ partials,
-          const TrigEntry* __restrict__ trig, unsigned* __restrict__ status, int S, int T)
+          unsigned* __restrict__ status, int S, int T)
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
     TrigEntry* st = reinterpret_cast<TrigEntry*>(s_raw);
-    int4* sp = reinterpret_cast<int4*>(s_raw + kTrigBytes);
+    int4* sp = reinterpret_cast<int4*>(s_raw + kRho64Trig);
     __shared__ int s_eb;
     __shared__ double s_red[2][32];
     const int tid = threadIdx.x, nt = blockDim.x, kt = blockIdx.x, c = blockIdx.y;
     const int64_t start = (int64_t)c * chunk_len, end = min(N, start + chunk_len);
     if (tid == 0) s_eb = 1;
     __syncthreads();
-    load_trig(trig, st);
+    load_trig(g_trig.entry, st, (int)kRho64Trig);
     // the largest exponent field of the chunk's charges, and the sum of their squares (inputs only)
     int eb = 1;
     double q2 = 0.0, zero = 0.0;
@@ -118,11 +138,14 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
     const bool act = ss < S && l < K;
     const int share = kRho64Stage / S, stage = share * S;
     const int4 mv = act ? m[l] : make_int4(0, 0, 0, 0);
+    const float mfx = (float)mv.x, mfy = (float)mv.y, mfz = (float)mv.z;
+    const TrigLow* sw = reinterpret_cast<const TrigLow*>(st + kTrigN);
     const FixScale scx = fs(ks->sc64[0]), scy = fs(ks->sc64[1]), scz = fs(ks->sc64[2]);
     __int128 re = 0, im = 0;
     for (int64_t base = start; base < end; base += stage) {
         __syncthreads();  // every thread is done with the previous tile
         const int here = (int)min((int64_t)stage, end - base);
+        int low = 0;
         for (int u = tid; u < here; u += nt) {
             const int64_t i = base + u;
             const unsigned long long bx = (unsigned long long)__double_as_longlong(pos[3 * i]);
@@ -130,40 +153,55 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
             const unsigned long long bz = (unsigned long long)__double_as_longlong(pos[3 * i + 2]);
             const unsigned long long bq = (unsigned long long)__double_as_longlong(q[i]);
             if (nonfinite_bits(bx) || nonfinite_bits(by) || nonfinite_bits(bz)) atomicOr(status, kStatusNonFinite);
-            // signed halves: 2^31 added, the low word's top bit flipped
-            const unsigned long long x = fixed_frac64(bx, scx) + kMulBias, y = fixed_frac64(by, scy) + kMulBias,
-                                     z = fixed_frac64(bz, scz) + kMulBias, a = fix_magnitude(bq, eb) + kMulBias;
-            sp[2 * u] = make_int4(fx_hi(x), fx_lo(x), fx_hi(y), fx_lo(y));
-            sp[2 * u + 1] = make_int4(fx_hi(z), fx_lo(z), (int)((uint32_t)fx_hi(a) | ((uint32_t)(bq >> 63) << 31)), fx_lo(a));
+            const Frac x = frac_of(fixed_frac64(bx, scx)), y = frac_of(fixed_frac64(by, scy)),
+                       z = frac_of(fixed_frac64(bz, scz));
+            const unsigned long long a = fix_magnitude(bq, eb) + (1ull << 27);
+            const int ql = (int)(a & 0xFFFFFFFull) - (1 << 27);
+            low |= ql;
+            sp[2 * u] = make_int4(x.hi, y.hi, z.hi, (int)((uint32_t)(a >> 28) | ((uint32_t)(bq >> 63) << 31)));
+            sp[2 * u + 1] = make_int4(__float_as_int(x.lo), __float_as_int(y.lo), __float_as_int(z.lo), ql);
         }
-        __syncthreads();
+        const bool has_low = __syncthreads_or(low) != 0;
         if (!act) continue;
         const int p1 = min(here, (ss + 1) * share);
-        for (int p = ss * share; p < p1; p += kRho64Group) {
-            const int n = min(kRho64Group, p1 - p);
-            unsigned long long ar = 0, ai = 0;
-#pragma unroll 2
+        auto group = [&](auto low_tag, int p, int n) {
+            constexpr bool LOW = decltype(low_tag)::value;
+            unsigned long long ar = 0, ai = 0, br = 0, bi = 0;
+            float cr = 0.0f, ci = 0.0f;
+#pragma unroll kRho64Unroll
             for (int u = p; u < p + n; ++u) {
                 const int4 a = sp[2 * u], b = sp[2 * u + 1];
-                unsigned long long t = mad_wide(mv.x, a.y, kPhaseStart);
-                t = mad_wide(mv.y, a.w, t);
-                t = mad_wide(mv.z, b.y, t);
-                uint32_t hi = (uint32_t)(t >> 32) + (uint32_t)mv.x * (uint32_t)a.x;
-                hi += (uint32_t)mv.y * (uint32_t)a.z;
-                hi += (uint32_t)mv.z * (uint32_t)b.x;
-                hi ^= (uint32_t)b.z & 0x80000000u;
-                const PhaseX x = phase_x(hi, (uint32_t)t);
-                const TrigEntry* e = st + (hi >> 21);
-                const TrigEntry es = e[0], ec = e[kTrigN / 4];
-                const unsigned long long vs = trig_value<1>(es.v, es.h, es.l, ec.h, ec.l, x);
-                const unsigned long long vc = trig_value<-1>(ec.v, ec.h, ec.l, es.h, es.l, x);
-                const int qh = b.z & 0x7fffffff, ql = b.w;
-                ar += mul_fix(fx_hi(vc), fx_lo(vc), qh, ql);
-                ai += mul_fix(fx_hi(vs), fx_lo(vs), qh, ql);
+                uint32_t hi = (uint32_t)mv.x * (uint32_t)a.x + kPhaseStart;
+                hi += (uint32_t)mv.y * (uint32_t)a.y;
+                hi += (uint32_t)mv.z * (uint32_t)a.z;
+                hi ^= (uint32_t)a.w & 0x80000000u;
+                const float lo = fmaf(mfx, __int_as_float(b.x), fmaf(mfy, __int_as_float(b.y), mfz * __int_as_float(b.z)));
+                const TrigEntry e = st[hi >> 21];
+                const TrigLow w = sw[hi >> 21];
+                const PhaseX x = phase_x(hi, lo);
+                const float sf = fx_i2f(e.sa), cf = fx_i2f(e.ca);
+                int sh, ch;
+                float sl, cl;
+                trig_value<1>(e.sa, sf, w.s, cf, w.c, x, sh, sl);
+                trig_value<-1>(e.ca, cf, w.c, sf, w.s, x, ch, cl);
+                const int qh = a.w & 0x7fffffff;
+                const float qf = fx_i2f(qh);
+                ar = mad_wide(ch, qh, ar);
+                ai = mad_wide(sh, qh, ai);
+                if (LOW) {
+                    br = mad_wide(ch, b.w, br);
+                    bi = mad_wide(sh, b.w, bi);
+                }
+                cr = fmaf(trig_low_f(e.cr, cl), qf, cr);
+                ci = fmaf(trig_low_f(e.sr, sl), qf, ci);
             }
-            const unsigned long long bias = (unsigned long long)n * kMulBias;
-            re += (long long)(ar - bias);
-            im += (long long)(ai - bias);
+            re += ((__int128)(long long)ar << 28) + (long long)br + __float2ll_rn(cr * 0x1.0p28f);
+            im += ((__int128)(long long)ai << 28) + (long long)bi + __float2ll_rn(ci * 0x1.0p28f);
+        };
+        for (int p = ss * share; p < p1; p += kRho64Group) {
+            const int n = min(kRho64Group, p1 - p);
+            if (has_low) group(std::true_type{}, p, n);
+            else group(std::false_type{}, p, n);
         }
     }
     __syncthreads();
@@ -182,7 +220,7 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
             }
     }
     if (act && ss == 0) {
-        const int e = eb - 1023 - 56;  // units of 2^-57 of 2^(eb - 1023 + 1)
+        const int e = eb - 1023 + 1 - 85;  // units of 2^-30 2^-55 of 2^(eb - 1023 + 1)
         partials[(size_t)l * nchunks + c] = make_double2(int128_to_double(re, e), int128_to_double(im, e));
     }
     if (kt == 0 && tid == 0) partials[(size_t)K * nchunks + c] = make_double2(q2, 0.0);
@@ -198,7 +236,7 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
 // table; and the remaining angle (below 2^-22) from Im(rho e^{-i phi}) / |rho|.
 __global__ void __launch_bounds__(kReduceThreads)
 k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int4* __restrict__ m,
-             const double* __restrict__ w, const KState* __restrict__ ks, const TrigEntry* __restrict__ trig,
+             const double* __restrict__ w, const KState* __restrict__ ks,
              double2* __restrict__ rho, double* __restrict__ terms, double2* __restrict__ coef,
              unsigned* __restrict__ status)
 {
@@ -240,16 +278,21 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
         const double cr = re * inv, ci = im * inv;  // (cos, sin) of arg rho
         const float rev = atan2f((float)ci, (float)cr) * 0.159154943f;
         phi = (unsigned long long)(long long)__float2int_rn(rev * 1073741824.0f) << 34;
-        const unsigned long long ph = phi + kPhaseStart;
-        const PhaseX x = phase_x((uint32_t)(ph >> 32), (uint32_t)ph);
-        const TrigEntry es = trig[ph >> 53], ec = trig[(ph >> 53) + kTrigN / 4];
-        const double s = (double)(long long)(trig_value<1>(es.v, es.h, es.l, ec.h, ec.l, x) - kMulBias);
-        const double co = (double)(long long)(trig_value<-1>(ec.v, ec.h, ec.l, es.h, es.l, x) - kMulBias);
-        // ci co - cr s = sin(arg rho - phi) in units of 2^62; revolutions in units of 2^-64: 4 / 2 pi
-        const double d = fma(ci, co, -(cr * s)) * 0.63661977236758134308;
+        const uint32_t ph = (uint32_t)(phi >> 32) + kPhaseStart;
+        const PhaseX x = phase_x(ph, 0.0f);
+        const TrigEntry te = g_trig.entry[ph >> 21];
+        const TrigLow tw = g_trig.low[ph >> 21];
+        const float sf = fx_i2f(te.sa), cf = fx_i2f(te.ca);
+        int sh, ch;
+        float sl, cl;
+        trig_value<1>(te.sa, sf, tw.s, cf, tw.c, x, sh, sl);
+        trig_value<-1>(te.ca, cf, tw.c, sf, tw.s, x, ch, cl);
+        const double s = (double)sh + (double)trig_low_f(te.sr, sl), co = (double)ch + (double)trig_low_f(te.cr, cl);
+        // ci co - cr s = sin(arg rho - phi) in units of 2^-30; revolutions in units of 2^-64: 2^34 / 2 pi
+        const double d = fma(ci, co, -(cr * s)) * 2734261102.3059327;
         phi += (unsigned long long)__double2ll_rn(d);
     }
-    coef[l] = make_double2(__longlong_as_double((long long)(kPhaseStart - phi)), R);
+    coef[l] = make_double2(__longlong_as_double((long long)(0ull - phi)), R);
 }
 
 // =================================================================================
@@ -257,13 +300,13 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
 // A block takes rounds of kForce64Threads / SL particles (lanes) with the frequencies of a staged tile split
 // over SL slices, whose integer sums are added at the end of the round: SL > 1 spreads small systems
 // over the GPU.  Per staged tile the amplitudes R_l become integers: scaled so that sum_l |m_l| R_l
-// (an FP32 bound, rounded up) is below 2^62, each product R sin is rounded to 2^-60 of that sum.
+// (an FP32 bound, rounded up) is below 2^60, each product R sin is rounded to 2^-60 of that sum.
 // The launch carries one extra block that computes the energy and virial sums (final_sums) meanwhile.
 template <int SL>
-__global__ void __launch_bounds__(kForce64Threads, 4)
+__global__ void __launch_bounds__(kForce64Threads, RBE_FORCE64_MINB)
 k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t N, int64_t per_block,
             const KState* __restrict__ ks, const int4* __restrict__ mk, const double2* __restrict__ coef, int K,
-            double* __restrict__ F, const TrigEntry* __restrict__ trig, unsigned* __restrict__ status,
+            double* __restrict__ F, unsigned* __restrict__ status,
             const double* __restrict__ terms, double* __restrict__ W_out, double* __restrict__ E_out)
 {
     if (blockIdx.x == gridDim.x - 1) {
@@ -273,14 +316,16 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
     }
     constexpr int PB = kForce64Threads / SL;
     extern __shared__ __align__(16) unsigned char s_raw[];
-    TrigEntry* st = reinterpret_cast<TrigEntry*>(s_raw);
-    int4* sk = reinterpret_cast<int4*>(s_raw + kTrigBytes);  // (mx, my, mz, R low), (phase low, high, R high, 0)
+    TrigSine* st = reinterpret_cast<TrigSine*>(s_raw);
+    const float* sw = reinterpret_cast<const float*>(st + kTrigN);
+    // per frequency: (mx, my, mz, phase high), the same m as floats and the phase low, (R high, R low)
+    int4* sk = reinterpret_cast<int4*>(s_raw + kForce64Trig);
     __shared__ unsigned long long s_sum[SL > 1 ? 3 : 1][SL > 1 ? kForce64Threads : 1];
     __shared__ int s_e;
     __shared__ float s_b[3][kForce64Threads / 32];
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int pl = tid % PB, sl = tid / PB;
-    load_trig(trig, st);
+    load_trig(g_trig.sine, st, (int)kForce64Trig);
     pdl_wait();  // (ks: see k_rho_f64)
     const FixScale scx = fs(ks->sc64[0]), scy = fs(ks->sc64[1]), scz = fs(ks->sc64[2]);
     const double cx = 2.0 * kPi * ks->inv[0], cy = 2.0 * kPi * ks->inv[1], cz = 2.0 * kPi * ks->inv[2];
@@ -289,13 +334,12 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
     int sh = 0;  // R as an integer is R 2^sh
     for (int64_t base = b0; base < b1; base += PB) {
         const int64_t i = base + pl;
-        unsigned long long x = 0, y = 0, z = 0;
+        Frac x{0, 0.0f}, y{0, 0.0f}, z{0, 0.0f};
         if (i < b1) {
-            x = fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i]), scx) + kMulBias;
-            y = fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i + 1]), scy) + kMulBias;
-            z = fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i + 2]), scz) + kMulBias;
+            x = frac_of(fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i]), scx));
+            y = frac_of(fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i + 1]), scy));
+            z = frac_of(fixed_frac64((unsigned long long)__double_as_longlong(pos[3 * i + 2]), scz));
         }
-        const int xh = fx_hi(x), xl = fx_lo(x), yh = fx_hi(y), yl = fx_lo(y), zh = fx_hi(z), zl = fx_lo(z);
         double fx = 0.0, fy = 0.0, fz = 0.0;
         for (int k0 = 0; k0 < K; k0 += kForce64Stage) {
             const int nk = min(kForce64Stage, K - k0);
@@ -343,16 +387,18 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
                 // the bound, at least 2 (the largest R itself), rounded up well above the FP32 sums' error
                 const float bound = fmaxf(2.0f, fmaxf(bx, fmaxf(by, bz)) * 1.0001f);
                 const int lg = (int)((__float_as_uint(bound) >> 23) & 0xffu) - 127 + 1;  // bound < 2^lg
-                sh = 62 - lg + 1023 - er;  // sum |m| R 2^sh < 2^62
+                sh = 60 - lg + 1023 - er;  // sum |m| R 2^sh < 2^60
                 if (tid < nk) {
                     // R 2^sh = mantissa 2^(e - 1075 + sh)
                     const unsigned long long mant = e > 0 ? (rb & 0xFFFFFFFFFFFFFull) | (1ull << 52) : 0ull;
                     const int k = e - 1075 + sh;
                     const unsigned long long A =
-                        (k >= 0 ? mant << min(k, 63) : (k > -64 ? mant >> -k : 0ull)) + kMulBias;
-                    const unsigned long long off = (unsigned long long)__double_as_longlong(co.x);
-                    sk[2 * tid] = make_int4(mm.x, mm.y, mm.z, fx_lo(A));
-                    sk[2 * tid + 1] = make_int4((int)(uint32_t)off, (int)(uint32_t)(off >> 32), fx_hi(A), 0);
+                        (k >= 0 ? mant << min(k, 63) : (k > -64 ? mant >> -k : 0ull)) + (1ull << 29);
+                    const Frac off = frac_of((unsigned long long)__double_as_longlong(co.x));
+                    sk[3 * tid] = make_int4(mm.x, mm.y, mm.z, (int)((uint32_t)off.hi + kPhaseStart));
+                    sk[3 * tid + 1] = make_int4(__float_as_int((float)mm.x), __float_as_int((float)mm.y),
+                                                __float_as_int((float)mm.z), __float_as_int(off.lo));
+                    sk[3 * tid + 2] = make_int4((int)(A >> 30), (int)(A & 0x3FFFFFFFull) - (1 << 29), 0, 0);
                 }
                 __syncthreads();
             }
@@ -360,21 +406,22 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
             uint32_t hx = 0, hy = 0, hz = 0;
             const int per = SL > 1 ? (nk + SL - 1) / SL : nk;
             const int l1 = SL > 1 ? min(nk, (sl + 1) * per) : nk;
-#pragma unroll 2
+#pragma unroll kForce64Unroll
             for (int l = SL > 1 ? sl * per : 0; l < l1; ++l) {
-                const int4 a = sk[2 * l], b = sk[2 * l + 1];
-                unsigned long long t = mad_wide(a.x, xl, ((unsigned long long)(uint32_t)b.y << 32) | (uint32_t)b.x);
-                t = mad_wide(a.y, yl, t);
-                t = mad_wide(a.z, zl, t);
-                uint32_t hi = (uint32_t)(t >> 32) + (uint32_t)a.x * (uint32_t)xh;
-                hi += (uint32_t)a.y * (uint32_t)yh;
-                hi += (uint32_t)a.z * (uint32_t)zh;
-                const PhaseX p = phase_x(hi, (uint32_t)t);
-                const TrigEntry* e = st + (hi >> 21);
-                const TrigEntry es = e[0];
-                const float2 ec = *reinterpret_cast<const float2*>(&e[kTrigN / 4].h);
-                const unsigned long long v = trig_value<1>(es.v, es.h, es.l, ec.x, ec.y, p);
-                const unsigned long long h = mul_fix(fx_hi(v), fx_lo(v), b.z, a.w);
+                const int4 a = sk[3 * l], b = sk[3 * l + 1];
+                const int2 r = *reinterpret_cast<const int2*>(sk + 3 * l + 2);
+                uint32_t hi = (uint32_t)a.x * (uint32_t)x.hi + (uint32_t)a.w;
+                hi += (uint32_t)a.y * (uint32_t)y.hi;
+                hi += (uint32_t)a.z * (uint32_t)z.hi;
+                const float lo = fmaf(__int_as_float(b.x), x.lo,
+                                      fmaf(__int_as_float(b.y), y.lo, fmaf(__int_as_float(b.z), z.lo, __int_as_float(b.w))));
+                const TrigSine e = st[hi >> 21];
+                const float vl0 = sw[hi >> 21];
+                const PhaseX p = phase_x(hi, lo);
+                int vh;
+                float vl;
+                trig_value<1>(e.sa, fx_i2f(e.sa), vl0, e.ch, e.cl, p, vh, vl);
+                const unsigned long long h = mul_fix(vh, trig_low_i(e.sr, vl), r.x, r.y);
                 const int hh = fx_hi(h), hl = fx_lo(h);
                 ax = mad_wide(a.x, hl, ax);
                 ay = mad_wide(a.y, hl, ay);
@@ -400,9 +447,9 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
                         az += s_sum[2][s * PB + pl];
                     }
             }
-            // units of 2^-62 (sine) times 2^64 (product's high half) over 2^sh
+            // units of 2^-30 (sine) times 2^30 (mul_fix's) over 2^sh
             if (sl == 0 && i < b1) {
-                const double u = ldexp(1.0, 2 - sh);
+                const double u = ldexp(1.0, -sh);
                 fx += u * (double)(long long)ax;
                 fy += u * (double)(long long)ay;
                 fz += u * (double)(long long)az;

@@ -23,13 +23,14 @@ def fix64():
 
     def run(lines):
         res = subprocess.run([EXE], input="\n".join(lines) + "\n", capture_output=True, text=True, check=True)
-        return [[int(x) for x in ln.split()] for ln in res.stdout.splitlines()]
+        return [[float(x) if "." in x or "e" in x else int(x) for x in ln.split()] for ln in res.stdout.splitlines()]
     return run
 
 
 def test_sine_and_cosine(fix64):
-    """Within 2^-51 (the low part's grid 2^-53 and a few float-float roundings below it), the exact
-    negative half a revolution on, at random phases and around every table boundary."""
+    """Within 2^-51 in either form of the remainder (the phase's FP32 part 2^-58 revolutions, the remainder's
+    rounding 2^-54, a few float-float roundings of that size), the exact negative half a revolution on, at
+    random phases and around table boundaries."""
     mp = pytest.importorskip("mpmath")
     mp.mp.prec = 120
     rng = np.random.default_rng(1)
@@ -39,11 +40,14 @@ def test_sine_and_cosine(fix64):
     ps = [p % 2**64 for p in ps]
     got = fix64([f"T {p:x}" for p in ps])
     opp = fix64([f"T {(p + 2**63) % 2**64:x}" for p in ps])
-    for p, (s, c), (s2, c2) in zip(ps, got, opp):
+    bound = mp.mpf(2) ** -51
+    for p, v, w in zip(ps, got, opp):
         a = 2 * mp.pi * mp.mpf(p) / 2**64
-        assert abs(mp.mpf(s) / 2**62 - mp.sin(a)) < mp.mpf(2) ** -51, hex(p)
-        assert abs(mp.mpf(c) / 2**62 - mp.cos(a)) < mp.mpf(2) ** -51, hex(p)
-        assert (s2, c2) == (-s, -c), hex(p)
+        for (h, f, i), exact in ((v[:3], mp.sin(a)), (v[3:], mp.cos(a))):
+            assert abs((h + mp.mpf(f)) / 2**30 - exact) < bound, hex(p)
+            assert abs((h + mp.mpf(i) / 2**24) / 2**30 - exact) < bound, hex(p)
+            assert abs(f) < 1.8
+        assert w == [-x for x in v], hex(p)
 
 
 def test_fractions(fix64):
@@ -60,15 +64,16 @@ def test_fractions(fix64):
 
 
 def test_products(fix64):
-    """a |b| to one unit plus the truncation of |b| to 59 bits, and exactly antisymmetric in a for a power
-    of two."""
+    """Products to 1.3 units (half of the rounding, and up to 0.7 of the left-out product of the low
+    words); charges to half a unit of their 55 bits and exact within a factor of 4."""
     rng = np.random.default_rng(3)
-    cases = [(int(a) - 2**61, float(b), -1) for a, b in zip(rng.integers(0, 2**62, 500), rng.uniform(0.0, 1.0, 500))]
-    cases += [(2**62 - 1, 0.8476, -1), (-2**62 + 1, 1.0, 0), (2**62 - 1, 1e-3, -1), (12345, 0.0, 0), (-5, 5e-324, 0)]
-    got = fix64([f"M {a} {b!r} {e}" for a, b, e in cases])
-    for (a, b, e), (g,) in zip(cases, got):
-        assert abs(Fraction(a, 2**62) * Fraction(b) / Fraction(2) ** (e + 1) * 2**57 - g) <= 1.25, (a, b, e)
-    odd = [int(a) | 1 for a in rng.integers(0, 2**62, 300)]
-    pos = fix64([f"M {a} 1.0 0" for a in odd])
-    neg = fix64([f"M {-a} 1.0 0" for a in odd])
-    assert all(x == -y for (x,), (y,) in zip(pos, neg))
+    cases = [(int(h), int(l), int(b)) for h, l, b in zip(rng.integers(-2**30, 2**30, 500),
+                                                         rng.integers(-20_000_000, 20_000_000, 500),
+                                                         rng.integers(0, 2**60, 500))]
+    cases += [(2**30, 21_000_000, 2**60 - 2**29 - 1), (-2**30, -21_000_000, 2**60 - 2**29 - 1), (5, 7, 0), (0, 0, 2**59)]
+    for (h, l, b), (g,) in zip(cases, fix64([f"M {h} {l} {b}" for h, l, b in cases])):
+        assert abs((h + Fraction(l, 2**24)) * Fraction(b, 2**30) - g) <= 1.3, (h, l, b)
+    qs = [(float(q), e) for q in rng.uniform(0.0, 2.0, 200) for e in (0, 3, 40)] + [(1.0, 0), (0.0, 0), (5e-324, 0)]
+    for (q, e), (g,) in zip(qs, fix64([f"Q {q!r} {e}" for q, e in qs])):
+        d = abs(Fraction(q) * Fraction(2) ** (54 - e) - g)
+        assert d <= Fraction(1, 2) and (d == 0 or q < 2.0 ** (e - 1)), (q, e)
