@@ -74,6 +74,12 @@ struct NptBuffers {
     int* sorted = nullptr;         // N particle indices grouped by cell, by index within a cell
     float4* spos32 = nullptr;      // N packed FP32 positions+charge in sorted order
     double4_32a* spos64 = nullptr; // N packed FP64 positions+charge (FP64 path)
+    // FP64 path: the pair terms' tables (rbe_pair64.cuh) and the parameters each was built for; a table is
+    // never rewritten (a captured step may hold it), so a context keeps a few and no more
+    static constexpr int kPairTabs = 8;
+    void* pair_tab[kPairTabs] = {};
+    double pair_key[kPairTabs][5] = {};
+    int pair_tabs = 0;
     double2* mprop = nullptr;      // N (1/m, sqrt(m)), set by rbe_npt_init
     void* cellc = nullptr;         // cell-list constants of the current box (rbe_npt.cu)
     int* nbr = nullptr;            // neighbour list: slots of the neighbours of slot u at [u * nbr_cap, ...)
@@ -210,6 +216,9 @@ rbe_status npt_step_phase(rbe_ctx ctx, rbe_system* sys, int phase);
 // constants in npt.cellc (nls: the neighbour-list state or NULL).
 rbe_status npt_ensure(rbe_ctx ctx, int64_t N, const double box[3], double rc, double skin);
 int pair_blocks(rbe_ctx ctx, int64_t N, bool fp64);
+int pair_blocks64(rbe_ctx ctx, int64_t N);
+struct Pair64Const;
+rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out);
 rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls, bool fp64);
 // Shared with the rigid-water step (rbe_npt.cu): parameter checks, the setup of rbe_npt_init
 // before its first forces, the device step index, the isotropic cell part of a step.

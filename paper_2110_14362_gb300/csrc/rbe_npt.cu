@@ -21,13 +21,15 @@
 
 #include <algorithm>
 #include <climits>
-#include <type_traits>
 #include <cmath>
+#include <cstring>
 #include <string>
+#include <type_traits>
 
 #include "rbe_context.h"
 #include "rbe_device.cuh"
 #include "rbe_npt_common.cuh"
+#include "rbe_pair64.cuh"
 
 namespace rbe {
 
@@ -659,7 +661,7 @@ k_cl_sort(const CellConsts* __restrict__ cc, const int* __restrict__ cnt, const 
 //   Search: FP32 positions; a candidate within the cutoff (FP64 path: within rc plus a
 //   margin above the FP32 rounding of the distance) is appended to the warp's buffer in
 //   shared memory (ballot order, so the order is fixed).
-//   Evaluation: every 32 buffered candidates, one per lane; the FP64 path recomputes the
+//   Evaluation: every 32 buffered candidates, one per lane; the FP64 path (k_pair64) recomputes the
 //   distance from the FP64 positions and applies the exact cutoff.
 //   f = -(dU/dr)/r for U = qqr2e q_i q_j erfc(sqrt(a) r)/r + 4 eps ((s/r)^12 - (s/r)^6); the
 //   lane sums go through a fixed shuffle tree, so the result does not depend on timing.  The
@@ -673,6 +675,8 @@ k_cl_sort(const CellConsts* __restrict__ cc, const int* __restrict__ cnt, const 
 // the list radius and write the list (only on a rebuild step), evaluate the listed pairs.
 enum PairMode { kPairCells = 0, kPairBuild = 1, kPairList = 2 };
 
+constexpr int kPairNoShift = 1 | (1 << 2) | (1 << 4);  // image code (two bits per axis, shift + 1) of no shift
+
 // Neighbour-list arguments of the pair kernel (unused without a list).
 struct ListArgs {
     NListState* nls;
@@ -683,46 +687,40 @@ struct ListArgs {
     int cap;
 };
 
-template <bool kF64, int kMode, bool kDiag = false>
-__global__ void __launch_bounds__(kPairWarps * 32, kF64 ? kPairBlocksPerSM64 : kPairBlocksPerSM)
+template <int kMode, bool kDiag = false>
+__global__ void __launch_bounds__(kPairWarps * 32, kPairBlocksPerSM)
 k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const int* __restrict__ cid,
        const int* __restrict__ cnt,
        const int* __restrict__ start, const int* __restrict__ sorted, const float4* __restrict__ spos32,
-       const double4_32a* __restrict__ spos64, double* __restrict__ Fr, double* __restrict__ partials,
-       const ListArgs la)
+       double* __restrict__ Fr, double* __restrict__ partials, const ListArgs la)
 {
-    using R = typename std::conditional<kF64, double, float>::type;
-    using Hit = typename std::conditional<kF64, int2, float4>::type;  // FP64: (slot, image code)
+    using R = float;
+    using Hit = float4;
     constexpr bool kBuild = kMode == kPairBuild, kList = kMode == kPairList;
     if (kBuild && !la.nls->rebuild) return;  // the list stands (the same for every thread)
     __shared__ Hit hits[kPairWarps][kHitCap];
     __shared__ double red[kDiag ? 5 : 3][kPairWarps];
-    __shared__ double sL[3], sInvL[3];
     __shared__ float sLf[3], sInvLf[3], sPass;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     // box constants once per block (shared memory)
     if (threadIdx.x < 3) {
-        sL[threadIdx.x] = cc->L[threadIdx.x];
-        sInvL[threadIdx.x] = cc->invL[threadIdx.x];
         sLf[threadIdx.x] = cc->Lf[threadIdx.x];
         sInvLf[threadIdx.x] = cc->invLf[threadIdx.x];
     } else if (threadIdx.x == 32) {
-        // FP64 path: the FP32 search keeps candidates within rc plus 2^-16 l_max, far above
-        // the FP32 rounding of a distance, and the exact cutoff is applied in FP64.  A build
-        // keeps every candidate within rl plus the same margin (a superset is harmless).
+        // a build keeps every candidate within rl plus 2^-16 l_max, far above the FP32 rounding of a
+        // distance (a superset is harmless)
         if (kBuild) {
             const double lmax = fmax(cc->L[0], fmax(cc->L[1], cc->L[2]));
             const double rp = (double)la.nls->rl + lmax * 0x1.0p-16;
             sPass = (float)(rp * rp);
         } else {
-            sPass = kF64 ? cc->pass64 : pc.rc2f;
+            sPass = pc.rc2f;
         }
     }
     __syncthreads();
     const int nc[3] = {cc->nc[0], cc->nc[1], cc->nc[2]};
-    // this warp's particles (lane 0): FP64 sums on the FP64 path; float-float sums on the FP32
-    // path, where no per-particle FP64 instruction runs (each costs a whole warp issue slot on
-    // GB300's narrow FP64 pipe)
+    // this warp's particles (lane 0): float-float sums, so that no per-particle FP64 instruction runs
+    // (each costs a whole warp many issue slots on GB300's narrow FP64 pipe)
     double wsum = 0.0, ecsum = 0.0, elsum = 0.0;
     float wh = 0.f, wl = 0.f, ech = 0.f, ecl = 0.f, elh = 0.f, ell = 0.f;
     // kDiag: w, wsum, (wh, wl) hold the x part of the virial; y and z here
@@ -736,8 +734,6 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
                  j += (int64_t)gridDim.x * blockDim.x)
                 Fr[j] = 0.0;
     } else {
-        const double* L = sL;
-        const double* invL = sInvL;
         const float* Lf = sLf;
         const float* invLf = sInvLf;
         // nearest image per pair on the axes with fewer than 3 cells, and on all axes for the
@@ -745,35 +741,18 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
         const bool mi[3] = {kList || nc[0] < 3, kList || nc[1] < 3, kList || nc[2] < 3};
         const float rc2_pass = sPass;
         R rc2, sa, aR, two_sa_pi, qk, s2, e4, e24;
-        if constexpr (kF64) {
-            rc2 = pc.rc2, sa = pc.sa, aR = pc.a, two_sa_pi = pc.two_sa_pi;
-            qk = pc.qk, s2 = pc.s2, e4 = pc.e4, e24 = pc.e24;
-        } else {
-            rc2 = pc.rc2f, sa = pc.saf, aR = pc.af, two_sa_pi = pc.two_sa_pif;
-            qk = pc.qkf, s2 = pc.s2f, e4 = pc.e4f, e24 = pc.e24f;
-        }
+        rc2 = pc.rc2f, sa = pc.saf, aR = pc.af, two_sa_pi = pc.two_sa_pif;
+        qk = pc.qkf, s2 = pc.s2f, e4 = pc.e4f, e24 = pc.e24f;
         const bool lj = pc.lj != 0;
         const int nwarps = gridDim.x * kPairWarps;
         for (int u = blockIdx.x * kPairWarps + wib; u < (int)N; u += nwarps) {
             const int i = sorted[u];
             const float4 me = spos32[u];
-            R xi, yi, zi, qi;
-            if constexpr (kF64) {
-                const double4_32a m64 = spos64[u];
-                xi = m64.x;
-                yi = m64.y;
-                zi = m64.z;
-                qi = m64.w;
-            } else {
-                xi = me.x;
-                yi = me.y;
-                zi = me.z;
-                qi = me.w;
-            }
+            const R qi = me.w;
             // Segments, one per lane (lanes 0..17): row r = lane / 2 of the 3 x 3 rows (dy, dz),
             // part lane % 2 (a row that wraps in x has two parts).  Each lane finds its slot
             // range [lo, hi), its image (sx, sy, sz) and the search centre me - shift.
-            int lo = 0, hi = 0, code = 0;
+            int lo = 0, hi = 0;
             float ctx = 0.f, cty = 0.f, ctz = 0.f;
             if (!kList) {
                 const int c = cid[i];
@@ -805,7 +784,6 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
                     if (a >= 0) {
                         lo = start[row + a];
                         hi = start[row + e] + cnt[row + e];
-                        code = (sx + 1) | ((sy + 1) << 2) | ((sz + 1) << 4);
                         ctx = me.x - (float)sx * Lf[0];
                         cty = me.y - (float)sy * Lf[1];
                         ctz = me.z - (float)sz * Lf[2];
@@ -819,40 +797,13 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
             auto evaluate = [&](int count, int base = 0) {
                 if (lane >= count) return;
                 const Hit h = hits[wib][base + lane];
-                R dx, dy, dz, qj;
-                if constexpr (kF64) {
-                    const double4_32a o = spos64[h.x];
-                    const int cd = h.y;
-                    dx = (o.x - xi) + (double)((cd & 3) - 1) * L[0];
-                    dy = (o.y - yi) + (double)(((cd >> 2) & 3) - 1) * L[1];
-                    dz = (o.z - zi) + (double)(((cd >> 4) & 3) - 1) * L[2];
-                    if (mi[0]) dx -= L[0] * rint(dx * invL[0]);
-                    if (mi[1]) dy -= L[1] * rint(dy * invL[1]);
-                    if (mi[2]) dz -= L[2] * rint(dz * invL[2]);
-                    qj = o.w;
-                } else {
-                    dx = h.x;
-                    dy = h.y;
-                    dz = h.z;
-                    qj = h.w;
-                }
+                const R dx = h.x, dy = h.y, dz = h.z, qj = h.w;
                 const R r2 = dx * dx + dy * dy + dz * dz;
                 if (!(r2 < rc2)) return;
-                R inv_r, r, ex;
-                if constexpr (kF64) {
-                    r = sqrt(r2);
-                    inv_r = 1.0 / r;
-                    ex = exp(-aR * r2);
-                } else {
-                    inv_r = rsqrtf(r2);
-                    r = r2 * inv_r;
-                    ex = __expf(-aR * r2);
-                }
+                const R inv_r = rsqrtf(r2), r = r2 * inv_r, ex = __expf(-aR * r2);
                 const R inv_r2 = inv_r * inv_r;
                 const R coul = qk * qi * qj * inv_r;  // qqr2e q_i q_j / r
-                R er;
-                if constexpr (kF64) er = erfc(sa * r);
-                else er = erfc_nr(sa * r);
+                const R er = erfc_nr(sa * r);
                 ec += coul * er;
                 R f = coul * (er + two_sa_pi * r * ex) * inv_r2;
                 if (lj) {
@@ -876,7 +827,7 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
             // the search over one segment; MI: some axis has fewer than 3 cells (nearest image
             // per candidate there).  The loop body has no divergent branch: out-of-range lanes
             // load an in-range slot and are masked out of the hit.
-            auto search = [&](auto mi_tag, int glo, int ghi, int gcode, float gx, float gy, float gz) {
+            auto search = [&](auto mi_tag, int glo, int ghi, float gx, float gy, float gz) {
                 constexpr bool MI = decltype(mi_tag)::value;
                 for (int s0 = glo; s0 < ghi; s0 += 32) {
                     const int s = s0 + lane;
@@ -900,8 +851,7 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
                     }
                     if (hit) {
                         const int p = nh + __popc(m & ((1u << lane) - 1u));
-                        if constexpr (kF64) hits[wib][p] = make_int2(s, gcode);
-                        else hits[wib][p] = make_float4(dx, dy, dz, o.w);
+                        hits[wib][p] = make_float4(dx, dy, dz, o.w);
                     }
                     nh += __popc(m);
                     if (nh >= 32) {
@@ -942,8 +892,7 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
                         const unsigned m = __ballot_sync(0xffffffffu, hit);
                         if (hit) {
                             const int p = nh + __popc(m & ((1u << lane) - 1u));
-                            if constexpr (kF64) hits[wib][p] = make_int2(sj[a], 1 | (1 << 2) | (1 << 4));  // no shift
-                            else hits[wib][p] = make_float4(dx, dy, dz, o[a].w);
+                            hits[wib][p] = make_float4(dx, dy, dz, o[a].w);
                         }
                         nh += __popc(m);
                     }
@@ -961,11 +910,10 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
                 for (int g = 0; g < 18; ++g) {
                     const int glo = __shfl_sync(0xffffffffu, lo, g), ghi = __shfl_sync(0xffffffffu, hi, g);
                     if (glo >= ghi) continue;  // the same for every lane
-                    const int gcode = __shfl_sync(0xffffffffu, code, g);
                     const float gx = __shfl_sync(0xffffffffu, ctx, g), gy = __shfl_sync(0xffffffffu, cty, g),
                                 gz = __shfl_sync(0xffffffffu, ctz, g);
-                    if (any_mi) search(std::true_type{}, glo, ghi, gcode, gx, gy, gz);
-                    else search(std::false_type{}, glo, ghi, gcode, gx, gy, gz);
+                    if (any_mi) search(std::true_type{}, glo, ghi, gx, gy, gz);
+                    else search(std::false_type{}, glo, ghi, gx, gy, gz);
                 }
             }
             if constexpr (kBuild) {
@@ -993,31 +941,18 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
                 el += __shfl_xor_sync(0xffffffffu, el, off);
             }
             if (lane == 0) {
-                if constexpr (kF64) {
-                    Fr[3 * (int64_t)i] = fx;
-                    Fr[3 * (int64_t)i + 1] = fy;
-                    Fr[3 * (int64_t)i + 2] = fz;
-                    wsum += 0.5 * w;
-                    if constexpr (kDiag) {
-                        wysum += 0.5 * wy;
-                        wzsum += 0.5 * wz;
-                    }
-                    ecsum += 0.5 * ec;
-                    elsum += 0.5 * el;
-                } else {
-                    // exact widening by integer operations
-                    unsigned long long* Fb = reinterpret_cast<unsigned long long*>(Fr);
-                    Fb[3 * (int64_t)i] = float_to_double_bits(__float_as_uint(fx));
-                    Fb[3 * (int64_t)i + 1] = float_to_double_bits(__float_as_uint(fy));
-                    Fb[3 * (int64_t)i + 2] = float_to_double_bits(__float_as_uint(fz));
-                    ff_add(wh, wl, 0.5f * w);
-                    if constexpr (kDiag) {
-                        ff_add(wyh, wyl, 0.5f * wy);
-                        ff_add(wzh, wzl, 0.5f * wz);
-                    }
-                    ff_add(ech, ecl, 0.5f * ec);
-                    ff_add(elh, ell, 0.5f * el);
+                // exact widening by integer operations
+                unsigned long long* Fb = reinterpret_cast<unsigned long long*>(Fr);
+                Fb[3 * (int64_t)i] = float_to_double_bits(__float_as_uint(fx));
+                Fb[3 * (int64_t)i + 1] = float_to_double_bits(__float_as_uint(fy));
+                Fb[3 * (int64_t)i + 2] = float_to_double_bits(__float_as_uint(fz));
+                ff_add(wh, wl, 0.5f * w);
+                if constexpr (kDiag) {
+                    ff_add(wyh, wyl, 0.5f * wy);
+                    ff_add(wzh, wzl, 0.5f * wz);
                 }
+                ff_add(ech, ecl, 0.5f * ec);
+                ff_add(elh, ell, 0.5f * el);
             }
         }
     }
@@ -1032,14 +967,12 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
     }
     // fixed-order block sums
     if (lane == 0) {
-        if (!kF64) {
-            wsum = (double)wh + (double)wl;
-            ecsum = (double)ech + (double)ecl;
-            elsum = (double)elh + (double)ell;
-            if (kDiag) {
-                wysum = (double)wyh + (double)wyl;
-                wzsum = (double)wzh + (double)wzl;
-            }
+        wsum = (double)wh + (double)wl;
+        ecsum = (double)ech + (double)ecl;
+        elsum = (double)elh + (double)ell;
+        if (kDiag) {
+            wysum = (double)wyh + (double)wyl;
+            wzsum = (double)wzh + (double)wzl;
         }
         constexpr int o = kDiag ? 2 : 0;
         red[0][wib] = wsum;
@@ -1057,6 +990,173 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
         for (int wv = 0; wv < kPairWarps; ++wv) t += red[threadIdx.x][wv];
         partials[kPartStride * (size_t)blockIdx.x + (kDiag ? 3 : 1) + threadIdx.x] = t;
     }
+}
+
+// ---------------------------------------------------------------------------------
+// The FP64 path's evaluation (from a cell search, or the list): the search of k_pair in FP32 with rc plus
+// a margin above the FP32 rounding of a distance, the hits as (slot, image code); their separations, the
+// cutoff and the sums in FP64, the pair terms from the tables of rbe_pair64.cuh.  One block of
+// kPair64Warps warps per SM shares the table; each block takes a contiguous run of slots.
+//
+// What bounds it: the FP64 pipe still (about 20 instructions of 76 clocks per 32 pairs, against about 115
+// with sqrt, exp, erfc and divisions), with the float-float polynomials beside it: N = 2e4, rc = 7 A, list
+// of 8 A: 875 -> 169 us; 9000 water sites, rc = 10 A, from the cells (k_water_pair): 1021 -> 261 us.  The image of a pair is
+// taken from the search (an addition of +-l only where some lane has one) except on an axis with fewer
+// than 3 cells, or, from a list, one whose half is within 0.1 % of rc, where the nearest image is rounded
+// in FP64.
+template <int kMode, bool kDiag>
+__global__ void __launch_bounds__(kPair64Warps * 32, 1)
+k_pair64(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, double rc, const int* __restrict__ cid,
+         const int* __restrict__ cnt, const int* __restrict__ start, const int* __restrict__ sorted,
+         const float4* __restrict__ spos32, const double4_32a* __restrict__ spos64, double* __restrict__ Fr,
+         double* __restrict__ partials, const ListArgs la)
+{
+    constexpr bool kList = kMode == kPairList;
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    PairWord* tab = reinterpret_cast<PairWord*>(s_raw);
+    __shared__ int2 hits[kPair64Warps][kHitCap];
+    __shared__ double red[kDiag ? 5 : 3][kPair64Warps];
+    const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    load_pair_table(pc.tab, tab);
+    Pair64Sums<kDiag> s{};
+    // no cell list this step (box beyond the cell arrays, flagged), or no list built yet
+    const bool cells_ok = kList ? la.nls->force == 0 : cc->ncell >= 0;
+    __syncthreads();
+    if (!cells_ok) {
+        for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < 3 * N; j += (int64_t)gridDim.x * blockDim.x)
+            Fr[j] = 0.0;
+    } else {
+        const double L[3] = {cc->L[0], cc->L[1], cc->L[2]};
+        const float Lf[3] = {cc->Lf[0], cc->Lf[1], cc->Lf[2]}, invLf[3] = {cc->invLf[0], cc->invLf[1], cc->invLf[2]};
+        const int nc[3] = {cc->nc[0], cc->nc[1], cc->nc[2]};
+        bool mi[3];  // the nearest image rounded in FP64
+#pragma unroll
+        for (int t = 0; t < 3; ++t) mi[t] = kList ? 2.0 * rc > 0.999 * L[t] : nc[t] < 3;
+        const bool any_mi = mi[0] || mi[1] || mi[2];
+        const float pass = cc->pass64;
+        const int64_t per = (N + gridDim.x - 1) / gridDim.x;
+        const int u1 = (int)min(N, (blockIdx.x + 1) * per);
+        for (int u = (int)(blockIdx.x * per) + wib; u < u1; u += kPair64Warps) {
+            const int i = sorted[u];
+            const float4 me = spos32[u];
+            const double4_32a m64 = spos64[u];
+            const double qki = pc.qk * m64.w;
+            s.fx = s.fy = s.fz = 0.0;
+            s.ecp = FF{0.0f, 0.0f};
+            int nh = 0;
+            // one buffered candidate per lane (lanes >= count idle)
+            auto evaluate = [&](int count, int base) {
+                const bool on = lane < count;
+                const int2 h = on ? hits[wib][base + lane] : make_int2(u, kPairNoShift);
+                const double4_32a o = spos64[h.x];
+                double dx = o.x - m64.x, dy = o.y - m64.y, dz = o.z - m64.z;
+                if (__any_sync(0xffffffffu, h.y != kPairNoShift)) {
+                    const int cx = h.y & 3, cy = (h.y >> 2) & 3, cz = (h.y >> 4) & 3;
+                    dx += cx == 1 ? 0.0 : (cx == 0 ? -L[0] : L[0]);
+                    dy += cy == 1 ? 0.0 : (cy == 0 ? -L[1] : L[1]);
+                    dz += cz == 1 ? 0.0 : (cz == 0 ? -L[2] : L[2]);
+                }
+                if (any_mi) {
+                    if (mi[0]) dx -= L[0] * rint(dx * cc->invL[0]);
+                    if (mi[1]) dy -= L[1] * rint(dy * cc->invL[1]);
+                    if (mi[2]) dz -= L[2] * rint(dz * cc->invL[2]);
+                }
+                const double r2 = dx * dx + dy * dy + dz * dz;
+                // r2 < rc^2 by the bits: both non-negative (and a NaN is above)
+                if (on && (unsigned long long)__double_as_longlong(r2) < pc.rc2)
+                    pair64_add<kDiag>(tab, pc, pc.lj != 0, dx, dy, dz, r2, m64.w, o.w, qki, s);
+                __syncwarp();
+            };
+            if constexpr (kList) {
+                const int nn = la.nnb[u];
+                const int* row = la.nbr + (int64_t)u * la.cap;
+                const float hx = 0.5f * Lf[0], hy = 0.5f * Lf[1], hz = 0.5f * Lf[2];
+                for (int k0 = 0; k0 < nn; k0 += 32 * kListBatch) {
+                    int sj[kListBatch];
+                    float4 o[kListBatch];
+#pragma unroll
+                    for (int a = 0; a < kListBatch; ++a) {
+                        const int k = k0 + 32 * a + lane;
+                        sj[a] = row[k < nn ? k : nn - 1];
+                    }
+#pragma unroll
+                    for (int a = 0; a < kListBatch; ++a) o[a] = spos32[sj[a]];
+#pragma unroll
+                    for (int a = 0; a < kListBatch; ++a) {
+                        const int k = k0 + 32 * a + lane;
+                        float dx = o[a].x - me.x, dy = o[a].y - me.y, dz = o[a].z - me.z;
+                        const int cx = dx > hx ? 0 : (dx < -hx ? 2 : 1), cy = dy > hy ? 0 : (dy < -hy ? 2 : 1),
+                                  cz = dz > hz ? 0 : (dz < -hz ? 2 : 1);
+                        dx += cx == 1 ? 0.0f : (cx == 0 ? -Lf[0] : Lf[0]);
+                        dy += cy == 1 ? 0.0f : (cy == 0 ? -Lf[1] : Lf[1]);
+                        dz += cz == 1 ? 0.0f : (cz == 0 ? -Lf[2] : Lf[2]);
+                        const bool hit = k < nn && dx * dx + dy * dy + dz * dz < pass;
+                        const unsigned m = __ballot_sync(0xffffffffu, hit);
+                        if (hit)  // on an axis with mi the code is 1: the image is rounded in FP64
+                            hits[wib][nh + __popc(m & ((1u << lane) - 1u))] =
+                                make_int2(sj[a], (mi[0] ? 1 : cx) | ((mi[1] ? 1 : cy) << 2) | ((mi[2] ? 1 : cz) << 4));
+                        nh += __popc(m);
+                    }
+                    // evaluate whole groups of 32 and keep the rest at the front
+                    __syncwarp();
+                    int b0 = 0;
+                    for (; b0 + 32 <= nh; b0 += 32) evaluate(32, b0);
+                    __syncwarp();
+                    const int2 keep = b0 > 0 && lane < nh - b0 ? hits[wib][b0 + lane] : make_int2(0, 0);
+                    __syncwarp();
+                    if (b0 > 0 && lane < nh - b0) hits[wib][lane] = keep;
+                    __syncwarp();
+                    nh -= b0;
+                }
+            } else {
+                // segments of the neighbouring cells' slots, one per lane (see k_pair)
+                int lo = 0, hi = 0, code = 0;
+                float ctx = 0.f, cty = 0.f, ctz = 0.f;
+                int sx, sy, sz;
+                if (pair_segment_of(cid[i], nc, lane, mi, cnt, start, lo, hi, sx, sy, sz)) {
+                    code = (sx + 1) | ((sy + 1) << 2) | ((sz + 1) << 4);
+                    ctx = me.x - (float)sx * Lf[0];
+                    cty = me.y - (float)sy * Lf[1];
+                    ctz = me.z - (float)sz * Lf[2];
+                }
+                for (int g = 0; g < 18; ++g) {
+                    const int glo = __shfl_sync(0xffffffffu, lo, g), ghi = __shfl_sync(0xffffffffu, hi, g);
+                    if (glo >= ghi) continue;  // the same for every lane
+                    const int gcode = __shfl_sync(0xffffffffu, code, g);
+                    const float gx = __shfl_sync(0xffffffffu, ctx, g), gy = __shfl_sync(0xffffffffu, cty, g),
+                                gz = __shfl_sync(0xffffffffu, ctz, g);
+                    for (int s0 = glo; s0 < ghi; s0 += 32) {
+                        const int sl = s0 + lane;
+                        const float4 o = spos32[sl < ghi ? sl : glo];
+                        float dx = o.x - gx, dy = o.y - gy, dz = o.z - gz;
+                        if (any_mi) {
+                            if (mi[0]) dx -= Lf[0] * rintf(dx * invLf[0]);
+                            if (mi[1]) dy -= Lf[1] * rintf(dy * invLf[1]);
+                            if (mi[2]) dz -= Lf[2] * rintf(dz * invLf[2]);
+                        }
+                        const bool hit = sl < ghi && sl != u && dx * dx + dy * dy + dz * dz < pass;
+                        const unsigned m = __ballot_sync(0xffffffffu, hit);
+                        if (hit) hits[wib][nh + __popc(m & ((1u << lane) - 1u))] = make_int2(sl, gcode);
+                        nh += __popc(m);
+                        if (nh >= 32) {
+                            __syncwarp();
+                            evaluate(32, 0);
+                            __syncwarp();
+                            if (lane < nh - 32) hits[wib][lane] = hits[wib][32 + lane];
+                            __syncwarp();
+                            nh -= 32;
+                        }
+                    }
+                }
+            }
+            __syncwarp();
+            if (nh > 0) evaluate(nh, 0);
+            __syncwarp();
+            warp_force_out(s.fx, s.fy, s.fz, lane, Fr + 3 * (int64_t)i);
+            ff_acc(s.ec, ff_mul(s.ecp, charge_fits(m64.w) ? ff_of_double(m64.w) : FF{0.0f, 0.0f}));
+        }
+    }
+    pair64_partials<kDiag>(s, pc.qk, red, partials + kPartStride * (size_t)blockIdx.x, kDiag ? 3 : 1);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1229,7 +1329,68 @@ static rbe_status npt_check(rbe_ctx ctx, const char* what)
     return e == cudaSuccess ? RBE_OK : npt_fail(ctx, e, what);
 }
 
-// Blocks of the pair kernel: one warp per particle, at most one resident wave (the warps
+// Blocks of the FP64 pair kernels: one per SM (its warps share the table), every SM from few particles on.
+int pair_blocks64(rbe_ctx ctx, int64_t N)
+{
+    return (int)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, (N + 3) / 4));
+}
+
+__global__ void k_pair_table(PairWord* __restrict__ t, int top, double alpha, double s2, double e24, double e4)
+{
+    const int seg = blockIdx.x * blockDim.x + threadIdx.x;
+    if (seg < kPairSegs) pair_segment(t, seg, top, alpha, s2, e24, e4);
+}
+
+// The FP64 pair kernels' constants, with the table of these parameters: found among the context's, or
+// built by one small launch.  Without a table (direct evaluation, the same results to rounding) where the
+// polynomials' coefficients could leave the float range, in a capture that meets the parameters for
+// the first time, and past kPairTabs sets of parameters.
+rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out)
+{
+    NptBuffers& b = ctx->npt;
+    const PairConst c = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
+    Pair64Const p{};
+    p.lj = c.lj;
+    p.alpha = c.a;
+    p.sa = c.sa;
+    p.two_sa_pi = c.two_sa_pi;
+    p.qk = c.qk;
+    p.s2 = c.s2;
+    p.e4 = c.e4;
+    p.e24 = c.e24;
+    std::memcpy(&p.rc2, &c.rc2, sizeof(p.rc2));
+    const bool rc_ok = prm.rc >= 1e-4 && prm.rc <= 1e4;
+    const int top = rc_ok ? std::ilogb(c.rc2) + 1 : 0;
+    const double y = c.s2 / std::ldexp(1.0, top - kPairOctaves), lj = 50.0 * std::fabs(c.e24) * std::pow(y, 6) / c.s2;
+    if (rc_ok && (!c.lj || (std::isfinite(lj) && lj * y < 1e30))) {
+        p.base = (1023 + top - kPairOctaves) << kPairSegBits;
+        const double key[5] = {ctx->alpha, c.rc2, c.s2, c.e24, c.e4};
+        int t = 0;
+        while (t < b.pair_tabs && std::memcmp(key, b.pair_key[t], sizeof(key)) != 0) ++t;
+        if (t == b.pair_tabs && t < NptBuffers::kPairTabs) {
+            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+            if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
+                cudaGetLastError();
+                cap = cudaStreamCaptureStatusActive;
+            }
+            if (cap == cudaStreamCaptureStatusNone) {
+                cudaError_t e = ctx_alloc(ctx, &b.pair_tab[t], kPairTabBytes);
+                if (e != cudaSuccess) return npt_fail(ctx, e, "cudaMalloc(pair tables)");
+                k_pair_table<<<kPairSegs / 32, 32, 0, ctx->stream>>>(static_cast<PairWord*>(b.pair_tab[t]), top, ctx->alpha,
+                                                                    c.s2, c.e24, c.e4);
+                rbe_status st = npt_check(ctx, "k_pair_table");
+                if (st != RBE_OK) return st;
+                std::memcpy(b.pair_key[t], key, sizeof(key));
+                ++b.pair_tabs;
+            }
+        }
+        if (t < b.pair_tabs) p.tab = static_cast<const PairWord*>(b.pair_tab[t]);
+    }
+    *out = p;
+    return RBE_OK;
+}
+
+// Blocks of the FP32 pair kernel: one warp per particle, at most one resident wave (the warps
 // stride over the rest).  The FP32 count is the larger one and sizes the partials.
 int pair_blocks(rbe_ctx ctx, int64_t N, bool fp64)
 {
@@ -1358,7 +1519,7 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, uint64_t batch, int d
     cudaStream_t s = ctx->stream;
     const int64_t N = sys->N;
     const int nb = (int)((N + kNptThreads - 1) / kNptThreads);
-    const int nbp = pair_blocks(ctx, N, ctx->precision == RBE_FP64);
+    const int nbp = ctx->precision == RBE_FP64 ? pair_blocks64(ctx, N) : pair_blocks(ctx, N, false);
     rbe_status st;
     if (prm.kspace && (parts & 1)) {
         // tables from the device box and the sampler (one launch), then the evaluation
@@ -1390,35 +1551,29 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, uint64_t batch, int d
         if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nls, fp64)) != RBE_OK) return st;
         const PairConst pc = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
         const ListArgs la{nls, b.nbr, b.nnb, b.sref, ctx->d.status, b.nbr_cap};
-        const double4_32a* s64 = fp64 ? b.spos64 : nullptr;
         const bool diag = prm.barostat >= 2;  // rectangular cell: the virial diagonal
-        auto pair = [&](auto f64_tag, auto mode_tag) {
-            constexpr bool F64 = decltype(f64_tag)::value;
-            constexpr int MODE = decltype(mode_tag)::value;
-            if constexpr (MODE == kPairBuild)
-                k_pair<F64, MODE><<<nbp, kPairWarps * 32, 0, s>>>(N, cc, pc, b.cid, b.cnt, b.start, b.sorted,
-                                                                  b.spos32, s64, b.Fr, b.partials, la);
-            else if (diag)
-                k_pair<F64, MODE, true><<<nbp, kPairWarps * 32, 0, s>>>(N, cc, pc, b.cid, b.cnt, b.start, b.sorted,
-                                                                        b.spos32, s64, b.Fr, b.partials, la);
-            else
-                k_pair<F64, MODE><<<nbp, kPairWarps * 32, 0, s>>>(N, cc, pc, b.cid, b.cnt, b.start, b.sorted,
-                                                                  b.spos32, s64, b.Fr, b.partials, la);
-        };
-        using T = std::true_type;
-        using F = std::false_type;
-        using Cells = std::integral_constant<int, kPairCells>;
-        using Build = std::integral_constant<int, kPairBuild>;
-        using List = std::integral_constant<int, kPairList>;
-        if (!list) {
-            if (fp64) pair(T{}, Cells{});
-            else pair(F{}, Cells{});
-        } else if (fp64) {
-            pair(T{}, Build{});
-            pair(T{}, List{});
+        if (list)
+            k_pair<kPairBuild><<<pair_blocks(ctx, N, false), kPairWarps * 32, 0, s>>>(N, cc, pc, b.cid, b.cnt, b.start,
+                                                                                     b.sorted, b.spos32, b.Fr, b.partials, la);
+        if (fp64) {
+            Pair64Const p64;
+            if ((st = pair64_const(ctx, prm, &p64)) != RBE_OK) return st;
+            auto kern = list ? (diag ? k_pair64<kPairList, true> : k_pair64<kPairList, false>)
+                             : (diag ? k_pair64<kPairCells, true> : k_pair64<kPairCells, false>);
+            static const cudaError_t attr = [] {
+                cudaError_t e = cudaSuccess;
+                for (auto k : {k_pair64<kPairList, true>, k_pair64<kPairList, false>, k_pair64<kPairCells, true>,
+                               k_pair64<kPairCells, false>})
+                    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairTabBytes);
+                return e;
+            }();
+            if (attr != cudaSuccess) return npt_fail(ctx, attr, "shared memory of k_pair64");
+            kern<<<nbp, kPair64Warps * 32, kPairTabBytes, s>>>(N, cc, p64, prm.rc, b.cid, b.cnt, b.start, b.sorted, b.spos32,
+                                                              b.spos64, b.Fr, b.partials, la);
         } else {
-            pair(F{}, Build{});
-            pair(F{}, List{});
+            auto kern = list ? (diag ? k_pair<kPairList, true> : k_pair<kPairList, false>)
+                             : (diag ? k_pair<kPairCells, true> : k_pair<kPairCells, false>);
+            kern<<<nbp, kPairWarps * 32, 0, s>>>(N, cc, pc, b.cid, b.cnt, b.start, b.sorted, b.spos32, b.Fr, b.partials, la);
         }
         if ((st = npt_check(ctx, "real-space kernels")) != RBE_OK) return st;
     }

@@ -23,6 +23,7 @@
 #include "rbe_context.h"
 #include "rbe_device.cuh"
 #include "rbe_npt_common.cuh"
+#include "rbe_pair64.cuh"
 
 namespace rbe {
 
@@ -301,98 +302,72 @@ k_water_drift(int64_t Nmol, double* __restrict__ pos, double* __restrict__ mom, 
 // the neighbouring cells (an axis with fewer than 3 cells visits each of its cells once) and
 // stride over their slots; the separation is the nearest image per pair (sites may sit up to a
 // bond outside the box).  The search runs on the FP32 packed positions with rc plus a margin above
-// their rounding; the hits (slots) go to a per-warp buffer in ballot order and are evaluated 32 at a
-// time, one per lane, in FP64 from the FP64 packed positions with the exact cutoff.  A hit of the
+// their rounding; the hits (slot, image code) go to a per-warp buffer in ballot order and are evaluated 32
+// at a time, one per lane, in FP64 from the FP64 packed positions with the exact cutoff; the pair terms come
+// from the tables of rbe_pair64.cuh (k_pair64 says what bounds it; on an axis shorter than 2 rc + 0.1 % the
+// image is rounded in FP64).  A hit of the
 // same molecule (site index / 3) is skipped; LJ acts between oxygens (site index divisible by 3).
-// Lane sums through a fixed shuffle tree.  Each pair is
+// Each pair is
 // visited from both ends: energies and the virial take half.  Per-block partials {W_r, E_coul,
 // E_lj} at slots 1..3 (the isotropic layout).  A box beyond the cell arrays leaves F_r = 0.
-__global__ void __launch_bounds__(kPairWarps * 32, kPairBlocksPerSM64)
-k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const int* __restrict__ cid,
+__global__ void __launch_bounds__(kPair64Warps * 32, 1)
+k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, double rc, const int* __restrict__ cid,
              const int* __restrict__ cnt, const int* __restrict__ start, const int* __restrict__ sorted,
              const float4* __restrict__ spos32, const double4_32a* __restrict__ spos64, double* __restrict__ Fr,
              double* __restrict__ partials)
 {
-    __shared__ int hits[kPairWarps][kWaterHitCap];  // slots of candidates within the FP32 search radius
-    __shared__ double red[3][kPairWarps];
+    extern __shared__ __align__(16) unsigned char s_raw[];
+    PairWord* tab = reinterpret_cast<PairWord*>(s_raw);
+    __shared__ int2 hits[kPair64Warps][kWaterHitCap];  // candidates within the FP32 search radius
+    __shared__ double red[3][kPair64Warps];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    const int nc[3] = {cc->nc[0], cc->nc[1], cc->nc[2]};
-    const double L[3] = {cc->L[0], cc->L[1], cc->L[2]}, inv[3] = {cc->invL[0], cc->invL[1], cc->invL[2]};
-    const float Lf[3] = {cc->Lf[0], cc->Lf[1], cc->Lf[2]}, invf[3] = {cc->invLf[0], cc->invLf[1], cc->invLf[2]};
-    // FP32 search radius: rc plus 2^-16 l_max, far above the FP32 rounding of a separation; the
-    // exact cutoff is applied in FP64
-    const float pass = cc->pass64;
-    double wsum = 0.0, ecsum = 0.0, elsum = 0.0;
+    load_pair_table(pc.tab, tab);
+    Pair64Sums<false> s{};
+    __syncthreads();
     if (cc->ncell < 0) {
         for (int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; j < 3 * N; j += (int64_t)gridDim.x * blockDim.x)
             Fr[j] = 0.0;
     } else {
-        const int nwarps = gridDim.x * kPairWarps;
-        for (int u = blockIdx.x * kPairWarps + wib; u < (int)N; u += nwarps) {
+        const int nc[3] = {cc->nc[0], cc->nc[1], cc->nc[2]};
+        const double L[3] = {cc->L[0], cc->L[1], cc->L[2]};
+        const float Lf[3] = {cc->Lf[0], cc->Lf[1], cc->Lf[2]}, invf[3] = {cc->invLf[0], cc->invLf[1], cc->invLf[2]};
+        const bool exact = 2.0 * rc > 0.999 * fmin(L[0], fmin(L[1], L[2]));
+        const bool mi[3] = {true, true, true};  // the segments carry no image: it is taken per pair
+        const float pass = cc->pass64;
+        const int64_t per = (N + gridDim.x - 1) / gridDim.x;
+        const int u1 = (int)min(N, (blockIdx.x + 1) * per);
+        for (int u = (int)(blockIdx.x * per) + wib; u < u1; u += kPair64Warps) {
             const int i = sorted[u];
             const double4_32a me = spos64[u];
             const float4 me32 = spos32[u];
             const int mol_i = i / 3;
-            const bool oxy_i = i % 3 == 0;
-            int lo = 0, hi = 0;
-            {
-                const int c = cid[i];
-                const int cxy = nc[0] * nc[1];
-                const int cz = c / cxy, cy = (c - cz * cxy) / nc[0], cx = c - cz * cxy - cy * nc[0];
-                const int r = lane >> 1, part = lane & 1;
-                const int dy = r % 3 - 1, dz = r / 3 - 1;
-                const bool row_ok = r < 9 && dy >= (nc[1] >= 3 ? -1 : 0) && dy <= (nc[1] >= 2 ? 1 : 0) &&
-                                    dz >= (nc[2] >= 3 ? -1 : 0) && dz <= (nc[2] >= 2 ? 1 : 0);
-                if (row_ok) {
-                    const int uy = cy + dy, uz = cz + dz;
-                    const int yy = uy < 0 ? uy + nc[1] : (uy >= nc[1] ? uy - nc[1] : uy);
-                    const int zz = uz < 0 ? uz + nc[2] : (uz >= nc[2] ? uz - nc[2] : uz);
-                    const int row = (zz * nc[1] + yy) * nc[0], nx = nc[0];
-                    int a = -1, b = -1;
-                    if (nx < 3) {
-                        if (part == 0) a = 0, b = nx - 1;
-                    } else if (cx == 0) {
-                        if (part == 0) a = 0, b = 1;
-                        else a = b = nx - 1;
-                    } else if (cx == nx - 1) {
-                        if (part == 0) a = nx - 2, b = nx - 1;
-                        else a = b = 0;
-                    } else if (part == 0) {
-                        a = cx - 1, b = cx + 1;
-                    }
-                    if (a >= 0) {
-                        lo = start[row + a];
-                        hi = start[row + b] + cnt[row + b];
-                    }
-                }
-            }
-            double fx = 0.0, fy = 0.0, fz = 0.0, w = 0.0, ec = 0.0, el = 0.0;
-            int nh = 0;
+            const bool oxy_i = i % 3 == 0 && pc.lj;
+            const double qki = pc.qk * me.w;
+            s.fx = s.fy = s.fz = 0.0;
+            s.ecp = FF{0.0f, 0.0f};
+            int lo = 0, hi = 0, sx, sy, sz, nh = 0;
+            pair_segment_of(cid[i], nc, lane, mi, cnt, start, lo, hi, sx, sy, sz);
             auto evaluate = [&](int count) {
-                if (lane >= count) return;
-                const int sj = hits[wib][lane];
-                const int j = sorted[sj];
-                if (j / 3 == mol_i) return;  // the same molecule (the site itself included)
-                const double4_32a o = spos64[sj];
-                double d[3] = {o.x - me.x, o.y - me.y, o.z - me.z};
-                #pragma unroll
-                for (int t = 0; t < 3; ++t) d[t] -= L[t] * rint(d[t] * inv[t]);
-                const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2];
-                if (!(r2 < pc.rc2)) return;
-                const double r = sqrt(r2), inv_r = 1.0 / r, inv_r2 = inv_r * inv_r;
-                const double coul = pc.qk * me.w * o.w * inv_r;
-                const double er = erfc(pc.sa * r);
-                ec += coul * er;
-                double f = coul * (er + pc.two_sa_pi * r * exp(-pc.a * r2)) * inv_r2;
-                if (oxy_i && j % 3 == 0 && pc.lj) {
-                    const double sr2 = pc.s2 * inv_r2, sr6 = sr2 * sr2 * sr2;
-                    el += pc.e4 * (sr6 * sr6 - sr6);
-                    f += pc.e24 * (2.0 * sr6 * sr6 - sr6) * inv_r2;
+                const bool on = lane < count;
+                const int2 h = on ? hits[wib][lane] : make_int2(u, 1 | (1 << 2) | (1 << 4));
+                const int j = sorted[h.x];
+                const double4_32a o = spos64[h.x];
+                double dx = o.x - me.x, dy = o.y - me.y, dz = o.z - me.z;
+                if (exact) {
+                    dx -= L[0] * rint(dx * cc->invL[0]);
+                    dy -= L[1] * rint(dy * cc->invL[1]);
+                    dz -= L[2] * rint(dz * cc->invL[2]);
+                } else if (__any_sync(0xffffffffu, h.y != (1 | (1 << 2) | (1 << 4)))) {
+                    const int cx = h.y & 3, cy = (h.y >> 2) & 3, cz = (h.y >> 4) & 3;
+                    dx += cx == 1 ? 0.0 : (cx == 0 ? -L[0] : L[0]);
+                    dy += cy == 1 ? 0.0 : (cy == 0 ? -L[1] : L[1]);
+                    dz += cz == 1 ? 0.0 : (cz == 0 ? -L[2] : L[2]);
                 }
-                fx -= f * d[0];
-                fy -= f * d[1];
-                fz -= f * d[2];
-                w += f * r2;
+                const double r2 = dx * dx + dy * dy + dz * dz;
+                // another molecule (the site itself excluded with its own) and r2 < rc^2 by the bits
+                if (on && j / 3 != mol_i && (unsigned long long)__double_as_longlong(r2) < pc.rc2)
+                    pair64_add<false>(tab, pc, oxy_i && j % 3 == 0, dx, dy, dz, r2, me.w, o.w, qki, s);
+                __syncwarp();
             };
             for (int g = 0; g < 18; ++g) {
                 const int glo = __shfl_sync(0xffffffffu, lo, g), ghi = __shfl_sync(0xffffffffu, hi, g);
@@ -400,12 +375,17 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, c
                     const int sl = s0 + lane;
                     const float4 o = spos32[sl < ghi ? sl : glo];
                     float dx = o.x - me32.x, dy = o.y - me32.y, dz = o.z - me32.z;
-                    dx -= Lf[0] * rintf(dx * invf[0]);
-                    dy -= Lf[1] * rintf(dy * invf[1]);
-                    dz -= Lf[2] * rintf(dz * invf[2]);
+                    // sites lie within a bond of [0, l), l >= 2 rc: the image is -1, 0 or 1
+                    const float kx = rintf(dx * invf[0]), ky = rintf(dy * invf[1]), kz = rintf(dz * invf[2]);
+                    dx -= Lf[0] * kx;
+                    dy -= Lf[1] * ky;
+                    dz -= Lf[2] * kz;
                     const bool hit = sl < ghi && sl != u && dx * dx + dy * dy + dz * dz < pass;
                     const unsigned m = __ballot_sync(0xffffffffu, hit);
-                    if (hit) hits[wib][nh + __popc(m & ((1u << lane) - 1u))] = sl;
+                    if (hit) {
+                        const int code = (1 - (int)kx) | ((1 - (int)ky) << 2) | ((1 - (int)kz) << 4);
+                        hits[wib][nh + __popc(m & ((1u << lane) - 1u))] = make_int2(sl, code);
+                    }
                     nh += __popc(m);
                     if (nh >= 32) {
                         __syncwarp();
@@ -418,38 +398,13 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, c
                 }
             }
             __syncwarp();
-            evaluate(nh);
+            if (nh > 0) evaluate(nh);
             __syncwarp();
-#pragma unroll
-            for (int off = 16; off > 0; off >>= 1) {
-                fx += __shfl_xor_sync(0xffffffffu, fx, off);
-                fy += __shfl_xor_sync(0xffffffffu, fy, off);
-                fz += __shfl_xor_sync(0xffffffffu, fz, off);
-                w += __shfl_xor_sync(0xffffffffu, w, off);
-                ec += __shfl_xor_sync(0xffffffffu, ec, off);
-                el += __shfl_xor_sync(0xffffffffu, el, off);
-            }
-            if (lane == 0) {
-                Fr[3 * (int64_t)i] = fx;
-                Fr[3 * (int64_t)i + 1] = fy;
-                Fr[3 * (int64_t)i + 2] = fz;
-                wsum += 0.5 * w;
-                ecsum += 0.5 * ec;
-                elsum += 0.5 * el;
-            }
+            warp_force_out(s.fx, s.fy, s.fz, lane, Fr + 3 * (int64_t)i);
+            ff_acc(s.ec, ff_mul(s.ecp, charge_fits(me.w) ? ff_of_double(me.w) : FF{0.0f, 0.0f}));
         }
     }
-    if (lane == 0) {
-        red[0][wib] = wsum;
-        red[1][wib] = ecsum;
-        red[2][wib] = elsum;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double t = 0.0;
-        for (int wv = 0; wv < kPairWarps; ++wv) t += red[threadIdx.x][wv];
-        partials[kPartStride * (size_t)blockIdx.x + 1 + threadIdx.x] = t;
-    }
+    pair64_partials<false>(s, pc.qk, red, partials + kPartStride * (size_t)blockIdx.x, 1);
 }
 
 // ---------------------------------------------------------------------------------
@@ -633,7 +588,7 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, int do_kick)
     const rbe_npt_params& prm = sys->params;
     cudaStream_t s = ctx->stream;
     const int64_t N = sys->N, Nmol = N / 3;
-    const int nbp = pair_blocks(ctx, N, true);
+    const int nbp = pair_blocks64(ctx, N);
     rbe_status st;
     if (prm.kspace) {
         if ((st = launch_tables_sample_device(ctx, ctx->P, sys->cell,
@@ -646,9 +601,14 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, int do_kick)
     if (prm.real) {
         if (b.n64 < N) return fail(ctx, RBE_ESTATE, "the FP64 packed positions are missing: call rbe_water_init again");
         if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nullptr, true)) != RBE_OK) return st;
-        const PairConst pc = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
-        k_water_pair<<<nbp, kPairWarps * 32, 0, s>>>(N, static_cast<const CellConsts*>(b.cellc), pc, b.cid, b.cnt,
-                                                     b.start, b.sorted, b.spos32, b.spos64, b.Fr, b.partials);
+        Pair64Const pc;
+        if ((st = pair64_const(ctx, prm, &pc)) != RBE_OK) return st;
+        static const cudaError_t attr =
+            cudaFuncSetAttribute(k_water_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairTabBytes);
+        if (attr != cudaSuccess) return cuda_fail(ctx, attr, "shared memory of k_water_pair");
+        k_water_pair<<<nbp, kPair64Warps * 32, kPairTabBytes, s>>>(N, static_cast<const CellConsts*>(b.cellc), pc, prm.rc,
+                                                                  b.cid, b.cnt, b.start, b.sorted, b.spos32, b.spos64,
+                                                                  b.Fr, b.partials);
         if ((st = water_check(ctx, "k_water_pair")) != RBE_OK) return st;
     }
     const int nbm = (int)std::max<int64_t>(1, (Nmol + kWaterThreads - 1) / kWaterThreads);
@@ -673,7 +633,7 @@ rbe_status water_init(rbe_ctx ctx, rbe_system* sys, const rbe_water_params* wp, 
     const int64_t Nmol = sys->N / 3;
     // block partials: the pair pass's blocks, then one slot row per finishing block
     NptBuffers& b = ctx->npt;
-    const int need = pair_blocks(ctx, sys->N, true) + (int)std::max<int64_t>(1, (Nmol + kWaterThreads - 1) / kWaterThreads);
+    const int need = pair_blocks64(ctx, sys->N) + (int)std::max<int64_t>(1, (Nmol + kWaterThreads - 1) / kWaterThreads);
     if (need > b.partcap) {
         ctx_free(ctx, b.partials);
         b.partials = nullptr;

@@ -1,0 +1,43 @@
+// Host-side driver for the tabulated pair terms of the FP64 real space.  Reads from stdin lines
+//   alpha rc sigma eps r2 ...   (r2 values to the end of the line)
+// and prints for each r2 the Coulomb force factor and energy and the Lennard-Jones ones (energies as float-float
+// sums), or "out" where the table has no segment.
+#include <cmath>
+#include <cstdio>
+#include <cstring>
+#include <iostream>
+#include <sstream>
+#include <string>
+#include <vector>
+
+#include "../../paper_2110_14362_gb300/csrc/rbe_pair64.cuh"
+
+using namespace rbe;
+
+int main()
+{
+    std::string line;
+    while (std::getline(std::cin, line)) {
+        std::istringstream in(line);
+        double alpha, rc, sigma, eps, u;
+        in >> alpha >> rc >> sigma >> eps;
+        const int top = std::ilogb(rc * rc) + 1;
+        std::vector<PairWord> t(kPairTabBytes / sizeof(PairWord));
+        for (int i = 0; i < kPairSegs; ++i) pair_segment(t.data(), i, top, alpha, sigma * sigma, 24.0 * eps, 4.0 * eps);
+        while (in >> u) {
+            unsigned long long b;
+            std::memcpy(&b, &u, 8);
+            const PairArg a = pair_arg((uint32_t)(b >> 32), (uint32_t)b, (1023 + top - kPairOctaves) << kPairSegBits);
+            if ((unsigned)a.seg >= (unsigned)kPairSegs) {
+                std::printf("out\n");
+                continue;
+            }
+            double f, g;
+            FF e, l;
+            pair_eval<0>(t.data(), a, f, e);
+            pair_eval<1>(t.data(), a, g, l);
+            std::printf("%.17g %.17g %.17g %.17g\n", f, (double)e.h + (double)e.l, g, (double)l.h + (double)l.l);
+        }
+    }
+    return 0;
+}
