@@ -1329,11 +1329,7 @@ static rbe_status npt_check(rbe_ctx ctx, const char* what)
     return e == cudaSuccess ? RBE_OK : npt_fail(ctx, e, what);
 }
 
-// Blocks of the FP64 pair kernels: one per SM (its warps share the table), every SM from few particles on.
-int pair_blocks64(rbe_ctx ctx, int64_t N)
-{
-    return (int)std::max<int64_t>(1, std::min<int64_t>(ctx->num_sms, (N + 3) / 4));
-}
+int pair_blocks64(rbe_ctx ctx, int64_t N) { return pair_blocks64_of(N, ctx->num_sms); }
 
 __global__ void k_pair_table(PairWord* __restrict__ t, int top, double alpha, double s2, double e24, double e4)
 {
@@ -1390,13 +1386,10 @@ rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out
     return RBE_OK;
 }
 
-// Blocks of the FP32 pair kernel: one warp per particle, at most one resident wave (the warps
-// stride over the rest).  The FP32 count is the larger one and sizes the partials.
+// Blocks of the FP32 pair kernel and (fp64) of the flexible cell's FP64 pairs.
 int pair_blocks(rbe_ctx ctx, int64_t N, bool fp64)
 {
-    const int64_t want = (N + kPairWarps - 1) / kPairWarps;
-    const int per_sm = fp64 ? kPairBlocksPerSM64 : kPairBlocksPerSM;
-    return (int)std::max<int64_t>(1, std::min<int64_t>(want, (int64_t)ctx->num_sms * per_sm));
+    return pair_blocks_of(N, ctx->num_sms, fp64 ? kPairBlocksPerSM64 : kPairBlocksPerSM);
 }
 
 // Grow the NPT scratch for N particles and a box whose edges may double; with skin > 0 also
@@ -1475,7 +1468,7 @@ rbe_status npt_ensure(rbe_ctx ctx, int64_t N, const double box[3], double rc, do
         }
         b.nbr_cap = cap;
     }
-    const int need = pair_blocks(ctx, N, false) + (int)((N + kNptThreads - 1) / kNptThreads);
+    const int need = (int)npt_partial_rows(N, ctx->num_sms);
     if (need > b.partcap) {
         ctx_free(ctx, b.partials);
         b.partials = nullptr;

@@ -9,16 +9,13 @@
 #include <cstdint>
 
 #include "rbe_device.cuh"
+#include "rbe_npt_plan.h"
 
 namespace rbe {
 
 constexpr double kFConv = 100.0;  // kJ/mol/A per g/mol -> A/ps^2
-constexpr int kNptThreads = 256;
 constexpr int kScanThreads = 1024;
 constexpr int kSortWarps = 8;        // k_cl_sort: warps (cells) per block
-constexpr int kPairWarps = 8;        // k_pair: warps (particles in flight) per block
-constexpr int kPairBlocksPerSM = 4;  // k_pair (FP32): resident blocks per SM the grid is sized for
-constexpr int kPairBlocksPerSM64 = 2;  // k_pair (FP64): more registers per thread
 constexpr int kListBatch = 4;        // k_pair (list): list entries per lane loaded together
 constexpr int kHitCap = 32 * (kListBatch + 1);  // k_pair: buffered candidates per warp (< 32 + 32 kListBatch)
 // Per-block partial sums of the pair and finishing kernels: 8 doubles per block.  Isotropic:
