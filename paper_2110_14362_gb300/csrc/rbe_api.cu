@@ -202,6 +202,12 @@ rbe_status rbe_destroy(rbe_ctx ctx)
     for (auto& e : ctx->pev)
         if (e) cudaEventDestroy(e);
     if (ctx->h_out) cudaFreeHost(ctx->h_out);
+    if (ctx->side) {
+        cudaStreamSynchronize(ctx->side);
+        cudaStreamDestroy(ctx->side);
+    }
+    for (auto& e : ctx->side_ev)
+        if (e) cudaEventDestroy(e);
     free_npt(ctx->npt);
     free_buffers(ctx->d);
     if (ctx->chain) cudaFree(ctx->chain);

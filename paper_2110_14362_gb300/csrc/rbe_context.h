@@ -165,6 +165,12 @@ struct rbe_ctx_s {
     cudaStream_t copy_stream = nullptr;
     cudaEvent_t pev[17] = {};  // 1 + 2 kMaxPieces
     double* h_out = nullptr;
+    // the NPT steps' side stream: the k-space chain beside the drift and the real space, forked from and
+    // joined to the context's stream by these events (created by the first rbe_npt_init)
+    cudaStream_t side = nullptr;
+    bool overlap = true;     // false: no side stream (the slots of a server, whose replicas fill the GPU already)
+    bool rho_plain = false;  // the next rho pass follows an event wait: no programmatic launch
+    cudaEvent_t side_ev[3] = {nullptr, nullptr, nullptr};  // after the cell update, after the drift, k-space done
     rbe::DeviceBuffers d;
     std::string last_error;
 };
@@ -223,6 +229,21 @@ rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const dou
 // Shared with the rigid-water step (rbe_npt.cu): parameter checks, the setup of rbe_npt_init
 // before its first forces, the device step index, the isotropic cell part of a step.
 rbe_status npt_validate(rbe_ctx ctx, const rbe_system* sys);
+// The k-space of an NPT or water step beside its other work (rbe_npt.cu).
+struct KspaceFork {
+    rbe_ctx ctx;
+    bool on;  // on the side stream; otherwise each call runs on the context's stream in order
+    KspaceFork(rbe_ctx c, const rbe_system* sys);
+    rbe_status tables(const rbe_system* sys);  // after the cell update: tables of the new box and the sampler
+    rbe_status passes(const rbe_system* sys);  // after the drift: rho, reduction, forces into npt.Fk and npt.WEk
+    rbe_status join();                         // before the finishing kernel
+    KspaceFork(const KspaceFork&) = delete;
+    ~KspaceFork();
+
+  private:
+    bool forked = false;
+    rbe_status branch(int ev);
+};
 rbe_status npt_prepare(rbe_ctx ctx, rbe_system* sys, uint64_t batch);
 rbe_status launch_npt_set_step(rbe_ctx ctx, double* cell, uint64_t step);
 rbe_status launch_npt_cell_iso(rbe_ctx ctx, rbe_system* sys);

@@ -473,10 +473,12 @@ static Plan make_plan(rbe_ctx ctx, int64_t N, int K, const RhoShape& rs, int rho
     return p;
 }
 
-// Launch with programmatic stream serialization (the kernel calls pdl_wait()).
+// Launch with programmatic stream serialization (the kernel calls pdl_wait()), or, with pdl false, in plain
+// stream order: a rho pass behind an event wait, which stages its particles before pdl_wait() and so must not
+// start before the event.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                              Args... args)
+static cudaError_t launch_ordered(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                  Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -487,20 +489,27 @@ static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, siz
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
-    cfg.numAttrs = 1;
+    cfg.numAttrs = pdl ? 1 : 0;
     return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
 }
 
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              Args... args)
+{
+    return launch_ordered(true, kern, grid, block, smem, s, args...);
+}
+
 // The FP32-phase rho pass of plan p on stream s (the wide two-frequency kernel when p.klanes > 0).
-static cudaError_t launch_rho_f32(int accum, bool xyzq, const Plan& p, dim3 grid, cudaStream_t s, const void* pos,
-                                  const double* q, int64_t N, const KState* ks, const int4* m, int K, int nchunks,
-                                  float4* part, unsigned* status)
+static cudaError_t launch_rho_f32(bool pdl, int accum, bool xyzq, const Plan& p, dim3 grid, cudaStream_t s,
+                                  const void* pos, const double* q, int64_t N, const KState* ks, const int4* m, int K,
+                                  int nchunks, float4* part, unsigned* status)
 {
     if (p.klanes > 0)
-        return launch_pdl(rho_wide_kernel(accum, xyzq), grid, dim3(p.kthreads), 0, s, pos, q, N, ks, m, K, p.chunk_len,
-                          nchunks, part, status, 0, p.ksub, p.klanes);
-    return launch_pdl(rho_kernel(accum, p.kf, xyzq), grid, dim3(p.kthreads), 0, s, pos, q, N, ks, m, K, p.chunk_len,
-                      nchunks, part, status, 0, p.ksub);
+        return launch_ordered(pdl, rho_wide_kernel(accum, xyzq), grid, dim3(p.kthreads), 0, s, pos, q, N, ks, m, K,
+                              p.chunk_len, nchunks, part, status, 0, p.ksub, p.klanes);
+    return launch_ordered(pdl, rho_kernel(accum, p.kf, xyzq), grid, dim3(p.kthreads), 0, s, pos, q, N, ks, m, K,
+                          p.chunk_len, nchunks, part, status, 0, p.ksub);
 }
 
 // The reduction's block: the fewest whole warps (up to kReduceThreads) that leave each thread at
@@ -650,8 +659,8 @@ static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* 
     const double* w = d.w + koff;
     const KState* ks = d.ks;
     double2* part = static_cast<double2*>(d.partials);
-    cudaError_t err = launch_pdl(k_rho_f64, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem, s, pos, q, N, ks, m,
-                                 K, p.chunk_len, p.nchunks, part, d.status, p.ksub, p.klanes);
+    cudaError_t err = launch_ordered(!ctx->rho_plain, k_rho_f64, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem,
+                                     s, pos, q, N, ks, m, K, p.chunk_len, p.nchunks, part, d.status, p.ksub, p.klanes);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f64");
     record_event(ctx, 2);
     int threads = 32;
@@ -721,8 +730,8 @@ static rbe_status launch_evaluate_range(rbe_ctx ctx, int64_t N, const void* pos,
     cudaStream_t s = ctx->stream;
     float4* part32 = static_cast<float4*>(d.partials);
     const KState* ks = d.ks;
-    cudaError_t err = launch_rho_f32(ctx->rho_accum, xyzq, p, dim3(p.ktiles, p.nchunks), s, pos, q, N, ks, m_in, K,
-                                     p.nchunks, part32, d.status);
+    cudaError_t err = launch_rho_f32(!ctx->rho_plain, ctx->rho_accum, xyzq, p, dim3(p.ktiles, p.nchunks), s, pos, q,
+                                     N, ks, m_in, K, p.nchunks, part32, d.status);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f32");
     if ((st = check_launch(ctx, "k_rho")) != RBE_OK) return st;
     record_event(ctx, 2);
@@ -815,7 +824,7 @@ rbe_status launch_evaluate_staged(rbe_ctx ctx, int64_t N, const double* h_pos, c
             (err = cudaStreamWaitEvent(s, ctx->pev[1 + g], 0)) != cudaSuccess)
             return cuda_fail(ctx, err, "staged: input event");
         // group g: rows of stride nchunks, its columns from coff[g]
-        err = launch_rho_f32(ctx->rho_accum, false, pl[g], dim3(pl[g].ktiles, pl[g].nchunks), s,
+        err = launch_rho_f32(true, ctx->rho_accum, false, pl[g], dim3(pl[g].ktiles, pl[g].nchunks), s,
                              (const double*)(d_pos + 3 * a), (const double*)(d_q + a), n, ks, (const int4*)d.m, K,
                              nchunks, part32 + coff[g], d.status);
         if (err != cudaSuccess) return cuda_fail(ctx, err, "staged: k_rho_f32");

@@ -8,7 +8,8 @@
 //                   sub-step coefficients, V/2, O^p, V/2, the cell-list constants
 //   k_water_drift   one thread per molecule: R^p/2, R/2, O, R/2 of the centre (exact flows) and of
 //                   the internal motion (kick, free move, SHAKE, momentum correction, projection)
-//   k-space         tables of the device box, sampler, rho, force pass over all sites
+//   k-space         tables of the device box, sampler, rho, force pass over all sites (on a side stream beside
+//                   the drift and the real space, KspaceFork in rbe_npt.cu)
 //   cell list       count, scan, fill, sort (rbe_npt.cu)
 //   k_water_pair    one warp per site: erfc Coulomb with sites of other molecules, LJ between
 //                   oxygens, nearest image per pair
@@ -580,24 +581,17 @@ static rbe_status water_validate(rbe_ctx ctx, const rbe_system* sys, const rbe_w
     return RBE_OK;
 }
 
-// Forces, molecular virial and energies at the current state (batch = the device step index),
-// then the finishing kernel.
-static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, int do_kick)
+// Forces, molecular virial and energies at the current state (batch = the device step index; the k-space
+// tables have been launched on `fork`), then the finishing kernel.
+static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, int do_kick)
 {
     NptBuffers& b = ctx->npt;
     const rbe_npt_params& prm = sys->params;
     cudaStream_t s = ctx->stream;
     const int64_t N = sys->N, Nmol = N / 3;
     const int nbp = pair_blocks64(ctx, N);
-    rbe_status st;
-    if (prm.kspace) {
-        if ((st = launch_tables_sample_device(ctx, ctx->P, sys->cell,
-                                              reinterpret_cast<const unsigned long long*>(sys->cell + kCellStep))) !=
-            RBE_OK)
-            return st;
-        ctx->tables_dirty = true;
-        if ((st = launch_rbe(ctx, N, sys->pos, sys->charge, ctx->P, b.Fk, b.WEk, b.WEk + 9)) != RBE_OK) return st;
-    }
+    rbe_status st = fork.passes(sys);
+    if (st != RBE_OK) return st;
     if (prm.real) {
         if (b.n64 < N) return fail(ctx, RBE_ESTATE, "the FP64 packed positions are missing: call rbe_water_init again");
         if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nullptr, true)) != RBE_OK) return st;
@@ -611,6 +605,7 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, int do_kick)
                                                                   b.Fr, b.partials);
         if ((st = water_check(ctx, "k_water_pair")) != RBE_OK) return st;
     }
+    if ((st = fork.join()) != RBE_OK) return st;
     const int nbm = (int)std::max<int64_t>(1, (Nmol + kWaterThreads - 1) / kWaterThreads);
     k_water_finish<<<nbm, kWaterThreads, 0, s>>>(Nmol, sys->mom, sys->force, sys->pos, sys->charge, sys->mass, b.Fk,
                                                  b.Fr, b.WEk, reinterpret_cast<const NptCoef*>(b.coef), b.partials, nbp,
@@ -645,7 +640,8 @@ rbe_status water_init(rbe_ctx ctx, rbe_system* sys, const rbe_water_params* wp, 
     k_water_whole<<<(unsigned)((Nmol + kWaterThreads - 1) / kWaterThreads), kWaterThreads, 0, ctx->stream>>>(
         Nmol, sys->pos, sys->cell);
     if ((st = water_check(ctx, "k_water_whole")) != RBE_OK) return st;
-    if ((st = water_forces(ctx, sys, 0)) != RBE_OK) return st;
+    KspaceFork fork(ctx, sys);
+    if ((st = fork.tables(sys)) != RBE_OK || (st = water_forces(ctx, sys, fork, 0)) != RBE_OK) return st;
     ctx->water_ready_N = sys->N;
     return launch_npt_set_step(ctx, sys->cell, sys->step);
 }
@@ -659,12 +655,13 @@ rbe_status water_run(rbe_ctx ctx, rbe_system* sys, const rbe_water_params* wp, i
     const int64_t Nmol = sys->N / 3;
     const unsigned nbm = (unsigned)((Nmol + kWaterThreads - 1) / kWaterThreads);
     for (int32_t k = 0; k < nsteps; ++k) {
-        if ((st = launch_npt_cell_iso(ctx, sys)) != RBE_OK) return st;
+        KspaceFork fork(ctx, sys);
+        if ((st = launch_npt_cell_iso(ctx, sys)) != RBE_OK || (st = fork.tables(sys)) != RBE_OK) return st;
         k_water_drift<<<nbm, kWaterThreads, 0, ctx->stream>>>(Nmol, sys->pos, sys->mom, sys->force, sys->mass,
                                                               reinterpret_cast<const NptCoef*>(ctx->npt.coef),
                                                               ctx->seed, sys->cell, *wp, sys->params.dt, ctx->d.status);
         if ((st = water_check(ctx, "k_water_drift")) != RBE_OK) return st;
-        if ((st = water_forces(ctx, sys, 1)) != RBE_OK) return st;
+        if ((st = water_forces(ctx, sys, fork, 1)) != RBE_OK) return st;
         sys->step += 1;
     }
     return RBE_OK;
