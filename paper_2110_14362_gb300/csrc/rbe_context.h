@@ -225,7 +225,9 @@ int pair_blocks(rbe_ctx ctx, int64_t N, bool fp64);
 int pair_blocks64(rbe_ctx ctx, int64_t N);
 struct Pair64Const;
 rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out);
-rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls, bool fp64);
+rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls, bool fp64, int unit);
+// launch_cell_list: FP64 positions packed as they are
+constexpr int kPairNoUnit = -(1 << 20);
 // Shared with the rigid-water step (rbe_npt.cu): parameter checks, the setup of rbe_npt_init
 // before its first forces, the device step index, the isotropic cell part of a step.
 rbe_status npt_validate(rbe_ctx ctx, const rbe_system* sys);

@@ -1176,7 +1176,8 @@ static rbe_status flex_forces(rbe_ctx ctx, rbe_flex_system* sys, int do_kick)
                 k_flex_nl_check<false><<<grid, kNptThreads, 0, s>>>(N, ctx->gpos, sys->charge, b.sorted,
                                                                   ctx->flex_cpos32, nullptr, b.sref, cf, nl);
         }
-        if ((st = launch_cell_list(ctx, N, ctx->gpos, sys->charge, list ? &nl->base : nullptr, fp64)) != RBE_OK)
+        if ((st = launch_cell_list(ctx, N, ctx->gpos, sys->charge, list ? &nl->base : nullptr, fp64,
+                                   kPairNoUnit)) != RBE_OK)
             return st;
         const PairConst pc = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
         const CellConsts* cc = static_cast<const CellConsts*>(b.cellc);

@@ -91,7 +91,7 @@ __global__ void k_cell_consts(const double* __restrict__ cell, double rc, double
 template <bool kF64>
 __global__ void __launch_bounds__(kNptThreads)
 k_nl_check(int64_t N, const double* __restrict__ pos, const double* __restrict__ q, const int* __restrict__ sorted,
-           float4* __restrict__ spos32, double4_32a* __restrict__ spos64, const float4* __restrict__ sref,
+           float4* __restrict__ spos32, double4_32a* __restrict__ spos64, int unit, const float4* __restrict__ sref,
            const CellConsts* __restrict__ cc, NListState* __restrict__ nls)
 {
     __shared__ float smax[kNptThreads / 32];
@@ -105,14 +105,7 @@ k_nl_check(int64_t N, const double* __restrict__ pos, const double* __restrict__
             const int64_t i = sorted[u];
             const double x = pos[3 * i], y = pos[3 * i + 1], z = pos[3 * i + 2], qq = q[i];
             spos32[u] = make_float4((float)x, (float)y, (float)z, (float)qq);
-            if (kF64) {
-                double4_32a v;
-                v.x = x;
-                v.y = y;
-                v.z = z;
-                v.w = qq;
-                spos64[u] = v;
-            }
+            if (kF64) spos64[u] = pair_pack(x, y, z, qq, unit);
             const float4 r0 = sref[u];
             float dx = (float)(x * inv[0]) - r0.x, dy = (float)(y * inv[1]) - r0.y, dz = (float)(z * inv[2]) - r0.z;
             dx = (dx - rintf(dx)) * Lr[0];
@@ -610,11 +603,12 @@ __global__ void k_cl_fill(int64_t N, const int* __restrict__ cid, int* __restric
 // Per cell, one warp: order the members by particle index (a fixed order for every run,
 // whatever order the fill's atomics gave): the member with index i goes to rank = number of
 // members with a smaller index.  Then pack positions and charges in that order: FP32 xyzq
-// always (the pair search runs on it), FP64 as well when spos64 is given.
+// always (the pair search runs on it), and when spos64 is given FP64, as they are or (unit not kPairNoUnit)
+// in fixed point.
 __global__ void __launch_bounds__(kSortWarps * 32)
 k_cl_sort(const CellConsts* __restrict__ cc, const int* __restrict__ cnt, const int* __restrict__ start,
           const int* __restrict__ fill, int* __restrict__ sorted, const double* __restrict__ pos,
-          const double* __restrict__ q, float4* __restrict__ spos32, double4_32a* __restrict__ spos64,
+          const double* __restrict__ q, float4* __restrict__ spos32, double4_32a* __restrict__ spos64, int unit,
           const NListState* __restrict__ nls)
 {
     if (nls && !nls->rebuild) return;
@@ -644,7 +638,7 @@ k_cl_sort(const CellConsts* __restrict__ cc, const int* __restrict__ cnt, const 
                 v.y = y;
                 v.z = z;
                 v.w = qq;
-                spos64[s0 + rank] = v;
+                spos64[s0 + rank] = unit == kPairNoUnit ? v : pair_pack(x, y, z, qq, unit);
             }
         }
     }
@@ -995,16 +989,17 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
 
 // ---------------------------------------------------------------------------------
 // The FP64 path's evaluation (from a cell search, or the list): the search of k_pair in FP32 with rc plus
-// a margin above the FP32 rounding of a distance, the hits as (slot, image code); their separations, the
-// cutoff and the sums in FP64, the pair terms from the tables of rbe_pair64.cuh.  One block of
+// a margin above the FP32 rounding of a distance, the hits as (slot, image code); their separations and the
+// cutoff in fixed point, the pair terms from the tables of rbe_pair64.cuh, the sums in FP64.  One block of
 // kPair64Warps warps per SM shares the table; each block takes a contiguous run of slots.
 //
-// What bounds it: the FP64 pipe still (about 20 instructions of 76 clocks per 32 pairs, against about 115
-// with sqrt, exp, erfc and divisions), with the float-float polynomials beside it: N = 2e4, rc = 7 A, list
-// of 8 A: 875 -> 169 us; 9000 water sites, rc = 10 A, from the cells (k_water_pair): 1021 -> 261 us.  The image of a pair is
-// taken from the search (an addition of +-l only where some lane has one) except on an axis with fewer
-// than 3 cells, or, from a list, one whose half is within 0.1 % of rc, where the nearest image is rounded
-// in FP64.
+// What bounds it: the FP64 pipe still (70 % busy: 11 instructions of about 76 clocks of a scheduler per 32 pairs,
+// and 8 per particle), with the float-float polynomials and the waits of four warps per scheduler beside it.
+// N = 2e4, rc = 7 A, list of 8 A: 875 us with sqrt, exp, erfc and divisions (about 115 FP64 instructions), 169 us
+// with the tables and FP64 separations (22), 125 us with fixed-point separations; 9000 water sites, rc = 10 A,
+// from the cells (k_water_pair): 1021, 261 and 150 us.  The image of a pair is taken from the search (an addition
+// of +-l only where some lane has one) except on an axis with fewer than 3 cells, or, from a list, one whose half
+// is within 0.1 % of rc, where it is taken per pair (pair_nearest).
 template <int kMode, bool kDiag>
 __global__ void __launch_bounds__(kPair64Warps * 32, 1)
 k_pair64(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, double rc, const int* __restrict__ cid,
@@ -1017,6 +1012,7 @@ k_pair64(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, dou
     PairWord* tab = reinterpret_cast<PairWord*>(s_raw);
     __shared__ int2 hits[kPair64Warps][kHitCap];
     __shared__ double red[kDiag ? 5 : 3][kPair64Warps];
+    __shared__ double pforce[kPair64Warps][3];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     load_pair_table(pc.tab, tab);
     Pair64Sums<kDiag> s{};
@@ -1030,134 +1026,141 @@ k_pair64(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, dou
         const double L[3] = {cc->L[0], cc->L[1], cc->L[2]};
         const float Lf[3] = {cc->Lf[0], cc->Lf[1], cc->Lf[2]}, invLf[3] = {cc->invLf[0], cc->invLf[1], cc->invLf[2]};
         const int nc[3] = {cc->nc[0], cc->nc[1], cc->nc[2]};
-        bool mi[3];  // the nearest image rounded in FP64
+        const PairBox box = pair_box(L, rc, pc.unit.s);
+        bool mi[3];  // the nearest image per pair
 #pragma unroll
         for (int t = 0; t < 3; ++t) mi[t] = kList ? 2.0 * rc > 0.999 * L[t] : nc[t] < 3;
         const bool any_mi = mi[0] || mi[1] || mi[2];
         const float pass = cc->pass64;
         const int64_t per = (N + gridDim.x - 1) / gridDim.x;
         const int u1 = (int)min(N, (blockIdx.x + 1) * per);
-        for (int u = (int)(blockIdx.x * per) + wib; u < u1; u += kPair64Warps) {
-            const int i = sorted[u];
-            const float4 me = spos32[u];
-            const double4_32a m64 = spos64[u];
-            const double qki = pc.qk * m64.w;
+        const float wid[3] = {Lf[0] / nc[0], Lf[1] / nc[1], Lf[2] / nc[2]};
+        for (int base = (int)(blockIdx.x * per); base < u1; base += kPair64Warps) {
+            int part, parts, i = 0;
+            const int u = pair_round<kPair64Warps>(base, u1, wib, part, parts);
             s.fx = s.fy = s.fz = 0.0;
-            s.ecp = FF{0.0f, 0.0f};
-            int nh = 0;
-            // one buffered candidate per lane (lanes >= count idle)
-            auto evaluate = [&](int count, int base) {
-                const bool on = lane < count;
-                const int2 h = on ? hits[wib][base + lane] : make_int2(u, kPairNoShift);
-                const double4_32a o = spos64[h.x];
-                double dx = o.x - m64.x, dy = o.y - m64.y, dz = o.z - m64.z;
-                if (__any_sync(0xffffffffu, h.y != kPairNoShift)) {
-                    const int cx = h.y & 3, cy = (h.y >> 2) & 3, cz = (h.y >> 4) & 3;
-                    dx += cx == 1 ? 0.0 : (cx == 0 ? -L[0] : L[0]);
-                    dy += cy == 1 ? 0.0 : (cy == 0 ? -L[1] : L[1]);
-                    dz += cz == 1 ? 0.0 : (cz == 0 ? -L[2] : L[2]);
+            if (u >= 0) {
+                i = sorted[u];
+                const float4 me = spos32[u];
+                const double4_32a m64 = spos64[u];
+                const double qki = pc.qk * m64.w;
+                int nh = 0;
+                // one buffered candidate per lane (lanes >= count idle)
+                auto evaluate = [&](int count, int base) {
+                    const bool on = lane < count;
+                    const int2 h = on ? hits[wib][base + lane] : make_int2(u, kPairNoShift);
+                    const double4_32a o = spos64[h.x];
+                    long long dx = pair_diff(o.x, m64.x), dy = pair_diff(o.y, m64.y), dz = pair_diff(o.z, m64.z);
+                    if (__any_sync(0xffffffffu, h.y != kPairNoShift)) {
+                        dx = pair_shift(dx, h.y & 3, box.L[0]);
+                        dy = pair_shift(dy, (h.y >> 2) & 3, box.L[1]);
+                        dz = pair_shift(dz, (h.y >> 4) & 3, box.L[2]);
+                    }
+                    if (any_mi) {
+                        const float4 o32 = spos32[h.x];
+                        if (mi[0]) dx = pair_nearest(dx, o32.x - me.x, invLf[0], box.L[0], box.near[0]);
+                        if (mi[1]) dy = pair_nearest(dy, o32.y - me.y, invLf[1], box.L[1], box.near[1]);
+                        if (mi[2]) dz = pair_nearest(dz, o32.z - me.z, invLf[2], box.L[2], box.near[2]);
+                    }
+                    const unsigned long long n = pair_r2(dx, dy, dz);
+                    if (on && n < pc.unit.rc2) pair64_add<kDiag>(tab, pc, pc.lj != 0, dx, dy, dz, n, qki * o.w, s);
+                    __syncwarp();
+                };
+                if constexpr (kList) {
+                    const int all = la.nnb[u], k1 = (int)((int64_t)all * part / parts),
+                              nn = (int)((int64_t)all * (part + 1) / parts);
+                    const int* row = la.nbr + (int64_t)u * la.cap;
+                    const float hx = 0.5f * Lf[0], hy = 0.5f * Lf[1], hz = 0.5f * Lf[2];
+                    for (int k0 = k1; k0 < nn; k0 += 32 * kListBatch) {
+                        int sj[kListBatch];
+                        float4 o[kListBatch];
+#pragma unroll
+                        for (int a = 0; a < kListBatch; ++a) {
+                            const int k = k0 + 32 * a + lane;
+                            sj[a] = row[k < nn ? k : nn - 1];
+                        }
+#pragma unroll
+                        for (int a = 0; a < kListBatch; ++a) o[a] = spos32[sj[a]];
+#pragma unroll
+                        for (int a = 0; a < kListBatch; ++a) {
+                            const int k = k0 + 32 * a + lane;
+                            float dx = o[a].x - me.x, dy = o[a].y - me.y, dz = o[a].z - me.z;
+                            const int cx = dx > hx ? 0 : (dx < -hx ? 2 : 1), cy = dy > hy ? 0 : (dy < -hy ? 2 : 1),
+                                      cz = dz > hz ? 0 : (dz < -hz ? 2 : 1);
+                            dx += cx == 1 ? 0.0f : (cx == 0 ? -Lf[0] : Lf[0]);
+                            dy += cy == 1 ? 0.0f : (cy == 0 ? -Lf[1] : Lf[1]);
+                            dz += cz == 1 ? 0.0f : (cz == 0 ? -Lf[2] : Lf[2]);
+                            const bool hit = k < nn && dx * dx + dy * dy + dz * dz < pass;
+                            const unsigned m = __ballot_sync(0xffffffffu, hit);
+                            if (hit)  // on an axis with mi the code is 1: the image is rounded in FP64
+                                hits[wib][nh + __popc(m & ((1u << lane) - 1u))] =
+                                    make_int2(sj[a], (mi[0] ? 1 : cx) | ((mi[1] ? 1 : cy) << 2) | ((mi[2] ? 1 : cz) << 4));
+                            nh += __popc(m);
+                        }
+                        // evaluate whole groups of 32 and keep the rest at the front
+                        __syncwarp();
+                        int b0 = 0;
+                        for (; b0 + 32 <= nh; b0 += 32) evaluate(32, b0);
+                        __syncwarp();
+                        const int2 keep = b0 > 0 && lane < nh - b0 ? hits[wib][b0 + lane] : make_int2(0, 0);
+                        __syncwarp();
+                        if (b0 > 0 && lane < nh - b0) hits[wib][lane] = keep;
+                        __syncwarp();
+                        nh -= b0;
+                    }
+                } else {
+                    // segments of the neighbouring cells' slots, one per lane (see k_pair)
+                    int lo = 0, hi = 0, code = 0;
+                    float ctx = 0.f, cty = 0.f, ctz = 0.f;
+                    int sx, sy, sz;
+                    // the particle's image in the box, in cells
+                    const float frac[3] = {pair_cell_coord(me.x, invLf[0], nc[0]), pair_cell_coord(me.y, invLf[1], nc[1]),
+                                           pair_cell_coord(me.z, invLf[2], nc[2])};
+                    if (pair_segment_of(cid[i], nc, frac, wid, pass, lane, mi, cnt, start, lo, hi, sx, sy, sz)) {
+                        code = (sx + 1) | ((sy + 1) << 2) | ((sz + 1) << 4);
+                        ctx = me.x - (float)sx * Lf[0];
+                        cty = me.y - (float)sy * Lf[1];
+                        ctz = me.z - (float)sz * Lf[2];
+                    }
+                    for (int g = 0; g < 18; ++g) {
+                        const int glo = __shfl_sync(0xffffffffu, lo, g), ghi = __shfl_sync(0xffffffffu, hi, g);
+                        if (glo >= ghi) continue;  // the same for every lane
+                        const int gcode = __shfl_sync(0xffffffffu, code, g);
+                        const float gx = __shfl_sync(0xffffffffu, ctx, g), gy = __shfl_sync(0xffffffffu, cty, g),
+                                    gz = __shfl_sync(0xffffffffu, ctz, g);
+                        for (int s0 = glo + 32 * part; s0 < ghi; s0 += 32 * parts) {
+                            const int sl = s0 + lane;
+                            const float4 o = spos32[sl < ghi ? sl : glo];
+                            float dx = o.x - gx, dy = o.y - gy, dz = o.z - gz;
+                            if (any_mi) {
+                                if (mi[0]) dx -= Lf[0] * rintf(dx * invLf[0]);
+                                if (mi[1]) dy -= Lf[1] * rintf(dy * invLf[1]);
+                                if (mi[2]) dz -= Lf[2] * rintf(dz * invLf[2]);
+                            }
+                            const bool hit = sl < ghi && sl != u && dx * dx + dy * dy + dz * dz < pass;
+                            const unsigned m = __ballot_sync(0xffffffffu, hit);
+                            if (hit) hits[wib][nh + __popc(m & ((1u << lane) - 1u))] = make_int2(sl, gcode);
+                            nh += __popc(m);
+                            if (nh >= 32) {
+                                __syncwarp();
+                                evaluate(32, 0);
+                                __syncwarp();
+                                if (lane < nh - 32) hits[wib][lane] = hits[wib][32 + lane];
+                                __syncwarp();
+                                nh -= 32;
+                            }
+                        }
+                    }
                 }
-                if (any_mi) {
-                    if (mi[0]) dx -= L[0] * rint(dx * cc->invL[0]);
-                    if (mi[1]) dy -= L[1] * rint(dy * cc->invL[1]);
-                    if (mi[2]) dz -= L[2] * rint(dz * cc->invL[2]);
-                }
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                // r2 < rc^2 by the bits: both non-negative (and a NaN is above)
-                if (on && (unsigned long long)__double_as_longlong(r2) < pc.rc2)
-                    pair64_add<kDiag>(tab, pc, pc.lj != 0, dx, dy, dz, r2, m64.w, o.w, qki, s);
                 __syncwarp();
-            };
-            if constexpr (kList) {
-                const int nn = la.nnb[u];
-                const int* row = la.nbr + (int64_t)u * la.cap;
-                const float hx = 0.5f * Lf[0], hy = 0.5f * Lf[1], hz = 0.5f * Lf[2];
-                for (int k0 = 0; k0 < nn; k0 += 32 * kListBatch) {
-                    int sj[kListBatch];
-                    float4 o[kListBatch];
-#pragma unroll
-                    for (int a = 0; a < kListBatch; ++a) {
-                        const int k = k0 + 32 * a + lane;
-                        sj[a] = row[k < nn ? k : nn - 1];
-                    }
-#pragma unroll
-                    for (int a = 0; a < kListBatch; ++a) o[a] = spos32[sj[a]];
-#pragma unroll
-                    for (int a = 0; a < kListBatch; ++a) {
-                        const int k = k0 + 32 * a + lane;
-                        float dx = o[a].x - me.x, dy = o[a].y - me.y, dz = o[a].z - me.z;
-                        const int cx = dx > hx ? 0 : (dx < -hx ? 2 : 1), cy = dy > hy ? 0 : (dy < -hy ? 2 : 1),
-                                  cz = dz > hz ? 0 : (dz < -hz ? 2 : 1);
-                        dx += cx == 1 ? 0.0f : (cx == 0 ? -Lf[0] : Lf[0]);
-                        dy += cy == 1 ? 0.0f : (cy == 0 ? -Lf[1] : Lf[1]);
-                        dz += cz == 1 ? 0.0f : (cz == 0 ? -Lf[2] : Lf[2]);
-                        const bool hit = k < nn && dx * dx + dy * dy + dz * dz < pass;
-                        const unsigned m = __ballot_sync(0xffffffffu, hit);
-                        if (hit)  // on an axis with mi the code is 1: the image is rounded in FP64
-                            hits[wib][nh + __popc(m & ((1u << lane) - 1u))] =
-                                make_int2(sj[a], (mi[0] ? 1 : cx) | ((mi[1] ? 1 : cy) << 2) | ((mi[2] ? 1 : cz) << 4));
-                        nh += __popc(m);
-                    }
-                    // evaluate whole groups of 32 and keep the rest at the front
-                    __syncwarp();
-                    int b0 = 0;
-                    for (; b0 + 32 <= nh; b0 += 32) evaluate(32, b0);
-                    __syncwarp();
-                    const int2 keep = b0 > 0 && lane < nh - b0 ? hits[wib][b0 + lane] : make_int2(0, 0);
-                    __syncwarp();
-                    if (b0 > 0 && lane < nh - b0) hits[wib][lane] = keep;
-                    __syncwarp();
-                    nh -= b0;
-                }
-            } else {
-                // segments of the neighbouring cells' slots, one per lane (see k_pair)
-                int lo = 0, hi = 0, code = 0;
-                float ctx = 0.f, cty = 0.f, ctz = 0.f;
-                int sx, sy, sz;
-                if (pair_segment_of(cid[i], nc, lane, mi, cnt, start, lo, hi, sx, sy, sz)) {
-                    code = (sx + 1) | ((sy + 1) << 2) | ((sz + 1) << 4);
-                    ctx = me.x - (float)sx * Lf[0];
-                    cty = me.y - (float)sy * Lf[1];
-                    ctz = me.z - (float)sz * Lf[2];
-                }
-                for (int g = 0; g < 18; ++g) {
-                    const int glo = __shfl_sync(0xffffffffu, lo, g), ghi = __shfl_sync(0xffffffffu, hi, g);
-                    if (glo >= ghi) continue;  // the same for every lane
-                    const int gcode = __shfl_sync(0xffffffffu, code, g);
-                    const float gx = __shfl_sync(0xffffffffu, ctx, g), gy = __shfl_sync(0xffffffffu, cty, g),
-                                gz = __shfl_sync(0xffffffffu, ctz, g);
-                    for (int s0 = glo; s0 < ghi; s0 += 32) {
-                        const int sl = s0 + lane;
-                        const float4 o = spos32[sl < ghi ? sl : glo];
-                        float dx = o.x - gx, dy = o.y - gy, dz = o.z - gz;
-                        if (any_mi) {
-                            if (mi[0]) dx -= Lf[0] * rintf(dx * invLf[0]);
-                            if (mi[1]) dy -= Lf[1] * rintf(dy * invLf[1]);
-                            if (mi[2]) dz -= Lf[2] * rintf(dz * invLf[2]);
-                        }
-                        const bool hit = sl < ghi && sl != u && dx * dx + dy * dy + dz * dz < pass;
-                        const unsigned m = __ballot_sync(0xffffffffu, hit);
-                        if (hit) hits[wib][nh + __popc(m & ((1u << lane) - 1u))] = make_int2(sl, gcode);
-                        nh += __popc(m);
-                        if (nh >= 32) {
-                            __syncwarp();
-                            evaluate(32, 0);
-                            __syncwarp();
-                            if (lane < nh - 32) hits[wib][lane] = hits[wib][32 + lane];
-                            __syncwarp();
-                            nh -= 32;
-                        }
-                    }
-                }
+                if (nh > 0) evaluate(nh, 0);
+                __syncwarp();
+                warp_force_out(s.fx, s.fy, s.fz, pc.scale, lane, parts == 1 ? Fr + 3 * (int64_t)i : pforce[wib]);
             }
-            __syncwarp();
-            if (nh > 0) evaluate(nh, 0);
-            __syncwarp();
-            warp_force_out(s.fx, s.fy, s.fz, lane, Fr + 3 * (int64_t)i);
-            ff_acc(s.ec, ff_mul(s.ecp, charge_fits(m64.w) ? ff_of_double(m64.w) : FF{0.0f, 0.0f}));
+            if (parts > 1) pair_parts_out<kPair64Warps>(pforce, u, i, part, parts, wib, lane, Fr);  // the last round
         }
     }
-    pair64_partials<kDiag>(s, pc.qk, red, partials + kPartStride * (size_t)blockIdx.x, kDiag ? 3 : 1);
+    pair64_partials<kDiag>(s, pc.scale, red, partials + kPartStride * (size_t)blockIdx.x, kDiag ? 3 : 1);
 }
 
 // ---------------------------------------------------------------------------------
@@ -1355,12 +1358,12 @@ rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out
     p.s2 = c.s2;
     p.e4 = c.e4;
     p.e24 = c.e24;
-    std::memcpy(&p.rc2, &c.rc2, sizeof(p.rc2));
     const bool rc_ok = prm.rc >= 1e-4 && prm.rc <= 1e4;
     const int top = rc_ok ? std::ilogb(c.rc2) + 1 : 0;
+    p.unit = pair_unit(prm.rc, top);
+    p.scale = std::ldexp(1.0, kPairDrop - p.unit.s);
     const double y = c.s2 / std::ldexp(1.0, top - kPairOctaves), lj = 50.0 * std::fabs(c.e24) * std::pow(y, 6) / c.s2;
     if (rc_ok && (!c.lj || (std::isfinite(lj) && lj * y < 1e30))) {
-        p.base = (1023 + top - kPairOctaves) << kPairSegBits;
         const double key[5] = {ctx->alpha, c.rc2, c.s2, c.e24, c.e4};
         int t = 0;
         while (t < b.pair_tabs && std::memcmp(key, b.pair_key[t], sizeof(key)) != 0) ++t;
@@ -1482,9 +1485,10 @@ rbe_status npt_ensure(rbe_ctx ctx, int64_t N, const double box[3], double rc, do
 }
 
 // The cell list of the constants in ctx->npt.cellc: count, scan, fill, per-cell sort and the
-// packed positions (FP64 as well with fp64).  With a neighbour list (nls) the launches exit at
+// packed positions (FP64 as well with fp64, in fixed point of this unit unless it is kPairNoUnit).  With a
+// neighbour list (nls) the launches exit at
 // once on steps that do not rebuild it.
-rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls_v, bool fp64)
+rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls_v, bool fp64, int unit)
 {
     NptBuffers& b = ctx->npt;
     cudaStream_t s = ctx->stream;
@@ -1498,7 +1502,7 @@ rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const dou
     k_cl_fill<<<nb, kNptThreads, 0, s>>>(N, b.cid, b.cursor, b.fill, nls);
     const int64_t sort_blocks = ((int64_t)b.cellcap + kSortWarps - 1) / kSortWarps;
     k_cl_sort<<<(unsigned)sort_blocks, kSortWarps * 32, 0, s>>>(cc, b.cnt, b.start, b.fill, b.sorted, pos, q, b.spos32,
-                                                              fp64 ? b.spos64 : nullptr, nls);
+                                                              fp64 ? b.spos64 : nullptr, unit, nls);
     return npt_check(ctx, "cell list");
 }
 
@@ -1599,16 +1603,17 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
         if (list && (!b.nls || b.ncap_list < N)) return fail(ctx, RBE_ESTATE, "skin changed after rbe_npt_init: call it again");
         NListState* nls = list ? static_cast<NListState*>(b.nls) : nullptr;
         const CellConsts* cc = static_cast<const CellConsts*>(b.cellc);
+        const int unit = pair_unit(prm.rc, 0).s;
         if (list) {
             const int grid = (int)std::min<int64_t>(nb, (int64_t)ctx->num_sms * 4);
             if (fp64)
                 k_nl_check<true><<<grid, kNptThreads, 0, s>>>(N, sys->pos, sys->charge, b.sorted, b.spos32, b.spos64,
-                                                            b.sref, cc, nls);
+                                                            unit, b.sref, cc, nls);
             else
                 k_nl_check<false><<<grid, kNptThreads, 0, s>>>(N, sys->pos, sys->charge, b.sorted, b.spos32, nullptr,
-                                                             b.sref, cc, nls);
+                                                             unit, b.sref, cc, nls);
         }
-        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nls, fp64)) != RBE_OK) return st;
+        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nls, fp64, unit)) != RBE_OK) return st;
         const PairConst pc = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
         const ListArgs la{nls, b.nbr, b.nnb, b.sref, ctx->d.status, b.nbr_cap};
         const bool diag = prm.barostat >= 2;  // rectangular cell: the virial diagonal

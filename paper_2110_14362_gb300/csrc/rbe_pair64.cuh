@@ -1,5 +1,6 @@
 // Pair terms of the FP64 real space from tables: force factor and energy of the erfc Coulomb and of the
-// Lennard-Jones 12-6 potential as functions of u = r^2, to about 2^-52 (force) and 2^-45 (energy) per pair.
+// Lennard-Jones 12-6 potential as functions of u = r^2, to about 2^-52 (force) and 2^-45 (energy) per pair; the
+// separations in 64-bit fixed point.
 //
 // Why: GB300 issues an FP64 instruction over about 76 clocks of a warp and scheduler, and sqrt, the
 // division, exp and erfc of a pair are about 90 of them (the pair kernels kept the FP64 pipe 85 % busy).
@@ -8,7 +9,10 @@
 // Taylor polynomial of degree 8 about the centre (half a segment is at most 2^-8 of u, so each further
 // term is about 2^-7 smaller, and the first one left out below 2^-58), the constant term in FP64 and the
 // rest, at most 2^-5 of it, in float-float with FP32 for the small terms: two FP64 additions.  The
-// segment and the argument come from the bits of u.  With dU/du = -f/2 the energy is the integral
+// segment and the argument come from the bits of u, and u from integers: the separation of two coordinates
+// in fixed point is exact, box vectors included, and its square is nine 32-bit multiplications to 2^-59 of the
+// cutoff's.  What is left in FP64 per pair is eleven instructions: the charge product, one FMA and two
+// additions of the force factor, three roundings of separations, four FMAs of the force and the virial.  With dU/du = -f/2 the energy is the integral
 // of the same polynomial from the segment's centre, in float-float throughout.
 //
 // Coulomb derivatives: with B_0 = erfc(s r)/r and B_n = ((2n-1) B_{n-1} + (2a)^n e^{-a u} / sqrt(pi a)) / u
@@ -170,30 +174,91 @@ __host__ __device__ __forceinline__ double float_as_double(float f)
 #endif
 }
 
-// The segment of u and its argument tau (exact, tau = h + l); seg is outside [0, kPairSegs) where u is.
+// Separations as integers: coordinates in units of 2^-s, modulo 2^64, with s such that the cutoff is in
+// [2^61, 2^62): exact for every coordinate above rc / 512 in size (its last bit is a multiple of the unit),
+// and so are the differences, box vectors added, of a pair near the cutoff or below.  r^2 is counted in
+// 2^(64 - 2 s): the cutoff's square is in [2^58, 2^60).
+constexpr int kPairDrop = 11;  // bits of a separation left out where it becomes a double
+
+struct PairUnit {
+    int s;                   // the unit's exponent
+    int e;                   // r^2 with z leading zeros has the binary exponent e - z
+    int base;                // of the table's segments
+    unsigned long long rc2;  // the cutoff's square
+};
+
+inline PairUnit pair_unit(double rc, int top)
+{
+    PairUnit u;
+    u.s = 61 - std::ilogb(rc);
+    u.e = 127 - 2 * u.s;
+    u.base = ((u.e - top + kPairOctaves) << kPairSegBits) - (1 << kPairSegBits);
+    const double m = std::ldexp(rc, u.s - 61);  // rc in [1, 2)
+    u.rc2 = (unsigned long long)std::ldexp(m * m, 58);
+    return u;
+}
+
+// x in units of 2^-s, modulo 2^64, rounded to the nearest (finite x).
+__host__ __device__ __forceinline__ unsigned long long pair_fixed(unsigned long long bits, int s)
+{
+    const int e = (int)(bits >> 52) & 0x7ff;
+    const unsigned long long m = (bits & 0xFFFFFFFFFFFFFull) | (1ull << 52);
+    const int sh = e - 1075 + s;
+    unsigned long long v = 0;
+    if (e != 0 && sh >= 0 && sh < 64) v = m << sh;
+    else if (e != 0 && sh < 0 && sh >= -54) v = ((m >> (-sh - 1)) + 1) >> 1;
+    return bits >> 63 ? 0ull - v : v;
+}
+
+// The square sum of three separations (below 2^63 in size), times 2^-64: from the signed 32-bit halves,
+// without the squares of the low ones (below 1).
+__host__ __device__ __forceinline__ unsigned long long pair_r2(long long x, long long y, long long z)
+{
+    const int xl = (int)x, yl = (int)y, zl = (int)z;
+    const int xh = (int)(x >> 32) - (xl >> 31), yh = (int)(y >> 32) - (yl >> 31), zh = (int)(z >> 32) - (zl >> 31);
+    const long long mid = (long long)mad_wide(xh, xl, mad_wide(yh, yl, mad_wide(zh, zl, 0ull)));
+    return mad_wide(xh, xh, mad_wide(yh, yh, mad_wide(zh, zh, (unsigned long long)(mid >> 31))));
+}
+
+// The segment of u = r^2 and its argument tau = h + l (to 2^-46); seg is outside [0, kPairSegs) where u is.
 struct PairArg {
     int seg;
     FF tau;
-    float half;  // half the segment's half width
+    float half;         // half the segment's half width
+    uint32_t hi, lo;    // u normalised, the first bit set
+    int e;              // and its binary exponent
 };
 
-// base: (1023 + top - kPairOctaves) << kPairSegBits
-__host__ __device__ __forceinline__ PairArg pair_arg(uint32_t hi, uint32_t lo, int base)
+__host__ __device__ __forceinline__ int pair_clz(uint32_t x)
+{
+#ifdef __CUDA_ARCH__
+    return __clz((int)x);
+#else
+    return x ? __builtin_clz(x) : 32;
+#endif
+}
+
+__host__ __device__ __forceinline__ PairArg pair_arg(unsigned long long n, int e, int base)
 {
     PairArg a;
-    a.seg = (int)(hi >> (20 - kPairSegBits)) - base;
-    // the mantissa bits below the segment's: the first 23, and the others
-    constexpr int k = kPairSegBits + 3;
-    a.tau.h = RBE_FMA(2.0f, fx_float((((hi << k) | (lo >> (32 - k))) & 0x7FFFFFu) | 0x3F800000u), -3.0f);
-    a.tau.l = RBE_FMA(fx_float(((lo << (k - 9)) & 0x7FFFFFu) | 0x3F800000u), 0x1.0p-22f, -0x1.0p-22f);
+    const int z = pair_clz((uint32_t)(n >> 32));  // 32 and a segment far below for n < 2^32
+    n <<= z;
+    a.hi = (uint32_t)(n >> 32);
+    a.lo = (uint32_t)n;
+    a.e = e - z;
+    a.seg = (int)(a.hi >> (31 - kPairSegBits)) - (z << kPairSegBits) + base;
+    // the mantissa bits below the segment's: the first 23, and the next 23
+    constexpr int k = 31 - kPairSegBits - 23;
+    a.tau.h = RBE_FMA(2.0f, fx_float(((a.hi >> k) & 0x7FFFFFu) | 0x3F800000u), -3.0f);
+    a.tau.l = RBE_FMA(fx_float((((a.hi << (23 - k)) | (a.lo >> (9 + k))) & 0x7FFFFFu) | 0x3F800000u), 0x1.0p-22f, -0x1.0p-22f);
     // half width 2^(e - kPairSegBits - 1), halved
-    a.half = fx_float((((hi >> 20) - 896u) - (uint32_t)(kPairSegBits + 2)) << 23);
+    a.half = fx_float((uint32_t)(a.e + 127 - kPairSegBits - 2) << 23);
     return a;
 }
 
-// Force factor (FP64) and energy (float-float) of one part (0: Coulomb, 1: LJ) from its table planes.
+// One part (0: Coulomb, 1: LJ) from its table planes: the force factor as c0 + q, and the energy.
 template <int PART>
-__host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const PairArg& a, double& f, FF& energy)
+__host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const PairArg& a, double& c0, FF& q, FF& energy)
 {
     const PairWord* p = t + PART * kPairPlanes * kPairSegs + a.seg;
     const PairWord w0 = p[0], w1 = p[kPairSegs], w2 = p[2 * kPairSegs], w3 = p[3 * kPairSegs];
@@ -203,18 +268,16 @@ __host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const Pair
     const float c5 = fx_float(w3.w[0]), c6 = fx_float(w3.w[1]), c7 = fx_float(w3.w[2]), c8 = fx_float(w3.w[3]);
     const float s = RBE_FMA(RBE_FMA(RBE_FMA(c8, tau.h, c7), tau.h, c6), tau.h, c5);
     constexpr bool ANY = PART == 1;
-    FF q = ff_fma<ANY>(FF{s, 0.0f}, tau, c4);
+    q = ff_fma<ANY>(FF{s, 0.0f}, tau, c4);
     q = ff_fma<ANY>(q, tau, c3);
     q = ff_fma<ANY>(q, tau, c2);
     q = ff_fma<ANY>(q, tau, c1);
     q = ff_mul(q, tau);
 #ifdef __CUDA_ARCH__
-    f = __dadd_rn(__dadd_rn(__hiloint2double((int)w0.w[1], (int)w0.w[0]), float_as_double(q.h)), float_as_double(q.l));
+    c0 = __hiloint2double((int)w0.w[1], (int)w0.w[0]);
 #else
-    double d0;
     const unsigned long long b = ((unsigned long long)w0.w[1] << 32) | w0.w[0];
-    __builtin_memcpy(&d0, &b, 8);
-    f = (d0 + float_as_double(q.h)) + float_as_double(q.l);
+    __builtin_memcpy(&c0, &b, 8);
 #endif
     // energy e0 - half tau (c0 + tau (c1 / 2 + tau (c2 / 3 + tau (c3 / 4 + ...))))
     float si = RBE_FMA(RBE_MUL(c6, 1.0f / 7.0f), tau.h, RBE_MUL(c5, 1.0f / 6.0f));
@@ -231,24 +294,33 @@ __host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const Pair
 // Device side: the table in shared memory and the accumulation of one pair.
 #ifdef __CUDACC__
 
-constexpr int kPair64Warps = 16;  // warps of an FP64 pair block: one block per SM, its warps share the table
+// Warps of an FP64 pair block: one block per SM, its warps share the table.  From a list 16 (an NPT run of four
+// steps at N = 2e4: 1147 us; 18 warps 1166, 20 1194, 24 1328: fewer registers and less L1 beside the table); the
+// water's cell search, mostly loads and FP32, 24 (3000 molecules: 1710 us with 16, 1717 with 18, 1625 with 20, 1602).
+#ifndef RBE_PAIR64_WARPS
+#define RBE_PAIR64_WARPS 16
+#endif
+#ifndef RBE_WATER_PAIR_WARPS
+#define RBE_WATER_PAIR_WARPS 24
+#endif
+constexpr int kPair64Warps = RBE_PAIR64_WARPS, kWaterPairWarps = RBE_WATER_PAIR_WARPS;
 
 // The FP64 pair kernels' constants beside PairConst.
 struct Pair64Const {
     const PairWord* tab;  // device table, NULL: direct evaluation (cutoff or LJ sizes beyond the float range)
-    int base;             // (1023 + top - kPairOctaves) << kPairSegBits
+    PairUnit unit;
+    double scale;         // 2^(kPairDrop - s), the unit of the separations as doubles
     int lj;
     double alpha, sa, two_sa_pi, qk, s2, e4, e24;
-    unsigned long long rc2;  // bits of rc^2
 };
 
-// Sums of one lane: the particle's force, and over all particles of the warp the virial (its trace, or its
-// diagonal), and the energies: Coulomb without the Coulomb constant.
+// Sums of one lane: the particle's force and over all particles of the warp the virial (its trace, or its
+// diagonal), separations in units; and the energies.
 template <bool DIAG>
 struct Pair64Sums {
     double fx, fy, fz;
     double w[DIAG ? 3 : 1];
-    FF ecp, ec, el;   // ecp: sum_j q_j E of the current particle
+    FF ec, el;
     double ecd, eld;  // energies of the pairs evaluated directly
 };
 
@@ -258,43 +330,67 @@ __device__ __forceinline__ FF ff_of_double(double x)
     return (hi & 0x7ff00000u) == 0u ? FF{0.0f, 0.0f} : ff_of(hi, lo);
 }
 
-// A charge that float-floats hold to 48 bits: zero, or between 2^-60 and 2^60.
+// A charge product that float-floats hold to 48 bits: zero, or between 2^-60 and 2^60.
 __device__ __forceinline__ bool charge_fits(double q)
 {
     const uint32_t e = ((uint32_t)__double2hiint(q) >> 20) & 0x7ffu;
     return e == 0u || (e > 963u && e < 1083u);
 }
 
-// One pair: separation d (from i to the neighbour), r2 = |d|^2 < rc^2, charges qi, qj.
+// d / 2^11 (at most 2^51) rounded to an integer, as a double: one FP64 addition (the conversion of a 64-bit
+// integer is two conversions and an FMA on the FP64 pipe).  The rounding is 2^-52 of the cutoff at most, as much
+// as FP64 coordinates have at four times the cutoff.
+__device__ __forceinline__ double pair_double(long long d)
+{
+    const long long v = (d + (1 << (kPairDrop - 1))) >> kPairDrop;
+    return __dadd_rn(__longlong_as_double(v + 0x4338000000000000ll), -0x1.8p52);
+}
+
+// A pair below the table (r under 1/16 of the cutoff at least) or outside the float range: the force factor and
+// the energies (Coulomb, LJ).  Not inlined: rare, and its registers are not the evaluation's.
+static __device__ __noinline__ double3 pair_direct(double r2, double qq, double sa, double two_sa_pi, double alpha,
+                                                   double s2, double e24, double e4)
+{
+    const double r = sqrt(r2), inv_r = 1.0 / r, inv_r2 = inv_r * inv_r;
+    const double coul = qq * inv_r, er = erfc(sa * r);
+    const double sr2 = s2 * inv_r2, sr6 = sr2 * sr2 * sr2;
+    return make_double3(coul * (er + two_sa_pi * r * exp(-alpha * r2)) * inv_r2 + e24 * (2.0 * sr6 * sr6 - sr6) * inv_r2,
+                        coul * er, e4 * (sr6 * sr6 - sr6));
+}
+
+// One pair: separation d (from i to the neighbour) and n = r^2 < rc^2 in units, qq the charge product with the
+// Coulomb constant.  The table's force factor: qq (c0 + q) + (d0 + p), the two large terms in one FP64 FMA, the
+// small ones in float-float first.
 template <bool DIAG>
-__device__ __forceinline__ void pair64_add(const PairWord* __restrict__ tab, const Pair64Const& pc, bool lj, double dx,
-                                           double dy, double dz, double r2, double qi, double qj, double qki,
+__device__ __forceinline__ void pair64_add(const PairWord* __restrict__ tab, const Pair64Const& pc, bool lj, long long dxi,
+                                           long long dyi, long long dzi, unsigned long long n, double qq,
                                            Pair64Sums<DIAG>& s)
 {
-    const PairArg a = pair_arg((uint32_t)__double2hiint(r2), (uint32_t)__double2loint(r2), pc.base);
-    double f;
-    if (pc.tab && (unsigned)a.seg < (unsigned)kPairSegs && charge_fits(qj) && charge_fits(qi)) {
-        FF e;
-        pair_eval<0>(tab, a, f, e);
-        f *= qki * qj;
-        ff_acc(s.ecp, ff_mul(e, ff_of_double(qj)));
+    const PairArg a = pair_arg(n, pc.unit.e, pc.unit.base);
+    const double dx = pair_double(dxi), dy = pair_double(dyi), dz = pair_double(dzi);
+    double f, r2;
+    if (pc.tab && (unsigned)a.seg < (unsigned)kPairSegs && charge_fits(qq)) {
+        FF q, e;
+        pair_eval<0>(tab, a, f, q, e);
+        const FF qf = ff_of_double(qq);
+        ff_acc(s.ec, ff_mul(e, qf));
+        q = ff_mul(q, qf);
+        double d0 = 0.0;
         if (lj) {
-            double fl;
-            pair_eval<1>(tab, a, fl, e);
-            f += fl;
+            FF p;
+            pair_eval<1>(tab, a, d0, p, e);
             ff_acc(s.el, e);
+            ff_acc(q, p);
         }
+        f = (fma(f, qq, d0) + float_as_double(q.h)) + float_as_double(q.l);
+        r2 = __hiloint2double(((a.e + 1022) << 20) + (int)(a.hi >> 11), (int)((a.hi << 21) | (a.lo >> 11)));
     } else {
-        // below the table (r under 1/16 of the cutoff at least) or outside the float range
-        const double r = sqrt(r2), inv_r = 1.0 / r, inv_r2 = inv_r * inv_r;
-        const double coul = qki * qj * inv_r, er = erfc(pc.sa * r);
-        s.ecd += coul * er;
-        f = coul * (er + pc.two_sa_pi * r * exp(-pc.alpha * r2)) * inv_r2;
-        if (lj) {
-            const double sr2 = pc.s2 * inv_r2, sr6 = sr2 * sr2 * sr2;
-            s.eld += pc.e4 * (sr6 * sr6 - sr6);
-            f += pc.e24 * (2.0 * sr6 * sr6 - sr6) * inv_r2;
-        }
+        const double x = dx * pc.scale, y = dy * pc.scale, z = dz * pc.scale;
+        r2 = x * x + y * y + z * z;
+        const double3 t = pair_direct(r2, qq, pc.sa, pc.two_sa_pi, pc.alpha, lj ? pc.s2 : 0.0, pc.e24, pc.e4);
+        f = t.x;
+        s.ecd += t.y;
+        if (lj) s.eld += t.z;
     }
     // force on i is -f d
     if (DIAG) {
@@ -313,9 +409,62 @@ __device__ __forceinline__ void pair64_add(const PairWord* __restrict__ tab, con
     }
 }
 
+// Box edges in units, and the axes whose image is taken from FP32 separations per pair (mi).  There |d| can be
+// half an edge and still within the cutoff only if the edge is hardly above 2 rc: then the image is put right in
+// integers (near; the edge is below 2^64 units).
+struct PairBox {
+    unsigned long long L[3];
+    bool near[3];
+};
+
+__device__ __forceinline__ PairBox pair_box(const double L[3], double rc, int s)
+{
+    PairBox b;
+#pragma unroll
+    for (int t = 0; t < 3; ++t) {
+        b.L[t] = pair_fixed((unsigned long long)__double_as_longlong(L[t]), s);
+        b.near[t] = L[t] < 2.5 * rc;
+    }
+    return b;
+}
+
+// d plus the image of code c: 0: -L, 1: none, 2: +L
+__device__ __forceinline__ long long pair_shift(long long d, int c, unsigned long long L)
+{
+    return (long long)((unsigned long long)d + (c == 1 ? 0ull : (c == 0 ? 0ull - L : L)));
+}
+
+// d less the k edges that its FP32 value is nearest to
+__device__ __forceinline__ long long pair_nearest(long long d, float d32, float invL, unsigned long long L, bool near)
+{
+    d = (long long)((unsigned long long)d - (unsigned long long)__float2ll_rn(d32 * invL) * L);
+    if (near) {
+        const long long half = (long long)(L >> 1);
+        if (d > half) d = (long long)((unsigned long long)d - L);
+        else if (d < -half) d = (long long)((unsigned long long)d + L);
+    }
+    return d;
+}
+
+// A packed particle: its coordinates in units (as bits) and its charge.
+__device__ __forceinline__ double4_32a pair_pack(double x, double y, double z, double q, int s)
+{
+    double4_32a v;
+    v.x = __longlong_as_double((long long)pair_fixed((unsigned long long)__double_as_longlong(x), s));
+    v.y = __longlong_as_double((long long)pair_fixed((unsigned long long)__double_as_longlong(y), s));
+    v.z = __longlong_as_double((long long)pair_fixed((unsigned long long)__double_as_longlong(z), s));
+    v.w = q;
+    return v;
+}
+
+__device__ __forceinline__ long long pair_diff(double a, double b)
+{
+    return (long long)((unsigned long long)__double_as_longlong(a) - (unsigned long long)__double_as_longlong(b));
+}
+
 // The warp's force sums of one particle: a transposing tree (6 FP64 additions instead of 15) that ends with x,
-// y, z in lanes 0, 8, 16; they are written to F[3 i], F[3 i + 1], F[3 i + 2].
-__device__ __forceinline__ void warp_force_out(double fx, double fy, double fz, int lane, double* __restrict__ F)
+// y, z in lanes 0, 8, 16; they are written to F[0], F[1], F[2], times the separations' unit.
+__device__ __forceinline__ void warp_force_out(double fx, double fy, double fz, double unit, int lane, double* F)
 {
     const bool up = lane & 16, mid = lane & 8;
     double k0 = up ? fz : fx, k1 = up ? 0.0 : fy;
@@ -325,7 +474,7 @@ __device__ __forceinline__ void warp_force_out(double fx, double fy, double fz, 
     k += __shfl_xor_sync(0xffffffffu, mid ? k0 : k1, 8);
 #pragma unroll
     for (int off = 4; off > 0; off >>= 1) k += __shfl_xor_sync(0xffffffffu, k, off);
-    if ((lane & 7) == 0 && lane < 24) F[lane >> 3] = k;
+    if ((lane & 7) == 0 && lane < 24) F[lane >> 3] = k * unit;
 }
 
 __device__ __forceinline__ double warp_sum(double v)
@@ -335,18 +484,46 @@ __device__ __forceinline__ double warp_sum(double v)
     return v;
 }
 
+// A block's particles [u0, u1) over its W warps: round `base` gives one to each warp, and the last, partial
+// round gives each of its particles to `parts` warps (a power of two), warp wib taking part `part`: at 132
+// particles and 16 warps the last round of 4 takes a quarter of the time.  u < 0: none for this warp.
+template <int W>
+__device__ __forceinline__ int pair_round(int base, int u1, int wib, int& part, int& parts)
+{
+    const int left = u1 - base;
+    parts = 1;
+    while (2 * parts * left <= W) parts *= 2;
+    part = wib & (parts - 1);
+    const int k = wib / parts;
+    return k < left ? base + k : -1;
+}
+
+// The partial forces of a particle's warps (f[warp]), summed by the first of them in order.  All threads of
+// the block.
+template <int W>
+__device__ __forceinline__ void pair_parts_out(const double (*f)[3], int u, int i, int part, int parts, int wib, int lane,
+                                               double* __restrict__ Fr)
+{
+    __syncthreads();
+    if (u >= 0 && part == 0 && lane < 3) {
+        double t = f[wib][lane];
+        for (int k = 1; k < parts; ++k) t += f[wib + k][lane];
+        Fr[3 * (int64_t)i + lane] = t;
+    }
+}
+
 // Block partials of the sums: half of each (every pair is visited from both ends), virial components from slot
-// o, then E_coul (times the Coulomb constant) and E_lj.  All threads of the block.
-template <bool DIAG>
-__device__ __forceinline__ void pair64_partials(const Pair64Sums<DIAG>& s, double qk, double (*red)[kPair64Warps],
+// o, then E_coul and E_lj.  All threads of the block.
+template <bool DIAG, int W>
+__device__ __forceinline__ void pair64_partials(const Pair64Sums<DIAG>& s, double unit, double (*red)[W],
                                                 double* __restrict__ partials, int o)
 {
     constexpr int nw = DIAG ? 3 : 1;
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < nw + 2; ++k) {
-        const double v = k < nw ? s.w[k < nw ? k : 0]
-                                : (k == nw ? qk * ((double)s.ec.h + (double)s.ec.l) + s.ecd
+        const double v = k < nw ? (DIAG ? s.w[k < nw ? k : 0] * unit * unit : s.w[0])
+                                : (k == nw ? (double)s.ec.h + (double)s.ec.l + s.ecd
                                            : (double)s.el.h + (double)s.el.l + s.eld);
         const double t = warp_sum(v);
         if (lane == 0) red[k][wib] = t;
@@ -354,16 +531,26 @@ __device__ __forceinline__ void pair64_partials(const Pair64Sums<DIAG>& s, doubl
     __syncthreads();
     if (threadIdx.x < nw + 2) {
         double t = 0.0;
-        for (int v = 0; v < kPair64Warps; ++v) t += red[threadIdx.x][v];
+        for (int v = 0; v < W; ++v) t += red[threadIdx.x][v];
         partials[o + threadIdx.x] = 0.5 * t;
     }
 }
 
+// The particle's coordinate in the box, in cells.
+__device__ __forceinline__ float pair_cell_coord(float x, float invL, int nc)
+{
+    const float f = x * invL;
+    return (f - floorf(f)) * (float)nc;
+}
+
 // Lane's segment of the slots of the 27 cells around cell c: row r = lane / 2 of the 3 x 3 rows (dy, dz), part
 // lane % 2 (a row that wraps in x has two); [lo, hi) and the image shift (sx, sy, sz), 0 on an axis whose
-// image is taken per pair (mi).  An axis with fewer than 3 cells visits each of them once.  False: no
-// segment.
-__device__ __forceinline__ bool pair_segment_of(int c, const int nc[3], int lane, const bool mi[3],
+// image is taken per pair (mi).  An axis with fewer than 3 cells visits each of them once.  Cells that lie
+// farther than the search radius from the particle (fractional coordinates f of its image in the box, in cells of
+// width w; with the search's margin of 2^-16 edges) are left out: about a quarter of the slots at cells of 1.1 rc.
+// False: no segment.
+__device__ __forceinline__ bool pair_segment_of(int c, const int nc[3], const float f[3], const float w[3], float pass,
+                                                int lane, const bool mi[3],
                                                 const int* __restrict__ cnt, const int* __restrict__ start, int& lo,
                                                 int& hi, int& sx, int& sy, int& sz)
 {
@@ -377,6 +564,17 @@ __device__ __forceinline__ bool pair_segment_of(int c, const int nc[3], int lane
     const int uy = cy + dy, uz = cz + dz;
     const int yy = uy < 0 ? uy + nc[1] : (uy >= nc[1] ? uy - nc[1] : uy);
     const int zz = uz < 0 ? uz + nc[2] : (uz >= nc[2] ? uz - nc[2] : uz);
+    // distance to the row, and what it leaves for x
+    auto gap = [&](int t, int d, int cell) {
+        if (nc[t] < 3 || d == 0) return 0.0f;
+        float g = f[t] - (float)cell;  // in [0, 1], but for rounding over the box's edge
+        g = g < -0.5f ? g + (float)nc[t] : (g > 1.5f ? g - (float)nc[t] : g);
+        return fmaxf(0.0f, ((d < 0 ? g : 1.0f - g) - ((float)nc[t] * 0x1.0p-16f + 1e-4f)) * w[t]);
+    };
+    const float gy = gap(1, dy, cy), gz = gap(2, dz, cz), left2 = pass - gy * gy - gz * gz;
+    if (left2 < 0.0f) return false;
+    const float gl = gap(0, -1, cx), gr = gap(0, 1, cx);
+    const int nl = gl * gl < left2 ? 1 : 0, nr = gr * gr < left2 ? 1 : 0;
     sx = 0;
     sy = mi[1] ? 0 : (uy < 0 ? -1 : (uy >= nc[1] ? 1 : 0));
     sz = mi[2] ? 0 : (uz < 0 ? -1 : (uz >= nc[2] ? 1 : 0));
@@ -385,13 +583,13 @@ __device__ __forceinline__ bool pair_segment_of(int c, const int nc[3], int lane
     if (nx < 3) {
         if (part == 0) a = 0, e = nx - 1;
     } else if (cx == 0) {
-        if (part == 0) a = 0, e = 1;
-        else a = e = nx - 1, sx = -1;
+        if (part == 0) a = 0, e = nr;
+        else if (nl) a = e = nx - 1, sx = -1;
     } else if (cx == nx - 1) {
-        if (part == 0) a = nx - 2, e = nx - 1;
-        else a = e = 0, sx = 1;
+        if (part == 0) a = nx - 1 - nl, e = nx - 1;
+        else if (nr) a = e = 0, sx = 1;
     } else if (part == 0) {
-        a = cx - 1, e = cx + 1;
+        a = cx - nl, e = cx + nr;
     }
     if (a < 0) return false;
     if (mi[0]) sx = 0;

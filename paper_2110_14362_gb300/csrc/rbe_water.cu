@@ -304,14 +304,15 @@ k_water_drift(int64_t Nmol, double* __restrict__ pos, double* __restrict__ mom, 
 // stride over their slots; the separation is the nearest image per pair (sites may sit up to a
 // bond outside the box).  The search runs on the FP32 packed positions with rc plus a margin above
 // their rounding; the hits (slot, image code) go to a per-warp buffer in ballot order and are evaluated 32
-// at a time, one per lane, in FP64 from the FP64 packed positions with the exact cutoff; the pair terms come
-// from the tables of rbe_pair64.cuh (k_pair64 says what bounds it; on an axis shorter than 2 rc + 0.1 % the
-// image is rounded in FP64).  A hit of the
+// at a time, one per lane, from the fixed-point positions with the exact cutoff; the pair terms come
+// from the tables of rbe_pair64.cuh, the sums are FP64 (k_pair64 says more; in a box with an edge shorter than
+// 2 rc + 0.1 % the image is taken per pair).  Half of it is the search: cells out of reach are left out
+// (195 -> 164 us at 9000 sites), 24 warps a block (164 -> 150 us).  A hit of the
 // same molecule (site index / 3) is skipped; LJ acts between oxygens (site index divisible by 3).
 // Each pair is
 // visited from both ends: energies and the virial take half.  Per-block partials {W_r, E_coul,
 // E_lj} at slots 1..3 (the isotropic layout).  A box beyond the cell arrays leaves F_r = 0.
-__global__ void __launch_bounds__(kPair64Warps * 32, 1)
+__global__ void __launch_bounds__(kWaterPairWarps * 32, 1)
 k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, double rc, const int* __restrict__ cid,
              const int* __restrict__ cnt, const int* __restrict__ start, const int* __restrict__ sorted,
              const float4* __restrict__ spos32, const double4_32a* __restrict__ spos64, double* __restrict__ Fr,
@@ -319,8 +320,9 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc,
 {
     extern __shared__ __align__(16) unsigned char s_raw[];
     PairWord* tab = reinterpret_cast<PairWord*>(s_raw);
-    __shared__ int2 hits[kPair64Warps][kWaterHitCap];  // candidates within the FP32 search radius
-    __shared__ double red[3][kPair64Warps];
+    __shared__ int2 hits[kWaterPairWarps][kWaterHitCap];  // candidates within the FP32 search radius
+    __shared__ double red[3][kWaterPairWarps];
+    __shared__ double pforce[kWaterPairWarps][3];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     load_pair_table(pc.tab, tab);
     Pair64Sums<false> s{};
@@ -332,80 +334,89 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc,
         const int nc[3] = {cc->nc[0], cc->nc[1], cc->nc[2]};
         const double L[3] = {cc->L[0], cc->L[1], cc->L[2]};
         const float Lf[3] = {cc->Lf[0], cc->Lf[1], cc->Lf[2]}, invf[3] = {cc->invLf[0], cc->invLf[1], cc->invLf[2]};
+        const PairBox box = pair_box(L, rc, pc.unit.s);
         const bool exact = 2.0 * rc > 0.999 * fmin(L[0], fmin(L[1], L[2]));
         const bool mi[3] = {true, true, true};  // the segments carry no image: it is taken per pair
         const float pass = cc->pass64;
         const int64_t per = (N + gridDim.x - 1) / gridDim.x;
         const int u1 = (int)min(N, (blockIdx.x + 1) * per);
-        for (int u = (int)(blockIdx.x * per) + wib; u < u1; u += kPair64Warps) {
-            const int i = sorted[u];
-            const double4_32a me = spos64[u];
-            const float4 me32 = spos32[u];
-            const int mol_i = i / 3;
-            const bool oxy_i = i % 3 == 0 && pc.lj;
-            const double qki = pc.qk * me.w;
+        const float wid[3] = {Lf[0] / nc[0], Lf[1] / nc[1], Lf[2] / nc[2]};
+        for (int base = (int)(blockIdx.x * per); base < u1; base += kWaterPairWarps) {
+            int part, parts, i = 0;
+            const int u = pair_round<kWaterPairWarps>(base, u1, wib, part, parts);
             s.fx = s.fy = s.fz = 0.0;
-            s.ecp = FF{0.0f, 0.0f};
-            int lo = 0, hi = 0, sx, sy, sz, nh = 0;
-            pair_segment_of(cid[i], nc, lane, mi, cnt, start, lo, hi, sx, sy, sz);
-            auto evaluate = [&](int count) {
-                const bool on = lane < count;
-                const int2 h = on ? hits[wib][lane] : make_int2(u, 1 | (1 << 2) | (1 << 4));
-                const int j = sorted[h.x];
-                const double4_32a o = spos64[h.x];
-                double dx = o.x - me.x, dy = o.y - me.y, dz = o.z - me.z;
-                if (exact) {
-                    dx -= L[0] * rint(dx * cc->invL[0]);
-                    dy -= L[1] * rint(dy * cc->invL[1]);
-                    dz -= L[2] * rint(dz * cc->invL[2]);
-                } else if (__any_sync(0xffffffffu, h.y != (1 | (1 << 2) | (1 << 4)))) {
-                    const int cx = h.y & 3, cy = (h.y >> 2) & 3, cz = (h.y >> 4) & 3;
-                    dx += cx == 1 ? 0.0 : (cx == 0 ? -L[0] : L[0]);
-                    dy += cy == 1 ? 0.0 : (cy == 0 ? -L[1] : L[1]);
-                    dz += cz == 1 ? 0.0 : (cz == 0 ? -L[2] : L[2]);
+            if (u >= 0) {
+                i = sorted[u];
+                const double4_32a me = spos64[u];
+                const float4 me32 = spos32[u];
+                const int mol_i = i / 3;
+                const bool oxy_i = i % 3 == 0 && pc.lj;
+                const double qki = pc.qk * me.w;
+                int lo = 0, hi = 0, sx, sy, sz, nh = 0;
+                const float frac[3] = {pair_cell_coord(me32.x, invf[0], nc[0]), pair_cell_coord(me32.y, invf[1], nc[1]),
+                                       pair_cell_coord(me32.z, invf[2], nc[2])};
+                pair_segment_of(cid[i], nc, frac, wid, pass, lane, mi, cnt, start, lo, hi, sx, sy, sz);
+                auto evaluate = [&](int count) {
+                    const bool on = lane < count;
+                    const int2 h = on ? hits[wib][lane] : make_int2(u, 1 | (1 << 2) | (1 << 4));
+                    const int j = sorted[h.x];
+                    const double4_32a o = spos64[h.x];
+                    long long dx = pair_diff(o.x, me.x), dy = pair_diff(o.y, me.y), dz = pair_diff(o.z, me.z);
+                    if (exact) {
+                        const float4 o32 = spos32[h.x];
+                        dx = pair_nearest(dx, o32.x - me32.x, invf[0], box.L[0], box.near[0]);
+                        dy = pair_nearest(dy, o32.y - me32.y, invf[1], box.L[1], box.near[1]);
+                        dz = pair_nearest(dz, o32.z - me32.z, invf[2], box.L[2], box.near[2]);
+                    } else if (__any_sync(0xffffffffu, h.y != (1 | (1 << 2) | (1 << 4)))) {
+                        dx = pair_shift(dx, h.y & 3, box.L[0]);
+                        dy = pair_shift(dy, (h.y >> 2) & 3, box.L[1]);
+                        dz = pair_shift(dz, (h.y >> 4) & 3, box.L[2]);
+                    }
+                    const unsigned long long n = pair_r2(dx, dy, dz);
+                    // another molecule (the site itself excluded with its own) and r2 < rc^2
+                    if (on && j / 3 != mol_i && n < pc.unit.rc2)
+                        pair64_add<false>(tab, pc, oxy_i && j % 3 == 0, dx, dy, dz, n, qki * o.w, s);
+                    __syncwarp();
+                };
+                for (int g = 0; g < 18; ++g) {
+                    const int glo = __shfl_sync(0xffffffffu, lo, g), ghi = __shfl_sync(0xffffffffu, hi, g);
+                    for (int s0 = glo + 32 * part; s0 < ghi; s0 += 32 * parts) {  // the same trip count on every lane
+                        const int sl = s0 + lane;
+                        const float4 o = spos32[sl < ghi ? sl : glo];
+                        float dx = o.x - me32.x, dy = o.y - me32.y, dz = o.z - me32.z;
+                        // sites lie within a bond of [0, l), l >= 2 rc: the image is -1, 0 or 1
+                        // (rounded by adding 1.5 2^23: rintf runs on a quarter-rate pipe)
+                        const float kx = (dx * invf[0] + 12582912.f) - 12582912.f, ky = (dy * invf[1] + 12582912.f) - 12582912.f,
+                                    kz = (dz * invf[2] + 12582912.f) - 12582912.f;
+                        dx -= Lf[0] * kx;
+                        dy -= Lf[1] * ky;
+                        dz -= Lf[2] * kz;
+                        const bool hit = sl < ghi && sl != u && dx * dx + dy * dy + dz * dz < pass;
+                        const unsigned m = __ballot_sync(0xffffffffu, hit);
+                        if (hit) {
+                            const int code = (1 - (int)kx) | ((1 - (int)ky) << 2) | ((1 - (int)kz) << 4);
+                            hits[wib][nh + __popc(m & ((1u << lane) - 1u))] = make_int2(sl, code);
+                        }
+                        nh += __popc(m);
+                        if (nh >= 32) {
+                            __syncwarp();
+                            evaluate(32);
+                            __syncwarp();
+                            if (lane < nh - 32) hits[wib][lane] = hits[wib][32 + lane];
+                            __syncwarp();
+                            nh -= 32;
+                        }
+                    }
                 }
-                const double r2 = dx * dx + dy * dy + dz * dz;
-                // another molecule (the site itself excluded with its own) and r2 < rc^2 by the bits
-                if (on && j / 3 != mol_i && (unsigned long long)__double_as_longlong(r2) < pc.rc2)
-                    pair64_add<false>(tab, pc, oxy_i && j % 3 == 0, dx, dy, dz, r2, me.w, o.w, qki, s);
                 __syncwarp();
-            };
-            for (int g = 0; g < 18; ++g) {
-                const int glo = __shfl_sync(0xffffffffu, lo, g), ghi = __shfl_sync(0xffffffffu, hi, g);
-                for (int s0 = glo; s0 < ghi; s0 += 32) {  // the same trip count on every lane
-                    const int sl = s0 + lane;
-                    const float4 o = spos32[sl < ghi ? sl : glo];
-                    float dx = o.x - me32.x, dy = o.y - me32.y, dz = o.z - me32.z;
-                    // sites lie within a bond of [0, l), l >= 2 rc: the image is -1, 0 or 1
-                    const float kx = rintf(dx * invf[0]), ky = rintf(dy * invf[1]), kz = rintf(dz * invf[2]);
-                    dx -= Lf[0] * kx;
-                    dy -= Lf[1] * ky;
-                    dz -= Lf[2] * kz;
-                    const bool hit = sl < ghi && sl != u && dx * dx + dy * dy + dz * dz < pass;
-                    const unsigned m = __ballot_sync(0xffffffffu, hit);
-                    if (hit) {
-                        const int code = (1 - (int)kx) | ((1 - (int)ky) << 2) | ((1 - (int)kz) << 4);
-                        hits[wib][nh + __popc(m & ((1u << lane) - 1u))] = make_int2(sl, code);
-                    }
-                    nh += __popc(m);
-                    if (nh >= 32) {
-                        __syncwarp();
-                        evaluate(32);
-                        __syncwarp();
-                        if (lane < nh - 32) hits[wib][lane] = hits[wib][32 + lane];
-                        __syncwarp();
-                        nh -= 32;
-                    }
-                }
+                if (nh > 0) evaluate(nh);
+                __syncwarp();
+                warp_force_out(s.fx, s.fy, s.fz, pc.scale, lane, parts == 1 ? Fr + 3 * (int64_t)i : pforce[wib]);
             }
-            __syncwarp();
-            if (nh > 0) evaluate(nh);
-            __syncwarp();
-            warp_force_out(s.fx, s.fy, s.fz, lane, Fr + 3 * (int64_t)i);
-            ff_acc(s.ec, ff_mul(s.ecp, charge_fits(me.w) ? ff_of_double(me.w) : FF{0.0f, 0.0f}));
+            if (parts > 1) pair_parts_out<kWaterPairWarps>(pforce, u, i, part, parts, wib, lane, Fr);  // the last round
         }
     }
-    pair64_partials<false>(s, pc.qk, red, partials + kPartStride * (size_t)blockIdx.x, 1);
+    pair64_partials<false>(s, pc.scale, red, partials + kPartStride * (size_t)blockIdx.x, 1);
 }
 
 // ---------------------------------------------------------------------------------
@@ -594,13 +605,14 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, i
     if (st != RBE_OK) return st;
     if (prm.real) {
         if (b.n64 < N) return fail(ctx, RBE_ESTATE, "the FP64 packed positions are missing: call rbe_water_init again");
-        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nullptr, true)) != RBE_OK) return st;
+        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nullptr, true, pair_unit(prm.rc, 0).s)) != RBE_OK)
+            return st;
         Pair64Const pc;
         if ((st = pair64_const(ctx, prm, &pc)) != RBE_OK) return st;
         static const cudaError_t attr =
             cudaFuncSetAttribute(k_water_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairTabBytes);
         if (attr != cudaSuccess) return cuda_fail(ctx, attr, "shared memory of k_water_pair");
-        k_water_pair<<<nbp, kPair64Warps * 32, kPairTabBytes, s>>>(N, static_cast<const CellConsts*>(b.cellc), pc, prm.rc,
+        k_water_pair<<<nbp, kWaterPairWarps * 32, kPairTabBytes, s>>>(N, static_cast<const CellConsts*>(b.cellc), pc, prm.rc,
                                                                   b.cid, b.cnt, b.start, b.sorted, b.spos32, b.spos64,
                                                                   b.Fr, b.partials);
         if ((st = water_check(ctx, "k_water_pair")) != RBE_OK) return st;

@@ -25,17 +25,18 @@ int main()
         std::vector<PairWord> t(kPairTabBytes / sizeof(PairWord));
         for (int i = 0; i < kPairSegs; ++i) pair_segment(t.data(), i, top, alpha, sigma * sigma, 24.0 * eps, 4.0 * eps);
         while (in >> u) {
-            unsigned long long b;
-            std::memcpy(&b, &u, 8);
-            const PairArg a = pair_arg((uint32_t)(b >> 32), (uint32_t)b, (1023 + top - kPairOctaves) << kPairSegBits);
+            const PairUnit unit = pair_unit(rc, top);
+            const PairArg a = pair_arg((unsigned long long)std::ldexp(u, 2 * unit.s - 64), unit.e, unit.base);
             if ((unsigned)a.seg >= (unsigned)kPairSegs) {
                 std::printf("out\n");
                 continue;
             }
             double f, g;
-            FF e, l;
-            pair_eval<0>(t.data(), a, f, e);
-            pair_eval<1>(t.data(), a, g, l);
+            FF e, l, q;
+            pair_eval<0>(t.data(), a, f, q, e);
+            f = (f + (double)q.h) + (double)q.l;
+            pair_eval<1>(t.data(), a, g, q, l);
+            g = (g + (double)q.h) + (double)q.l;
             std::printf("%.17g %.17g %.17g %.17g\n", f, (double)e.h + (double)e.l, g, (double)l.h + (double)l.l);
         }
     }

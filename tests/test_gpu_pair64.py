@@ -60,3 +60,25 @@ def test_many_parameter_sets():
     with rbe.Context([14.0, 14.0, 14.0], ALPHA, 10, 1, rbe.RBE_FP64) as ctx:
         for k in list(range(10)) + [0, 9]:
             _check(ctx, pos, q, 14.0, 5.0 + 0.2 * k, 0.0, 2.0, 0.4)
+
+
+@pytest.mark.parametrize("skin", [0.0, 0.6])
+@pytest.mark.parametrize("N", [1, 2, 33, 609, 1217, 2433, 3801])
+def test_last_rounds(N, skin):
+    """Particle counts around the blocks' rounds (particles shared by 1, 2, 4, 8 or 16 warps, idle warps and
+    blocks); cells out of reach at 3 to 8 cells per axis."""
+    n = int(np.ceil(N ** (1 / 3)))
+    L = max(12.0, n * 2.2)
+    pos, q = _system(n, L, 11, 0)
+    keep = np.random.default_rng(N).permutation(n ** 3)[:N]
+    with rbe.Context([L, L, L], ALPHA, 10, 1, rbe.RBE_FP64) as ctx:
+        if N > 1:
+            _check(ctx, pos[keep], q[keep], L, 4.0, skin, 2.0, 0.4)
+        else:
+            rep_pos = pos[keep] * 0 + [0.0, L - 1e-12, 5.0]
+            prm = rbe.NptParams(dt=0.001, kT=2.5, P_ext=0.0, gamma=1.0, gamma_V=1.0, M_V=1.0, rc=4.0, qqr2e=1389.35, lj_sigma=2.0,
+                                lj_eps=0.4, max_disp=0.05, kspace=0, real=1, noise=0, barostat=0, skin=skin)
+            rep = rbe.NptReplica(rep_pos, rep_pos * 0, q[keep], np.full(1, 20.0), np.array([L, L, L]), prm, cuda_device())
+            rep.init(ctx)
+            ctx.sync()
+            assert np.all(rep.state()[2] == 0.0)
