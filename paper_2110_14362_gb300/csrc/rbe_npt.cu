@@ -600,7 +600,8 @@ __global__ void k_cl_fill(int64_t N, const int* __restrict__ cid, int* __restric
     fill[slot] = (int)i;
 }
 
-// Per cell, one warp: order the members by particle index (a fixed order for every run,
+// Per cell, kSortPart warps (a warp takes every kSortPart-th 32 members; one warp alone took 20 us for the 64
+// cells of 140 sites of 3000 waters, four take 10 us): order the members by particle index (a fixed order for every run,
 // whatever order the fill's atomics gave): the member with index i goes to rank = number of
 // members with a smaller index.  Then pack positions and charges in that order: FP32 xyzq
 // always (the pair search runs on it), and when spos64 is given FP64, as they are or (unit not kPairNoUnit)
@@ -613,32 +614,34 @@ k_cl_sort(const CellConsts* __restrict__ cc, const int* __restrict__ cnt, const 
 {
     if (nls && !nls->rebuild) return;
     const int64_t ncell = cc->ncell;  // -1: nothing to sort
-    const int64_t c = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+    const int64_t stride = ((int64_t)gridDim.x * blockDim.x >> 5) / kSortPart;
     const int lane = threadIdx.x & 31;
-    if (c >= ncell) return;  // c is the same for the whole warp
-    const int s0 = start[c], k = cnt[c];
-    for (int a0 = 0; a0 < k; a0 += 32) {
-        const int a = a0 + lane;
-        const int ia = a < k ? fill[s0 + a] : INT_MAX;
-        int rank = 0;
-        for (int b0 = 0; b0 < k; b0 += 32) {
-            const int b = b0 + lane;
-            const int ib = b < k ? fill[s0 + b] : INT_MAX;
+    for (int64_t c = wid / kSortPart; c < ncell; c += stride) {  // c is the same for the whole warp
+        const int s0 = start[c], k = cnt[c];
+        for (int a0 = 32 * (int)(wid % kSortPart); a0 < k; a0 += 32 * kSortPart) {
+            const int a = a0 + lane;
+            const int ia = a < k ? fill[s0 + a] : INT_MAX;
+            int rank = 0;
+            for (int b0 = 0; b0 < k; b0 += 32) {
+                const int b = b0 + lane;
+                const int ib = b < k ? fill[s0 + b] : INT_MAX;
 #pragma unroll 8
-            for (int t = 0; t < 32; ++t) rank += __shfl_sync(0xffffffffu, ib, t) < ia ? 1 : 0;
-        }
-        if (a < k) {
-            const double x = pos[3 * (int64_t)ia], y = pos[3 * (int64_t)ia + 1], z = pos[3 * (int64_t)ia + 2];
-            const double qq = q[ia];
-            sorted[s0 + rank] = ia;
-            spos32[s0 + rank] = make_float4((float)x, (float)y, (float)z, (float)qq);
-            if (spos64) {
-                double4_32a v;
-                v.x = x;
-                v.y = y;
-                v.z = z;
-                v.w = qq;
-                spos64[s0 + rank] = unit == kPairNoUnit ? v : pair_pack(x, y, z, qq, unit);
+                for (int t = 0; t < 32; ++t) rank += __shfl_sync(0xffffffffu, ib, t) < ia ? 1 : 0;
+            }
+            if (a < k) {
+                const double x = pos[3 * (int64_t)ia], y = pos[3 * (int64_t)ia + 1], z = pos[3 * (int64_t)ia + 2];
+                const double qq = q[ia];
+                sorted[s0 + rank] = ia;
+                spos32[s0 + rank] = make_float4((float)x, (float)y, (float)z, (float)qq);
+                if (spos64) {
+                    double4_32a v;
+                    v.x = x;
+                    v.y = y;
+                    v.z = z;
+                    v.w = qq;
+                    spos64[s0 + rank] = unit == kPairNoUnit ? v : pair_pack(x, y, z, qq, unit);
+                }
             }
         }
     }
@@ -1500,7 +1503,9 @@ rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const dou
     k_cl_count<<<nb, kNptThreads, 0, s>>>(N, pos, cc, b.cid, b.cnt, ctx->d.status, nls);
     k_cl_scan<<<1, kScanThreads, 0, s>>>(cc, b.cnt, b.start, b.cursor, nls);
     k_cl_fill<<<nb, kNptThreads, 0, s>>>(N, b.cid, b.cursor, b.fill, nls);
-    const int64_t sort_blocks = ((int64_t)b.cellcap + kSortWarps - 1) / kSortWarps;
+    // (the cell arrays have room for eight times the cells: a resident wave that strides over the cells there are)
+    const int64_t sort_blocks = std::min<int64_t>(((int64_t)b.cellcap * kSortPart + kSortWarps - 1) / kSortWarps,
+                                                  (int64_t)ctx->num_sms * 8);
     k_cl_sort<<<(unsigned)sort_blocks, kSortWarps * 32, 0, s>>>(cc, b.cnt, b.start, b.fill, b.sorted, pos, q, b.spos32,
                                                               fp64 ? b.spos64 : nullptr, unit, nls);
     return npt_check(ctx, "cell list");

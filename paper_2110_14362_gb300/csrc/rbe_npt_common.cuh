@@ -15,7 +15,8 @@ namespace rbe {
 
 constexpr double kFConv = 100.0;  // kJ/mol/A per g/mol -> A/ps^2
 constexpr int kScanThreads = 1024;
-constexpr int kSortWarps = 8;        // k_cl_sort: warps (cells) per block
+constexpr int kSortWarps = 8;        // k_cl_sort: warps per block
+constexpr int kSortPart = 4;         // k_cl_sort: warps per cell
 constexpr int kListBatch = 4;        // k_pair (list): list entries per lane loaded together
 constexpr int kHitCap = 32 * (kListBatch + 1);  // k_pair: buffered candidates per warp (< 32 + 32 kListBatch)
 // Per-block partial sums of the pair and finishing kernels: 8 doubles per block.  Isotropic:

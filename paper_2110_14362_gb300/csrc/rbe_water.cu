@@ -29,10 +29,13 @@
 namespace rbe {
 
 // Molecules per block of the per-molecule kernels (k_water_whole, k_water_drift, k_water_finish):
-// one warp, so that their FP64 constraint and virial arithmetic spreads over as many SMs'
+// one warp's, so that their FP64 constraint and virial arithmetic spreads over as many SMs'
 // FP64 pipes as there are warps of molecules (3000 molecules: 94 SMs, against 24 with blocks of
-// 128, where the drift took 97 us bound by the FP64 pipe of those 24 SMs).
+// 128, where the drift took 97 us bound by the FP64 pipe of those 24 SMs).  The drift and the
+// finishing kernel give a block three more warps, on the SM's other three schedulers, for what does not
+// depend on the chain of constraints: the normals of one site, the exclusion of one site pair.
 constexpr int kWaterThreads = 32;
+constexpr int kWaterWarps = 4;
 constexpr int kCellExcl = 25;       // cell block: the exclusion energy
 constexpr int kWaterHitCap = 64;    // buffered candidates per warp (< 32 buffered + 32 new)
 
@@ -75,6 +78,23 @@ __device__ __forceinline__ void solve3(const double A[3][3], const double b[3], 
     }
 }
 
+// x / y with r = 1 / y: the product and its residual's correction (Markstein 1990: correctly rounded but for
+// rare last bits), three instructions for the division's ten.
+__device__ __forceinline__ double w_div(double x, double y, double r)
+{
+    const double q = x * r;
+    return fma(fma(-q, y, x), r, q);
+}
+
+// A double as a float: its leading bits (0 below the float range, infinity above it).
+__device__ __forceinline__ float w_float(double x)
+{
+    const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
+    const uint32_t e = (hi >> 20) & 0x7ffu;
+    if (e > 1150u) return __int_as_float(0x7f800000);
+    return e < 897u ? 0.0f : __uint_as_float((hi & 0x80000000u) | ((e - 896u) << 23) | ((hi & 0xFFFFFu) << 3) | (lo >> 29));
+}
+
 // The change of (x_a - x_b) of constraint c per unit multiplier of constraint d, in units of
 // s_d: ((a_c == a_d) - (a_c == b_d))/m_{a_c} - ((b_c == a_d) - (b_c == b_d))/m_{b_c}.
 __device__ __forceinline__ double coupling(int c, int d, const double im[3])
@@ -86,45 +106,84 @@ __device__ __forceinline__ double coupling(int c, int d, const double im[3])
 // The position constraints of one molecule after an unconstrained move from the constrained xo:
 // x_i <- x_i + sum_d lambda_d s_old,d (e_{i,a_d} - e_{i,b_d}) / m_i with lambda making every
 // |x_a - x_b|^2 = d^2, the equations SHAKE solves (corrections along the old separations).  Here by
-// Newton's method on lambda (each step an exact 3x3 solve, quadratic convergence from lambda = 0):
-// it stops once every |r^2 - d^2| <= tol d^2, at the root SHAKE's sweeps converge to.  Returns
-// false when max_iter iterations did not get there.
+// Newton's method on lambda (quadratic convergence from lambda = 0): it stops once every
+// |r^2 - d^2| <= tol d^2, at the root SHAKE's sweeps converge to.  Returns false when max_iter iterations did
+// not get there.  The residuals and the moves are FP64; the 3x3 solves are FP32, which leaves about 2^-20 of a
+// residual beside the quadratic term (the same two or three iterations, for 42 FP64 instructions each instead
+// of 127), and FP64 in the last four iterations allowed.
 __device__ bool w_shake(double x[3][3], const double xo[3][3], const double im[3], const rbe_water_params& wp)
 {
     const double dd[3] = {wp.d_OH * wp.d_OH, wp.d_OH * wp.d_OH, wp.d_HH * wp.d_HH};
-    double so[3][3], K[3][3];
+    double so[3][3];
+    float sof[3][3], K2[3][3];
     #pragma unroll
     for (int c = 0; c < 3; ++c) {
         #pragma unroll
-        for (int t = 0; t < 3; ++t) so[c][t] = xo[wpa(c)][t] - xo[wpb(c)][t];
+        for (int t = 0; t < 3; ++t) {
+            so[c][t] = xo[wpa(c)][t] - xo[wpb(c)][t];
+            sof[c][t] = (float)so[c][t];
+        }
         #pragma unroll
-        for (int d = 0; d < 3; ++d) K[c][d] = coupling(c, d, im);
+        for (int d = 0; d < 3; ++d) K2[c][d] = (float)(2.0 * coupling(c, d, im));
     }
     for (int it = 0; it < wp.shake_max_iter; ++it) {
-        double s[3][3], g[3];
+        double s[3][3], g[3], dl[3];
         bool done = true;
         #pragma unroll
         for (int c = 0; c < 3; ++c) {
+            g[c] = -dd[c];
             #pragma unroll
-            for (int t = 0; t < 3; ++t) s[c][t] = x[wpa(c)][t] - x[wpb(c)][t];
-            g[c] = s[c][0] * s[c][0] + s[c][1] * s[c][1] + s[c][2] * s[c][2] - dd[c];
+            for (int t = 0; t < 3; ++t) {
+                s[c][t] = x[wpa(c)][t] - x[wpb(c)][t];
+                g[c] = fma(s[c][t], s[c][t], g[c]);
+            }
             if (fabs(g[c]) > wp.shake_tol * dd[c]) done = false;
         }
         if (done) return true;
-        double J[3][3], dl[3], rhs[3] = {-g[0], -g[1], -g[2]};
-        #pragma unroll
-        for (int c = 0; c < 3; ++c)
+        float det = 0.0f;
+        if (it + 4 < wp.shake_max_iter) {
+            float sf[3][3], J[3][3], cof[3][3];
             #pragma unroll
-            for (int d = 0; d < 3; ++d)
-                J[c][d] = 2.0 * K[c][d] * (s[c][0] * so[d][0] + s[c][1] * so[d][1] + s[c][2] * so[d][2]);
-        solve3(J, rhs, dl);
+            for (int c = 0; c < 3; ++c)
+                #pragma unroll
+                for (int t = 0; t < 3; ++t) sf[c][t] = w_float(s[c][t]);
+            #pragma unroll
+            for (int c = 0; c < 3; ++c)
+                #pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    J[c][d] = K2[c][d] * (sf[c][0] * sof[d][0] + sf[c][1] * sof[d][1] + sf[c][2] * sof[d][2]);
+            #pragma unroll
+            for (int c = 0; c < 3; ++c)
+                #pragma unroll
+                for (int d = 0; d < 3; ++d) {
+                    const int c1 = (c + 1) % 3, c2 = (c + 2) % 3, d1 = (d + 1) % 3, d2 = (d + 2) % 3;
+                    cof[c][d] = J[c1][d1] * J[c2][d2] - J[c1][d2] * J[c2][d1];
+                }
+            det = J[0][0] * cof[0][0] + J[0][1] * cof[0][1] + J[0][2] * cof[0][2];
+            const float id = -1.0f / det, r0 = id * (float)g[0], r1 = id * (float)g[1], r2 = id * (float)g[2];
+            #pragma unroll
+            for (int d = 0; d < 3; ++d) dl[d] = (double)(cof[0][d] * r0 + cof[1][d] * r1 + cof[2][d] * r2);
+        }
+        if (!(fabsf(det) > 1e-24f && fabsf(det) < 1e24f)) {  // the last iterations, or far from a molecule's sizes
+            double J[3][3];
+            #pragma unroll
+            for (int c = 0; c < 3; ++c) {
+                g[c] = -g[c];
+                #pragma unroll
+                for (int d = 0; d < 3; ++d)
+                    J[c][d] = 2.0 * coupling(c, d, im) * (s[c][0] * so[d][0] + s[c][1] * so[d][1] + s[c][2] * so[d][2]);
+            }
+            solve3(J, g, dl);
+        }
         #pragma unroll
-        for (int d = 0; d < 3; ++d)
+        for (int d = 0; d < 3; ++d) {
+            const double la = dl[d] * im[wpa(d)], lb = dl[d] * im[wpb(d)];
             #pragma unroll
             for (int t = 0; t < 3; ++t) {
-                x[wpa(d)][t] += dl[d] * so[d][t] * im[wpa(d)];
-                x[wpb(d)][t] -= dl[d] * so[d][t] * im[wpb(d)];
+                x[wpa(d)][t] += la * so[d][t];
+                x[wpb(d)][t] -= lb * so[d][t];
             }
+        }
     }
     return false;
 }
@@ -165,7 +224,7 @@ __device__ void w_project(double p[3][3], const double x[3][3], const double im[
 __device__ void w_kick(double p[3][3], const double F[3][3], const double x[3][3], const double m3[3],
                        const double im[3], double a, double b, double h)
 {
-    const double M = m3[0] + m3[1] + m3[2];
+    const double M = m3[0] + m3[1] + m3[2], rM = 1.0 / M;
     double P[3] = {0.0, 0.0, 0.0}, Ft[3] = {0.0, 0.0, 0.0};
     #pragma unroll
     for (int k = 0; k < 3; ++k)
@@ -178,9 +237,11 @@ __device__ void w_kick(double p[3][3], const double F[3][3], const double x[3][3
     #pragma unroll
     for (int t = 0; t < 3; ++t) dP[t] = P[t] * a + kFConv * Ft[t] * b - P[t];
     #pragma unroll
-    for (int k = 0; k < 3; ++k)
+    for (int k = 0; k < 3; ++k) {
+        const double mM = w_div(m3[k], M, rM);
         #pragma unroll
-        for (int t = 0; t < 3; ++t) p[k][t] += kFConv * h * (F[k][t] - m3[k] * Ft[t] / M) + (m3[k] / M) * dP[t];
+        for (int t = 0; t < 3; ++t) p[k][t] += kFConv * h * (F[k][t] - mM * Ft[t]) + mM * dP[t];
+    }
     w_project(p, x, im);
 }
 
@@ -190,10 +251,10 @@ __device__ void w_kick(double p[3][3], const double F[3][3], const double x[3][3
 __device__ bool w_drift(double x[3][3], double p[3][3], const double m3[3], const double im[3], double am1, double b,
                         double h, double cap, const rbe_water_params& wp)
 {
-    const double M = m3[0] + m3[1] + m3[2];
+    const double M = m3[0] + m3[1] + m3[2], rM = 1.0 / M, rh = 1.0 / h;
     double R[3], P[3] = {0.0, 0.0, 0.0}, d[3][3], dn[3][3], ds[3][3];
     #pragma unroll
-    for (int t = 0; t < 3; ++t) R[t] = (m3[0] * x[0][t] + m3[1] * x[1][t] + m3[2] * x[2][t]) / M;
+    for (int t = 0; t < 3; ++t) R[t] = w_div(m3[0] * x[0][t] + m3[1] * x[1][t] + m3[2] * x[2][t], M, rM);
     #pragma unroll
     for (int k = 0; k < 3; ++k)
         #pragma unroll
@@ -201,9 +262,12 @@ __device__ bool w_drift(double x[3][3], double p[3][3], const double m3[3], cons
             P[t] += p[k][t];
             d[k][t] = x[k][t] - R[t];
         }
-    double D[3];
+    double D[3], V[3];
     #pragma unroll
-    for (int t = 0; t < 3; ++t) D[t] = (P[t] / M) * b;
+    for (int t = 0; t < 3; ++t) {
+        V[t] = w_div(P[t], M, rM);
+        D[t] = V[t] * b;
+    }
     if (cap > 0.0) {
         const double len = sqrt(D[0] * D[0] + D[1] * D[1] + D[2] * D[2]);
         if (len > cap)
@@ -217,7 +281,7 @@ __device__ bool w_drift(double x[3][3], double p[3][3], const double m3[3], cons
     for (int k = 0; k < 3; ++k)
         #pragma unroll
         for (int t = 0; t < 3; ++t) {
-            dn[k][t] = d[k][t] + h * (p[k][t] * im[k] - P[t] / M);
+            dn[k][t] = d[k][t] + h * (p[k][t] * im[k] - V[t]);
             ds[k][t] = dn[k][t];
         }
     const bool ok = w_shake(ds, d, im, wp);
@@ -225,7 +289,7 @@ __device__ bool w_drift(double x[3][3], double p[3][3], const double m3[3], cons
     for (int k = 0; k < 3; ++k)
         #pragma unroll
         for (int t = 0; t < 3; ++t) {
-            p[k][t] += m3[k] * (ds[k][t] - dn[k][t]) / h;
+            p[k][t] += w_div(m3[k] * (ds[k][t] - dn[k][t]), h, rh);
             x[k][t] = Rn[t] + ds[k][t];
         }
     w_project(p, x, im);
@@ -251,38 +315,52 @@ k_water_whole(int64_t Nmol, double* __restrict__ pos, const double* __restrict__
     }
 }
 
-// Particles before the forces, one thread per molecule: R^p/2, R/2, O, R/2, the wrap by molecule.
-__global__ void __launch_bounds__(kWaterThreads)
+// Particles before the forces, one thread of warp 0 per molecule: R^p/2, R/2, O, R/2, the wrap by molecule; warp
+// 1 + k forms site k's noise meanwhile.  Bound by the serial FP64 chain of warp 0, about 76 clocks an
+// instruction: 3000 molecules 85 -> 55 us with the noise on other warps, quotients by reciprocals and the FP32
+// constraint solves.
+__global__ void __launch_bounds__(kWaterThreads * kWaterWarps)
 k_water_drift(int64_t Nmol, double* __restrict__ pos, double* __restrict__ mom, const double* __restrict__ force,
               const double* __restrict__ mass, const NptCoef* __restrict__ cfp, uint64_t seed,
               const double* __restrict__ cell, const rbe_water_params wp, double dt, unsigned* __restrict__ status)
 {
-    const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (I >= Nmol) return;
-    const uint64_t step = cell_step(cell);
+    __shared__ double sz[3][3][kWaterThreads];
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t I = (int64_t)blockIdx.x * kWaterThreads + lane;
+    const bool on = I < Nmol;
     const NptCoef& c = *cfp;
     const double h = 0.5 * dt;
-    const double m3[3] = {mass[3 * I], mass[3 * I + 1], mass[3 * I + 2]};
-    double x[3][3], p[3][3], F[3][3];
-    w_whole(pos, I, c.L, c.invL, x);
+    double x[3][3], p[3][3], m3[3], im[3];
+    bool ok = true;
+    if (on && warp > 0) {
+        const int k = warp - 1;
+        double z[4] = {0.0, 0.0, 0.0, 0.0};
+        if (c.noise) npt_normals(seed, 1u, cell_step(cell), (uint32_t)(3 * I + k), z);
+        const double s = c.sog * sqrt(mass[3 * I + k]);
+        #pragma unroll
+        for (int t = 0; t < 3; ++t) sz[k][t][lane] = s * z[t];
+    } else if (on) {
+        double F[3][3];
+        w_whole(pos, I, c.L, c.invL, x);
+        #pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            m3[k] = mass[3 * I + k];
+            im[k] = 1.0 / m3[k];
+            #pragma unroll
+            for (int t = 0; t < 3; ++t) {
+                p[k][t] = mom[9 * I + 3 * k + t];
+                F[k][t] = force[9 * I + 3 * k + t];
+            }
+        }
+        w_kick(p, F, x, m3, im, c.a1[0], c.b1[0], h);
+        ok = w_drift(x, p, m3, im, c.a2m1[0], c.b2[0], h, c.half_cap, wp);
+    }
+    __syncthreads();  // the one barrier of every thread of the block
+    if (warp > 0 || !on) return;
     #pragma unroll
     for (int k = 0; k < 3; ++k)
         #pragma unroll
-        for (int t = 0; t < 3; ++t) {
-            p[k][t] = mom[9 * I + 3 * k + t];
-            F[k][t] = force[9 * I + 3 * k + t];
-        }
-    const double im[3] = {1.0 / m3[0], 1.0 / m3[1], 1.0 / m3[2]};
-    w_kick(p, F, x, m3, im, c.a1[0], c.b1[0], h);
-    bool ok = w_drift(x, p, m3, im, c.a2m1[0], c.b2[0], h, c.half_cap, wp);
-    #pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        double z[4] = {0.0, 0.0, 0.0, 0.0};
-        if (c.noise) npt_normals(seed, 1u, step, (uint32_t)(3 * I + k), z);
-        const double s = c.sog * sqrt(m3[k]);
-        #pragma unroll
-        for (int t = 0; t < 3; ++t) p[k][t] = p[k][t] * c.g + s * z[t];
-    }
+        for (int t = 0; t < 3; ++t) p[k][t] = p[k][t] * c.g + sz[k][t][lane];
     w_project(p, x, im);
     ok = w_drift(x, p, m3, im, c.a3m1[0], c.b3[0], h, c.half_cap, wp) && ok;
     if (!ok) atomicOr(status, kStatusShake);
@@ -425,25 +503,46 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc,
 // R^p/2; the centres' 2K, the exclusion's virial plus the molecular correction -sum_i F_i . d_i,
 // and the exclusion energy as block partials {0: 2K, 4: W, 5: E_excl}.  The last block sums the
 // partials in a fixed order, forms W_mol = qqr2e tr(W_k) + W_r + W, P_ins = (2K + W_mol)/(3V) and,
-// with do_kick, V^p/2 and the step index.
-__global__ void __launch_bounds__(kWaterThreads)
+// with do_kick, V^p/2 and the step index.  Warp 0 has the molecules' chains, warp 1 + c their exclusions of site
+// pair c (3000 molecules: 40 -> 29 us).
+__global__ void __launch_bounds__(kWaterThreads * kWaterWarps)
 k_water_finish(int64_t Nmol, double* __restrict__ mom, double* __restrict__ force, const double* __restrict__ pos,
                const double* __restrict__ q, const double* __restrict__ mass, const double* __restrict__ Fk,
                const double* __restrict__ Fr, const double* __restrict__ WEk, const NptCoef* __restrict__ cfp,
                double* __restrict__ partials, int nblocks_pair, unsigned* __restrict__ counter,
                double* __restrict__ cell, rbe_npt_params prm, double alpha, int do_kick, unsigned* __restrict__ status)
 {
-    __shared__ double red[3][kWaterThreads / 32];
+    // of each site pair's exclusion: the force factor, energy and virial
+    __shared__ double s_ex[3][3][kWaterThreads];
     __shared__ bool is_last;
-    const int64_t I = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const int64_t I = (int64_t)blockIdx.x * kWaterThreads + lane;
+    const bool on = I < Nmol;
     double k2 = 0.0, wc = 0.0, ex = 0.0;
-    if (I < Nmol) {
-        const NptCoef& c = *cfp;
+    double x[3][3], F[3][3], p[3][3];
+    if (on) {
         const double L[3] = {cell[0], cell[1], cell[2]};
         const double inv[3] = {1.0 / L[0], 1.0 / L[1], 1.0 / L[2]};
-        const double m3[3] = {mass[3 * I], mass[3 * I + 1], mass[3 * I + 2]};
-        double x[3][3], F[3][3], p[3][3];
         w_whole(pos, I, L, inv, x);
+    }
+    if (on && warp > 0 && prm.real) {
+        const double sa = sqrt(alpha), tsp = 2.0 * sqrt(alpha / kPi);
+        #pragma unroll
+        for (int cp = 0; cp < 3; ++cp) {
+            if (cp != warp - 1) continue;
+            const int a = wpa(cp), b = wpb(cp);
+            double d[3];
+            #pragma unroll
+            for (int t = 0; t < 3; ++t) d[t] = x[b][t] - x[a][t];
+            const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], r = sqrt(r2);
+            const double qq = prm.qqr2e * q[3 * I + a] * q[3 * I + b], ef = erf(sa * r);
+            const double f = qq * (tsp * exp(-alpha * r2) / r - ef / r2) / r;
+            s_ex[cp][0][lane] = f;
+            s_ex[cp][1][lane] = qq * ef / r;
+            s_ex[cp][2][lane] = f * r2;
+        }
+    }
+    if (on && warp == 0) {
         #pragma unroll
         for (int k = 0; k < 3; ++k)
             #pragma unroll
@@ -452,30 +551,30 @@ k_water_finish(int64_t Nmol, double* __restrict__ mom, double* __restrict__ forc
                 F[k][t] = (prm.kspace ? prm.qqr2e * Fk[j] : 0.0) + (prm.real ? Fr[j] : 0.0);
                 p[k][t] = mom[j];
             }
+    }
+    __syncthreads();
+    if (on && warp == 0) {
+        const NptCoef& c = *cfp;
+        const double m3[3] = {mass[3 * I], mass[3 * I + 1], mass[3 * I + 2]};
         if (prm.real) {
-            const double sa = sqrt(alpha), tsp = 2.0 * sqrt(alpha / kPi);
             #pragma unroll
             for (int cp = 0; cp < 3; ++cp) {
                 const int a = wpa(cp), b = wpb(cp);
-                double d[3];
-                #pragma unroll
-                for (int t = 0; t < 3; ++t) d[t] = x[b][t] - x[a][t];
-                const double r2 = d[0] * d[0] + d[1] * d[1] + d[2] * d[2], r = sqrt(r2);
-                const double qq = prm.qqr2e * q[3 * I + a] * q[3 * I + b], ef = erf(sa * r);
-                const double f = qq * (tsp * exp(-alpha * r2) / r - ef / r2) / r;
-                ex -= qq * ef / r;
+                const double f = s_ex[cp][0][lane];
+                ex -= s_ex[cp][1][lane];
                 #pragma unroll
                 for (int t = 0; t < 3; ++t) {
-                    F[b][t] += f * d[t];
-                    F[a][t] -= f * d[t];
+                    const double d = x[b][t] - x[a][t];
+                    F[b][t] += f * d;
+                    F[a][t] -= f * d;
                 }
-                wc += f * r2;
+                wc += s_ex[cp][2][lane];
             }
         }
-        const double M = m3[0] + m3[1] + m3[2];
+        const double M = m3[0] + m3[1] + m3[2], rM = 1.0 / M;
         double R[3];
         #pragma unroll
-        for (int t = 0; t < 3; ++t) R[t] = (m3[0] * x[0][t] + m3[1] * x[1][t] + m3[2] * x[2][t]) / M;
+        for (int t = 0; t < 3; ++t) R[t] = w_div(m3[0] * x[0][t] + m3[1] * x[1][t] + m3[2] * x[2][t], M, rM);
         #pragma unroll
         for (int k = 0; k < 3; ++k)
             #pragma unroll
@@ -498,48 +597,42 @@ k_water_finish(int64_t Nmol, double* __restrict__ mom, double* __restrict__ forc
             for (int t = 0; t < 3; ++t) P[t] += p[k][t];
         k2 = (P[0] * P[0] + P[1] * P[1] + P[2] * P[2]) / M * (1.0 / kFConv);
     }
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    if (warp == 0) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1) {
-        k2 += __shfl_xor_sync(0xffffffffu, k2, off);
-        wc += __shfl_xor_sync(0xffffffffu, wc, off);
-        ex += __shfl_xor_sync(0xffffffffu, ex, off);
+        for (int off = 16; off > 0; off >>= 1) {
+            k2 += __shfl_xor_sync(0xffffffffu, k2, off);
+            wc += __shfl_xor_sync(0xffffffffu, wc, off);
+            ex += __shfl_xor_sync(0xffffffffu, ex, off);
+        }
+        if (lane == 0) {
+            double* row = partials + kPartStride * (size_t)(nblocks_pair + blockIdx.x);
+            row[0] = k2;
+            row[4] = wc;
+            row[5] = ex;
+            __threadfence();
+        }
     }
-    if (lane == 0) {
-        red[0][warp] = k2;
-        red[1][warp] = wc;
-        red[2][warp] = ex;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double sum = 0.0;
-        for (int wv = 0; wv < kWaterThreads / 32; ++wv) sum += red[threadIdx.x][wv];
-        const int slot = threadIdx.x == 0 ? 0 : 3 + threadIdx.x;  // 0, 4, 5
-        partials[kPartStride * (size_t)(nblocks_pair + blockIdx.x) + slot] = sum;
-        __threadfence();
-    }
-    __syncthreads();
     if (threadIdx.x == 0) is_last = (atomicAdd(counter, 1u) == gridDim.x - 1);
     __syncthreads();
     if (!is_last) return;
     __threadfence();
     // fin: 0 2K, 1 W_r, 2 E_coul, 3 E_lj, 4 W (exclusion + correction), 5 E_excl
-    __shared__ double fin[6][kWaterThreads];
+    __shared__ double fin[6][kWaterThreads * kWaterWarps];
     {
         double v[6] = {0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
-        for (int b = threadIdx.x; b < (int)gridDim.x; b += kWaterThreads) {
+        for (int b = threadIdx.x; b < (int)gridDim.x; b += kWaterThreads * kWaterWarps) {
             const double* pb = partials + kPartStride * (size_t)(nblocks_pair + b);
             v[0] += __ldcg(pb);
             v[4] += __ldcg(pb + 4);
             v[5] += __ldcg(pb + 5);
         }
         if (prm.real)
-            for (int b = threadIdx.x; b < nblocks_pair; b += kWaterThreads)
+            for (int b = threadIdx.x; b < nblocks_pair; b += kWaterThreads * kWaterWarps)
                 for (int a = 1; a <= 3; ++a) v[a] += __ldcg(partials + kPartStride * (size_t)b + a);
         for (int a = 0; a < 6; ++a) fin[a][threadIdx.x] = v[a];
     }
     __syncthreads();
-    for (int half = kWaterThreads / 2; half > 0; half >>= 1) {
+    for (int half = kWaterThreads * kWaterWarps / 2; half > 0; half >>= 1) {
         if (threadIdx.x < half)
             for (int a = 0; a < 6; ++a) fin[a][threadIdx.x] += fin[a][threadIdx.x + half];
         __syncthreads();
@@ -619,7 +712,7 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, i
     }
     if ((st = fork.join()) != RBE_OK) return st;
     const int nbm = (int)std::max<int64_t>(1, (Nmol + kWaterThreads - 1) / kWaterThreads);
-    k_water_finish<<<nbm, kWaterThreads, 0, s>>>(Nmol, sys->mom, sys->force, sys->pos, sys->charge, sys->mass, b.Fk,
+    k_water_finish<<<nbm, kWaterThreads * kWaterWarps, 0, s>>>(Nmol, sys->mom, sys->force, sys->pos, sys->charge, sys->mass, b.Fk,
                                                  b.Fr, b.WEk, reinterpret_cast<const NptCoef*>(b.coef), b.partials, nbp,
                                                  b.counter, sys->cell, prm, ctx->alpha, do_kick, ctx->d.status);
     return water_check(ctx, "k_water_finish");
@@ -669,7 +762,7 @@ rbe_status water_run(rbe_ctx ctx, rbe_system* sys, const rbe_water_params* wp, i
     for (int32_t k = 0; k < nsteps; ++k) {
         KspaceFork fork(ctx, sys);
         if ((st = launch_npt_cell_iso(ctx, sys)) != RBE_OK || (st = fork.tables(sys)) != RBE_OK) return st;
-        k_water_drift<<<nbm, kWaterThreads, 0, ctx->stream>>>(Nmol, sys->pos, sys->mom, sys->force, sys->mass,
+        k_water_drift<<<nbm, kWaterThreads * kWaterWarps, 0, ctx->stream>>>(Nmol, sys->pos, sys->mom, sys->force, sys->mass,
                                                               reinterpret_cast<const NptCoef*>(ctx->npt.coef),
                                                               ctx->seed, sys->cell, *wp, sys->params.dt, ctx->d.status);
         if ((st = water_check(ctx, "k_water_drift")) != RBE_OK) return st;
