@@ -237,7 +237,8 @@ struct KspaceFork {
     bool on;  // on the side stream; otherwise each call runs on the context's stream in order
     KspaceFork(rbe_ctx c, const rbe_system* sys);
     rbe_status tables(const rbe_system* sys);  // after the cell update: tables of the new box and the sampler
-    rbe_status passes(const rbe_system* sys);  // after the drift: rho, reduction, forces into npt.Fk and npt.WEk
+    // after the drift: (in order: the tables and the sampler,) rho, reduction, forces into npt.Fk and npt.WEk
+    rbe_status passes(const rbe_system* sys);
     rbe_status join();                         // before the finishing kernel
     KspaceFork(const KspaceFork&) = delete;
     ~KspaceFork();
@@ -245,6 +246,7 @@ struct KspaceFork {
   private:
     bool forked = false;
     rbe_status branch(int ev);
+    rbe_status launch_tables(const rbe_system* sys);
 };
 rbe_status npt_prepare(rbe_ctx ctx, rbe_system* sys, uint64_t batch);
 rbe_status launch_npt_set_step(rbe_ctx ctx, double* cell, uint64_t step);

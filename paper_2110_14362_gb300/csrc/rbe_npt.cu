@@ -1552,11 +1552,13 @@ static rbe_status on_side(rbe_ctx ctx, bool on, Fn f)
 
 rbe_status KspaceFork::tables(const rbe_system* sys)
 {
-    if (!sys->params.kspace) return RBE_OK;
-    if (on) {
-        const rbe_status st = branch(0);
-        if (st != RBE_OK) return st;
-    }
+    if (!on || !sys->params.kspace) return RBE_OK;
+    const rbe_status st = branch(0);
+    return st == RBE_OK ? launch_tables(sys) : st;
+}
+
+rbe_status KspaceFork::launch_tables(const rbe_system* sys)
+{
     ctx->tables_dirty = true;  // the snapshot API must rebuild from its own box
     // tables from the device box and the sampler at the device-resident step index (one launch)
     return on_side(ctx, on, [&] {
@@ -1568,13 +1570,13 @@ rbe_status KspaceFork::tables(const rbe_system* sys)
 rbe_status KspaceFork::passes(const rbe_system* sys)
 {
     if (!sys->params.kspace) return RBE_OK;
-    if (on) {
-        const rbe_status st = branch(1);
-        if (st != RBE_OK) return st;
-    }
+    // in order, the sampler stands between the drift and the rho pass, which starts early behind the kernel
+    // before it and reads the positions then
+    rbe_status st = on ? branch(1) : launch_tables(sys);
+    if (st != RBE_OK) return st;
     NptBuffers& b = ctx->npt;
     ctx->rho_plain = on;
-    const rbe_status st = on_side(
+    st = on_side(
         ctx, on, [&] { return launch_rbe(ctx, sys->N, sys->pos, sys->charge, ctx->P, b.Fk, b.WEk, b.WEk + 9); });
     ctx->rho_plain = false;
     return st;
