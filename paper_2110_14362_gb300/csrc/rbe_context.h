@@ -190,6 +190,33 @@ inline void ctx_free(rbe_ctx ctx, void* p)
     if (p) cudaFreeAsync(p, ctx->stream);
 }
 
+// Launch with programmatic stream serialization (the kernel calls pdl_wait()), or, with pdl false, in plain
+// stream order: a rho pass behind an event wait, which stages its particles before pdl_wait() and so must not
+// start before the event.
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_ordered(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                                  Args... args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
+}
+
+template <typename... KArgs, typename... Args>
+inline cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
+                              Args... args)
+{
+    return launch_ordered(true, kern, grid, block, smem, s, args...);
+}
+
 // Device validation helpers (rbe_api.cu).
 rbe_status fail(rbe_ctx ctx, rbe_status st, const std::string& msg);
 rbe_status cuda_fail(rbe_ctx ctx, cudaError_t err, const char* what);
@@ -224,8 +251,8 @@ rbe_status npt_ensure(rbe_ctx ctx, int64_t N, const double box[3], double rc, do
 int pair_blocks(rbe_ctx ctx, int64_t N, bool fp64);
 int pair_blocks64(rbe_ctx ctx, int64_t N);
 struct Pair64Const;
-rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out);
-rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls, bool fp64, int unit);
+rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out, bool* built);
+rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls, bool fp64, int unit, bool zeroed);
 // launch_cell_list: FP64 positions packed as they are
 constexpr int kPairNoUnit = -(1 << 20);
 // Shared with the rigid-water step (rbe_npt.cu): parameter checks, the setup of rbe_npt_init

@@ -1177,7 +1177,7 @@ static rbe_status flex_forces(rbe_ctx ctx, rbe_flex_system* sys, int do_kick)
                                                                   ctx->flex_cpos32, nullptr, b.sref, cf, nl);
         }
         if ((st = launch_cell_list(ctx, N, ctx->gpos, sys->charge, list ? &nl->base : nullptr, fp64,
-                                   kPairNoUnit)) != RBE_OK)
+                                   kPairNoUnit, false)) != RBE_OK)
             return st;
         const PairConst pc = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
         const CellConsts* cc = static_cast<const CellConsts*>(b.cellc);

@@ -473,33 +473,6 @@ static Plan make_plan(rbe_ctx ctx, int64_t N, int K, const RhoShape& rs, int rho
     return p;
 }
 
-// Launch with programmatic stream serialization (the kernel calls pdl_wait()), or, with pdl false, in plain
-// stream order: a rho pass behind an event wait, which stages its particles before pdl_wait() and so must not
-// start before the event.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_ordered(bool pdl, void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                                  Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<KArgs>(args)...);
-}
-
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_pdl(void (*kern)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s,
-                              Args... args)
-{
-    return launch_ordered(true, kern, grid, block, smem, s, args...);
-}
-
 // The FP32-phase rho pass of plan p on stream s (the wide two-frequency kernel when p.klanes > 0).
 static cudaError_t launch_rho_f32(bool pdl, int accum, bool xyzq, const Plan& p, dim3 grid, cudaStream_t s,
                                   const void* pos, const double* q, int64_t N, const KState* ks, const int4* m, int K,

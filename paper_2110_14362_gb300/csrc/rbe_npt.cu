@@ -86,16 +86,19 @@ __global__ void k_cell_consts(const double* __restrict__ cell, double rc, double
 
 
 // Per step, before the cell list: refresh the packed positions in the list's slot order and
-// decide whether the list must be rebuilt.  Until the first build there is no slot order:
+// decide whether the list must be rebuilt; and the cells' counts to zero.  Until the first build there is no slot order:
 // the kernel then only asks for a build.
 template <bool kF64>
 __global__ void __launch_bounds__(kNptThreads)
 k_nl_check(int64_t N, const double* __restrict__ pos, const double* __restrict__ q, const int* __restrict__ sorted,
            float4* __restrict__ spos32, double4_32a* __restrict__ spos64, int unit, const float4* __restrict__ sref,
-           const CellConsts* __restrict__ cc, NListState* __restrict__ nls)
+           const CellConsts* __restrict__ cc, NListState* __restrict__ nls, int* __restrict__ cnt, int cellcap)
 {
     __shared__ float smax[kNptThreads / 32];
     __shared__ bool last;
+    pdl_wait();
+    pdl_trigger();
+    for (int j = blockIdx.x * blockDim.x + threadIdx.x; j < cellcap; j += gridDim.x * blockDim.x) cnt[j] = 0;
     const bool force = nls->force != 0;
     float d2max = 0.f;
     if (!force) {
@@ -476,6 +479,8 @@ k_npt_drift(int64_t N, double* __restrict__ pos, double* __restrict__ mom, const
             const double* __restrict__ cell)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (i >= N) return;
     const uint64_t step = cell_step(cell);
     const NptCoef& c = *cfp;
@@ -533,6 +538,8 @@ k_cl_count(int64_t N, const double* __restrict__ pos, const CellConsts* __restri
            int* __restrict__ cnt, unsigned* __restrict__ status, const NListState* __restrict__ nls)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (i >= N) return;
     if (i == 0 && !cc->ok) atomicOr(status, kStatusBox);
     if (nls && !nls->rebuild) return;  // the neighbour list stands: no cell list this step
@@ -555,6 +562,8 @@ k_cl_scan(const CellConsts* __restrict__ cc, const int* __restrict__ cnt, int* _
           int* __restrict__ cursor, const NListState* __restrict__ nls)
 {
     __shared__ int wsum[kScanThreads / 32];
+    pdl_wait();
+    pdl_trigger();
     if (nls && !nls->rebuild) return;
     // a box beyond the cell arrays put every particle in cell 0 with a count of 0: start and
     // cursor of cell 0 are still written (0), so the fill stays in bounds
@@ -594,6 +603,8 @@ __global__ void k_cl_fill(int64_t N, const int* __restrict__ cid, int* __restric
                           const NListState* __restrict__ nls)
 {
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    pdl_wait();
+    pdl_trigger();
     if (i >= N) return;
     if (nls && !nls->rebuild) return;
     const int slot = atomicAdd(&cursor[cid[i]], 1);
@@ -612,6 +623,8 @@ k_cl_sort(const CellConsts* __restrict__ cc, const int* __restrict__ cnt, const 
           const double* __restrict__ q, float4* __restrict__ spos32, double4_32a* __restrict__ spos64, int unit,
           const NListState* __restrict__ nls)
 {
+    pdl_wait();
+    pdl_trigger();
     if (nls && !nls->rebuild) return;
     const int64_t ncell = cc->ncell;  // -1: nothing to sort
     const int64_t wid = ((int64_t)blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -695,6 +708,8 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
     using R = float;
     using Hit = float4;
     constexpr bool kBuild = kMode == kPairBuild, kList = kMode == kPairList;
+    pdl_wait();
+    pdl_trigger();
     if (kBuild && !la.nls->rebuild) return;  // the list stands (the same for every thread)
     __shared__ Hit hits[kPairWarps][kHitCap];
     __shared__ double red[kDiag ? 5 : 3][kPairWarps];
@@ -1017,7 +1032,8 @@ k_pair64(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, dou
     __shared__ double red[kDiag ? 5 : 3][kPair64Warps];
     __shared__ double pforce[kPair64Warps][3];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    load_pair_table(pc.tab, tab);
+    load_pair_table(pc.tab, tab);  // before the wait: the table is an earlier launch's (pair64_const)
+    pdl_wait();
     Pair64Sums<kDiag> s{};
     // no cell list this step (box beyond the cell arrays, flagged), or no list built yet
     const bool cells_ok = kList ? la.nls->force == 0 : cc->ncell >= 0;
@@ -1347,9 +1363,11 @@ __global__ void k_pair_table(PairWord* __restrict__ t, int top, double alpha, do
 // The FP64 pair kernels' constants, with the table of these parameters: found among the context's, or
 // built by one small launch.  Without a table (direct evaluation, the same results to rounding) where the
 // polynomials' coefficients could leave the float range, in a capture that meets the parameters for
-// the first time, and past kPairTabs sets of parameters.
-rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out)
+// the first time, and past kPairTabs sets of parameters.  built: the table's launch is the stream's last, and the
+// pair kernel, which loads the table before pdl_wait(), must not be launched programmatically.
+rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out, bool* built)
 {
+    *built = false;
     NptBuffers& b = ctx->npt;
     const PairConst c = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
     Pair64Const p{};
@@ -1385,6 +1403,7 @@ rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out
                 if (st != RBE_OK) return st;
                 std::memcpy(b.pair_key[t], key, sizeof(key));
                 ++b.pair_tabs;
+                *built = true;
             }
         }
         if (t < b.pair_tabs) p.tab = static_cast<const PairWord*>(b.pair_tab[t]);
@@ -1487,28 +1506,34 @@ rbe_status npt_ensure(rbe_ctx ctx, int64_t N, const double box[3], double rc, do
     return RBE_OK;
 }
 
+// The NPT step's kernels from the drift to the pairs start programmatically behind one another (each waits at its
+// start for the one before to complete): on most steps the five of the list's rebuild exit at once, and their
+// launches were a fifth of the real space.  N = 2e4, FP32, ten steps: 1120 -> 979 us.
 // The cell list of the constants in ctx->npt.cellc: count, scan, fill, per-cell sort and the
 // packed positions (FP64 as well with fp64, in fixed point of this unit unless it is kPairNoUnit).  With a
 // neighbour list (nls) the launches exit at
-// once on steps that do not rebuild it.
-rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls_v, bool fp64, int unit)
+// once on steps that do not rebuild it.  zeroed: the launch before (k_nl_check) has set the counts to zero.
+rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls_v, bool fp64, int unit,
+                            bool zeroed)
 {
     NptBuffers& b = ctx->npt;
     cudaStream_t s = ctx->stream;
     NListState* nls = static_cast<NListState*>(nls_v);
     const CellConsts* cc = static_cast<const CellConsts*>(b.cellc);
     const int nb = (int)((N + kNptThreads - 1) / kNptThreads);
-    cudaError_t e = cudaMemsetAsync(b.cnt, 0, sizeof(int) * b.cellcap, s);
-    if (e != cudaSuccess) return npt_fail(ctx, e, "cudaMemsetAsync(cells)");
-    k_cl_count<<<nb, kNptThreads, 0, s>>>(N, pos, cc, b.cid, b.cnt, ctx->d.status, nls);
-    k_cl_scan<<<1, kScanThreads, 0, s>>>(cc, b.cnt, b.start, b.cursor, nls);
-    k_cl_fill<<<nb, kNptThreads, 0, s>>>(N, b.cid, b.cursor, b.fill, nls);
+    cudaError_t e = zeroed ? cudaSuccess : cudaMemsetAsync(b.cnt, 0, sizeof(int) * b.cellcap, s);
+    if (e == cudaSuccess)
+        e = launch_ordered(zeroed, k_cl_count, dim3(nb), dim3(kNptThreads), 0, s, N, pos, cc, b.cid, b.cnt, ctx->d.status, nls);
+    if (e == cudaSuccess)
+        e = launch_pdl(k_cl_scan, dim3(1), dim3(kScanThreads), 0, s, cc, b.cnt, b.start, b.cursor, nls);
+    if (e == cudaSuccess) e = launch_pdl(k_cl_fill, dim3(nb), dim3(kNptThreads), 0, s, N, b.cid, b.cursor, b.fill, nls);
     // (the cell arrays have room for eight times the cells: a resident wave that strides over the cells there are)
     const int64_t sort_blocks = std::min<int64_t>(((int64_t)b.cellcap * kSortPart + kSortWarps - 1) / kSortWarps,
                                                   (int64_t)ctx->num_sms * 8);
-    k_cl_sort<<<(unsigned)sort_blocks, kSortWarps * 32, 0, s>>>(cc, b.cnt, b.start, b.fill, b.sorted, pos, q, b.spos32,
-                                                              fp64 ? b.spos64 : nullptr, unit, nls);
-    return npt_check(ctx, "cell list");
+    if (e == cudaSuccess)
+        e = launch_pdl(k_cl_sort, dim3((unsigned)sort_blocks), dim3(kSortWarps * 32), 0, s, cc, b.cnt, b.start, b.fill,
+                       b.sorted, pos, q, b.spos32, fp64 ? b.spos64 : nullptr, unit, nls);
+    return e == cudaSuccess ? RBE_OK : npt_fail(ctx, e, "cell list");
 }
 
 // ---------------------------------------------------------------------------------
@@ -1519,7 +1544,7 @@ rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const dou
 // With kernel timing on (events on the context's stream around each kernel) everything stays in order, and a
 // server of several slots does without (12 requests on 8 slots: 18.0 ms with it, 18.0 without, and 0.5 ms more
 // for the streams of a new server).  A step at 2e4 charges, FP32: 136 -> 112 us, FP64: 391 -> 341 us; of 3000
-// rigid waters: 580 -> 540 us.
+// rigid waters: 580 -> 540 us (as measured when this came in).
 KspaceFork::KspaceFork(rbe_ctx c, const rbe_system* sys)
     : ctx(c), on(c->side && !c->timing && sys->params.kspace && sys->params.real && sys->N > 0)
 {
@@ -1613,23 +1638,23 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
         const int unit = pair_unit(prm.rc, 0).s;
         if (list) {
             const int grid = (int)std::min<int64_t>(nb, (int64_t)ctx->num_sms * 4);
-            if (fp64)
-                k_nl_check<true><<<grid, kNptThreads, 0, s>>>(N, sys->pos, sys->charge, b.sorted, b.spos32, b.spos64,
-                                                            unit, b.sref, cc, nls);
-            else
-                k_nl_check<false><<<grid, kNptThreads, 0, s>>>(N, sys->pos, sys->charge, b.sorted, b.spos32, nullptr,
-                                                             unit, b.sref, cc, nls);
+            const cudaError_t e = launch_pdl(fp64 ? k_nl_check<true> : k_nl_check<false>, dim3(grid), dim3(kNptThreads), 0, s, N,
+                                             sys->pos, sys->charge, b.sorted, b.spos32, fp64 ? b.spos64 : nullptr, unit,
+                                             b.sref, cc, nls, b.cnt, b.cellcap);
+            if (e != cudaSuccess) return npt_fail(ctx, e, "k_nl_check");
         }
-        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nls, fp64, unit)) != RBE_OK) return st;
+        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nls, fp64, unit, list)) != RBE_OK) return st;
         const PairConst pc = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
         const ListArgs la{nls, b.nbr, b.nnb, b.sref, ctx->d.status, b.nbr_cap};
         const bool diag = prm.barostat >= 2;  // rectangular cell: the virial diagonal
+        cudaError_t e = cudaSuccess;
         if (list)
-            k_pair<kPairBuild><<<pair_blocks(ctx, N, false), kPairWarps * 32, 0, s>>>(N, cc, pc, b.cid, b.cnt, b.start,
-                                                                                     b.sorted, b.spos32, b.Fr, b.partials, la);
+            e = launch_pdl(k_pair<kPairBuild>, dim3(pair_blocks(ctx, N, false)), dim3(kPairWarps * 32), 0, s, N, cc, pc, b.cid,
+                           b.cnt, b.start, b.sorted, b.spos32, b.Fr, b.partials, la);
         if (fp64) {
             Pair64Const p64;
-            if ((st = pair64_const(ctx, prm, &p64)) != RBE_OK) return st;
+            bool built;
+            if ((st = pair64_const(ctx, prm, &p64, &built)) != RBE_OK) return st;
             auto kern = list ? (diag ? k_pair64<kPairList, true> : k_pair64<kPairList, false>)
                              : (diag ? k_pair64<kPairCells, true> : k_pair64<kPairCells, false>);
             static const cudaError_t attr = [] {
@@ -1640,13 +1665,17 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
                 return e;
             }();
             if (attr != cudaSuccess) return npt_fail(ctx, attr, "shared memory of k_pair64");
-            kern<<<nbp, kPair64Warps * 32, kPairTabBytes, s>>>(N, cc, p64, prm.rc, b.cid, b.cnt, b.start, b.sorted, b.spos32,
-                                                              b.spos64, b.Fr, b.partials, la);
+            if (e == cudaSuccess)
+                e = launch_ordered(!built, kern, dim3(nbp), dim3(kPair64Warps * 32), kPairTabBytes, s, N, cc, p64, prm.rc, b.cid,
+                                   b.cnt, b.start, b.sorted, b.spos32, b.spos64, b.Fr, b.partials, la);
         } else {
             auto kern = list ? (diag ? k_pair<kPairList, true> : k_pair<kPairList, false>)
                              : (diag ? k_pair<kPairCells, true> : k_pair<kPairCells, false>);
-            kern<<<nbp, kPairWarps * 32, 0, s>>>(N, cc, pc, b.cid, b.cnt, b.start, b.sorted, b.spos32, b.Fr, b.partials, la);
+            if (e == cudaSuccess)
+                e = launch_pdl(kern, dim3(nbp), dim3(kPairWarps * 32), 0, s, N, cc, pc, b.cid, b.cnt, b.start, b.sorted, b.spos32,
+                               b.Fr, b.partials, la);
         }
+        if (e != cudaSuccess) return npt_fail(ctx, e, "real-space kernels");
         if ((st = npt_check(ctx, "real-space kernels")) != RBE_OK) return st;
     }
     if (!(parts & 4)) return RBE_OK;
@@ -1787,14 +1816,15 @@ static rbe_status npt_move(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork)
     if (st != RBE_OK) return st;
     const bool rect = sys->params.barostat >= 2;
     auto drift = [&](auto f32_tag, auto rect_tag) {
-        k_npt_drift<decltype(f32_tag)::value, decltype(rect_tag)::value><<<nb, kNptThreads, 0, s>>>(
-            N, sys->pos, sys->mom, sys->force, b.mprop, cf, ctx->seed, sys->cell);
+        return launch_pdl(k_npt_drift<decltype(f32_tag)::value, decltype(rect_tag)::value>, dim3(nb), dim3(kNptThreads),
+                          0, s, N, sys->pos, sys->mom, sys->force, b.mprop, cf, ctx->seed, sys->cell);
     };
     using T = std::true_type;
     using F = std::false_type;
-    if (ctx->precision == RBE_FP64) rect ? drift(F{}, T{}) : drift(F{}, F{});
-    else rect ? drift(T{}, T{}) : drift(T{}, F{});
-    return npt_check(ctx, "k_npt_drift");
+    cudaError_t e;
+    if (ctx->precision == RBE_FP64) e = rect ? drift(F{}, T{}) : drift(F{}, F{});
+    else e = rect ? drift(T{}, T{}) : drift(T{}, F{});
+    return e == cudaSuccess ? RBE_OK : npt_fail(ctx, e, "k_npt_drift");
 }
 
 rbe_status npt_run(rbe_ctx ctx, rbe_system* sys, int32_t nsteps)

@@ -402,7 +402,8 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc,
     __shared__ double red[3][kWaterPairWarps];
     __shared__ double pforce[kWaterPairWarps][3];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
-    load_pair_table(pc.tab, tab);
+    load_pair_table(pc.tab, tab);  // before the wait, as in k_pair64
+    pdl_wait();
     Pair64Sums<false> s{};
     __syncthreads();
     if (cc->ncell < 0) {
@@ -698,17 +699,18 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, i
     if (st != RBE_OK) return st;
     if (prm.real) {
         if (b.n64 < N) return fail(ctx, RBE_ESTATE, "the FP64 packed positions are missing: call rbe_water_init again");
-        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nullptr, true, pair_unit(prm.rc, 0).s)) != RBE_OK)
+        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nullptr, true, pair_unit(prm.rc, 0).s, false)) != RBE_OK)
             return st;
         Pair64Const pc;
-        if ((st = pair64_const(ctx, prm, &pc)) != RBE_OK) return st;
+        bool built;
+        if ((st = pair64_const(ctx, prm, &pc, &built)) != RBE_OK) return st;
         static const cudaError_t attr =
             cudaFuncSetAttribute(k_water_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairTabBytes);
         if (attr != cudaSuccess) return cuda_fail(ctx, attr, "shared memory of k_water_pair");
-        k_water_pair<<<nbp, kWaterPairWarps * 32, kPairTabBytes, s>>>(N, static_cast<const CellConsts*>(b.cellc), pc, prm.rc,
-                                                                  b.cid, b.cnt, b.start, b.sorted, b.spos32, b.spos64,
-                                                                  b.Fr, b.partials);
-        if ((st = water_check(ctx, "k_water_pair")) != RBE_OK) return st;
+        const cudaError_t e = launch_ordered(!built, k_water_pair, dim3(nbp), dim3(kWaterPairWarps * 32), kPairTabBytes, s, N,
+                                             static_cast<const CellConsts*>(b.cellc), pc, prm.rc, b.cid, b.cnt, b.start,
+                                             b.sorted, b.spos32, b.spos64, b.Fr, b.partials);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "k_water_pair");
     }
     if ((st = fork.join()) != RBE_OK) return st;
     const int nbm = (int)std::max<int64_t>(1, (Nmol + kWaterThreads - 1) / kWaterThreads);
