@@ -216,6 +216,11 @@ static rbe_status ensure_slot_buffers(rbe_server_s* s, Slot& sl, int64_t N)
     return RBE_OK;
 }
 
+// Chunks of a request from which its graph pays: capturing and instantiating one costs the host what launching
+// about four chunks directly does (12 requests on 8 slots, graphs against direct launches: 1 chunk 11.9 and 8.2 ms,
+// 2 chunks 16.1 and 13.8, 4 chunks 25.4 and 25.2, 8 chunks 43.5 and 46.7).
+constexpr int32_t kGraphChunks = 5;
+
 // Admit request `id` into slot `sl`: upload its state, initialise the forces, capture the
 // chunk graph.  Everything runs on the slot's stream; no device-wide synchronisation.
 static rbe_status admit(rbe_server_s* s, Slot& sl, int64_t id)
@@ -259,7 +264,7 @@ static rbe_status admit(rbe_server_s* s, Slot& sl, int64_t id)
         sl.graph = nullptr;
     }
     sl.graph_steps = 0;
-    if (s->cfg.use_graphs && !s->cfg.batched && rq.r.nsteps >= s->cfg.chunk_steps) {
+    if (s->cfg.use_graphs && !s->cfg.batched && rq.r.nsteps / s->cfg.chunk_steps >= kGraphChunks) {
         // one chunk of launches, captured; the device step index makes it replayable
         cudaGraph_t g = nullptr;
         rbe_system probe = sl.sys;
