@@ -250,6 +250,7 @@ rbe_status rbe_set_precision(rbe_ctx ctx, int32_t precision, int32_t rho_accum)
     if (precision != RBE_FP64 && precision != RBE_FP32_PHASE) return fail(ctx, RBE_EINVAL, "unknown precision");
     if (rho_accum != RBE_RHO_FP64 && rho_accum != RBE_RHO_COMP32 && rho_accum != RBE_RHO_FP32)
         return fail(ctx, RBE_EINVAL, "unknown rho accumulation");
+    if (precision != ctx->precision) ctx->tables_dirty = true;  // the FP64 path's scales come with its tables
     ctx->precision = precision;
     ctx->rho_accum = rho_accum;
     return RBE_OK;

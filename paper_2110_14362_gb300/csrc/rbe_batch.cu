@@ -171,7 +171,7 @@ __device__ __forceinline__ void pass_tables(const BArgs& a)
         const int r = a.which[w];
         const double* b = a.boxes + 3 * (size_t)r;
         tables_body(b[0], b[1], b[2], a.items[r].box_dev, a.alpha, a.P, a.cum + (size_t)r * 3 * a.cap, a.cap, a.ks + r,
-                    a.items[r].status);
+                    a.items[r].status, false);
         __syncthreads();
     }
 }

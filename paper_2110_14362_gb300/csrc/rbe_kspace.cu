@@ -60,9 +60,9 @@ constexpr double kRhoLatencyPairs = RBE_RHO_LATENCY_PAIRS;
 
 __global__ void __launch_bounds__(kTableThreads)
 k_tables(double bx, double by, double bz, const double* __restrict__ box_dev, double alpha, int P,
-         unsigned long long* __restrict__ cum, int cap, KState* __restrict__ ks, unsigned* __restrict__ status)
+         unsigned long long* __restrict__ cum, int cap, KState* __restrict__ ks, unsigned* __restrict__ status, bool scale64)
 {
-    tables_body(bx, by, bz, box_dev, alpha, P, cum, cap, ks, status);
+    tables_body(bx, by, bz, box_dev, alpha, P, cum, cap, ks, status, scale64);
 }
 
 // Tables of the device box and the sampler in one block (the NPT step, where the box changes
@@ -75,9 +75,9 @@ k_tables_sample(const double* __restrict__ box_dev, double alpha, int Pf, int P,
                 int cap, int smem_cap, KState* __restrict__ ks, uint64_t seed,
                 const unsigned long long* __restrict__ step_dev, int4* __restrict__ m_out,
                 double* __restrict__ w_out, unsigned* __restrict__ status, int mode, int4* __restrict__ chain,
-                int reuse, int4* __restrict__ m_all)
+                int reuse, int4* __restrict__ m_all, bool scale64)
 {
-    tables_body(0.0, 0.0, 0.0, box_dev, alpha, Pf, cum, cap, ks, status);
+    tables_body(0.0, 0.0, 0.0, box_dev, alpha, Pf, cum, cap, ks, status, scale64);
     __syncthreads();
     if (reuse <= 1) {
         for (int lb = 0; lb < P; lb += kTableThreads) {
@@ -268,7 +268,8 @@ rbe_status ensure_table_capacity(rbe_ctx ctx, int need)
 rbe_status launch_tables(rbe_ctx ctx, const double* box_dev)
 {
     k_tables<<<1, kTableThreads, 0, ctx->stream>>>(ctx->box[0], ctx->box[1], ctx->box[2], box_dev, ctx->alpha,
-                                                   ctx->P, ctx->d.cum, ctx->d.tab_cap, ctx->d.ks, ctx->d.status);
+                                                   ctx->P, ctx->d.cum, ctx->d.tab_cap, ctx->d.ks, ctx->d.status,
+                                                   ctx->precision == RBE_FP64);
     return check_launch(ctx, "k_tables");
 }
 
@@ -277,7 +278,7 @@ rbe_status launch_tables(rbe_ctx ctx, const double* box_dev)
 rbe_status launch_tables_box(rbe_ctx ctx, const double box[3])
 {
     k_tables<<<1, kTableThreads, 0, ctx->stream>>>(box[0], box[1], box[2], nullptr, ctx->alpha, ctx->P, ctx->d.cum,
-                                                   ctx->d.tab_cap, ctx->d.ks, ctx->d.status);
+                                                   ctx->d.tab_cap, ctx->d.ks, ctx->d.status, ctx->precision == RBE_FP64);
     ctx->tables_dirty = true;
     return check_launch(ctx, "k_tables");
 }
@@ -391,7 +392,8 @@ rbe_status launch_tables_sample_device(rbe_ctx ctx, int P, const double* box_dev
     const bool mh = ctx->sampler == kSamplerMH;
     k_tables_sample<<<1, kTableThreads, smem_cap ? smem : 0, ctx->stream>>>(
         box_dev, ctx->alpha, P, mh ? 0 : Ptot, ctx->d.cum, ctx->d.tab_cap, smem_cap, ctx->d.ks, ctx->seed, step_dev,
-        ctx->d.m, ctx->d.w, ctx->d.status, ctx->sampler, ctx->chain, reuse, ctx->m_all);
+        ctx->d.m, ctx->d.w, ctx->d.status, ctx->sampler, ctx->chain, reuse, ctx->m_all,
+        ctx->precision == RBE_FP64);
     if (mh) {
         if ((st = check_launch(ctx, "k_tables_sample")) != RBE_OK) return st;
         k_sample_mh<<<(Ptot + kMhSlots - 1) / kMhSlots, kMhWarps * 32, 0, ctx->stream>>>(

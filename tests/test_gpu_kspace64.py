@@ -35,3 +35,28 @@ def test_fp64_plan_edges(N, P):
     assert rel_max_force(F.cpu().numpy(), F0) <= 2e-12 * max(1.0, np.max(np.abs(q)) / np.sqrt(np.mean(q * q)))
     assert rel_frob(W.cpu().numpy().reshape(3, 3), W0) <= 2e-12
     assert abs(E[0].item() - Ek0) <= 2e-12 * abs(Ek0)
+
+
+def test_precision_switched_on_the_same_box():
+    """FP32-phase first, FP64 next on the same box and context, and back: the bits of contexts of their own."""
+    import torch
+    dev = cuda_device()
+    rng = np.random.default_rng(8)
+    box, alpha, P, N = np.array([21.0, 18.0, 25.5]), 0.4, 100, 3000
+    pos = torch.as_tensor(rng.uniform(0, 1, (N, 3)) * box).to(dev)
+    q = torch.as_tensor(rng.choice([-1.0, 1.0], N)).to(dev)
+
+    def evaluate(ctx):
+        F = torch.empty((N, 3), dtype=torch.float64, device=dev)
+        ctx.forces_virial(pos, q, 5, F)
+        ctx.sync()
+        return F.cpu().numpy()
+
+    alone = {}
+    for precision in (rbe.RBE_FP32_PHASE, rbe.RBE_FP64):
+        with rbe.Context(box, alpha, P, 77, precision) as ctx:
+            alone[precision] = evaluate(ctx)
+    with rbe.Context(box, alpha, P, 77, rbe.RBE_FP32_PHASE) as ctx:
+        for precision in (rbe.RBE_FP32_PHASE, rbe.RBE_FP64, rbe.RBE_FP32_PHASE, rbe.RBE_FP64):
+            ctx.set_precision(precision)
+            assert np.array_equal(evaluate(ctx), alone[precision])
