@@ -169,6 +169,7 @@ struct rbe_ctx_s {
     // joined to the context's stream by these events (created by the first rbe_npt_init)
     cudaStream_t side = nullptr;
     bool overlap = true;     // false: no side stream (the slots of a server, whose replicas fill the GPU already)
+    bool early = true;       // the step's real-space launches start early behind one another
     bool rho_plain = false;  // the next rho pass follows an event wait: no programmatic launch
     cudaEvent_t side_ev[3] = {nullptr, nullptr, nullptr};  // after the cell update, after the drift, k-space done
     rbe::DeviceBuffers d;

@@ -1523,15 +1523,17 @@ rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const dou
     const int nb = (int)((N + kNptThreads - 1) / kNptThreads);
     cudaError_t e = zeroed ? cudaSuccess : cudaMemsetAsync(b.cnt, 0, sizeof(int) * b.cellcap, s);
     if (e == cudaSuccess)
-        e = launch_ordered(zeroed, k_cl_count, dim3(nb), dim3(kNptThreads), 0, s, N, pos, cc, b.cid, b.cnt, ctx->d.status, nls);
+        e = launch_ordered(zeroed && ctx->early, k_cl_count, dim3(nb), dim3(kNptThreads), 0, s, N, pos, cc, b.cid, b.cnt,
+                           ctx->d.status, nls);
     if (e == cudaSuccess)
-        e = launch_pdl(k_cl_scan, dim3(1), dim3(kScanThreads), 0, s, cc, b.cnt, b.start, b.cursor, nls);
-    if (e == cudaSuccess) e = launch_pdl(k_cl_fill, dim3(nb), dim3(kNptThreads), 0, s, N, b.cid, b.cursor, b.fill, nls);
+        e = launch_ordered(ctx->early, k_cl_scan, dim3(1), dim3(kScanThreads), 0, s, cc, b.cnt, b.start, b.cursor, nls);
+    if (e == cudaSuccess)
+        e = launch_ordered(ctx->early, k_cl_fill, dim3(nb), dim3(kNptThreads), 0, s, N, b.cid, b.cursor, b.fill, nls);
     // (the cell arrays have room for eight times the cells: a resident wave that strides over the cells there are)
     const int64_t sort_blocks = std::min<int64_t>(((int64_t)b.cellcap * kSortPart + kSortWarps - 1) / kSortWarps,
                                                   (int64_t)ctx->num_sms * 8);
     if (e == cudaSuccess)
-        e = launch_pdl(k_cl_sort, dim3((unsigned)sort_blocks), dim3(kSortWarps * 32), 0, s, cc, b.cnt, b.start, b.fill,
+        e = launch_ordered(ctx->early, k_cl_sort, dim3((unsigned)sort_blocks), dim3(kSortWarps * 32), 0, s, cc, b.cnt, b.start, b.fill,
                        b.sorted, pos, q, b.spos32, fp64 ? b.spos64 : nullptr, unit, nls);
     return e == cudaSuccess ? RBE_OK : npt_fail(ctx, e, "cell list");
 }
@@ -1638,8 +1640,8 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
         const int unit = pair_unit(prm.rc, 0).s;
         if (list) {
             const int grid = (int)std::min<int64_t>(nb, (int64_t)ctx->num_sms * 4);
-            const cudaError_t e = launch_pdl(fp64 ? k_nl_check<true> : k_nl_check<false>, dim3(grid), dim3(kNptThreads), 0, s, N,
-                                             sys->pos, sys->charge, b.sorted, b.spos32, fp64 ? b.spos64 : nullptr, unit,
+            const cudaError_t e = launch_ordered(ctx->early, fp64 ? k_nl_check<true> : k_nl_check<false>, dim3(grid),
+                                                 dim3(kNptThreads), 0, s, N, sys->pos, sys->charge, b.sorted, b.spos32, fp64 ? b.spos64 : nullptr, unit,
                                              b.sref, cc, nls, b.cnt, b.cellcap);
             if (e != cudaSuccess) return npt_fail(ctx, e, "k_nl_check");
         }
@@ -1649,8 +1651,8 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
         const bool diag = prm.barostat >= 2;  // rectangular cell: the virial diagonal
         cudaError_t e = cudaSuccess;
         if (list)
-            e = launch_pdl(k_pair<kPairBuild>, dim3(pair_blocks(ctx, N, false)), dim3(kPairWarps * 32), 0, s, N, cc, pc, b.cid,
-                           b.cnt, b.start, b.sorted, b.spos32, b.Fr, b.partials, la);
+            e = launch_ordered(ctx->early, k_pair<kPairBuild>, dim3(pair_blocks(ctx, N, false)), dim3(kPairWarps * 32), 0, s, N,
+                               cc, pc, b.cid, b.cnt, b.start, b.sorted, b.spos32, b.Fr, b.partials, la);
         if (fp64) {
             Pair64Const p64;
             bool built;
@@ -1666,14 +1668,14 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
             }();
             if (attr != cudaSuccess) return npt_fail(ctx, attr, "shared memory of k_pair64");
             if (e == cudaSuccess)
-                e = launch_ordered(!built, kern, dim3(nbp), dim3(kPair64Warps * 32), kPairTabBytes, s, N, cc, p64, prm.rc, b.cid,
-                                   b.cnt, b.start, b.sorted, b.spos32, b.spos64, b.Fr, b.partials, la);
+                e = launch_ordered(!built && ctx->early, kern, dim3(nbp), dim3(kPair64Warps * 32), kPairTabBytes, s, N, cc, p64,
+                                   prm.rc, b.cid, b.cnt, b.start, b.sorted, b.spos32, b.spos64, b.Fr, b.partials, la);
         } else {
             auto kern = list ? (diag ? k_pair<kPairList, true> : k_pair<kPairList, false>)
                              : (diag ? k_pair<kPairCells, true> : k_pair<kPairCells, false>);
             if (e == cudaSuccess)
-                e = launch_pdl(kern, dim3(nbp), dim3(kPairWarps * 32), 0, s, N, cc, pc, b.cid, b.cnt, b.start, b.sorted, b.spos32,
-                               b.Fr, b.partials, la);
+                e = launch_ordered(ctx->early, kern, dim3(nbp), dim3(kPairWarps * 32), 0, s, N, cc, pc, b.cid, b.cnt, b.start,
+                                   b.sorted, b.spos32, b.Fr, b.partials, la);
         }
         if (e != cudaSuccess) return npt_fail(ctx, e, "real-space kernels");
         if ((st = npt_check(ctx, "real-space kernels")) != RBE_OK) return st;
@@ -1816,8 +1818,8 @@ static rbe_status npt_move(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork)
     if (st != RBE_OK) return st;
     const bool rect = sys->params.barostat >= 2;
     auto drift = [&](auto f32_tag, auto rect_tag) {
-        return launch_pdl(k_npt_drift<decltype(f32_tag)::value, decltype(rect_tag)::value>, dim3(nb), dim3(kNptThreads),
-                          0, s, N, sys->pos, sys->mom, sys->force, b.mprop, cf, ctx->seed, sys->cell);
+        return launch_ordered(ctx->early, k_npt_drift<decltype(f32_tag)::value, decltype(rect_tag)::value>, dim3(nb),
+                              dim3(kNptThreads), 0, s, N, sys->pos, sys->mom, sys->force, b.mprop, cf, ctx->seed, sys->cell);
     };
     using T = std::true_type;
     using F = std::false_type;

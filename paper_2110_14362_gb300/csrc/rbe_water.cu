@@ -707,7 +707,7 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, i
         static const cudaError_t attr =
             cudaFuncSetAttribute(k_water_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairTabBytes);
         if (attr != cudaSuccess) return cuda_fail(ctx, attr, "shared memory of k_water_pair");
-        const cudaError_t e = launch_ordered(!built, k_water_pair, dim3(nbp), dim3(kWaterPairWarps * 32), kPairTabBytes, s, N,
+        const cudaError_t e = launch_ordered(!built && ctx->early, k_water_pair, dim3(nbp), dim3(kWaterPairWarps * 32), kPairTabBytes, s, N,
                                              static_cast<const CellConsts*>(b.cellc), pc, prm.rc, b.cid, b.cnt, b.start,
                                              b.sorted, b.spos32, b.spos64, b.Fr, b.partials);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "k_water_pair");
