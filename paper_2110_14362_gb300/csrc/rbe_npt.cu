@@ -86,7 +86,7 @@ __global__ void k_cell_consts(const double* __restrict__ cell, double rc, double
 
 
 // Per step, before the cell list: refresh the packed positions in the list's slot order and
-// decide whether the list must be rebuilt; and the cells' counts to zero.  Until the first build there is no slot order:
+// decide whether the list must be rebuilt; and (cellcap > 0) the cells' counts to zero.  Until the first build there is no slot order:
 // the kernel then only asks for a build.
 template <bool kF64>
 __global__ void __launch_bounds__(kNptThreads)
@@ -1531,7 +1531,7 @@ rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const dou
         e = launch_ordered(ctx->early, k_cl_fill, dim3(nb), dim3(kNptThreads), 0, s, N, b.cid, b.cursor, b.fill, nls);
     // the cell arrays have room for eight times the initial cells: warps for those, striding over what there is (on
     // most steps with a list the blocks exit at once, and each costs the other replicas of a server: 64 slots
-    // 21.2 thousand replica-steps/s with blocks for the whole arrays, 21.5 with these)
+    // 21.2 thousand replica-steps/s with blocks for the whole arrays, 21.5 with these and 22.2 with the memset)
     const int64_t sort_blocks = std::min<int64_t>(((int64_t)b.cellcap * kSortPart / 8 + kSortWarps - 1) / kSortWarps,
                                                   (int64_t)ctx->num_sms * 8);
     if (e == cudaSuccess)
@@ -1640,14 +1640,17 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
         NListState* nls = list ? static_cast<NListState*>(b.nls) : nullptr;
         const CellConsts* cc = static_cast<const CellConsts*>(b.cellc);
         const int unit = pair_unit(prm.rc, 0).s;
+        // the counts set to zero by the list check, or (launches in order, many replicas) by a memset, which does
+        // not wait for a place on an SM: 64 slots of a server 22.2 against 21.6 thousand replica-steps/s
+        const bool zero = list && ctx->early;
         if (list) {
             const int grid = (int)std::min<int64_t>(nb, (int64_t)ctx->num_sms * 4);
             const cudaError_t e = launch_ordered(ctx->early, fp64 ? k_nl_check<true> : k_nl_check<false>, dim3(grid),
                                                  dim3(kNptThreads), 0, s, N, sys->pos, sys->charge, b.sorted, b.spos32, fp64 ? b.spos64 : nullptr, unit,
-                                             b.sref, cc, nls, b.cnt, b.cellcap);
+                                             b.sref, cc, nls, b.cnt, zero ? b.cellcap : 0);
             if (e != cudaSuccess) return npt_fail(ctx, e, "k_nl_check");
         }
-        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nls, fp64, unit, list)) != RBE_OK) return st;
+        if ((st = launch_cell_list(ctx, N, sys->pos, sys->charge, nls, fp64, unit, zero)) != RBE_OK) return st;
         const PairConst pc = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
         const ListArgs la{nls, b.nbr, b.nnb, b.sref, ctx->d.status, b.nbr_cap};
         const bool diag = prm.barostat >= 2;  // rectangular cell: the virial diagonal
