@@ -1529,11 +1529,14 @@ rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const dou
         e = launch_ordered(ctx->early, k_cl_scan, dim3(1), dim3(kScanThreads), 0, s, cc, b.cnt, b.start, b.cursor, nls);
     if (e == cudaSuccess)
         e = launch_ordered(ctx->early, k_cl_fill, dim3(nb), dim3(kNptThreads), 0, s, N, b.cid, b.cursor, b.fill, nls);
-    // the cell arrays have room for eight times the initial cells: warps for those, striding over what there is (on
-    // most steps with a list the blocks exit at once, and each costs the other replicas of a server: 64 slots
-    // 21.2 thousand replica-steps/s with blocks for the whole arrays, 21.5 with these and 22.2 with the memset)
-    const int64_t sort_blocks = std::min<int64_t>(((int64_t)b.cellcap * kSortPart / 8 + kSortWarps - 1) / kSortWarps,
-                                                  (int64_t)ctx->num_sms * 8);
+    // The cell arrays have room for eight times the initial cells.  Launched in order (many replicas) there are warps
+    // for the initial cells, striding over what there is: on most steps with a list the blocks exit at once, and each
+    // costs the other replicas (64 slots of a server: 21.2 thousand replica-steps/s with warps for the whole arrays,
+    // 21.5 with these).  Launched early, one replica is faster with warps for the whole arrays, a resident wave at
+    // most (N = 2e4, ten steps: 991 us, with warps for the initial cells 1023).
+    const int64_t sort_warps = (int64_t)b.cellcap * kSortPart / (ctx->early ? 1 : 8);
+    const int64_t sort_blocks =
+        std::max<int64_t>(1, std::min<int64_t>((sort_warps + kSortWarps - 1) / kSortWarps, (int64_t)ctx->num_sms * 8));
     if (e == cudaSuccess)
         e = launch_ordered(ctx->early, k_cl_sort, dim3((unsigned)sort_blocks), dim3(kSortWarps * 32), 0, s, cc, b.cnt,
                            b.start, b.fill, b.sorted, pos, q, b.spos32, fp64 ? b.spos64 : nullptr, unit, nls);
