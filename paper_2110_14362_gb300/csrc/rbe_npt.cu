@@ -1362,8 +1362,8 @@ __global__ void k_pair_table(PairWord* __restrict__ t, int top, double alpha, do
 
 // The FP64 pair kernels' constants, with the table of these parameters: found among the context's, or
 // built by one small launch.  Without a table (direct evaluation, the same results to rounding) where the
-// polynomials' coefficients could leave the float range, in a capture that meets the parameters for
-// the first time, and past kPairTabs sets of parameters.  built: the table's launch is the stream's last, and the
+// polynomials' coefficients would leave the float range (pair_lj_fits; pair_segs for the pairs far out), in a
+// capture that meets the parameters for the first time, and past kPairTabs sets of parameters.  built: the table's launch is the stream's last, and the
 // pair kernel, which loads the table before pdl_wait(), must not be launched programmatically.
 rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out, bool* built)
 {
@@ -1383,8 +1383,8 @@ rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out
     const int top = rc_ok ? std::ilogb(c.rc2) + 1 : 0;
     p.unit = pair_unit(prm.rc, top);
     p.scale = std::ldexp(1.0, kPairDrop - p.unit.s);
-    const double y = c.s2 / std::ldexp(1.0, top - kPairOctaves), lj = 50.0 * std::fabs(c.e24) * std::pow(y, 6) / c.s2;
-    if (rc_ok && (!c.lj || (std::isfinite(lj) && lj * y < 1e30))) {
+    p.segs = rc_ok ? (unsigned)pair_segs(ctx->alpha, top) : 0u;
+    if (rc_ok && (!c.lj || pair_lj_fits(c.s2, c.e24, top))) {
         const double key[5] = {ctx->alpha, c.rc2, c.s2, c.e24, c.e4};
         int t = 0;
         while (t < b.pair_tabs && std::memcmp(key, b.pair_key[t], sizeof(key)) != 0) ++t;

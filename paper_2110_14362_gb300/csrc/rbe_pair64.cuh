@@ -146,16 +146,18 @@ __host__ __device__ __forceinline__ void ff_acc(FF& s, FF x)
     s.l = RBE_ADD(s.l, RBE_ADD(x.l, e));
 }
 
-// A double's top 48 bits as a float-float, by its bits (normal and within the float range).
+// A double's top 48 bits as a float-float, by its bits; below 2^-103 zero (the low part keeps every bit that is at
+// least a float's smallest step), above the float range undefined.
 __host__ __device__ __forceinline__ FF ff_of(uint32_t hi, uint32_t lo)
 {
     const uint32_t sign = hi & 0x80000000u, e = (hi >> 20) & 0x7ffu;
     const uint32_t m = ((hi & 0xFFFFFu) << 3) | (lo >> 29);  // 23 bits
     FF r;
     r.h = fx_float(sign | ((e - 896u) << 23) | m);
-    // the next 24 bits times the unit 2^(e - 1023 - 47)
-    const float rest = RBE_MUL(fx_i2f((int)((lo >> 5) & 0xFFFFFFu)), fx_float((e - 896u - 47u) << 23));
+    // the next 24 bits as a fraction, times the unit 2^(e - 1023 - 23) of the high part
+    const float rest = RBE_MUL(RBE_MUL(fx_i2f((int)((lo >> 5) & 0xFFFFFFu)), 0x1.0p-24f), fx_float((e - 919u) << 23));
     r.l = fx_float(fx_bits(rest) | sign);
+    if (e < 920u) r.h = r.l = 0.0f;
     return r;
 }
 
@@ -186,6 +188,26 @@ struct PairUnit {
     int base;                // of the table's segments
     unsigned long long rc2;  // the cutoff's square
 };
+
+// The tables' range.  Coulomb: segments up to alpha u = 40 (there a force factor of cutoffs up to 1e4 is above
+// 2^-97, where ff_of keeps all of it; half a segment's alpha h is 0.16, for a series good to 2^-42 of itself);
+// pairs beyond are evaluated directly, as those below the table are.
+inline int pair_segs(double alpha, int top)
+{
+    const double u = 40.0 / alpha;
+    if (!(u < std::ldexp(1.0, top))) return kPairSegs;
+    const int e = std::ilogb(u), oct = e - (top - kPairOctaves);
+    return oct < 0 ? 0 : (oct << kPairSegBits) + (int)((std::ldexp(u, -e) - 1.0) * (1 << kPairSegBits));
+}
+
+// LJ: coefficients below 2^100 at the table's inner end, terms above 2^-97 at its outer end, and above 2^-58 where
+// the force passes through zero (a constant term there is a small part of them).
+inline bool pair_lj_fits(double s2, double e24, int top)
+{
+    const double in = std::ldexp(1.0, top - kPairOctaves), out = std::ldexp(1.0, top), yi = s2 / in, yo = s2 / out;
+    const double big = 50.0 * std::fabs(e24) * std::pow(yi, 6) / s2, far = std::fabs(e24) * yo * yo * yo / out;
+    return std::isfinite(big) && big < 1e30 && big * yi < 1e30 && far > 0x1.0p-97 && std::fabs(e24) / s2 > 0x1.0p-56;
+}
 
 inline PairUnit pair_unit(double rc, int top)
 {
@@ -307,7 +329,8 @@ constexpr int kPair64Warps = RBE_PAIR64_WARPS, kWaterPairWarps = RBE_WATER_PAIR_
 
 // The FP64 pair kernels' constants beside PairConst.
 struct Pair64Const {
-    const PairWord* tab;  // device table, NULL: direct evaluation (cutoff or LJ sizes beyond the float range)
+    const PairWord* tab;  // device table, NULL: direct evaluation (cutoff or LJ sizes outside the table's range)
+    unsigned segs;        // its usable segments (pair_segs)
     PairUnit unit;
     double scale;         // 2^(kPairDrop - s), the unit of the separations as doubles
     int lj;
@@ -346,7 +369,7 @@ __device__ __forceinline__ double pair_double(long long d)
     return __dadd_rn(__longlong_as_double(v + 0x4338000000000000ll), -0x1.8p52);
 }
 
-// A pair below the table (r under 1/16 of the cutoff at least) or outside the float range: the force factor and
+// A pair below the table (r under 1/16 of the cutoff at least) or beyond its range: the force factor and
 // the energies (Coulomb, LJ).  Not inlined: rare, and its registers are not the evaluation's.
 static __device__ __noinline__ double3 pair_direct(double r2, double qq, double sa, double two_sa_pi, double alpha,
                                                    double s2, double e24, double e4)
@@ -369,7 +392,7 @@ __device__ __forceinline__ void pair64_add(const PairWord* __restrict__ tab, con
     const PairArg a = pair_arg(n, pc.unit.e, pc.unit.base);
     const double dx = pair_double(dxi), dy = pair_double(dyi), dz = pair_double(dzi);
     double f, r2;
-    if (pc.tab && (unsigned)a.seg < (unsigned)kPairSegs && charge_fits(qq)) {
+    if (pc.tab && (unsigned)a.seg < pc.segs && charge_fits(qq)) {
         FF q, e;
         pair_eval<0>(tab, a, f, q, e);
         const FF qf = ff_of_double(qq);

@@ -1,0 +1,75 @@
+"""The FP64 real space at the edges of its tables, against the oracle's pair sum through rbe_npt_init and
+rbe_water_init: cutoffs where erfc leaves the float range, tiny Lennard-Jones terms.  Tolerance 1e-11 of the
+summed sizes of the energies' terms and of the largest force, as for the ordinary sizes: separations are exact to
+2^-53 of the coordinates, up to 40 times the distance and 14 times amplified by u^-7."""
+import numpy as np
+import pytest
+
+import oracle
+import paper_2110_14362_gb300 as rbe
+from gpu_util import cuda_device
+
+pytestmark = pytest.mark.gpu
+
+
+def _system(n, L, seed):
+    """n^3 charges on a jittered grid."""
+    rng = np.random.default_rng(seed)
+    g = (np.arange(n) + 0.5) * (L / n)
+    pos = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3) + rng.uniform(-0.15, 0.15, (n ** 3, 3)) * L / n
+    q = rng.choice([-1.0, 1.0], n ** 3) * rng.uniform(0.3, 1.2, n ** 3)
+    return np.mod(pos, L), q
+
+
+def _params(rc, skin, sigma, eps):
+    return rbe.NptParams(dt=0.001, kT=2.5, P_ext=0.0, gamma=1.0, gamma_V=1.0, M_V=1.0, rc=rc, qqr2e=1389.35, lj_sigma=sigma,
+                         lj_eps=eps, max_disp=0.05, kspace=0, real=1, noise=0, barostat=0, skin=skin)
+
+
+def _init(ctx, pos, q, L, prm):
+    rep = rbe.NptReplica(pos, np.zeros_like(pos), q, np.full(len(q), 20.0), np.array([L, L, L]), prm, cuda_device())
+    rep.init(ctx)
+    ctx.sync()
+    return rep.state()
+
+
+@pytest.mark.parametrize("skin", [0.0, 0.7])
+@pytest.mark.parametrize("alpha,rc,sigma,eps", [
+    (0.2, 16.0, 2.0, 0.4),     # alpha rc^2 = 51
+    (0.5, 12.0, 2.0, 0.4),     # 72
+    (5.0, 10.0, 2.0, 0.4),     # 500
+    (0.2, 7.0, 5e-4, 0.5),     # LJ far below the Coulomb terms
+    (0.2, 7.0, 2.0, 1e-24),
+])
+def test_energies_beyond_the_tables(alpha, rc, sigma, eps, skin):
+    L, box = 34.0, np.array([34.0, 34.0, 34.0])
+    pos, q = _system(11, L, 3)
+    with rbe.Context(box, alpha, 10, 1, rbe.RBE_FP64) as ctx:
+        _, _, F, _, cell = _init(ctx, pos, q, L, _params(rc, skin, sigma, eps))
+    F0, W0, Ec, El = oracle.pair_real(pos, q, box, alpha, rc, 1389.35, sigma, eps)
+    assert np.abs(F - F0).max() <= 1e-11 * np.abs(F0).max()
+    assert abs(cell[4] - np.trace(W0)) <= 1e-11 * max(abs(np.trace(W0)), np.abs(F0).max() * L)
+    assert abs(cell[8] - Ec) <= 1e-11 * (abs(Ec) + 1389.35 * np.sum(q * q) / L)
+    # each LJ term is at most eps (sigma / 2.1)^6 4 in size, the nearest pairs 2.1 apart at least; about 6 per particle
+    assert abs(cell[9] - El) <= 1e-11 * (abs(El) + 4 * eps * (sigma / 2.1) ** 6 * 3 * len(q))
+
+
+def test_water_energies_beyond_the_tables():
+    n, L, alpha, rc = 6, 20.0, 0.7, 9.5  # alpha rc^2 = 63
+    rng = np.random.default_rng(4)
+    g = (np.arange(n) + 0.5) * (L / n)
+    c = np.stack(np.meshgrid(g, g, g, indexing="ij"), -1).reshape(-1, 3) + rng.uniform(-0.2, 0.2, (n ** 3, 3))
+    half = np.radians(109.47) / 2
+    mol = np.array([[0.0, 0.0, 0.0], [np.sin(half), 0.0, np.cos(half)], [-np.sin(half), 0.0, np.cos(half)]])
+    pos = (c[:, None, :] + mol).reshape(-1, 3)
+    q, m = np.tile([-0.8476, 0.4238, 0.4238], n ** 3), np.tile([15.9994, 1.008, 1.008], n ** 3)
+    box = np.array([L, L, L])
+    with rbe.Context(box, alpha, 10, 1, rbe.RBE_FP64) as ctx:
+        rep = rbe.WaterReplica(pos, np.zeros_like(pos), q, m, box, _params(rc, 0.0, 3.166, 0.65), cuda_device())
+        rep.init(ctx)
+        ctx.sync()
+        _, _, F, _, cell = rep.state()
+    F0, _, *E = oracle.water_real(pos, q, box, alpha, rc, 1389.35, 3.166, 0.65)
+    assert np.abs(F - F0).max() <= 1e-11 * np.abs(F0).max()
+    for got, ref in ((cell[8], E[0]), (cell[9], E[1]), (cell[rbe.CELL_EXCL], E[2])):
+        assert abs(got - ref) <= 1e-11 * (abs(ref) + 1389.35 * np.sum(q * q) / L), (got, ref)
