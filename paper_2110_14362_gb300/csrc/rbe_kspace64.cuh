@@ -274,7 +274,7 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
     double R = 0.0;
     if (rho2 > 0.0) {
         const double inv = rsqrt(rho2);
-        R = c[7] * (rho2 * inv);
+        R = fabs(c[7]) * (rho2 * inv);
         const double cr = re * inv, ci = im * inv;  // (cos, sin) of arg rho
         const float rev = atan2f((float)ci, (float)cr) * 0.159154943f;
         phi = (unsigned long long)(long long)__float2int_rn(rev * 1073741824.0f) << 34;
@@ -291,6 +291,7 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
         // ci co - cr s = sin(arg rho - phi) in units of 2^-30; revolutions in units of 2^-64: 2^34 / 2 pi
         const double d = fma(ci, co, -(cr * s)) * 2734261102.3059327;
         phi += (unsigned long long)__double2ll_rn(d);
+        if (c[7] < 0.0) phi += 1ull << 63;  // a negative weight is half a revolution: R enters the force pass as a magnitude
     }
     coef[l] = make_double2(__longlong_as_double((long long)(0ull - phi)), R);
 }
