@@ -170,6 +170,7 @@ struct rbe_ctx_s {
     cudaStream_t side = nullptr;
     bool overlap = true;     // false: no side stream (the slots of a server, whose replicas fill the GPU already)
     bool early = true;       // the step's real-space launches start early behind one another
+    bool m_narrow = false;   // the frequencies in d.m are known to be within kPhaseNarrow (rbe_fix64.cuh)
     bool rho_plain = false;  // the next rho pass follows an event wait: no programmatic launch
     cudaEvent_t side_ev[3] = {nullptr, nullptr, nullptr};  // after the cell update, after the drift, k-space done
     rbe::DeviceBuffers d;
@@ -292,6 +293,7 @@ rbe_status launch_evaluate(rbe_ctx ctx, int64_t N, const double* pos, const doub
 rbe_status launch_rbe(rbe_ctx ctx, int64_t N, const void* pos, const double* q, int P, double* F, double* W,
                       double* E, bool xyzq = false);
 rbe_status launch_tables_box(rbe_ctx ctx, const double box[3]);
+bool tables_narrow(rbe_ctx ctx);
 // Pieces of the pipelined host-buffer evaluation (copy stream events: 1 + 2 kMaxPieces).
 constexpr int kMaxPieces = 8;
 rbe_status launch_evaluate_staged(rbe_ctx ctx, int64_t N, const double* h_pos, const double* h_q, double* h_F,

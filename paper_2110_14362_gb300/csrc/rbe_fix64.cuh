@@ -8,7 +8,7 @@
 //
 // Phase.  s = r / l is a fraction of a revolution with 64 bits, kept as an integer in units of 2^-32 and
 // an FP32 remainder (error at most 2^-58).  m.s is the wrapping integer sum of the m s_hi and the FP32
-// sum of the m s_lo: an error of about |m| 2^-59 revolutions (FP64: |m| 2^-54 from s alone).
+// sum of the m s_lo: an error of about |m| 2^-57 revolutions (FP64: |m| 2^-54 from s alone).
 // The top 11 bits, rounded, pick an entry a of a table of 2048 angles; the rest is x, |x| <= 2 pi 2^-12
 // (and a little more: the FP32 sum is at most |m| units), a float-float.
 //   sin(a + x) = S + sin x (C - S t),  cos(a + x) = C - sin x (S + C t),  t = tan(x / 2)
@@ -175,6 +175,25 @@ struct Frac {
     int hi;
     float lo;
 };
+
+// The FP32 sum of the low words, m.s_lo, is up to 3/2 of the largest |m| in units of 2^-32.  phase_x and
+// trig_value take it up to about 2^17 (the series of the remainder, the integer part below 2^22), with the lengths
+// |m| up to kPhaseNarrow as it is.  Beyond, phase_whole moves its whole part into the integer sum first: errors
+// then grow as |m| 2^-56 revolutions (FP64 phases: |m| 2^-54) for any 32-bit m.
+constexpr uint32_t kPhaseNarrow = 1u << 16;
+
+__host__ __device__ __forceinline__ bool phase_is_wide(int mx, int my, int mz)
+{
+    constexpr uint32_t n = kPhaseNarrow;
+    return (uint32_t)mx + n > 2u * n || (uint32_t)my + n > 2u * n || (uint32_t)mz + n > 2u * n;
+}
+
+__host__ __device__ __forceinline__ void phase_whole(uint32_t& hi, float& lo)
+{
+    const float k = rintf(lo);
+    hi += (uint32_t)(unsigned long long)(long long)k;
+    lo = RBE_ADD(lo, -k);
+}
 
 // The remainder of a phase: sin x = sh + sl, tan(x / 2) = th + tl.
 struct PhaseX {

@@ -1151,6 +1151,7 @@ static rbe_status flex_forces(rbe_ctx ctx, rbe_flex_system* sys, int do_kick)
             k_flex_mh<<<(P + 127) / 128, 128, 0, s>>>(ctx->seed, sys->cell, P, ctx->d.cum, ctx->d.tab_cap, ctx->d.ks,
                                                       ctx->gchain, gc, ctx->d.m, ctx->d.w, ctx->d.status);
         if ((st = flex_check(ctx, "k_flex_mh")) != RBE_OK) return st;
+        ctx->m_narrow = tables_narrow(ctx);
         const double unit[3] = {1.0, 1.0, 1.0};
         if ((st = launch_tables_box(ctx, unit)) != RBE_OK) return st;
         if ((st = launch_evaluate(ctx, N, ctx->gpos, sys->charge, P, false, b.Fk, nullptr, b.WEk + 9)) != RBE_OK)

@@ -197,6 +197,7 @@ rbe_status rbe_kspace_forces_virial_general(rbe_ctx ctx, int64_t N, const double
     if (P > 0)
         k_gen_mh<<<(P + 127) / 128, 128, 0, s>>>(ctx->seed, step, P, ctx->d.cum, ctx->d.tab_cap, ctx->d.ks, ctx->gchain,
                                                  g, ctx->d.m, ctx->d.w, ctx->d.status);
+    ctx->m_narrow = tables_narrow(ctx);
     const double unit[3] = {1.0, 1.0, 1.0};
     if ((st = launch_tables_box(ctx, unit)) != RBE_OK) return st;
     const int nb = (int)((N + 255) / 256);

@@ -317,6 +317,10 @@ rbe_status ensure_k_capacity(rbe_ctx ctx, int K)
     return RBE_OK;
 }
 
+// Batches drawn from tables of this size stay within kPhaseNarrow: the exact sampler's |m| within half the tables' room,
+// the others' within 12 sigma, 1.32 times that.
+bool tables_narrow(rbe_ctx ctx) { return ctx->d.tab_cap <= (int)kPhaseNarrow; }
+
 constexpr int kSampleSmemMax = 48 * 1024;
 
 rbe_status launch_sample(rbe_ctx ctx, uint64_t step, int P)
@@ -345,6 +349,7 @@ rbe_status launch_sample_device_box(rbe_ctx ctx, uint64_t step, int P, const uns
     rbe_status st = ensure_k_capacity(ctx, Ptot);
     if (st != RBE_OK) return st;
     if ((st = check_chain(ctx, Ptot)) != RBE_OK) return st;
+    ctx->m_narrow = tables_narrow(ctx);
     record_event(ctx, 0);
     if (ctx->sampler == kSamplerMH) {
         k_sample_mh<<<(Ptot + kMhSlots - 1) / kMhSlots, kMhWarps * 32, 0, ctx->stream>>>(
@@ -385,6 +390,7 @@ rbe_status launch_tables_sample_device(rbe_ctx ctx, int P, const double* box_dev
             ctx->m_all_cap = need;
         }
     }
+    ctx->m_narrow = tables_narrow(ctx);
     record_event(ctx, 0);
     const size_t smem = sizeof(unsigned long long) * 3 * (size_t)ctx->d.tab_cap;
     const int smem_cap = smem <= (size_t)kSampleSmemMax ? ctx->d.tab_cap : 0;
@@ -410,6 +416,7 @@ rbe_status launch_weights_from_list(rbe_ctx ctx, int K, const int32_t* m, const 
     if (st != RBE_OK) return st;
     st = ensure_k_capacity(ctx, K);
     if (st != RBE_OK) return st;
+    ctx->m_narrow = false;  // the caller's frequencies
     const int threads = 128;
     k_weights_from_list<<<(K + threads - 1) / threads, threads, 0, ctx->stream>>>(K, m, w, ctx->d.m, ctx->d.w);
     return check_launch(ctx, "k_weights_from_list");
@@ -613,14 +620,31 @@ static rbe_status ensure_partials(rbe_ctx ctx, size_t need)
     return RBE_OK;
 }
 
+using Force64Kernel = decltype(&k_force_f64<1, false>);
+static Force64Kernel force64_kernel(int slices, bool check)
+{
+    switch (slices) {
+    case 8: return check ? k_force_f64<8, true> : k_force_f64<8, false>;
+    case 4: return check ? k_force_f64<4, true> : k_force_f64<4, false>;
+    case 2: return check ? k_force_f64<2, true> : k_force_f64<2, false>;
+    default: return check ? k_force_f64<1, true> : k_force_f64<1, false>;
+    }
+}
+
 // launch_evaluate_range on the FP64 path.
 static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* pos, const double* q, int koff, int K,
                                           bool forces, double* F, double* W, double* E)
 {
     DeviceBuffers& d = ctx->d;
+    const bool check = !ctx->m_narrow;
+    const auto rho = check ? k_rho_f64<true> : k_rho_f64<false>;
     static const cudaError_t attr = [] {
-        cudaError_t e = cudaFuncSetAttribute(k_rho_f64, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRho64Smem);
-        for (auto k : {k_force_f64<1>, k_force_f64<2>, k_force_f64<4>, k_force_f64<8>})
+        cudaError_t e = cudaSuccess;
+        for (auto k : {k_rho_f64<false>, k_rho_f64<true>})
+            if (e == cudaSuccess)
+                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRho64Smem);
+        for (auto k : {k_force_f64<1, false>, k_force_f64<2, false>, k_force_f64<4, false>, k_force_f64<8, false>,
+                       k_force_f64<1, true>, k_force_f64<2, true>, k_force_f64<4, true>, k_force_f64<8, true>})
             if (e == cudaSuccess)
                 e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kForce64Smem);
         return e;
@@ -634,7 +658,7 @@ static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* 
     const double* w = d.w + koff;
     const KState* ks = d.ks;
     double2* part = static_cast<double2*>(d.partials);
-    cudaError_t err = launch_ordered(!ctx->rho_plain, k_rho_f64, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem,
+    cudaError_t err = launch_ordered(!ctx->rho_plain, rho, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem,
                                      s, pos, q, N, ks, m, K, p.chunk_len, p.nchunks, part, d.status, p.ksub, p.klanes);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f64");
     record_event(ctx, 2);
@@ -644,7 +668,7 @@ static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* 
                      d.rho, d.terms, d.coef_d, d.status);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_reduce_f64");
     record_event(ctx, 3);
-    auto force = p.ppt == 8 ? k_force_f64<8> : (p.ppt == 4 ? k_force_f64<4> : (p.ppt == 2 ? k_force_f64<2> : k_force_f64<1>));
+    const auto force = force64_kernel(p.ppt, check);
     err = launch_pdl(force, dim3((forces ? p.fblocks : 0) + 1), dim3(kForce64Threads), kForce64Smem, s, pos, q, N,
                      p.per_block, ks, m, (const double2*)d.coef_d, K, F, d.status, (const double*)d.terms, W, E);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_force_f64");

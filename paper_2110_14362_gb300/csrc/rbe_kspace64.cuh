@@ -101,6 +101,11 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double (*scratc
 // 2^-78); the groups' sums are added in 128 bits.  Where every charge of the staged tile has ql = 0 (27
 // significant bits do: integers, equal magnitudes that are a power of two) v ql is left out.
 // Partials: (Re, Im) at [l * nchunks + c]; row K holds the chunk's sum of q^2 in FP64.
+// CHECK: a list whose |m| the host does not bound (rbe_ctx_s::m_narrow): the warps with a frequency beyond kPhaseNarrow
+// move the low phase's whole part into the integer sum.  Kernels of their own, because the second loop beside the
+// ordinary one took its registers: N = 3e5, P = 200 391 us per evaluation against 387, 1e6 x 500 2.93 against 2.87 ms
+// (a weighted call of the former size: 388.2 us with CHECK, 387.1 without).
+template <bool CHECK>
 __global__ void __launch_bounds__(kRho64Threads, RBE_RHO64_MINB)
 k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t N, const KState* __restrict__ ks,
           const int4* __restrict__ m, int K, int64_t chunk_len, int nchunks, double2* __restrict__ partials,
@@ -139,6 +144,7 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
     const int share = kRho64Stage / S, stage = share * S;
     const int4 mv = act ? m[l] : make_int4(0, 0, 0, 0);
     const float mfx = (float)mv.x, mfy = (float)mv.y, mfz = (float)mv.z;
+    const bool wide = CHECK && __any_sync(0xffffffffu, phase_is_wide(mv.x, mv.y, mv.z));
     const TrigLow* sw = reinterpret_cast<const TrigLow*>(st + kTrigN);
     const FixScale scx = fs(ks->sc64[0]), scy = fs(ks->sc64[1]), scz = fs(ks->sc64[2]);
     __int128 re = 0, im = 0;
@@ -164,8 +170,8 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
         const bool has_low = __syncthreads_or(low) != 0;
         if (!act) continue;
         const int p1 = min(here, (ss + 1) * share);
-        auto group = [&](auto low_tag, int p, int n) {
-            constexpr bool LOW = decltype(low_tag)::value;
+        auto group = [&](auto low_tag, auto wide_tag, int p, int n) {
+            constexpr bool LOW = decltype(low_tag)::value, WIDE = decltype(wide_tag)::value;
             unsigned long long ar = 0, ai = 0, br = 0, bi = 0;
             float cr = 0.0f, ci = 0.0f;
 #pragma unroll kRho64Unroll
@@ -175,7 +181,8 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
                 hi += (uint32_t)mv.y * (uint32_t)a.y;
                 hi += (uint32_t)mv.z * (uint32_t)a.z;
                 hi ^= (uint32_t)a.w & 0x80000000u;
-                const float lo = fmaf(mfx, __int_as_float(b.x), fmaf(mfy, __int_as_float(b.y), mfz * __int_as_float(b.z)));
+                float lo = fmaf(mfx, __int_as_float(b.x), fmaf(mfy, __int_as_float(b.y), mfz * __int_as_float(b.z)));
+                if (WIDE) phase_whole(hi, lo);
                 const TrigEntry e = st[hi >> 21];
                 const TrigLow w = sw[hi >> 21];
                 const PhaseX x = phase_x(hi, lo);
@@ -200,8 +207,14 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
         };
         for (int p = ss * share; p < p1; p += kRho64Group) {
             const int n = min(kRho64Group, p1 - p);
-            if (has_low) group(std::true_type{}, p, n);
-            else group(std::false_type{}, p, n);
+            if constexpr (CHECK) {
+                if (wide) {
+                    group(std::true_type{}, std::true_type{}, p, n);
+                    continue;
+                }
+            }
+            if (has_low) group(std::true_type{}, std::false_type{}, p, n);
+            else group(std::false_type{}, std::false_type{}, p, n);
         }
     }
     __syncthreads();
@@ -303,7 +316,8 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
 // over the GPU.  Per staged tile the amplitudes R_l become integers: scaled so that sum_l |m_l| R_l
 // (an FP32 bound, rounded up) is below 2^60, each product R sin is rounded to 2^-60 of that sum.
 // The launch carries one extra block that computes the energy and virial sums (final_sums) meanwhile.
-template <int SL>
+// CHECK: as in k_rho_f64, by the staged tile.
+template <int SL, bool CHECK>
 __global__ void __launch_bounds__(kForce64Threads, RBE_FORCE64_MINB)
 k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t N, int64_t per_block,
             const KState* __restrict__ ks, const int4* __restrict__ mk, const double2* __restrict__ coef, int K,
@@ -333,6 +347,7 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
     const int64_t b0 = (int64_t)blockIdx.x * per_block, b1 = min(N, b0 + per_block);
     const bool one_tile = K <= kForce64Stage;
     int sh = 0;  // R as an integer is R 2^sh
+    [[maybe_unused]] int wide = 0;  // the staged tile has frequencies beyond kPhaseNarrow
     for (int64_t base = b0; base < b1; base += PB) {
         const int64_t i = base + pl;
         Frac x{0, 0.0f}, y{0, 0.0f}, z{0, 0.0f};
@@ -401,35 +416,42 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
                                                 __float_as_int((float)mm.z), __float_as_int(off.lo));
                     sk[3 * tid + 2] = make_int4((int)(A >> 30), (int)(A & 0x3FFFFFFFull) - (1 << 29), 0, 0);
                 }
-                __syncthreads();
+                if (CHECK) wide = __syncthreads_or(phase_is_wide(mm.x, mm.y, mm.z));
+                else __syncthreads();
             }
             unsigned long long ax = 0, ay = 0, az = 0;
             uint32_t hx = 0, hy = 0, hz = 0;
             const int per = SL > 1 ? (nk + SL - 1) / SL : nk;
             const int l1 = SL > 1 ? min(nk, (sl + 1) * per) : nk;
+            // the pair loop, and with CHECK before it a copy that moves the low phase's whole part: one of them runs
+#pragma unroll
+            for (int mode = CHECK ? 1 : 0; mode >= 0; --mode) {
+                if (CHECK && (mode == 1) != (wide != 0)) continue;
 #pragma unroll kForce64Unroll
-            for (int l = SL > 1 ? sl * per : 0; l < l1; ++l) {
-                const int4 a = sk[3 * l], b = sk[3 * l + 1];
-                const int2 r = *reinterpret_cast<const int2*>(sk + 3 * l + 2);
-                uint32_t hi = (uint32_t)a.x * (uint32_t)x.hi + (uint32_t)a.w;
-                hi += (uint32_t)a.y * (uint32_t)y.hi;
-                hi += (uint32_t)a.z * (uint32_t)z.hi;
-                const float lo = fmaf(__int_as_float(b.x), x.lo,
-                                      fmaf(__int_as_float(b.y), y.lo, fmaf(__int_as_float(b.z), z.lo, __int_as_float(b.w))));
-                const TrigSine e = st[hi >> 21];
-                const float vl0 = sw[hi >> 21];
-                const PhaseX p = phase_x(hi, lo);
-                int vh;
-                float vl;
-                trig_value<1>(e.sa, fx_i2f(e.sa), vl0, e.ch, e.cl, p, vh, vl);
-                const unsigned long long h = mul_fix(vh, trig_low_i(e.sr, vl), r.x, r.y);
-                const int hh = fx_hi(h), hl = fx_lo(h);
-                ax = mad_wide(a.x, hl, ax);
-                ay = mad_wide(a.y, hl, ay);
-                az = mad_wide(a.z, hl, az);
-                hx += (uint32_t)a.x * (uint32_t)hh;
-                hy += (uint32_t)a.y * (uint32_t)hh;
-                hz += (uint32_t)a.z * (uint32_t)hh;
+                for (int l = SL > 1 ? sl * per : 0; l < l1; ++l) {
+                    const int4 a = sk[3 * l], b = sk[3 * l + 1];
+                    const int2 r = *reinterpret_cast<const int2*>(sk + 3 * l + 2);
+                    uint32_t hi = (uint32_t)a.x * (uint32_t)x.hi + (uint32_t)a.w;
+                    hi += (uint32_t)a.y * (uint32_t)y.hi;
+                    hi += (uint32_t)a.z * (uint32_t)z.hi;
+                    float lo = fmaf(__int_as_float(b.x), x.lo,
+                                    fmaf(__int_as_float(b.y), y.lo, fmaf(__int_as_float(b.z), z.lo, __int_as_float(b.w))));
+                    if (mode == 1) phase_whole(hi, lo);
+                    const TrigSine e = st[hi >> 21];
+                    const float vl0 = sw[hi >> 21];
+                    const PhaseX p = phase_x(hi, lo);
+                    int vh;
+                    float vl;
+                    trig_value<1>(e.sa, fx_i2f(e.sa), vl0, e.ch, e.cl, p, vh, vl);
+                    const unsigned long long h = mul_fix(vh, trig_low_i(e.sr, vl), r.x, r.y);
+                    const int hh = fx_hi(h), hl = fx_lo(h);
+                    ax = mad_wide(a.x, hl, ax);
+                    ay = mad_wide(a.y, hl, ay);
+                    az = mad_wide(a.z, hl, az);
+                    hx += (uint32_t)a.x * (uint32_t)hh;
+                    hy += (uint32_t)a.y * (uint32_t)hh;
+                    hz += (uint32_t)a.z * (uint32_t)hh;
+                }
             }
             ax += (unsigned long long)hx << 32;
             ay += (unsigned long long)hy << 32;

@@ -50,3 +50,66 @@ def test_weights_of_both_signs(N, K):
     e = 2 * np.pi / np.prod(BOX) * np.abs(w) * np.abs(rho0) ** 2 / kk
     assert abs(E[0] - Ek0) <= 2e-12 * e.sum()
     assert np.linalg.norm(W - W0) <= 2e-12 * np.sum(e * (4 + kk / 0.8))
+
+
+def _exact(S, q, m, w, box, alpha):
+    """(F, E_k, rho, bound of the force) for positions S 2^-64 box (S uint64): the phases in wrapping integers."""
+    p = sum(m[:, t].astype(np.int64).astype(np.uint64)[None, :] * S[:, t][:, None] for t in range(3))
+    t = 2 * np.pi * (p.astype(np.int64) / 2.0 ** 64)
+    c, s = np.cos(t), np.sin(t)
+    rho = q @ c + 1j * (q @ s)
+    k = 2 * np.pi * m / box
+    kk = np.sum(k * k, axis=1)
+    beta = w * 4 * np.pi / (np.prod(box) * kk)
+    F = q[:, None] * ((s * (beta * rho.real) - c * (beta * rho.imag)) @ k)
+    size = np.abs(q).max() * np.max(np.sum(np.abs(beta * np.abs(rho))[:, None] * np.abs(k), axis=0))
+    return F, 2 * np.pi / np.prod(box) * np.sum(w * np.abs(rho) ** 2 / kk), rho, size
+
+
+def _dyadic(N, box, seed):
+    """Positions on a grid of 2^-50 box, exact in FP64 for boxes that are powers of two, and the same times 2^64 / box."""
+    S = np.random.default_rng(seed).integers(0, 2 ** 50, (N, 3), dtype=np.int64)
+    return S / 2.0 ** 50 * box, S.astype(np.uint64) << np.uint64(14)
+
+
+@pytest.mark.parametrize("N,K,most", [(60, 300, 10**7), (60, 600, 3 * 10**5), (40000, 20, 2**20), (3000, 40, 2**31 - 1),
+                                      (70000, 8, 10**6)])
+def test_large_frequencies(N, K, most):
+    """Lists with |m| up to any 32-bit size, small rows among them; each sine to 2 pi |m| 2^-54 (test_phase_host)
+    in rho and again in the force, beside 2e-12 of the sums of the terms' sizes."""
+    box = np.array([16.0, 32.0, 8.0])
+    rng = np.random.default_rng(K)
+    pos, S = _dyadic(N, box, N)
+    q = rng.choice([-1.0, 1.0], N) * rng.uniform(0.5, 1.0, N)
+    m = rng.integers(-most, most, (K, 3), endpoint=True)
+    m[::3] = rng.integers(1, 12, (len(m[::3]), 3))
+    w = rng.uniform(0.5, 1.0, K) * np.sum(m.astype(float) ** 2, axis=1) ** 0.5  # every size counts in the force
+    F, _, E, rho, status = _weighted(pos, q, m, w, box)
+    F0, E0, rho0, size = _exact(S, q, m, w, box, 0.4)
+    err = 2 * np.pi * most * 2.0 ** -54 + 2e-12
+    assert status == rbe.RBE_OK
+    assert np.max(np.abs(rho - rho0)) <= err * np.sum(np.abs(q))
+    # sin(theta_i - arg rho): the phase's error and that of arg rho, N err / |rho|
+    assert np.max(np.abs(F - F0)) <= size * err * (1 + np.sum(np.abs(q)) / np.abs(rho0).min())
+    assert abs(E[0] - E0) <= 2 * err * E0 * np.sum(np.abs(q)) / np.abs(rho0).min()
+
+
+def test_large_frequencies_sampled():
+    """A batch of a box where the sampler draws |m| of some 1e5."""
+    import torch
+    dev = cuda_device()
+    box, alpha, P, N = np.array([2.0 ** 18, 2.0 ** 18, 2.0 ** 17]), 1.0, 64, 500
+    pos, S = _dyadic(N, box, 2)
+    q = np.random.default_rng(3).choice([-1.0, 1.0], N)
+    F = torch.empty((N, 3), dtype=torch.float64, device=dev)
+    with rbe.Context(box, alpha, P, 9, rbe.RBE_FP64) as ctx:
+        ctx.forces_virial(torch.as_tensor(pos).to(dev), torch.as_tensor(q).to(dev), 4, F)
+        ctx.sync()
+        rho = ctx.rho()
+        m, total = ctx.sample_k(4)
+    m = np.asarray(m)
+    assert np.abs(m).max() > 10**5
+    F0, _, rho0, size = _exact(S, q, m, np.full(P, total / P), box, alpha)
+    err = 2 * np.pi * np.abs(m).max() * 2.0 ** -54 + 2e-12
+    assert np.max(np.abs(rho - rho0)) <= err * N
+    assert np.max(np.abs(F.cpu().numpy() - F0)) <= size * err * (1 + N / np.abs(rho0).min())
