@@ -8,6 +8,7 @@
 #include <cuda_runtime.h>
 
 #include "../../include/rbe.h"
+#include "rbe_optin.h"
 
 namespace rbe {
 
@@ -170,6 +171,7 @@ struct rbe_ctx_s {
     cudaStream_t side = nullptr;
     bool overlap = true;     // false: no side stream (the slots of a server, whose replicas fill the GPU already)
     bool early = true;       // the step's real-space launches start early behind one another
+    rbe::SmemOptIn smem;     // dynamic shared memory beyond 48 KB
     bool m_narrow = false;   // the frequencies in d.m are known to be within kPhaseNarrow (rbe_fix64.cuh)
     bool rho_plain = false;  // the next rho pass follows an event wait: no programmatic launch
     cudaEvent_t side_ev[3] = {nullptr, nullptr, nullptr};  // after the cell update, after the drift, k-space done
@@ -190,6 +192,15 @@ inline cudaError_t ctx_alloc(rbe_ctx ctx, T** p, size_t bytes)
 inline void ctx_free(rbe_ctx ctx, void* p)
 {
     if (p) cudaFreeAsync(p, ctx->stream);
+}
+
+// `bytes` of dynamic shared memory for kern on the context's device.
+template <typename... KArgs>
+inline cudaError_t smem_opt_in(rbe_ctx ctx, int kernel, void (*kern)(KArgs...), size_t bytes)
+{
+    return ctx->smem.once(kernel, [&] {
+        return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
+    });
 }
 
 // Launch with programmatic stream serialization (the kernel calls pdl_wait()), or, with pdl false, in plain

@@ -638,19 +638,12 @@ static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* 
     DeviceBuffers& d = ctx->d;
     const bool check = !ctx->m_narrow;
     const auto rho = check ? k_rho_f64<true> : k_rho_f64<false>;
-    static const cudaError_t attr = [] {
-        cudaError_t e = cudaSuccess;
-        for (auto k : {k_rho_f64<false>, k_rho_f64<true>})
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kRho64Smem);
-        for (auto k : {k_force_f64<1, false>, k_force_f64<2, false>, k_force_f64<4, false>, k_force_f64<8, false>,
-                       k_force_f64<1, true>, k_force_f64<2, true>, k_force_f64<4, true>, k_force_f64<8, true>})
-            if (e == cudaSuccess)
-                e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kForce64Smem);
-        return e;
-    }();
-    if (attr != cudaSuccess) return cuda_fail(ctx, attr, "shared memory of the FP64 passes");
     const Plan p = make_plan64(ctx, N, K);
+    const auto force = force64_kernel(p.ppt, check);
+    const int slices_log2 = p.ppt == 8 ? 3 : (p.ppt == 4 ? 2 : (p.ppt == 2 ? 1 : 0));
+    cudaError_t err = smem_opt_in(ctx, kSmemRho64 + check, rho, kRho64Smem);
+    if (err == cudaSuccess) err = smem_opt_in(ctx, kSmemForce64 + 2 * slices_log2 + check, force, kForce64Smem);
+    if (err != cudaSuccess) return cuda_fail(ctx, err, "shared memory of the FP64 passes");
     rbe_status st = ensure_partials(ctx, (size_t)(K + 1) * p.nchunks);
     if (st != RBE_OK) return st;
     cudaStream_t s = ctx->stream;
@@ -658,8 +651,8 @@ static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* 
     const double* w = d.w + koff;
     const KState* ks = d.ks;
     double2* part = static_cast<double2*>(d.partials);
-    cudaError_t err = launch_ordered(!ctx->rho_plain, rho, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem,
-                                     s, pos, q, N, ks, m, K, p.chunk_len, p.nchunks, part, d.status, p.ksub, p.klanes);
+    err = launch_ordered(!ctx->rho_plain, rho, dim3(p.ktiles, p.nchunks), dim3(p.kthreads), kRho64Smem, s, pos, q, N, ks,
+                         m, K, p.chunk_len, p.nchunks, part, d.status, p.ksub, p.klanes);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_rho_f64");
     record_event(ctx, 2);
     int threads = 32;
@@ -668,7 +661,6 @@ static rbe_status launch_evaluate_range64(rbe_ctx ctx, int64_t N, const double* 
                      d.rho, d.terms, d.coef_d, d.status);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_reduce_f64");
     record_event(ctx, 3);
-    const auto force = force64_kernel(p.ppt, check);
     err = launch_pdl(force, dim3((forces ? p.fblocks : 0) + 1), dim3(kForce64Threads), kForce64Smem, s, pos, q, N,
                      p.per_block, ks, m, (const double2*)d.coef_d, K, F, d.status, (const double*)d.terms, W, E);
     if (err != cudaSuccess) return cuda_fail(ctx, err, "launch k_force_f64");

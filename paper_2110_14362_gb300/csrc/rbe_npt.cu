@@ -1667,14 +1667,7 @@ static rbe_status npt_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork* fork, int
             if ((st = pair64_const(ctx, prm, &p64, &built)) != RBE_OK) return st;
             auto kern = list ? (diag ? k_pair64<kPairList, true> : k_pair64<kPairList, false>)
                              : (diag ? k_pair64<kPairCells, true> : k_pair64<kPairCells, false>);
-            static const cudaError_t attr = [] {
-                cudaError_t e = cudaSuccess;
-                for (auto k : {k_pair64<kPairList, true>, k_pair64<kPairList, false>, k_pair64<kPairCells, true>,
-                               k_pair64<kPairCells, false>})
-                    if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairTabBytes);
-                return e;
-            }();
-            if (attr != cudaSuccess) return npt_fail(ctx, attr, "shared memory of k_pair64");
+            if (e == cudaSuccess) e = smem_opt_in(ctx, kSmemPair64 + 2 * (list ? 1 : 0) + (diag ? 1 : 0), kern, kPairTabBytes);
             if (e == cudaSuccess)
                 e = launch_ordered(!built && ctx->early, kern, dim3(nbp), dim3(kPair64Warps * 32), kPairTabBytes, s, N, cc, p64,
                                    prm.rc, b.cid, b.cnt, b.start, b.sorted, b.spos32, b.spos64, b.Fr, b.partials, la);

@@ -704,12 +704,11 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, i
         Pair64Const pc;
         bool built;
         if ((st = pair64_const(ctx, prm, &pc, &built)) != RBE_OK) return st;
-        static const cudaError_t attr =
-            cudaFuncSetAttribute(k_water_pair, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPairTabBytes);
-        if (attr != cudaSuccess) return cuda_fail(ctx, attr, "shared memory of k_water_pair");
-        const cudaError_t e = launch_ordered(!built && ctx->early, k_water_pair, dim3(nbp), dim3(kWaterPairWarps * 32), kPairTabBytes, s, N,
-                                             static_cast<const CellConsts*>(b.cellc), pc, prm.rc, b.cid, b.cnt, b.start,
-                                             b.sorted, b.spos32, b.spos64, b.Fr, b.partials);
+        cudaError_t e = smem_opt_in(ctx, kSmemWaterPair, k_water_pair, kPairTabBytes);
+        if (e != cudaSuccess) return cuda_fail(ctx, e, "shared memory of k_water_pair");
+        e = launch_ordered(!built && ctx->early, k_water_pair, dim3(nbp), dim3(kWaterPairWarps * 32), kPairTabBytes, s, N,
+                           static_cast<const CellConsts*>(b.cellc), pc, prm.rc, b.cid, b.cnt, b.start, b.sorted, b.spos32,
+                           b.spos64, b.Fr, b.partials);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "k_water_pair");
     }
     if ((st = fork.join()) != RBE_OK) return st;
