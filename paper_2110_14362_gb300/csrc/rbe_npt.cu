@@ -1011,7 +1011,7 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
 // cutoff in fixed point, the pair terms from the tables of rbe_pair64.cuh, the sums in FP64.  One block of
 // kPair64Warps warps per SM shares the table; each block takes a contiguous run of slots.
 //
-// What bounds it: the FP64 pipe still (70 % busy: 11 instructions of about 76 clocks of a scheduler per 32 pairs,
+// What bounds it: the FP64 pipe still (70 % busy: 13 instructions of about 76 clocks of a scheduler per 32 pairs,
 // and 8 per particle), with the float-float polynomials and the waits of four warps per scheduler beside it.
 // N = 2e4, rc = 7 A, list of 8 A: 875 us with sqrt, exp, erfc and divisions (about 115 FP64 instructions), 169 us
 // with the tables and FP64 separations (22), 125 us with fixed-point separations; 9000 water sites, rc = 10 A,
@@ -1081,7 +1081,7 @@ k_pair64(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, dou
                         if (mi[1]) dy = pair_nearest(dy, o32.y - me.y, invLf[1], box.L[1], box.near[1]);
                         if (mi[2]) dz = pair_nearest(dz, o32.z - me.z, invLf[2], box.L[2], box.near[2]);
                     }
-                    const unsigned long long n = pair_r2(dx, dy, dz);
+                    const unsigned long long n = pair_r2(dx, dy, dz, kPairHalf);
                     if (on && n < pc.unit.rc2) pair64_add<kDiag>(tab, pc, pc.lj != 0, dx, dy, dz, n, qki * o.w, s);
                     __syncwarp();
                 };

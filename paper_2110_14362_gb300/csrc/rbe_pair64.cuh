@@ -1,6 +1,6 @@
 // Pair terms of the FP64 real space from tables: force factor and energy of the erfc Coulomb and of the
-// Lennard-Jones 12-6 potential as functions of u = r^2, to about 2^-52 (force) and 2^-45 (energy) per pair; the
-// separations in 64-bit fixed point.
+// Lennard-Jones 12-6 potential as functions of u = r^2, to about 2^-52 per pair;
+// the separations in 64-bit fixed point.
 //
 // Why: GB300 issues an FP64 instruction over about 76 clocks of a warp and scheduler, and sqrt, the
 // division, exp and erfc of a pair are about 90 of them (the pair kernels kept the FP64 pipe 85 % busy).
@@ -11,9 +11,12 @@
 // rest, at most 2^-5 of it, in float-float with FP32 for the small terms: two FP64 additions.  The
 // segment and the argument come from the bits of u, and u from integers: the separation of two coordinates
 // in fixed point is exact, box vectors included, and its square is nine 32-bit multiplications to 2^-59 of the
-// cutoff's.  What is left in FP64 per pair is eleven instructions: the charge product, one FMA and two
-// additions of the force factor, three roundings of separations, four FMAs of the force and the virial.  With dU/du = -f/2 the energy is the integral
-// of the same polynomial from the segment's centre, in float-float throughout.
+// cutoff's.  With dU/du = -f/2 the energy is the integral of the same polynomial from the segment's centre: the
+// value there in FP64, the rest, 2^-8 of it, in float-float.  What is left in FP64 per pair is thirteen
+// instructions: the charge product, one FMA and two additions of the force factor, three roundings of separations,
+// four FMAs of the force and the virial, two of the energies.  (All of an energy in float-float took eleven, 1137
+// against 1185 us for an NPT run of four steps at N = 2e4, with sums 4 to 20 times further off than FP64 pair terms
+// give: 1.6e-11 against 1.1e-12 for E_lj there; with the constant terms in FP64 they are as near.)
 //
 // Coulomb derivatives: with B_0 = erfc(s r)/r and B_n = ((2n-1) B_{n-1} + (2a)^n e^{-a u} / sqrt(pi a)) / u
 // (a = alpha, s = sqrt(alpha)) the force factor is B_1 and d B_n / du = -B_{n+1} / 2: a recurrence of
@@ -43,7 +46,7 @@ __host__ __device__ inline void pair_split(double x, float& h, float& l)
     l = (float)(x - (double)h);
 }
 
-__host__ __device__ inline void pair_put_double(PairWord& p, double x)
+__host__ __device__ inline void pair_put_double(PairWord& p, int j, double x)
 {
     unsigned long long b;
 #ifdef __CUDA_ARCH__
@@ -51,13 +54,32 @@ __host__ __device__ inline void pair_put_double(PairWord& p, double x)
 #else
     __builtin_memcpy(&b, &x, 8);
 #endif
-    p.w[0] = (uint32_t)b;
-    p.w[1] = (uint32_t)(b >> 32);
+    p.w[j] = (uint32_t)b;
+    p.w[j + 1] = (uint32_t)(b >> 32);
+}
+
+__host__ __device__ __forceinline__ double pair_get_double(const PairWord& p, int j)
+{
+#ifdef __CUDA_ARCH__
+    return __hiloint2double((int)p.w[j + 1], (int)p.w[j]);
+#else
+    const unsigned long long b = ((unsigned long long)p.w[j + 1] << 32) | p.w[j];
+    double x;
+    __builtin_memcpy(&x, &b, 8);
+    return x;
+#endif
+}
+
+// a b for a, b as sums of two doubles.
+__host__ __device__ inline double2 pair_dd_mul(double2 a, double2 b)
+{
+    const double p = a.x * b.x, e = fma(a.x, b.x, -p) + (a.x * b.y + a.y * b.x), s = p + e;
+    return make_double2(s, e - (s - p));
 }
 
 // Segment `seg` of the table whose octaves end at 2^top, both parts (Coulomb, LJ): coefficients c[k] of the
 // polynomial in tau in [-1, 1] and the energy e0 at the centre.  Planes (kPairSegs entries each):
-// {c0 FP64, e0 h, l}, {c1 h, l, c2 h, l}, {c3 h, l, c4 h, l}, {c5, c6, c7, c8}.
+// {c0 FP64, e0 FP64}, {c1 h, l, c2 h, l}, {c3 h, l, c4 h, l}, {c5, c6, c7, c8}.
 __host__ __device__ inline void pair_segment(PairWord* t, int seg, int top, double alpha, double lj_s2, double lj_e24,
                                              double lj_e4)
 {
@@ -68,7 +90,9 @@ __host__ __device__ inline void pair_segment(PairWord* t, int seg, int top, doub
     const double r = sqrt(u), iu = 1.0 / u, au = alpha * u, aul = fma(alpha, u, -au), x = sqrt(au);
     const double dx = (fma(-x, x, au) + aul) / (2.0 * x), ga = exp(-au) * (1.0 - aul);
     const double ex = ga / sqrt(kPi * alpha);
-    double c[9], e0 = (erfc(x) - 1.12837916709551257390 * ga * dx) / r, B = e0, a2 = 1.0, f = 1.0;
+    // erfc / r with the rounding errors of the root and the quotient put back too
+    const double er = erfc(x), de = -1.12837916709551257390 * ga * dx, q0 = er / r, dr = fma(-r, r, u) / (2.0 * r);
+    double c[9], e0 = q0 + ((fma(-q0, r, er) + de) - q0 * dr) / r, B = e0, a2 = 1.0, f = 1.0;
     for (int n = 1; n <= 9; ++n) {
         a2 *= 2.0 * alpha;
         B = ((2 * n - 1) * B + a2 * ex) * iu;
@@ -77,11 +101,17 @@ __host__ __device__ inline void pair_segment(PairWord* t, int seg, int top, doub
     }
     for (int part = 0; part < 2; ++part) {
         if (part == 1) {
-            const double y = lj_s2 * iu, y3 = y * y * y, hu = h * iu;
-            double p7 = 2.0 * lj_e24 * y3 * y3 * iu, p4 = -lj_e24 * y3 * iu;  // u^-7 and u^-4 terms of f
-            e0 = lj_e4 * (y3 * y3 - y3);
+            // the sixth power of y = s^2 / u to about 2^-100: a segment's constants serve all its pairs, and their
+            // errors do not average out
+            const double2 i1 = make_double2(iu, fma(-u, iu, 1.0) * iu), y = pair_dd_mul(i1, make_double2(lj_s2, 0.0));
+            const double2 y3 = pair_dd_mul(pair_dd_mul(y, y), y), y6 = pair_dd_mul(y3, y3);
+            const double2 a3 = pair_dd_mul(y3, i1), a6 = pair_dd_mul(y6, i1);
+            const double hu = h * iu;
+            double p7 = 2.0 * lj_e24 * a6.x, p4 = -lj_e24 * a3.x;  // u^-7 and u^-4 terms of f
+            e0 = lj_e4 * ((y6.x - y3.x) + (y6.y - y3.y));
+            c[0] = lj_e24 * ((2.0 * a6.x - a3.x) + (2.0 * a6.y - a3.y));
             for (int k = 0; k < 9; ++k) {
-                c[k] = p7 + p4;
+                if (k > 0) c[k] = p7 + p4;
                 p7 *= -hu * (7 + k) / (double)(k + 1);
                 p4 *= -hu * (4 + k) / (double)(k + 1);
             }
@@ -93,8 +123,8 @@ __host__ __device__ inline void pair_segment(PairWord* t, int seg, int top, doub
             pair_put(p[(size_t)plane * kPairSegs], j, fh);
             pair_put(p[(size_t)plane * kPairSegs], j + 1, fl);
         };
-        pair_put_double(p[0], c[0]);
-        two(0, 2, e0);
+        pair_put_double(p[0], 0, c[0]);
+        pair_put_double(p[0], 2, e0);
         two(1, 0, c[1]);
         two(1, 2, c[2]);
         two(2, 0, c[3]);
@@ -148,6 +178,8 @@ __host__ __device__ __forceinline__ void ff_acc(FF& s, FF x)
 
 // A double's top 48 bits as a float-float, by its bits; below 2^-103 zero (the low part keeps every bit that is at
 // least a float's smallest step), above the float range undefined.
+// ANY false: at least 2^-103 by the caller's word.
+template <bool ANY = true>
 __host__ __device__ __forceinline__ FF ff_of(uint32_t hi, uint32_t lo)
 {
     const uint32_t sign = hi & 0x80000000u, e = (hi >> 20) & 0x7ffu;
@@ -157,7 +189,7 @@ __host__ __device__ __forceinline__ FF ff_of(uint32_t hi, uint32_t lo)
     // the next 24 bits as a fraction, times the unit 2^(e - 1023 - 23) of the high part
     const float rest = RBE_MUL(RBE_MUL(fx_i2f((int)((lo >> 5) & 0xFFFFFFu)), 0x1.0p-24f), fx_float((e - 919u) << 23));
     r.l = fx_float(fx_bits(rest) | sign);
-    if (e < 920u) r.h = r.l = 0.0f;
+    if (ANY && e < 920u) r.h = r.l = 0.0f;
     return r;
 }
 
@@ -233,12 +265,14 @@ __host__ __device__ __forceinline__ unsigned long long pair_fixed(unsigned long 
 }
 
 // The square sum of three separations (below 2^63 in size), times 2^-64: from the signed 32-bit halves,
-// without the squares of the low ones (below 1).
-__host__ __device__ __forceinline__ unsigned long long pair_r2(long long x, long long y, long long z)
+// without the squares of the low ones (a quarter in the mean), rounded down after adding `start` 2^-31.
+constexpr unsigned long long kPairHalf = 3ull << 29;  // the mean of what is left out: sums over pairs are unbiased
+__host__ __device__ __forceinline__ unsigned long long pair_r2(long long x, long long y, long long z,
+                                                               unsigned long long start = 0)
 {
     const int xl = (int)x, yl = (int)y, zl = (int)z;
     const int xh = (int)(x >> 32) - (xl >> 31), yh = (int)(y >> 32) - (yl >> 31), zh = (int)(z >> 32) - (zl >> 31);
-    const long long mid = (long long)mad_wide(xh, xl, mad_wide(yh, yl, mad_wide(zh, zl, 0ull)));
+    const long long mid = (long long)mad_wide(xh, xl, mad_wide(yh, yl, mad_wide(zh, zl, start)));
     return mad_wide(xh, xh, mad_wide(yh, yh, mad_wide(zh, zh, (unsigned long long)(mid >> 31))));
 }
 
@@ -272,15 +306,19 @@ __host__ __device__ __forceinline__ PairArg pair_arg(unsigned long long n, int e
     // the mantissa bits below the segment's: the first 23, and the next 23
     constexpr int k = 31 - kPairSegBits - 23;
     a.tau.h = RBE_FMA(2.0f, fx_float(((a.hi >> k) & 0x7FFFFFu) | 0x3F800000u), -3.0f);
-    a.tau.l = RBE_FMA(fx_float((((a.hi << (23 - k)) | (a.lo >> (9 + k))) & 0x7FFFFFu) | 0x3F800000u), 0x1.0p-22f, -0x1.0p-22f);
+    // (and half of their last, the mean of what is below)
+    a.tau.l = RBE_FMA(fx_float((((a.hi << (23 - k)) | (a.lo >> (9 + k))) & 0x7FFFFFu) | 0x3F800000u), 0x1.0p-22f,
+                      0x1.0p-46f - 0x1.0p-22f);
     // half width 2^(e - kPairSegBits - 1), halved
     a.half = fx_float((uint32_t)(a.e + 127 - kPairSegBits - 2) << 23);
     return a;
 }
 
-// One part (0: Coulomb, 1: LJ) from its table planes: the force factor as c0 + q, and the energy.
+// One part (0: Coulomb, 1: LJ) from its table planes: the force factor as c0 + q, the energy as e0 + de, |de| at most
+// about 2^-8 of it where it has its full size.
 template <int PART>
-__host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const PairArg& a, double& c0, FF& q, FF& energy)
+__host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const PairArg& a, double& c0, FF& q, double& e0,
+                                                   FF& de)
 {
     const PairWord* p = t + PART * kPairPlanes * kPairSegs + a.seg;
     const PairWord w0 = p[0], w1 = p[kPairSegs], w2 = p[2 * kPairSegs], w3 = p[3 * kPairSegs];
@@ -295,21 +333,28 @@ __host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const Pair
     q = ff_fma<ANY>(q, tau, c2);
     q = ff_fma<ANY>(q, tau, c1);
     q = ff_mul(q, tau);
-#ifdef __CUDA_ARCH__
-    c0 = __hiloint2double((int)w0.w[1], (int)w0.w[0]);
-#else
-    const unsigned long long b = ((unsigned long long)w0.w[1] << 32) | w0.w[0];
-    __builtin_memcpy(&c0, &b, 8);
-#endif
-    // energy e0 - half tau (c0 + tau (c1 / 2 + tau (c2 / 3 + tau (c3 / 4 + ...))))
+    c0 = pair_get_double(w0, 0);
+    e0 = pair_get_double(w0, 2);
+    // -half tau (c0 + tau (c1 / 2 + tau (c2 / 3 + tau (c3 / 4 + ...))))
     float si = RBE_FMA(RBE_MUL(c6, 1.0f / 7.0f), tau.h, RBE_MUL(c5, 1.0f / 6.0f));
     si = RBE_FMA(si, tau.h, RBE_MUL(c4.h, 0.2f));
     si = RBE_FMA(si, tau.h, RBE_MUL(c3.h, 0.25f));
     const FF third{(float)(1.0 / 3.0), (float)(1.0 / 3.0 - (double)(float)(1.0 / 3.0))};
     FF in = ff_fma<ANY>(FF{si, 0.0f}, tau, ff_mul(c2, third));
     in = ff_fma<ANY>(in, tau, FF{RBE_MUL(0.5f, c1.h), RBE_MUL(0.5f, c1.l)});
-    in = ff_fma<ANY>(in, tau, ff_of(w0.w[1], w0.w[0]));
-    energy = ff_fma<ANY>(in, FF{RBE_MUL(-a.half, tau.h), RBE_MUL(-a.half, tau.l)}, FF{fx_float(w0.w[2]), fx_float(w0.w[3])});
+    in = ff_fma<ANY>(in, tau, ff_of<ANY>(w0.w[1], w0.w[0]));  // (pair_segs)
+    de = ff_mul(in, FF{RBE_MUL(-a.half, tau.h), RBE_MUL(-a.half, tau.l)});
+}
+
+// The same with the energy as one float-float (2^-45 of it).
+template <int PART>
+__host__ __device__ __forceinline__ void pair_eval(const PairWord* t, const PairArg& a, double& c0, FF& q, FF& energy)
+{
+    double e0;
+    FF de;
+    pair_eval<PART>(t, a, c0, q, e0, de);
+    pair_split(e0, energy.h, energy.l);
+    ff_acc(energy, de);
 }
 
 // ---------------------------------------------------------------------------------
@@ -343,14 +388,14 @@ template <bool DIAG>
 struct Pair64Sums {
     double fx, fy, fz;
     double w[DIAG ? 3 : 1];
-    FF ec, el;
-    double ecd, eld;  // energies of the pairs evaluated directly
+    double ecd, eld;  // energies: the table's constant terms, and the pairs evaluated directly
+    FF ec, el;        // the polynomials' rest, small beside them
 };
 
 __device__ __forceinline__ FF ff_of_double(double x)
 {
     const uint32_t hi = (uint32_t)__double2hiint(x), lo = (uint32_t)__double2loint(x);
-    return (hi & 0x7ff00000u) == 0u ? FF{0.0f, 0.0f} : ff_of(hi, lo);
+    return (hi & 0x7ff00000u) == 0u ? FF{0.0f, 0.0f} : ff_of<false>(hi, lo);  // (charge_fits)
 }
 
 // A charge product that float-floats hold to 48 bits: zero, or between 2^-60 and 2^60.
@@ -393,20 +438,25 @@ __device__ __forceinline__ void pair64_add(const PairWord* __restrict__ tab, con
     const double dx = pair_double(dxi), dy = pair_double(dyi), dz = pair_double(dzi);
     double f, r2;
     if (pc.tab && (unsigned)a.seg < pc.segs && charge_fits(qq)) {
-        FF q, e;
-        pair_eval<0>(tab, a, f, q, e);
+        FF q, de;
+        double e0;
+        pair_eval<0>(tab, a, f, q, e0, de);
         const FF qf = ff_of_double(qq);
-        ff_acc(s.ec, ff_mul(e, qf));
+        s.ecd = fma(qq, e0, s.ecd);
+        ff_acc(s.ec, ff_mul(de, qf));
         q = ff_mul(q, qf);
         double d0 = 0.0;
         if (lj) {
             FF p;
-            pair_eval<1>(tab, a, d0, p, e);
-            ff_acc(s.el, e);
+            pair_eval<1>(tab, a, d0, p, e0, de);
+            s.eld += e0;
+            ff_acc(s.el, de);
             ff_acc(q, p);
         }
         f = (fma(f, qq, d0) + float_as_double(q.h)) + float_as_double(q.l);
-        r2 = __hiloint2double(((a.e + 1022) << 20) + (int)(a.hi >> 11), (int)((a.hi << 21) | (a.lo >> 11)));
+        // the mantissa rounded: truncated it made the virial 3e-16 smaller than it is
+        const unsigned long long m = ((unsigned long long)a.hi << 32) | a.lo;
+        r2 = __longlong_as_double(((long long)(a.e + 1022) << 52) + (long long)((m >> 11) + (m >> 10 & 1)));
     } else {
         const double x = dx * pc.scale, y = dy * pc.scale, z = dz * pc.scale;
         r2 = x * x + y * y + z * z;

@@ -451,7 +451,7 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc,
                         dy = pair_shift(dy, (h.y >> 2) & 3, box.L[1]);
                         dz = pair_shift(dz, (h.y >> 4) & 3, box.L[2]);
                     }
-                    const unsigned long long n = pair_r2(dx, dy, dz);
+                    const unsigned long long n = pair_r2(dx, dy, dz, kPairHalf);
                     // another molecule (the site itself excluded with its own) and r2 < rc^2
                     if (on && j / 3 != mol_i && n < pc.unit.rc2)
                         pair64_add<false>(tab, pc, oxy_i && j % 3 == 0, dx, dy, dz, n, qki * o.w, s);
