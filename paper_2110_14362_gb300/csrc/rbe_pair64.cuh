@@ -435,7 +435,7 @@ __device__ __forceinline__ void pair64_add(const PairWord* __restrict__ tab, con
                                            Pair64Sums<DIAG>& s)
 {
     const PairArg a = pair_arg(n, pc.unit.e, pc.unit.base);
-    const double dx = pair_double(dxi), dy = pair_double(dyi), dz = pair_double(dzi);
+    double dx = pair_double(dxi), dy = pair_double(dyi), dz = pair_double(dzi);
     double f, r2;
     if (pc.tab && (unsigned)a.seg < pc.segs && charge_fits(qq)) {
         FF q, de;
@@ -458,6 +458,10 @@ __device__ __forceinline__ void pair64_add(const PairWord* __restrict__ tab, con
         const unsigned long long m = ((unsigned long long)a.hi << 32) | a.lo;
         r2 = __longlong_as_double(((long long)(a.e + 1022) << 52) + (long long)((m >> 11) + (m >> 10 & 1)));
     } else {
+        // close pairs: the separations to 53 bits of their own size, in the same unit
+        dx = (double)dxi * (1.0 / (1 << kPairDrop));
+        dy = (double)dyi * (1.0 / (1 << kPairDrop));
+        dz = (double)dzi * (1.0 / (1 << kPairDrop));
         const double x = dx * pc.scale, y = dy * pc.scale, z = dz * pc.scale;
         r2 = x * x + y * y + z * z;
         const double3 t = pair_direct(r2, qq, pc.sa, pc.two_sa_pi, pc.alpha, lj ? pc.s2 : 0.0, pc.e24, pc.e4);

@@ -73,3 +73,23 @@ def test_water_energies_beyond_the_tables():
     assert np.abs(F - F0).max() <= 1e-11 * np.abs(F0).max()
     for got, ref in ((cell[8], E[0]), (cell[9], E[1]), (cell[rbe.CELL_EXCL], E[2])):
         assert abs(got - ref) <= 1e-11 * (abs(ref) + 1389.35 * np.sum(q * q) / L), (got, ref)
+
+
+@pytest.mark.parametrize("skin", [0.0, 0.7])
+@pytest.mark.parametrize("gap", [1e-2, 1e-4, 1e-6])
+def test_close_pairs(gap, skin):
+    """Forces of charges `gap` apart to 1e-13 of their size: the difference of two FP64 coordinates is exact there, and
+    the pair terms are a few roundings of it (the other pairs' forces are below 1e-5 of theirs)."""
+    L, rc, box = 40.0, 7.0, np.array([40.0, 40.0, 40.0])
+    rng = np.random.default_rng(6)
+    a = (np.stack(np.meshgrid(*[[5.0, 18.0, 31.0]] * 3, indexing="ij"), -1).reshape(-1, 3) + rng.uniform(-1, 1, (27, 3)))
+    v = rng.normal(size=a.shape)
+    b = a + gap * v / np.linalg.norm(v, axis=1)[:, None]
+    pos = np.stack([a, b], 1).reshape(-1, 3)
+    q = rng.choice([-1.0, 1.0], len(pos)) * rng.uniform(0.3, 1.2, len(pos))
+    with rbe.Context(box, 0.2, 10, 1, rbe.RBE_FP64) as ctx:
+        _, _, F, _, cell = _init(ctx, pos, q, L, _params(rc, skin, 2.0, 0.0))
+    F0, W0, Ec, _ = oracle.pair_real(pos, q, box, 0.2, rc, 1389.35, 2.0, 0.0)
+    assert np.max(np.linalg.norm(F - F0, axis=1) / np.linalg.norm(F0, axis=1)) <= 1e-13
+    assert abs(cell[4] - np.trace(W0)) <= 1e-13 * 1389.35 * len(a) * 1.44 / gap
+    assert abs(cell[8] - Ec) <= 1e-13 * 1389.35 * len(a) * 1.44 / gap
