@@ -284,10 +284,21 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
     rho[l] = make_double2(re, im);
     if (!isfinite(re) || !isfinite(im)) atomicOr(status, kStatusNonFinite);
     unsigned long long phi = 0ull;
-    double R = 0.0;
-    if (rho2 > 0.0) {
-        const double inv = rsqrt(rho2);
-        R = fabs(c[7]) * (rho2 * inv);
+    double R = 0.0, h2 = rho2;
+    if (((uint32_t)__double2hiint(rho2) >> 20) - 93u > 1860u) {
+        // a square below 2^-930, above 2^930 or not finite: the forces are linear in rho, whose size is within FP64's
+        const double big = fmax(fabs(re), fabs(im));
+        if (big > 0.0 && big < 1.7e308) {
+            const int e = ilogb(big);
+            re = ldexp(re, -e);
+            im = ldexp(im, -e);
+            c[7] = ldexp(c[7], e);
+            h2 = re * re + im * im;
+        }
+    }
+    if (h2 > 0.0) {
+        const double inv = rsqrt(h2);
+        R = fabs(c[7]) * (h2 * inv);
         const double cr = re * inv, ci = im * inv;  // (cos, sin) of arg rho
         const float rev = atan2f((float)ci, (float)cr) * 0.159154943f;
         phi = (unsigned long long)(long long)__float2int_rn(rev * 1073741824.0f) << 34;

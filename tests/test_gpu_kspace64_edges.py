@@ -113,3 +113,17 @@ def test_large_frequencies_sampled():
     err = 2 * np.pi * np.abs(m).max() * 2.0 ** -54 + 2e-12
     assert np.max(np.abs(rho - rho0)) <= err * N
     assert np.max(np.abs(F.cpu().numpy() - F0)) <= size * err * (1 + N / np.abs(rho0).min())
+
+
+@pytest.mark.parametrize("e", [-560, -505, 505, 560])
+def test_rho_whose_square_leaves_fp64(e):
+    """Forces are linear in rho and in the weights: charges times 2^e and weights times 2^(-2 e + 100) give forces
+    times 2^100, whatever |rho|^2 does (it is 0 or infinite at 2^(+-1120), subnormal terms left out)."""
+    rng = np.random.default_rng(1)
+    N, K = 300, 40
+    pos, q = rng.uniform(0, 1, (N, 3)) * BOX, rng.choice([-1.0, 1.0], N)
+    m, w = rng.integers(1, 12, (K, 3)), rng.uniform(0.5, 1.0, K)
+    F, _, _, _, _ = _weighted(pos, q, m, w)
+    G, _, _, _, _ = _weighted(pos, np.ldexp(q, e), m, np.ldexp(w, max(-1000, min(1000, -2 * e + 100))))
+    back = 100 if abs(2 * e - 100) <= 1000 else 2 * e + (1000 if e < 0 else -1000)
+    assert rel_max_force(np.ldexp(G, -back), F) <= 1e-13
