@@ -88,6 +88,16 @@ __device__ __forceinline__ void block_sum2(double& a, double& b, double (*scratc
     }
 }
 
+// A coordinate that is not finite, or whose r / l is not.  Not inlined: the pair loop keeps its registers (inlined,
+// the rho pass took 5 % longer).
+static __device__ __noinline__ bool coord_bad(const KState* ks, unsigned long long bx, unsigned long long by,
+                                              unsigned long long bz)
+{
+    const double s = __longlong_as_double((long long)bx) * ks->inv[0], t = __longlong_as_double((long long)by) * ks->inv[1],
+                 u = __longlong_as_double((long long)bz) * ks->inv[2];
+    return !isfinite(s) || !isfinite(t) || !isfinite(u);
+}
+
 // =================================================================================
 // rho pass.  Block (kt, c): T frequency lanes (thread j of sub-stream s owns frequency kt T + j) in S
 // particle sub-streams over the particles of chunk c, staged kRho64Stage at a time as 64-bit
@@ -114,11 +124,14 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
     extern __shared__ __align__(16) unsigned char s_raw[];
     TrigEntry* st = reinterpret_cast<TrigEntry*>(s_raw);
     int4* sp = reinterpret_cast<int4*>(s_raw + kRho64Trig);
-    __shared__ int s_eb;
+    __shared__ int s_eb, s_bad;
     __shared__ double s_red[2][32];
     const int tid = threadIdx.x, nt = blockDim.x, kt = blockIdx.x, c = blockIdx.y;
     const int64_t start = (int64_t)c * chunk_len, end = min(N, start + chunk_len);
-    if (tid == 0) s_eb = 1;
+    if (tid == 0) {
+        s_eb = 1;
+        s_bad = 0;
+    }
     __syncthreads();
     load_trig(g_trig.entry, st, (int)kRho64Trig);
     // the largest exponent field of the chunk's charges, and the sum of their squares (inputs only)
@@ -138,15 +151,20 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
     const bool bad_q = s_eb == 0x7ff;
     pdl_wait();
     pdl_trigger();
-    if (bad_q && tid == 0) atomicOr(status, kStatusNonFinite);
+    if (bad_q && tid == 0) {
+        atomicOr(status, kStatusNonFinite);
+        s_bad = 1;
+    }
     const int j = tid % T, ss = tid / T, l = kt * T + j;
     const bool act = ss < S && l < K;
     const int share = kRho64Stage / S, stage = share * S;
     const int4 mv = act ? m[l] : make_int4(0, 0, 0, 0);
     const float mfx = (float)mv.x, mfy = (float)mv.y, mfz = (float)mv.z;
+    const FixScale scx = fs(ks->sc64[0]), scy = fs(ks->sc64[1]), scz = fs(ks->sc64[2]);
+    // r / l is below 2^(exponent field - 958 + sc.e): finite up to this field
+    const int far = min(1982 - max(max(scx.e, scy.e), scz.e), 0x7fe);
     const bool wide = CHECK && __any_sync(0xffffffffu, phase_is_wide(mv.x, mv.y, mv.z));
     const TrigLow* sw = reinterpret_cast<const TrigLow*>(st + kTrigN);
-    const FixScale scx = fs(ks->sc64[0]), scy = fs(ks->sc64[1]), scz = fs(ks->sc64[2]);
     __int128 re = 0, im = 0;
     for (int64_t base = start; base < end; base += stage) {
         __syncthreads();  // every thread is done with the previous tile
@@ -158,7 +176,11 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
             const unsigned long long by = (unsigned long long)__double_as_longlong(pos[3 * i + 1]);
             const unsigned long long bz = (unsigned long long)__double_as_longlong(pos[3 * i + 2]);
             const unsigned long long bq = (unsigned long long)__double_as_longlong(q[i]);
-            if (nonfinite_bits(bx) || nonfinite_bits(by) || nonfinite_bits(bz)) atomicOr(status, kStatusNonFinite);
+            const int ex = (int)(bx >> 52) & 0x7ff, ey = (int)(by >> 52) & 0x7ff, ez = (int)(bz >> 52) & 0x7ff;
+            if (max(max(ex, ey), ez) > far && coord_bad(ks, bx, by, bz)) {
+                atomicOr(status, kStatusNonFinite);
+                s_bad = 1;
+            }
             const Frac x = frac_of(fixed_frac64(bx, scx)), y = frac_of(fixed_frac64(by, scy)),
                        z = frac_of(fixed_frac64(bz, scz));
             const unsigned long long a = fix_magnitude(bq, eb) + (1ull << 27);
@@ -234,7 +256,10 @@ k_rho_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_t 
     }
     if (act && ss == 0) {
         const int e = eb - 1023 + 1 - 85;  // units of 2^-30 2^-55 of 2^(eb - 1023 + 1)
-        partials[(size_t)l * nchunks + c] = make_double2(int128_to_double(re, e), int128_to_double(im, e));
+        const double nan = __longlong_as_double(0x7ff8000000000000ll);
+        // an input that is not finite shows in every output, beside the latched status
+        partials[(size_t)l * nchunks + c] =
+            s_bad ? make_double2(nan, nan) : make_double2(int128_to_double(re, e), int128_to_double(im, e));
     }
     if (kt == 0 && tid == 0) partials[(size_t)K * nchunks + c] = make_double2(q2, 0.0);
 }
@@ -282,13 +307,16 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
     for (int a = 1; a < 7; ++a) t[a] = e * c[a];
     t[7] = 0.0;
     rho[l] = make_double2(re, im);
-    if (!isfinite(re) || !isfinite(im)) atomicOr(status, kStatusNonFinite);
     unsigned long long phi = 0ull;
     double R = 0.0, h2 = rho2;
     if (((uint32_t)__double2hiint(rho2) >> 20) - 93u > 1860u) {
         // a square below 2^-930, above 2^930 or not finite: the forces are linear in rho, whose size is within FP64's
         const double big = fmax(fabs(re), fabs(im));
-        if (big > 0.0 && big < 1.7e308) {
+        if (!isfinite(re) || !isfinite(im)) {
+            atomicOr(status, kStatusNonFinite);
+            c[7] = re - re + (im - im);  // NaN
+            h2 = 0.0;
+        } else if (big > 0.0) {
             const int e = ilogb(big);
             re = ldexp(re, -e);
             im = ldexp(im, -e);
@@ -316,6 +344,8 @@ k_reduce_f64(const double2* __restrict__ partials, int nchunks, int K, const int
         const double d = fma(ci, co, -(cr * s)) * 2734261102.3059327;
         phi += (unsigned long long)__double2ll_rn(d);
         if (c[7] < 0.0) phi += 1ull << 63;  // a negative weight is half a revolution: R enters the force pass as a magnitude
+    } else {
+        R = c[7] * 0.0;  // NaN for a rho, a weight or a 1 / |k|^2 that is not finite
     }
     coef[l] = make_double2(__longlong_as_double((long long)(0ull - phi)), R);
 }
@@ -483,7 +513,8 @@ k_force_f64(const double* __restrict__ pos, const double* __restrict__ q, int64_
             }
             // units of 2^-30 (sine) times 2^30 (mul_fix's) over 2^sh
             if (sl == 0 && i < b1) {
-                const double u = ldexp(1.0, -sh);
+                // (an R that is not finite: no force is)
+                const double u = s_e == 0x7ff ? __longlong_as_double(0x7ff8000000000000ll) : ldexp(1.0, -sh);
                 fx += u * (double)(long long)ax;
                 fy += u * (double)(long long)ay;
                 fz += u * (double)(long long)az;

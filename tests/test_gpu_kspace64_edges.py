@@ -127,3 +127,28 @@ def test_rho_whose_square_leaves_fp64(e):
     G, _, _, _, _ = _weighted(pos, np.ldexp(q, e), m, np.ldexp(w, max(-1000, min(1000, -2 * e + 100))))
     back = 100 if abs(2 * e - 100) <= 1000 else 2 * e + (1000 if e < 0 else -1000)
     assert rel_max_force(np.ldexp(G, -back), F) <= 1e-13
+
+
+@pytest.mark.parametrize("N,K", [(700, 600), (40000, 20), (70000, 8)])
+@pytest.mark.parametrize("what", ["position", "infinite position", "charge", "infinite charge", "far position", "zero row",
+                                  "weight"])
+def test_non_finite_inputs_show(what, N, K):
+    """One input that is not finite (or whose r / l is not): no force, energy or virial is, and the status tells.  A
+    frequency of zero or a weight of NaN leaves rho alone."""
+    rng = np.random.default_rng(1)
+    box = np.array([0.4, 0.5, 0.3])
+    pos, q = rng.uniform(0, 1, (N, 3)) * box, np.where(np.arange(N) % 2, 1.0, -1.0)
+    m, w = rng.integers(1, 12, (K, 3)), rng.uniform(0.5, 1.0, K)
+    i, l = int(rng.integers(N)), int(rng.integers(K))
+    if what.endswith("position"):
+        pos[i, 1] = {"position": np.nan, "infinite position": np.inf, "far position": 1.2e308}[what]
+    elif what.endswith("charge"):
+        q[i] = np.nan if what == "charge" else np.inf
+    elif what == "weight":
+        w[l] = np.nan
+    else:
+        m[l] = 0
+    F, W, E, rho, status = _weighted(pos, q, m, w, box=box, alpha=400.0)
+    assert status == rbe.RBE_ENONFINITE
+    assert not np.isfinite(F).any() and not np.isfinite(E[0]) and not np.isfinite(W).any()
+    assert np.isfinite(rho).all() if what in ("zero row", "weight") else not np.isfinite(rho).any()
