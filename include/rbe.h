@@ -369,7 +369,9 @@ rbe_status rbe_npt_init(rbe_ctx ctx, rbe_system* sys, uint64_t batch);
  * advances by nsteps.  The context's box is not used: each step rebuilds the sampling tables
  * from the device box in sys->cell.  The step index also lives on the device (cell[11], as
  * 64-bit integer bits, set by rbe_npt_init and advanced by every step), so the launches of
- * one call may be captured once in a CUDA graph and replayed for later steps. */
+ * one call may be captured once in a CUDA graph and replayed for later steps (on the FP64 path a
+ * captured set of alpha, rc and Lennard-Jones parameters keeps 128 KB of tables until the context
+ * is destroyed; results do not depend on the sets that a context has seen). */
 rbe_status rbe_npt_step(rbe_ctx ctx, rbe_system* sys, int32_t nsteps);
 
 /* ---------------------------------------------------------------------------------

@@ -124,7 +124,7 @@ static void free_npt(NptBuffers& b)
 {
     cudaFree(b.Fk); cudaFree(b.Fr); cudaFree(b.WEk); cudaFree(b.coef); cudaFree(b.cid); cudaFree(b.fill);
     cudaFree(b.sorted); cudaFree(b.spos32); cudaFree(b.spos64); cudaFree(b.mprop);
-    for (void* t : b.pair_tab) cudaFree(t);
+    for (const auto& t : b.pair_tabs) cudaFree(t.tab);
     cudaFree(b.cellc); cudaFree(b.cnt);
     cudaFree(b.nbr); cudaFree(b.nnb); cudaFree(b.sref); cudaFree(b.nls); cudaFree(b.start); cudaFree(b.cursor); cudaFree(b.partials);
     cudaFree(b.counter);

@@ -4,6 +4,7 @@
 
 #include <cstdint>
 #include <string>
+#include <vector>
 
 #include <cuda_runtime.h>
 
@@ -75,12 +76,17 @@ struct NptBuffers {
     int* sorted = nullptr;         // N particle indices grouped by cell, by index within a cell
     float4* spos32 = nullptr;      // N packed FP32 positions+charge in sorted order
     double4_32a* spos64 = nullptr; // N packed FP64 positions+charge (FP64 path)
-    // FP64 path: the pair terms' tables (rbe_pair64.cuh) and the parameters each was built for; a table is
-    // never rewritten (a captured step may hold it), so a context keeps a few and no more
+    // FP64 path: the pair terms' tables (rbe_pair64.cuh), each with the parameters it was built for.  At most kPairTabs
+    // that no captured step holds; the least recently used of them is rewritten, in the stream's order, for others
     static constexpr int kPairTabs = 8;
-    void* pair_tab[kPairTabs] = {};
-    double pair_key[kPairTabs][5] = {};
-    int pair_tabs = 0;
+    struct PairTab {
+        void* tab;
+        double key[5];
+        uint64_t used;  // time of the last use
+        bool held;      // a captured step has the pointer: never rewritten (npt_release_tables)
+    };
+    std::vector<PairTab> pair_tabs;
+    uint64_t pair_clock = 0;
     double2* mprop = nullptr;      // N (1/m, sqrt(m)), set by rbe_npt_init
     void* cellc = nullptr;         // cell-list constants of the current box (rbe_npt.cu)
     int* nbr = nullptr;            // neighbour list: slots of the neighbours of slot u at [u * nbr_cap, ...)
@@ -265,6 +271,7 @@ int pair_blocks(rbe_ctx ctx, int64_t N, bool fp64);
 int pair_blocks64(rbe_ctx ctx, int64_t N);
 struct Pair64Const;
 rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out, bool* built);
+void npt_release_tables(rbe_ctx ctx);  // the captured steps of this context are gone
 rbe_status launch_cell_list(rbe_ctx ctx, int64_t N, const double* pos, const double* q, void* nls, bool fp64, int unit, bool zeroed);
 // launch_cell_list: FP64 positions packed as they are
 constexpr int kPairNoUnit = -(1 << 20);

@@ -24,6 +24,7 @@
 #include <climits>
 #include <cmath>
 #include <cstring>
+#include <new>
 #include <string>
 #include <type_traits>
 
@@ -1360,15 +1361,89 @@ __global__ void k_pair_table(PairWord* __restrict__ t, int top, double alpha, do
     if (seg < kPairSegs) pair_segment(t, seg, top, alpha, s2, e24, e4);
 }
 
-// The FP64 pair kernels' constants, with the table of these parameters: found among the context's, or
-// built by one small launch.  Without a table (direct evaluation, the same results to rounding) where the
-// polynomials' coefficients would leave the float range (pair_lj_fits; pair_segs for the pairs far out), in a
-// capture that meets the parameters for the first time, and past kPairTabs sets of parameters.  built: the table's launch is the stream's last, and the
-// pair kernel, which loads the table before pdl_wait(), must not be launched programmatically.
+void npt_release_tables(rbe_ctx ctx)
+{
+    for (auto& t : ctx->npt.pair_tabs) t.held = false;
+}
+
+// The table of these parameters among the context's, built by one small launch if there is none: on the context's
+// stream, or, while that is being captured, beside the capture, on a stream of its own and complete on return.  built:
+// the launch is the stream's last, and the pair kernel, which loads the table before pdl_wait(), must not be launched
+// programmatically.
+static rbe_status pair_table(rbe_ctx ctx, int top, const PairConst& c, const PairWord** out, bool* built)
+{
+    NptBuffers& b = ctx->npt;
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    cudaError_t e = cudaStreamIsCapturing(ctx->stream, &cap);
+    if (e != cudaSuccess) cudaGetLastError();  // the legacy stream beside another stream's capture: treated as one
+    const bool capture = e != cudaSuccess || cap != cudaStreamCaptureStatusNone;
+    const double key[5] = {ctx->alpha, c.rc2, c.s2, c.e24, c.e4};
+    NptBuffers::PairTab* t = nullptr;
+    size_t oldest = 0;
+    int free_tabs = 0;
+    for (size_t k = 0; k < b.pair_tabs.size(); ++k) {
+        NptBuffers::PairTab& x = b.pair_tabs[k];
+        if (std::memcmp(key, x.key, sizeof(key)) == 0) t = &x;
+        if (x.held) continue;
+        if (free_tabs++ == 0 || x.used < b.pair_tabs[oldest].used) oldest = k;
+    }
+    if (!t) {
+        NptBuffers::PairTab fresh{};
+        std::memcpy(fresh.key, key, sizeof(key));
+        try {
+            b.pair_tabs.reserve(b.pair_tabs.size() + 1);
+        } catch (const std::bad_alloc&) {
+            return fail(ctx, RBE_ENOMEM, "host allocation failed");
+        }
+        const auto build = [&](cudaStream_t s) {
+            k_pair_table<<<kPairSegs / 32, 32, 0, s>>>(static_cast<PairWord*>(fresh.tab), top, ctx->alpha, c.s2, c.e24, c.e4);
+            return cudaGetLastError();
+        };
+        if (capture) {
+            cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+            cudaStream_t s = nullptr;
+            e = cudaThreadExchangeStreamCaptureMode(&mode);
+            if (e != cudaSuccess) return npt_fail(ctx, e, "capture mode");
+            e = cudaMalloc(&fresh.tab, kPairTabBytes);
+            if (e == cudaSuccess) e = cudaStreamCreateWithFlags(&s, cudaStreamNonBlocking);
+            if (e == cudaSuccess) e = build(s);
+            if (e == cudaSuccess) e = cudaStreamSynchronize(s);
+            if (s) cudaStreamDestroy(s);
+            if (e != cudaSuccess && fresh.tab) cudaFree(fresh.tab);
+            cudaThreadExchangeStreamCaptureMode(&mode);
+            if (e != cudaSuccess) return npt_fail(ctx, e, "pair tables beside a capture");
+            b.pair_tabs.push_back(fresh);
+            t = &b.pair_tabs.back();
+        } else {
+            if (free_tabs < NptBuffers::kPairTabs) {
+                e = ctx_alloc(ctx, &fresh.tab, kPairTabBytes);
+                if (e != cudaSuccess) return npt_fail(ctx, e, "cudaMalloc(pair tables)");
+                b.pair_tabs.push_back(fresh);
+                t = &b.pair_tabs.back();
+            } else {
+                t = &b.pair_tabs[oldest];
+                fresh.tab = t->tab;
+                *t = fresh;
+            }
+            if ((e = build(ctx->stream)) != cudaSuccess) {
+                t->key[0] = -1.0;  // no parameters' table
+                return npt_fail(ctx, e, "k_pair_table");
+            }
+            *built = true;
+        }
+    }
+    t->used = ++b.pair_clock;
+    t->held = t->held || capture;
+    *out = static_cast<const PairWord*>(t->tab);
+    return RBE_OK;
+}
+
+// The FP64 pair kernels' constants, with the table of these parameters; without one (direct evaluation, the same
+// results to rounding) where the polynomials' coefficients would leave the float range (pair_lj_fits; pair_segs for
+// the pairs far out): the parameters alone decide.
 rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out, bool* built)
 {
     *built = false;
-    NptBuffers& b = ctx->npt;
     const PairConst c = make_pair_const(prm.rc, ctx->alpha, prm.qqr2e, prm.lj_sigma, prm.lj_eps);
     Pair64Const p{};
     p.lj = c.lj;
@@ -1385,28 +1460,8 @@ rbe_status pair64_const(rbe_ctx ctx, const rbe_npt_params& prm, Pair64Const* out
     p.scale = std::ldexp(1.0, kPairDrop - p.unit.s);
     p.segs = rc_ok ? (unsigned)pair_segs(ctx->alpha, top) : 0u;
     if (rc_ok && (!c.lj || pair_lj_fits(c.s2, c.e24, top))) {
-        const double key[5] = {ctx->alpha, c.rc2, c.s2, c.e24, c.e4};
-        int t = 0;
-        while (t < b.pair_tabs && std::memcmp(key, b.pair_key[t], sizeof(key)) != 0) ++t;
-        if (t == b.pair_tabs && t < NptBuffers::kPairTabs) {
-            cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
-            if (cudaStreamIsCapturing(ctx->stream, &cap) != cudaSuccess) {
-                cudaGetLastError();
-                cap = cudaStreamCaptureStatusActive;
-            }
-            if (cap == cudaStreamCaptureStatusNone) {
-                cudaError_t e = ctx_alloc(ctx, &b.pair_tab[t], kPairTabBytes);
-                if (e != cudaSuccess) return npt_fail(ctx, e, "cudaMalloc(pair tables)");
-                k_pair_table<<<kPairSegs / 32, 32, 0, ctx->stream>>>(static_cast<PairWord*>(b.pair_tab[t]), top, ctx->alpha,
-                                                                    c.s2, c.e24, c.e4);
-                rbe_status st = npt_check(ctx, "k_pair_table");
-                if (st != RBE_OK) return st;
-                std::memcpy(b.pair_key[t], key, sizeof(key));
-                ++b.pair_tabs;
-                *built = true;
-            }
-        }
-        if (t < b.pair_tabs) p.tab = static_cast<const PairWord*>(b.pair_tab[t]);
+        const rbe_status st = pair_table(ctx, top, c, &p.tab, built);
+        if (st != RBE_OK) return st;
     }
     *out = p;
     return RBE_OK;

@@ -263,13 +263,14 @@ static rbe_status admit(rbe_server_s* s, Slot& sl, int64_t id)
         (e = cudaMemcpyAsync(sl.mass, rq.m.data(), sizeof(double) * N, cudaMemcpyHostToDevice, sl.stream)) != cudaSuccess ||
         (e = cudaMemcpyAsync(sl.cell, cell, sizeof(cell), cudaMemcpyHostToDevice, sl.stream)) != cudaSuccess)
         return sfail(s, RBE_ECUDA, std::string("upload: ") + cudaGetErrorString(e));
-    sl.sys = rbe_system{N, sl.pos, sl.mom, sl.force, sl.charge, sl.mass, sl.cell, 0, rq.r.params};
-    if ((st = rbe_npt_init(sl.ctx, &sl.sys, 0)) != RBE_OK) return sfail(s, st, rbe_last_error(sl.ctx));
     if (sl.graph) {
         cudaGraphExecDestroy(sl.graph);
         sl.graph = nullptr;
     }
     sl.graph_steps = 0;
+    npt_release_tables(sl.ctx);
+    sl.sys = rbe_system{N, sl.pos, sl.mom, sl.force, sl.charge, sl.mass, sl.cell, 0, rq.r.params};
+    if ((st = rbe_npt_init(sl.ctx, &sl.sys, 0)) != RBE_OK) return sfail(s, st, rbe_last_error(sl.ctx));
     if (s->cfg.use_graphs && !s->cfg.batched && rq.r.nsteps / s->cfg.chunk_steps >= kGraphChunks) {
         // one chunk of launches, captured; the device step index makes it replayable
         cudaGraph_t g = nullptr;

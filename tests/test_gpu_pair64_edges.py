@@ -93,3 +93,67 @@ def test_close_pairs(gap, skin):
     assert np.max(np.linalg.norm(F - F0, axis=1) / np.linalg.norm(F0, axis=1)) <= 1e-13
     assert abs(cell[4] - np.trace(W0)) <= 1e-13 * 1389.35 * len(a) * 1.44 / gap
     assert abs(cell[8] - Ec) <= 1e-13 * 1389.35 * len(a) * 1.44 / gap
+
+
+def _replica(pos, q, L, eps, rc=5.0):
+    return rbe.NptReplica(pos, np.zeros_like(pos), q, np.full(len(q), 20.0), np.array([L, L, L]), _params(rc, 0.0, 2.0, eps),
+                          cuda_device())
+
+
+def test_results_do_not_depend_on_earlier_parameters():
+    """Twelve sets of Lennard-Jones parameters one after the other on one context, and the first and the last again: the
+    bits of a context of its own for each."""
+    L = 14.0
+    pos, q = _system(6, L, 5)
+    box = np.array([L, L, L])
+
+    def run(ctx, k):
+        rep = _replica(pos, q, L, 0.1 + 0.05 * k)
+        rep.init(ctx)
+        rep.step(ctx, 2)
+        ctx.sync()
+        return rep.state()
+
+    with rbe.Context(box, 0.2, 10, 1, rbe.RBE_FP64) as shared:
+        for k in [*range(12), 0, 11, 3]:
+            with rbe.Context(box, 0.2, 10, 1, rbe.RBE_FP64) as own:
+                for a, b in zip(run(shared, k), run(own, k)):
+                    assert np.array_equal(a, b), k
+
+
+def test_captured_steps_keep_their_tables():
+    """A step captured with parameters that its context meets first in the capture, replayed after twenty other sets
+    have been through the context: the bits of the same step launched directly."""
+    import torch
+    L = 14.0
+    pos, q = _system(6, L, 5)
+    box = np.array([L, L, L])
+    with rbe.Context(box, 0.2, 10, 1, rbe.RBE_FP64) as ctx:
+        rep = _replica(pos, q, L, 0.1)
+        rep.init(ctx)
+        rep.sys.params.lj_eps = 0.33
+        rep.step(ctx, 3)
+        ctx.sync()
+        want = rep.state()
+    stream = torch.cuda.Stream()
+    with rbe.Context(box, 0.2, 10, 1, rbe.RBE_FP64) as ctx:
+        ctx.set_stream(stream.cuda_stream)
+        rep = _replica(pos, q, L, 0.1)
+        torch.cuda.synchronize()
+        rep.init(ctx)
+        rep.sys.params.lj_eps = 0.33
+        ctx.sync()
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g, stream=stream, capture_error_mode="thread_local"):
+            rep.step(ctx, 1)
+        for k in range(20):
+            other = _replica(pos, q, L, 0.5 + 0.01 * k)
+            torch.cuda.synchronize()
+            other.init(ctx)
+            ctx.sync()
+        with torch.cuda.stream(stream):
+            for _ in range(3):
+                g.replay()
+        ctx.sync()
+        for a, b in zip(want, rep.state()):
+            assert np.array_equal(a, b)
