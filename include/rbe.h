@@ -587,7 +587,8 @@ const char* rbe_batch_last_error(rbe_batch b);
  * admitted when a slot is free and its device memory fits the budget, and its state stays
  * resident in HBM until it finishes.  Each resident replica runs on its own non-blocking
  * stream and context, in chunks of chunk_steps NPT steps (rbe_npt_step), captured once per
- * replica as a CUDA graph when use_graphs != 0; chunks of different replicas run
+ * replica as a CUDA graph when use_graphs != 0 and the request has at least five whole chunks (for fewer
+ * the capture costs more than it saves); chunks of different replicas run
  * concurrently, and requests are admitted while others run.  A replica's result does not
  * depend on what else is resident (no shared state; fixed-order reductions). */
 typedef struct rbe_server_s* rbe_server;
@@ -604,7 +605,9 @@ typedef struct {
                             neighbour list (cap = 2 x the expected neighbours within rc + skin, + 64,
                             rounded up to 32), plus 128 (P + ptilde) + 16 reuse (P + ptilde) for the
                             frequency buffers (the reuse term when reuse > 1) */
-    int32_t use_graphs;  /* 1: replay a captured graph per chunk; 0: launch the steps directly */
+    int32_t use_graphs;  /* 1: replay a captured graph per chunk (requests of five whole chunks and more;
+                            the same launches directly for shorter ones, and the same results);
+                            0: launch the steps directly */
     int32_t batched;     /* 0: every replica runs its own chunks (its own stream and graph).  1: the
                             resident replicas advance in lockstep chunks; each step's k-space of all
                             of them is one persistent batched launch (rbe_batch, the tiles autotuned
@@ -679,6 +682,9 @@ rbe_status rbe_server_result(rbe_server s, int64_t id, double* pos, double* mom,
  * retirement. */
 rbe_status rbe_server_stats(rbe_server s, double* chunk_latency, int64_t capacity, int64_t* n_chunks,
                             int64_t* steps_done, double* span_seconds);
+
+/* Chunks so far that were replayed from a captured graph, batched = 0 (test support). */
+rbe_status rbe_server_graph_replays(rbe_server s, int64_t* n);
 
 /* Message for the server's last failure. */
 const char* rbe_server_last_error(rbe_server s);

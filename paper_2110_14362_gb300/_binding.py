@@ -180,6 +180,7 @@ SIGNATURES = [
                                                 ctypes.POINTER(ctypes.c_int)]),
     ("rbe_server_stats", ctypes.c_int, [_vp, _dp, ctypes.c_int64, ctypes.POINTER(ctypes.c_int64),
                                         ctypes.POINTER(ctypes.c_int64), _dp]),
+    ("rbe_server_graph_replays", ctypes.c_int, [_vp, ctypes.POINTER(ctypes.c_int64)]),
     ("rbe_server_last_error", ctypes.c_char_p, [_vp]),
     ("rbe_status_string", ctypes.c_char_p, [ctypes.c_int]),
     ("rbe_last_error", ctypes.c_char_p, [_vp]),
@@ -674,6 +675,11 @@ class Server:
         load().rbe_server_stats(self.h, lat.ctypes.data_as(_dp), n.value, ctypes.byref(n), ctypes.byref(steps),
                                 ctypes.byref(span))
         return lat[:n.value], steps.value, span.value
+
+    def graph_replays(self) -> int:
+        n = ctypes.c_int64()
+        self._check(load().rbe_server_graph_replays(self.h, ctypes.byref(n)))
+        return n.value
 
 
 def rbe_version() -> int:

@@ -92,6 +92,7 @@ struct rbe_server_s {
     int64_t mem_used = 0;
     std::vector<double> latencies;
     int64_t steps_done = 0;
+    int64_t graph_replays = 0;          // chunks launched from a captured graph
     int64_t n_done = 0;
     Clock::time_point t0;
     double t_first_admit = -1.0, t_last_done = 0.0;
@@ -311,6 +312,7 @@ static rbe_status launch_chunk(rbe_server_s* s, Slot& sl)
     if (sl.graph && n == sl.graph_steps) {
         cudaError_t e = cudaGraphLaunch(sl.graph, sl.stream);
         if (e != cudaSuccess) return sfail(s, RBE_ECUDA, std::string("cudaGraphLaunch: ") + cudaGetErrorString(e));
+        ++s->graph_replays;
         sl.sys.step += (uint64_t)n;
     } else {
         st = rbe_npt_step(sl.ctx, &sl.sys, n);
@@ -824,6 +826,13 @@ rbe_status rbe_server_result(rbe_server s, int64_t id, double* pos, double* mom,
     if (pos) std::memcpy(pos, rq.out_pos.data(), sizeof(double) * 3 * N);
     if (mom) std::memcpy(mom, rq.out_mom.data(), sizeof(double) * 3 * N);
     if (cell) std::memcpy(cell, rq.out_cell.data(), sizeof(double) * RBE_CELL_DOUBLES);
+    return RBE_OK;
+}
+
+rbe_status rbe_server_graph_replays(rbe_server s, int64_t* n)
+{
+    if (!s || !n) return RBE_EINVAL;
+    *n = s->graph_replays;
     return RBE_OK;
 }
 
