@@ -384,15 +384,16 @@ k_water_drift(int64_t Nmol, double* __restrict__ pos, double* __restrict__ mom, 
 // their rounding; the hits (slot, image code) go to a per-warp buffer in ballot order and are evaluated 32
 // at a time, one per lane, from the fixed-point positions with the exact cutoff; the pair terms come
 // from the tables of rbe_pair64.cuh, the sums are FP64 (k_pair64 says more; in a box with an edge shorter than
-// 2 rc + 0.1 % the image is taken per pair).  Half of it is the search: cells out of reach are left out
+// 2 rc + 0.1 %, or than `few`, five bonds, where sites on opposite sides can be 1.5 edges apart, the image is taken
+// per pair).  Half of it is the search: cells out of reach are left out
 // (195 -> 164 us at 9000 sites), 24 warps a block (164 -> 150 us).  A hit of the
 // same molecule (site index / 3) is skipped; LJ acts between oxygens (site index divisible by 3).
 // Each pair is
 // visited from both ends: energies and the virial take half.  Per-block partials {W_r, E_coul,
 // E_lj} at slots 1..3 (the isotropic layout).  A box beyond the cell arrays leaves F_r = 0.
 __global__ void __launch_bounds__(kWaterPairWarps * 32, 1)
-k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, double rc, const int* __restrict__ cid,
-             const int* __restrict__ cnt, const int* __restrict__ start, const int* __restrict__ sorted,
+k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc, double rc, double few,
+             const int* __restrict__ cid, const int* __restrict__ cnt, const int* __restrict__ start, const int* __restrict__ sorted,
              const float4* __restrict__ spos32, const double4_32a* __restrict__ spos64, double* __restrict__ Fr,
              double* __restrict__ partials)
 {
@@ -414,7 +415,8 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc,
         const double L[3] = {cc->L[0], cc->L[1], cc->L[2]};
         const float Lf[3] = {cc->Lf[0], cc->Lf[1], cc->Lf[2]}, invf[3] = {cc->invLf[0], cc->invLf[1], cc->invLf[2]};
         const PairBox box = pair_box(L, rc, pc.unit.s);
-        const bool exact = 2.0 * rc > 0.999 * fmin(L[0], fmin(L[1], L[2]));
+        const double lmin = fmin(L[0], fmin(L[1], L[2]));
+        const bool exact = 2.0 * rc > 0.999 * lmin || lmin < few;
         const bool mi[3] = {true, true, true};  // the segments carry no image: it is taken per pair
         const float pass = cc->pass64;
         const int64_t per = (N + gridDim.x - 1) / gridDim.x;
@@ -463,7 +465,7 @@ k_water_pair(int64_t N, const CellConsts* __restrict__ cc, const Pair64Const pc,
                         const int sl = s0 + lane;
                         const float4 o = spos32[sl < ghi ? sl : glo];
                         float dx = o.x - me32.x, dy = o.y - me32.y, dz = o.z - me32.z;
-                        // sites lie within a bond of [0, l), l >= 2 rc: the image is -1, 0 or 1
+                        // sites lie within a bond of [0, l): in boxes of more than a few bonds the image is -1, 0 or 1
                         // (rounded by adding 1.5 2^23: rintf runs on a quarter-rate pipe)
                         const float kx = (dx * invf[0] + 12582912.f) - 12582912.f, ky = (dy * invf[1] + 12582912.f) - 12582912.f,
                                     kz = (dz * invf[2] + 12582912.f) - 12582912.f;
@@ -688,7 +690,7 @@ static rbe_status water_validate(rbe_ctx ctx, const rbe_system* sys, const rbe_w
 
 // Forces, molecular virial and energies at the current state (batch = the device step index; the k-space
 // tables have been launched on `fork`), then the finishing kernel.
-static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, int do_kick)
+static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, const rbe_water_params& wp, KspaceFork& fork, int do_kick)
 {
     NptBuffers& b = ctx->npt;
     const rbe_npt_params& prm = sys->params;
@@ -707,8 +709,8 @@ static rbe_status water_forces(rbe_ctx ctx, rbe_system* sys, KspaceFork& fork, i
         cudaError_t e = smem_opt_in(ctx, kSmemWaterPair, k_water_pair, kPairTabBytes);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "shared memory of k_water_pair");
         e = launch_ordered(!built && ctx->early, k_water_pair, dim3(nbp), dim3(kWaterPairWarps * 32), kPairTabBytes, s, N,
-                           static_cast<const CellConsts*>(b.cellc), pc, prm.rc, b.cid, b.cnt, b.start, b.sorted, b.spos32,
-                           b.spos64, b.Fr, b.partials);
+                           static_cast<const CellConsts*>(b.cellc), pc, prm.rc, 5.0 * wp.d_OH, b.cid, b.cnt, b.start,
+                           b.sorted, b.spos32, b.spos64, b.Fr, b.partials);
         if (e != cudaSuccess) return cuda_fail(ctx, e, "k_water_pair");
     }
     if ((st = fork.join()) != RBE_OK) return st;
@@ -747,7 +749,7 @@ rbe_status water_init(rbe_ctx ctx, rbe_system* sys, const rbe_water_params* wp, 
         Nmol, sys->pos, sys->cell);
     if ((st = water_check(ctx, "k_water_whole")) != RBE_OK) return st;
     KspaceFork fork(ctx, sys);
-    if ((st = fork.tables(sys)) != RBE_OK || (st = water_forces(ctx, sys, fork, 0)) != RBE_OK) return st;
+    if ((st = fork.tables(sys)) != RBE_OK || (st = water_forces(ctx, sys, *wp, fork, 0)) != RBE_OK) return st;
     ctx->water_ready_N = sys->N;
     return launch_npt_set_step(ctx, sys->cell, sys->step);
 }
@@ -767,7 +769,7 @@ rbe_status water_run(rbe_ctx ctx, rbe_system* sys, const rbe_water_params* wp, i
                                                               reinterpret_cast<const NptCoef*>(ctx->npt.coef),
                                                               ctx->seed, sys->cell, *wp, sys->params.dt, ctx->d.status);
         if ((st = water_check(ctx, "k_water_drift")) != RBE_OK) return st;
-        if ((st = water_forces(ctx, sys, fork, 1)) != RBE_OK) return st;
+        if ((st = water_forces(ctx, sys, *wp, fork, 1)) != RBE_OK) return st;
         sys->step += 1;
     }
     return RBE_OK;

@@ -157,3 +157,21 @@ def test_captured_steps_keep_their_tables():
         ctx.sync()
         for a, b in zip(want, rep.state()):
             assert np.array_equal(a, b)
+
+
+def test_water_in_a_box_of_a_few_bonds():
+    """Two molecules in a box of 3.6 bonds, hydrogens of both a bond outside it on opposite sides: the separation of their
+    storage is 1.55 edges, and their nearest images are within rc."""
+    L, rc, alpha = 3.6, 1.79, 1.0
+    pos = np.array([[3.55, 0.5, 0.6], [4.55, 0.5, 0.6], [3.3, 1.4, 0.9], [0.03, 1.0, 0.8], [-0.97, 1.0, 0.8], [0.4, 1.9, 1.1]])
+    q, m = np.tile([-0.8476, 0.4238, 0.4238], 2), np.tile([15.9994, 1.008, 1.008], 2)
+    box = np.array([L, L, L])
+    with rbe.Context(box, alpha, 10, 1, rbe.RBE_FP64) as ctx:
+        rep = rbe.WaterReplica(pos, np.zeros_like(pos), q, m, box, _params(rc, 0.0, 1.2, 0.65), cuda_device())
+        rep.init(ctx)
+        ctx.sync()
+        _, _, F, _, cell = rep.state()
+    F0, _, *E = oracle.water_real(pos, q, box, alpha, rc, 1389.35, 1.2, 0.65)
+    assert np.abs(F - F0).max() <= 1e-11 * np.abs(F0).max()
+    for got, ref in ((cell[8], E[0]), (cell[9], E[1]), (cell[rbe.CELL_EXCL], E[2])):
+        assert abs(got - ref) <= 1e-11 * (abs(ref) + 1389.35 * np.sum(q * q) / L), (got, ref)
