@@ -218,9 +218,11 @@ static rbe_status ensure_slot_buffers(rbe_server_s* s, Slot& sl, int64_t N)
 }
 
 // Slots up to which a step's launches start early behind one another: blocks that are resident and wait take room
-// from other replicas' kernels (12 requests on 8 slots: 14.4-14.9 ms early, 15.1 in order; 256 requests on 64 slots:
-// 20.0-20.9 thousand replica-steps/s early, 21.4-21.8 in order).
-constexpr int kEarlySlots = 8;
+// from other replicas' kernels.  Thousand replica-steps/s early and in order, four requests a slot of 1e3 to 1e5 charges
+// and 100 steps (replayed chunks): 2 slots 17.8 and 17.1, 4: 16.9 and 16.5, 8: 21.8 and 21.5, 12: 25.8 and 25.3, 16: 24.7
+// and 24.6, 24: 22.2 and 22.6, 32: 22.2 and 23.3, 48: 21.8 and 23.3 (20 steps, launched directly: early 3 to 8 % faster at
+// each of them).  By configured slots, not by resident replicas: a replayed chunk keeps the launches it was captured with.
+constexpr int kEarlySlots = 16;
 
 // Chunks of a request from which its graph pays: capturing and instantiating one costs the host what launching
 // about four chunks directly does (12 requests on 8 slots, graphs against direct launches: 1 chunk 11.9 and 8.2 ms,

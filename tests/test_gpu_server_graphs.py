@@ -1,6 +1,6 @@
 """Requests long enough for their chunks to be replayed from a captured graph: the same bits as launched directly and as
 the NPT step called on its own, on servers with one slot (the k-space on a side stream inside the capture), several,
-and more than eight (launches in order), from a cell search and a neighbour list."""
+and more than sixteen (launches in order), from a cell search and a neighbour list."""
 import time
 
 import numpy as np
@@ -48,7 +48,7 @@ def _serve(precision, slots, skin, use_graphs):
 
 
 @pytest.mark.parametrize("skin", [0.0, 0.4])
-@pytest.mark.parametrize("slots", [1, 4, 9])
+@pytest.mark.parametrize("slots", [1, 4, 9, 17])
 @pytest.mark.parametrize("precision", [rbe.RBE_FP64, rbe.RBE_FP32_PHASE])
 def test_replayed_chunks(precision, slots, skin):
     dev = cuda_device()
