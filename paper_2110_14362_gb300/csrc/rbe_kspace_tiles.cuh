@@ -50,7 +50,8 @@ __device__ __forceinline__ FixScale fs(const FixScaleH& h) { return FixScale{h.q
 // library's own exponential, W_j = rint(w_{|j-M|} 2^sh) with sh = 62 - bitlength(2M+1),
 // C_j = W_0 + ... + W_j (exact integers: any summation order gives the same bits, so the
 // prefix sum runs in parallel), H = C_2M 2^-sh, S = H_x H_y H_z - 1.  scale64: also the FP64 path's scale, a
-// serial chain of about 4 us that the FP32-phase path leaves out (64 systems in one batch: 233 and 229 us).
+// serial chain.  The batch leaves it out at compile time: its fused kernel took 233 us for 64 systems with it and 229
+// without, although no table was built in those calls (the kernel's code, not the chain's time).
 __device__ __forceinline__ int bitlength(unsigned x) { return 32 - __clz(x); }
 
 __device__ __forceinline__ void tables_body(double bx, double by, double bz, const double* __restrict__ box_dev,

@@ -1012,11 +1012,12 @@ k_pair(int64_t N, const CellConsts* __restrict__ cc, const PairConst pc, const i
 // cutoff in fixed point, the pair terms from the tables of rbe_pair64.cuh, the sums in FP64.  One block of
 // kPair64Warps warps per SM shares the table; each block takes a contiguous run of slots.
 //
-// What bounds it: the FP64 pipe still (70 % busy: 13 instructions of about 76 clocks of a scheduler per 32 pairs,
+// What bounds it: the FP64 pipe still (75 % busy: 13 instructions of about 76 clocks of a scheduler per 32 pairs,
 // and 8 per particle), with the float-float polynomials and the waits of four warps per scheduler beside it.
 // N = 2e4, rc = 7 A, list of 8 A: 875 us with sqrt, exp, erfc and divisions (about 115 FP64 instructions), 169 us
-// with the tables and FP64 separations (22), 125 us with fixed-point separations; 9000 water sites, rc = 10 A,
-// from the cells (k_water_pair): 1021, 261 and 150 us.  The image of a pair is taken from the search (an addition
+// with the tables and FP64 separations (22), 125 us with fixed-point separations (11), 134 us with the energies'
+// constant terms in FP64 (13; see rbe_pair64.cuh); 9000 water sites, rc = 10 A,
+// from the cells (k_water_pair): 1021, 261, 150 and 146 us.  The image of a pair is taken from the search (an addition
 // of +-l only where some lane has one) except on an axis with fewer than 3 cells, or, from a list, one whose half
 // is within 0.1 % of rc, where it is taken per pair (pair_nearest).
 template <int kMode, bool kDiag>

@@ -15,7 +15,8 @@
 //                   oxygens, nearest image per pair
 //   k_water_finish  one thread per molecule: total forces with the intramolecular exclusion,
 //                   R^p/2, the centres' 2K and the molecular virial; last block: P_ins, V^p/2
-// Everything runs in FP64 except the k-space, which follows the context's precision.
+// FP64 state and sums; the pair terms as in rbe_pair64.cuh, the constraints' 3x3 solves in FP32 on FP64 residuals
+// (w_shake); the k-space follows the context's precision.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -386,7 +387,7 @@ k_water_drift(int64_t Nmol, double* __restrict__ pos, double* __restrict__ mom, 
 // from the tables of rbe_pair64.cuh, the sums are FP64 (k_pair64 says more; in a box with an edge shorter than
 // 2 rc + 0.1 %, or than `few`, five bonds, where sites on opposite sides can be 1.5 edges apart, the image is taken
 // per pair).  Half of it is the search: cells out of reach are left out
-// (195 -> 164 us at 9000 sites), 24 warps a block (164 -> 150 us).  A hit of the
+// (195 -> 164 us at 9000 sites), 24 warps a block (164 -> 150 us; 146 with energies in FP64).  A hit of the
 // same molecule (site index / 3) is skipped; LJ acts between oxygens (site index divisible by 3).
 // Each pair is
 // visited from both ends: energies and the virial take half.  Per-block partials {W_r, E_coul,
