@@ -152,3 +152,24 @@ def test_non_finite_inputs_show(what, N, K):
     assert status == rbe.RBE_ENONFINITE
     assert not np.isfinite(F).any() and not np.isfinite(E[0]) and not np.isfinite(W).any()
     assert np.isfinite(rho).all() if what in ("zero row", "weight") else not np.isfinite(rho).any()
+
+
+@pytest.mark.parametrize("N,K", [(60, 300), (3000, 40), (40000, 20), (70000, 8)])
+def test_lists_equal_batches(N, K):
+    """A sampled batch (its |m| bounded by the tables) and the same frequencies as a list (bounded by nothing): the same
+    bits."""
+    import torch
+    dev = cuda_device()
+    rng = np.random.default_rng(N)
+    pos, q = rng.uniform(0, 1, (N, 3)) * BOX, rng.choice([-1.0, 1.0], N) * rng.uniform(0.5, 1.0, N)
+    F = torch.empty((N, 3), dtype=torch.float64, device=dev)
+    W = torch.empty(9, dtype=torch.float64, device=dev)
+    E = torch.empty(2, dtype=torch.float64, device=dev)
+    with rbe.Context(BOX, 0.4, K, 9, rbe.RBE_FP64) as ctx:
+        ctx.forces_virial(torch.as_tensor(pos).to(dev), torch.as_tensor(q).to(dev), 4, F, W, E)
+        ctx.sync()
+        rho = ctx.rho()
+        m, S = ctx.sample_k(4)
+    F1, W1, E1, rho1, _ = _weighted(pos, q, np.asarray(m), np.full(K, S / K))
+    assert np.array_equal(F.cpu().numpy(), F1) and np.array_equal(W.cpu().numpy().reshape(3, 3), W1)
+    assert np.array_equal(E.cpu().numpy(), E1) and np.array_equal(rho, rho1)
